@@ -71,7 +71,7 @@ struct lattice_batch {
     // colour 0 / 1
     unsigned *d_counters = nullptr;
     int grid_tiled_ising = 0, grid_tiled_ne = 0, grid_generic = 0, grid_wide[2] = {0, 0}, grid_potts = 0;
-    int grid_any[2] = {0, 0};     // 2D any-L, Ising / North-East
+    int grid_any[3] = {0, 0, 0};  // 2D any-L: Ising, North-East at T, North-East in c-mode
     // resident lattices
     cudaStream_t res_stream = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
@@ -173,6 +173,17 @@ struct BatchTune {
     int passes, gsteps;
 };
 
+// One colour of the 2D spin-1/2 items of kind m: Ising, North-East at
+// temperature T, North-East in c-mode.
+cudaError_t batch_2d(lattice_batch *b, const Phase &ph, const uint2 *items, int n, int counter, int colour, int m,
+                     bool aligned, cudaStream_t st)
+{
+    const int grid = std::min(b->grid_any[m], n);
+    unsigned *next = b->d_counters + counter;
+    return m == 2 ? launch_batch_ne(ph.geoms, items, n, next, colour, aligned, ph.passes, grid, st)
+                  : launch_batch_any(ph.geoms, items, n, next, colour, m == 1, aligned, ph.passes, grid, st);
+}
+
 // Queue `steps` sweep steps of one phase.
 int enqueue_steps(lattice_batch *b, const Phase &ph, int steps, cudaStream_t st)
 {
@@ -190,14 +201,12 @@ int enqueue_steps(lattice_batch *b, const Phase &ph, int steps, cudaStream_t st)
         static const int kCtrW2[3] = {6, 8, 18}, kCtrGrp[3] = {12, 14, 20};
         for (int m = 0; m < 3; ++m) {   // L % 32 == 0
             for (int colour = 0; colour < 2 && e == cudaSuccess && sh.n_w2[m] > 0; ++colour)
-                e = launch_batch_any(ph.geoms, w2, sh.n_w2[m], b->d_counters + kCtrW2[m] + colour, colour, m >= 1,
-                                     m == 2, true, ph.passes, std::min(b->grid_any[m ? 1 : 0], sh.n_w2[m]), st);
+                e = batch_2d(b, ph, w2, sh.n_w2[m], kCtrW2[m] + colour, colour, m, true, st);
             w2 += sh.n_w2[m];
         }
         for (int m = 0; m < 3; ++m) {   // other even L
             for (int colour = 0; colour < 2 && e == cudaSuccess && sh.n_grp[m] > 0; ++colour)
-                e = launch_batch_any(ph.geoms, w2, sh.n_grp[m], b->d_counters + kCtrGrp[m] + colour, colour, m >= 1,
-                                     m == 2, false, ph.passes, std::min(b->grid_any[m ? 1 : 0], sh.n_grp[m]), st);
+                e = batch_2d(b, ph, w2, sh.n_grp[m], kCtrGrp[m] + colour, colour, m, false, st);
             w2 += sh.n_grp[m];
         }
         const uint2 *wide = w2;
@@ -510,6 +519,7 @@ int lattice_batch_create(lattice_batch_t **out, void *cuda_stream)
     b->grid_potts = batch_potts_grid();
     b->grid_any[0] = batch_any_grid(false);
     b->grid_any[1] = batch_any_grid(true);
+    b->grid_any[2] = batch_ne_grid();
     *out = b;
     return LAT_OK;
 }

@@ -190,7 +190,7 @@ int ensure_series(lattice *lt, unsigned long long need)
                             lt->stream);
     if (e == cudaSuccess)
         e = launch_set_ctrl(lt->ctrl, (unsigned long long)lt->sweeps, np, base, cap, np + 4 * cap, np + 5 * cap,
-                            lt->stream);
+                            (unsigned long long)lt->unfl_base, lt->stream);
     if (e != cudaSuccess) {
         dev_free(p, lt->stream);
         return cuda_fail(e, "series grow");
@@ -257,13 +257,141 @@ int choose_kernel(const lattice *lt)
     return LAT_KERNEL_GENERIC;
 }
 
+int *band_error_word()
+{
+    static std::mutex mu;
+    static int *page = nullptr;
+    static unsigned next = 0;
+    constexpr unsigned kWords = 1024;
+    std::lock_guard<std::mutex> g(mu);
+    if (page == nullptr && cudaHostAlloc((void **)&page, kWords * sizeof(int), cudaHostAllocPortable) != cudaSuccess) {
+        (void)cudaGetLastError();
+        page = nullptr;
+        return nullptr;
+    }
+    int *w = page + next++ % kWords;
+    *w = 0;
+    return w;
+}
+
+// One event per device, recorded after every band launch.
+static std::mutex g_band_mu;
+static std::map<int, cudaEvent_t> g_band_last;
+
+BandTurn::BandTurn(cudaStream_t st) : st_(st)
+{
+    g_band_mu.lock();
+    int dev = 0;
+    status = cudaGetDevice(&dev);
+    auto it = g_band_last.find(dev);
+    if (status == cudaSuccess && it != g_band_last.end()) status = cudaStreamWaitEvent(st, it->second, 0);
+}
+
+BandTurn::~BandTurn()
+{
+    int dev = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess) {
+        auto it = g_band_last.find(dev);
+        if (it == g_band_last.end()) {
+            cudaEvent_t ev = nullptr;
+            if (cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) == cudaSuccess) it = g_band_last.emplace(dev, ev).first;
+        }
+        if (it != g_band_last.end()) cudaEventRecord(it->second, st_);
+    }
+    g_band_mu.unlock();
+}
+
+// The band-resident kernel takes calls of at least this many sweeps: its
+// launch and its copy in and out cost about three half-sweep launches (more
+// bytes more), and a half-sweep saves more than half a launch (L = 1000: 1
+// sweep 10.4 us in a band, 7.8 in launches; 2 sweeps 12.6 and 15.7; 4 sweeps
+// 19 and 31; L = 3000: 30 and 19, 42 and 38, 67 and 77).  On lattices the
+// resident kernel is made for it saves little more than nothing.
+static int64_t band_min_sweeps(const lattice *lt)
+{
+    if (lt->P.L <= 128) return 16;
+    return lt->P.N * (lt->geom.cpl != nullptr ? 2u : 1u) > 6000000u ? 5 : 3;
+}
+
+// Whether the host's sweep number may go into a launch on st: not while the
+// caller captures the stream.
+static bool not_capturing(cudaStream_t st)
+{
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    return cs == cudaStreamCaptureStatusNone;
+}
+
+// CTAs of the band-resident kernel for a call of n sweeps, or 0: lattices on
+// the wide kernel that fit the chip's shared memory, unless the caller chose
+// a graph size (which asks for launches) or is capturing the stream (the
+// launch carries the host's sweep number, so it cannot be replayed).
+static int band_bands(const lattice *lt, int64_t n)
+{
+    if (n < band_min_sweeps(lt) || lt->graph_pinned || lt->P.layout != LAT_INT8 ||
+        lt->dynamics != LAT_DYNAMICS_CHECKERBOARD || choose_kernel(lt) != LAT_KERNEL_WIDE)
+        return 0;
+    const int bands = band_count_for(lt->geom);
+    if (bands == 0) return 0;
+    return not_capturing(lt->stream) ? bands : 0;
+}
+
+// Queue n sweeps on the band-resident kernel (sets *done to the sweeps
+// queued, 0 when its packet buffer cannot be allocated: the launches take over).
+// Each launch is kept well under a second.
+static int band_sweeps(lattice *lt, int bands, int64_t n, int64_t *done)
+{
+    *done = 0;
+    if (lt->band_err == nullptr && (lt->band_err = band_error_word()) == nullptr) return LAT_OK;
+    const size_t bytes = band_mail_bytes(lt->geom, bands);
+    if (lt->band_mail == nullptr) {
+        if (dev_alloc(&lt->band_mail, bytes, lt->stream) != cudaSuccess) {
+            (void)cudaGetLastError();
+            lt->band_mail = nullptr;
+            return LAT_OK;
+        }
+        lt->band_epoch = 1u << 30;   // clear below
+    }
+    const int64_t most = std::max<int64_t>(8, std::min<int64_t>(1 << 16, (int64_t)(1e11 / (double)lt->P.N)));
+    while (*done < n) {
+        const int k = (int)std::min<int64_t>(most, n - *done);
+        cudaError_t e = cudaSuccess;
+        if (lt->band_epoch >= 1u << 30) {
+            e = cudaMemsetAsync(lt->band_mail, 0, bytes, lt->stream);
+            lt->band_epoch = 0;
+        }
+        if (e == cudaSuccess) {
+            BandTurn turn(lt->stream);
+            e = turn.status;
+            if (e == cudaSuccess)
+                e = launch_sweep_band(lt->geom, lt->has_fields, bands, (unsigned long long)(lt->sweeps + *done), k,
+                                      lt->band_mail, lt->band_epoch, lt->band_err, lt->stream);
+        }
+        if (e != cudaSuccess) return cuda_fail(e, "band sweep launch");
+        lt->band_epoch += 2u * (unsigned)k;
+        *done += k;
+    }
+    return LAT_OK;
+}
+
+// Whether a bounded wait of an earlier launch gave up (after a synchronise).
+static int band_status(const lattice *lt)
+{
+    return lt->band_err != nullptr && *(volatile int *)lt->band_err != 0 ? LAT_ETIMEOUT : LAT_OK;
+}
+
 // Queue k sweeps with sweep offsets 0..k-1 relative to ctrl->sweep, then
-// advance ctrl->sweep by k.  Used directly and under stream capture.
+// advance ctrl->sweep by k.  Used directly and under stream capture; direct:
+// not captured, so kernels that can take the sweep number from the host do,
+// and move the counter on themselves.
 // Sweeps per resident launch (a launch runs about a microsecond per sweep at
 // L = 64, so this bounds one kernel to well under a second).
 constexpr int64_t kResidentChunk = 1 << 16;
 
-int enqueue_sweeps(lattice *lt, int64_t k, cudaStream_t st)
+int enqueue_sweeps(lattice *lt, int64_t k, cudaStream_t st, bool direct = false)
 {
     if (lt->dynamics != LAT_DYNAMICS_CHECKERBOARD) {
         const bool balanced = lt->dynamics == LAT_DYNAMICS_RANDOM_SITE_BALANCED;
@@ -276,17 +404,27 @@ int enqueue_sweeps(lattice *lt, int64_t k, cudaStream_t st)
         if (e != cudaSuccess) return cuda_fail(e, "advance launch");
         return LAT_OK;
     }
-    const int kern = choose_kernel(lt);
+    int kern = choose_kernel(lt);
+    // Under AUTO a short call on a small lattice takes the kernel that is
+    // cheaper for it, tuned or not: two launches for one sweep (L = 64: 4.0
+    // us, resident 5.8), one resident launch for more (1.1 us a sweep on top).
+    if (direct && lt->kernel == LAT_KERNEL_AUTO && lt->P.L <= 128 && resident_supported(lt->geom) &&
+        lt->geom.cpl == nullptr && (kern == LAT_KERNEL_WIDE || kern == LAT_KERNEL_RESIDENT) && sweep_at_known(lt->geom))
+        kern = k == 1 ? LAT_KERNEL_WIDE : LAT_KERNEL_RESIDENT;
     if (kern == LAT_KERNEL_RESIDENT) {
         for (int64_t off = 0; off < k; off += kResidentChunk) {
             const int m = (int)std::min<int64_t>(kResidentChunk, k - off);
-            cudaError_t e = launch_sweep_resident(lt->geom, (int)off, m, st);
+            cudaError_t e = launch_sweep_resident(
+                lt->geom, SweepAt{(unsigned long long)(lt->sweeps + off), (int)off, direct ? 1 : 0}, m, st);
             if (e != cudaSuccess) return cuda_fail(e, "resident sweep launch");
         }
+        if (direct) return LAT_OK;
         cudaError_t e = launch_advance(lt->ctrl, (unsigned long long)k, st);
         if (e != cudaSuccess) return cuda_fail(e, "advance launch");
         return LAT_OK;
     }
+    direct = direct && lt->P.layout == LAT_INT8 && kern == LAT_KERNEL_WIDE && wide2_supported(lt->geom) &&
+             sweep_at_known(lt->geom);
     for (int off = 0; off < k; ++off) {
         cudaError_t e;
         if (lt->P.layout == LAT_BITPACKED) {
@@ -294,7 +432,8 @@ int enqueue_sweeps(lattice *lt, int64_t k, cudaStream_t st)
         } else if (kern == LAT_KERNEL_TILED) {
             e = launch_sweep_tiled(lt->geom, lt->tile_w, lt->tile_h, off, st);
         } else if (kern == LAT_KERNEL_WIDE) {
-            e = wide2_supported(lt->geom)   ? launch_sweep_wide(lt->geom, lt->has_fields, off, st)
+            const SweepAt at{(unsigned long long)(lt->sweeps + off), off, direct ? 1 : 0};
+            e = wide2_supported(lt->geom)   ? launch_sweep_wide(lt->geom, lt->has_fields, at, st)
                 : potts_supported(lt->geom) ? launch_sweep_potts(lt->geom, off, st)
                                             : launch_sweep_wide3(lt->geom, off, st);
         } else {
@@ -303,6 +442,7 @@ int enqueue_sweeps(lattice *lt, int64_t k, cudaStream_t st)
         }
         if (e != cudaSuccess) return cuda_fail(e, "sweep launch");
     }
+    if (direct) return LAT_OK;
     cudaError_t e = launch_advance(lt->ctrl, (unsigned long long)k, st);
     if (e != cudaSuccess) return cuda_fail(e, "advance launch");
     return LAT_OK;
@@ -427,14 +567,27 @@ bool tune_choice_ok(const lattice *lt, const TuneChoice &c)
     }
 }
 
+// n sweeps of the band-resident kernel, `ahead` sweeps after the lattice's
+// count (the tuner moves the count on after a candidate).
+int band_candidate(lattice *lt, int bands, int ahead, int n)
+{
+    int64_t done = 0;
+    lt->sweeps += ahead;
+    const int rc = band_sweeps(lt, bands, n, &done);
+    lt->sweeps -= ahead;
+    return rc != LAT_OK || done == n ? rc : LAT_ENOMEM;
+}
+
 // Time one replay of a graph of n sweeps after one untimed replay (the
-// resident kernel: two launches of n sweeps, the second timed); 2n sweeps
-// are enqueued on the lattice's stream.
-int time_candidate(lattice *lt, int n, cudaEvent_t ev0, cudaEvent_t ev1, float &ms)
+// resident and band-resident kernels: two launches of n sweeps, the second
+// timed); 2n sweeps are enqueued on the lattice's stream.  graph_only: as a
+// graph whichever way the sweep loop would run them.
+int time_candidate(lattice *lt, int n, cudaEvent_t ev0, cudaEvent_t ev1, float &ms, bool graph_only = false)
 {
     cudaGraphExec_t exec = nullptr;
     int rc = LAT_OK;
-    const bool graphed = choose_kernel(lt) != LAT_KERNEL_RESIDENT;
+    const int bands = graph_only ? 0 : band_bands(lt, n);
+    const bool graphed = choose_kernel(lt) != LAT_KERNEL_RESIDENT && bands == 0;
     if (graphed) {
         if (lt->cap_stream == nullptr &&
             cudaStreamCreateWithFlags(&lt->cap_stream, cudaStreamNonBlocking) != cudaSuccess)
@@ -453,6 +606,7 @@ int time_candidate(lattice *lt, int n, cudaEvent_t ev0, cudaEvent_t ev1, float &
         if (rep == 1 && cudaEventRecord(ev0, lt->stream) != cudaSuccess) rc = LAT_ECUDA;
         if (rc == LAT_OK) {
             if (graphed) rc = cudaGraphLaunch(exec, lt->stream) == cudaSuccess ? LAT_OK : LAT_ECUDA;
+            else if (bands > 0) rc = band_candidate(lt, bands, rep * n, n);
             else rc = enqueue_sweeps(lt, n, lt->stream);
         }
     }
@@ -538,7 +692,7 @@ static int autotune(lattice *lt, int64_t &left)
             const int gs = std::max(2, g0 * f / 2);
             if (left < 2 * (int64_t)gs) break;
             float ms = 0.f;
-            rc = time_candidate(lt, gs, ev[0], ev[1], ms);
+            rc = time_candidate(lt, gs, ev[0], ev[1], ms, true);
             if (rc != LAT_OK) break;
             lt->sweeps += 2 * gs;
             left -= 2 * gs;
@@ -563,7 +717,8 @@ int sweep_impl(lattice *lt, int64_t n)
 {
     if (n < 0) return LAT_EINVAL;
     if (n == 0) return LAT_OK;
-    int rc = ensure_series(lt, (unsigned long long)(lt->sweeps + n));
+    int rc = band_status(lt);
+    if (rc == LAT_OK) rc = ensure_series(lt, (unsigned long long)(lt->sweeps + n));
     if (rc != LAT_OK) return rc;
     int64_t left = n;
     if (lt->kernel == LAT_KERNEL_AUTO && lt->tuned_kernel == 0 && lt->P.layout == LAT_INT8 &&
@@ -573,6 +728,14 @@ int sweep_impl(lattice *lt, int64_t n)
         if (rc != LAT_OK) return rc;
         n -= lt->sweeps - before;   // sweeps already done (and counted) by the tuner
         if (left == 0) return LAT_OK;
+    }
+    if (const int bands = band_bands(lt, left)) {
+        int64_t done = 0;
+        rc = band_sweeps(lt, bands, left, &done);
+        lt->sweeps += done;
+        if (rc != LAT_OK || done == left) return rc;
+        left -= done;
+        n -= done;
     }
     // The resident kernel runs many sweeps per launch: no graph needed.
     const int gk = (lt->dynamics == LAT_DYNAMICS_CHECKERBOARD && choose_kernel(lt) == LAT_KERNEL_RESIDENT)
@@ -587,7 +750,9 @@ int sweep_impl(lattice *lt, int64_t n)
         }
     }
     if (left > 0) {
-        rc = enqueue_sweeps(lt, left, lt->stream);
+        lt->sweeps += n - left;   // graph replays queued above
+        rc = enqueue_sweeps(lt, left, lt->stream, not_capturing(lt->stream));
+        lt->sweeps -= n - left;
         if (rc != LAT_OK) return rc;
     }
     lt->sweeps += n;
@@ -613,6 +778,7 @@ static void release(lattice *lt)
     dev_free(lt->ref_bits, st);
     dev_free(lt->rs_scratch, st);
     dev_free(lt->cpl, st);
+    dev_free(lt->band_mail, st);
     delete lt;
 }
 
@@ -702,6 +868,7 @@ int create_impl(lattice_t **out, int dims, int L, int two_S, int model, double J
         release(lt);
         return rc;
     }
+    lt->unfl_base = model == LAT_NE ? (int64_t)P.N : 0;
     lt->kernel = LAT_KERNEL_AUTO;
     lt->tile_w = 0;
     lt->tile_h = 0;
@@ -775,7 +942,7 @@ static int current_counters(lattice *lt, long long c[5])
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(lt->stream);
     if (e != cudaSuccess) return cuda_fail(e, "counters");
-    return LAT_OK;
+    return band_status(lt);
 }
 
 int lattice_observables(lattice_t *lt, double *E, double *M, double *density, double *persistence)
@@ -818,7 +985,7 @@ int lattice_series(lattice_t *lt, int64_t first, int64_t count, int64_t *bond, i
         if (up) up[k] = buf[4 * k + 2];
         if (unflipped) unflipped[k] = buf[4 * k + 3];
     }
-    return LAT_OK;
+    return band_status(lt);
 }
 
 int lattice_set_reference(lattice_t *lt, int64_t *ref_sweep)
@@ -1018,7 +1185,7 @@ int lattice_field_series(lattice_t *lt, int64_t first, int64_t count, int64_t *f
                                     (size_t)count * sizeof(int64_t), cudaMemcpyDeviceToHost, lt->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(lt->stream);
     if (e != cudaSuccess) return cuda_fail(e, "field series copy");
-    return LAT_OK;
+    return band_status(lt);
 }
 
 int lattice_clear_reference(lattice_t *lt)
@@ -1060,7 +1227,7 @@ int lattice_autocorrelation(lattice_t *lt, int64_t first, int64_t count, double 
         if (overlap) overlap[k] = buf[(size_t)k];
         if (phi) phi[k] = ((double)buf[(size_t)k] / N - m2) / (1.0 - m2);
     }
-    return LAT_OK;
+    return band_status(lt);
 }
 
 int lattice_get_spins(lattice_t *lt, int8_t *host_out)
@@ -1074,7 +1241,7 @@ int lattice_get_spins(lattice_t *lt, int8_t *host_out)
         e = cudaMemcpyAsync(host_out, lin, (size_t)lt->P.N, cudaMemcpyDeviceToHost, lt->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(lt->stream);
     if (e != cudaSuccess) return cuda_fail(e, "get spins");
-    return LAT_OK;
+    return band_status(lt);
 }
 
 static bool spins_allowed(const Params &P, const int8_t *s)
@@ -1211,6 +1378,13 @@ int lattice_set_state(lattice_t *lt, const int8_t *spins, const uint8_t *flags, 
         lt->sweeps = old_sweeps;
         return cuda_fail(e, "set state");
     }
+    if (lt->flags) {
+        int64_t changed = 0;
+        for (uint8_t f : dev) changed += __builtin_popcount(f);
+        lt->unfl_base = (int64_t)lt->P.N - changed;
+    }
+    if (lt->band_err != nullptr) *lt->band_err = 0;   // the state is whole again
+    lt->band_epoch = 1u << 30;                         // (clears the packet buffer)
     // The recorded series restarts at the restored sweep index.
     dev_free(lt->series, lt->stream);
     lt->series = nullptr;
@@ -1308,7 +1482,7 @@ int lattice_synchronize(lattice_t *lt)
     if (lt == nullptr) return LAT_EINVAL;
     cudaError_t e = cudaStreamSynchronize(lt->stream);
     if (e != cudaSuccess) return cuda_fail(e, "synchronize");
-    return LAT_OK;
+    return band_status(lt);
 }
 
 void lattice_destroy(lattice_t *lt) { release(lt); }

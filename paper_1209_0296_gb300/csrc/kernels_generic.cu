@@ -364,9 +364,10 @@ __global__ void k_advance(Ctrl *ctrl, unsigned long long k) { ctrl->sweep += k; 
 
 __global__ void k_set_ctrl(Ctrl *ctrl, unsigned long long sweep, unsigned long long *series,
                            unsigned long long base, unsigned long long cap, unsigned long long *acf,
-                           unsigned long long *fld)
+                           unsigned long long *fld, unsigned long long unfl_base)
 {
     ctrl->sweep = sweep;
+    ctrl->unfl_base = unfl_base;
     ctrl->series = series;
     ctrl->series_base = base;
     ctrl->series_cap = cap;
@@ -463,9 +464,9 @@ cudaError_t launch_advance(Ctrl *ctrl, unsigned long long k, cudaStream_t st)
 
 cudaError_t launch_set_ctrl(Ctrl *ctrl, unsigned long long sweep, unsigned long long *series,
                             unsigned long long base, unsigned long long cap, unsigned long long *acf,
-                            unsigned long long *fld, cudaStream_t st)
+                            unsigned long long *fld, unsigned long long unfl_base, cudaStream_t st)
 {
-    k_set_ctrl<<<1, 1, 0, st>>>(ctrl, sweep, series, base, cap, acf, fld);
+    k_set_ctrl<<<1, 1, 0, st>>>(ctrl, sweep, series, base, cap, acf, fld, unfl_base);
     return cudaGetLastError();
 }
 

@@ -476,6 +476,23 @@ Geom tiled_geom(const Geom &g)
     Geom k = g;
     for (int i = 0; i < 16; ++i)
         k.thr16[i] = ((g.always16 >> i) & 1u) ? 0xFFFFFFFFu : g.thr16[i] - 1u;
+    // sd << 3 | nd indexes thr16: unlike neighbours of an up spin are the
+    // down ones, of a down spin the others
+    k.acc_sym = 1;
+    for (int nd = 0; nd <= 4; ++nd)
+        if (k.thr16[nd] != k.thr16[8 + 4 - nd] || (nd >= 2 && k.thr16[nd] != 0xFFFFFFFFu)) k.acc_sym = 0;
+    for (uint32_t &w : k.acc) w = 0;
+    if (k.acc_sym) {
+        k.acc[0] = (k.thr16[0] >> 16) | (k.thr16[1] & 0xFFFF0000u);
+        k.acc[1] = 0xFFFFFFFFu;
+    } else {
+        for (int sd = 0; sd < 2; ++sd)
+            for (int nd = 0; nd <= 4; ++nd) {
+                const uint32_t t = k.thr16[sd << 3 | nd] >> 16, sh = 8u * (uint32_t)(nd & 3);
+                k.acc[4 * sd + (nd >> 2)] |= (t & 0xFFu) << sh;
+                k.acc[4 * sd + 2 + (nd >> 2)] |= (t >> 8) << sh;
+            }
+    }
     return k;
 }
 

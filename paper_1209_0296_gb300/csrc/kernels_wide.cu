@@ -21,13 +21,11 @@
 // CTA's shared memory.
 #include <algorithm>
 
-#include "lattice_internal.cuh"
+#include "ising_walk.cuh"
 
 namespace lat {
 
 namespace {
-
-constexpr int kThreads = 256;
 
 // Byte permute in PTX's generic mode, where bit 3 of a selector nibble
 // replicates the sign bit of the selected byte over the output byte.
@@ -42,37 +40,6 @@ LAT_D int byte_sum(uint32_t x)
 {
     const uint32_t s = (x & 0x00FF00FFu) + ((x >> 8) & 0x00FF00FFu);
     return (int)((s & 0xFFFFu) + (s >> 16));
-}
-
-struct Counts {
-    int bond = 0, mag = 0, up = 0, unfl = 0, acf = 0, fld = 0;
-};
-
-// W consecutive 4-byte words (4W same-colour sites) from p.
-template <int W>
-LAT_D void load_words(const int8_t *p, uint32_t (&v)[W])
-{
-    if constexpr (W == 4) {
-        const uint4 q = *reinterpret_cast<const uint4 *>(p);
-        v[0] = q.x;
-        v[1] = q.y;
-        v[2] = q.z;
-        v[3] = q.w;
-    } else if constexpr (W == 2) {
-        const uint2 q = *reinterpret_cast<const uint2 *>(p);
-        v[0] = q.x;
-        v[1] = q.y;
-    } else {
-        v[0] = *reinterpret_cast<const uint32_t *>(p);
-    }
-}
-
-template <int W>
-LAT_D void store_words(int8_t *p, const uint32_t (&v)[W])
-{
-    if constexpr (W == 4) *reinterpret_cast<uint4 *>(p) = make_uint4(v[0], v[1], v[2], v[3]);
-    else if constexpr (W == 2) *reinterpret_cast<uint2 *>(p) = make_uint2(v[0], v[1]);
-    else *reinterpret_cast<uint32_t *>(p) = v[0];
 }
 
 // Sweep colour `colour` of the chunk k (4W sites, W Philox groups) of plane
@@ -218,62 +185,6 @@ LAT_D void wide_chunk(const SweepView g, const uint32_t *sthr, int colour, unsig
     }
 }
 
-// Add the block's counters to the sweep's slot (bond, mag, up[, unflipped]).
-// Warp sums go to shared memory and warp 0 adds them up.  32-bit partial
-// sums are enough: a block's |bond| is at most 2 per site it updated, and a
-// block never updates 2^30 sites in one call.
-// acf: the sweep's autocorrelation slot, or null when no reference is set.
-LAT_D void flush_slot(unsigned long long *slot, unsigned long long *acf, const Counts &c, bool ne,
-                      int (*red)[5])
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int rb = __reduce_add_sync(0xffffffffu, c.bond);
-    const int rm = __reduce_add_sync(0xffffffffu, c.mag);
-    const int ru = __reduce_add_sync(0xffffffffu, c.up);
-    const int rf = __reduce_add_sync(0xffffffffu, c.unfl);
-    const int ra = acf ? __reduce_add_sync(0xffffffffu, c.acf) : 0;
-    if (lane == 0) {
-        red[warp][0] = rb;
-        red[warp][1] = rm;
-        red[warp][2] = ru;
-        red[warp][3] = rf;
-        red[warp][4] = ra;
-    }
-    __syncthreads();
-    if (warp == 0) {
-        const bool in = lane < (int)(blockDim.x >> 5);
-        const int b = __reduce_add_sync(0xffffffffu, in ? red[lane][0] : 0);
-        const int m = __reduce_add_sync(0xffffffffu, in ? red[lane][1] : 0);
-        const int u = __reduce_add_sync(0xffffffffu, in ? red[lane][2] : 0);
-        const int f = __reduce_add_sync(0xffffffffu, in ? red[lane][3] : 0);
-        if (lane < (ne ? 4 : 3)) add_counter(slot + lane, (long long)(lane == 0 ? b : lane == 1 ? m : lane == 2 ? u : f));
-        if (acf) {
-            const int a = __reduce_add_sync(0xffffffffu, in ? red[lane][4] : 0);
-            if (lane == 0) add_counter(acf, (long long)a);
-        }
-    }
-    __syncthreads();
-}
-
-LAT_D void flush(const SweepView &g, unsigned long long sweep, const Counts &c, bool ne, int (*red)[5])
-{
-    flush_slot(series_slot(g.ctrl, sweep), g.ref ? acf_slot(g.ctrl, sweep) : nullptr, c, ne, red);
-}
-
-// Add one int per thread, summed over the block, to *dst (all threads call).
-LAT_D void flush_one(unsigned long long *dst, int v, int (*red)[5])
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int r = __reduce_add_sync(0xffffffffu, v);
-    if (lane == 0) red[warp][0] = r;
-    __syncthreads();
-    if (warp == 0) {
-        const int t = __reduce_add_sync(0xffffffffu, lane < (int)(blockDim.x >> 5) ? red[lane][0] : 0);
-        if (lane == 0) add_counter(dst, (long long)t);
-    }
-    __syncthreads();
-}
-
 // ---------------------------------------------------------------------
 // Software-pipelined two-launch Ising sweep, uniform or with per-bond
 // coupling signs (kCpl) and per-site field signs (kFld).  Same chunks,
@@ -349,167 +260,46 @@ LAT_D void col_load(const ColWalk<kColour> &c, uint32_t y, WideIn &in)
     if constexpr (kCpl) load_words<4>(c.pC + oy, in.C);
 }
 
-// The four Philox groups of the walk's chunk in plane row y.
-template <int kColour>
-LAT_D void col_draws(const PhiloxPre &pp, const ColWalk<kColour> &c, uint32_t y, U4 (&u)[4])
-{
-    const uint32_t g0 = y * c.G + 4u * c.k;
-#pragma unroll
-    for (int w = 0; w < 4; ++w) u[w] = philox_item(pp, g0 + (uint32_t)w, (uint32_t)kColour);
-}
-
-// The Metropolis step of one loaded chunk: neighbour counts, table, accept
-// iff u <= t', write; colour 1 also counts bonds, magnetisation and up
-// sites (and the overlap with the reference when kRef); with kFld each
-// colour adds the field sum of its own sites.
-template <int kColour, bool kRef, bool kCpl = false, bool kFld = false>
-LAT_D void col_step(const ColWalk<kColour> &c, const uint32_t *sthr, uint32_t y, const WideIn &in,
-                    const U4 (&u)[4], Counts &cnt)
-{
-    const uint32_t oy = y * c.half;
-    const bool p1 = ((kColour + y) & 1) != 0;
-    const char *tb = reinterpret_cast<const char *>(sthr);
-    const uint32_t M1 = 0x02020202u;
-    uint32_t Sn[4], ue = 0, dn = 0, ed = 0;
-#pragma unroll
-    for (int w = 0; w < 4; ++w) {
-        uint32_t Lf, R;
-        if (!p1) {   // x = 2j: west is j-1 of the other plane, east is j
-            Lf = __funnelshift_l(w == 0 ? in.adj : in.O[w - 1], in.O[w], 8);
-            R = in.O[w];
-        } else {     // x = 2j+1: west is j, east is j+1
-            Lf = in.O[w];
-            R = __funnelshift_r(in.O[w], w == 3 ? in.adj : in.O[w + 1], 8);
-        }
-        uint32_t Uw = in.U[w], Dw = in.D[w];
-        if constexpr (kCpl) {
-            // Eq. 1 couplings: a negative bond enters as a flipped neighbour
-            // (XOR 0xFE turns +1 into -1 and back); bits 0-3 of a disorder
-            // byte are the west, east, north and south bonds
-            const uint32_t Cw = in.C[w];
-            Lf ^= (Cw & 0x01010101u) * 0xFEu;
-            R ^= ((Cw >> 1) & 0x01010101u) * 0xFEu;
-            Uw ^= ((Cw >> 2) & 0x01010101u) * 0xFEu;
-            Dw ^= ((Cw >> 3) & 0x01010101u) * 0xFEu;
-        }
-        const uint32_t s1 = Uw ^ Dw ^ Lf;
-        const uint32_t c1 = (Uw & Dw) | (Uw & Lf) | (Dw & Lf);
-        const uint32_t b0 = s1 ^ R;
-        const uint32_t b1 = c1 ^ (s1 & R);
-        const uint32_t b2 = c1 & s1 & R;
-        uint32_t idx = (b0 & 0x04040404u) | (b1 & 0x08080808u) | (b2 & 0x10101010u) | (in.S[w] & 0x20202020u);
-        if constexpr (kFld) idx |= in.C[w] & 0x40404040u;   // eta_i = -1: the -h entries 16..31
-        const uint32_t t0 = *reinterpret_cast<const uint32_t *>(tb + (idx & 0xFFu));
-        const uint32_t t1 = *reinterpret_cast<const uint32_t *>(tb + ((idx >> 8) & 0xFFu));
-        const uint32_t t2 = *reinterpret_cast<const uint32_t *>(tb + ((idx >> 16) & 0xFFu));
-        const uint32_t t3 = *reinterpret_cast<const uint32_t *>(tb + (idx >> 24));
-        const uint32_t acc = (u[w].x <= t0 ? 1u : 0u) | (u[w].y <= t1 ? 2u : 0u) | (u[w].z <= t2 ? 4u : 0u) |
-                             (u[w].w <= t3 ? 8u : 0u);
-        // (the spread multiplies run on the FMA pipe, which has room; the
-        // logic pipe is the busier one)
-        const uint32_t F = ((acc * 0x00204081u) & 0x01010101u) * 0xFEu;   // 0xFE at flipped sites
-        Sn[w] = in.S[w] ^ F;
-        // eta_i s_i is down when exactly one of (s_i down: bit 1, eta_i = -1: bit 6) holds
-        if constexpr (kFld) ed += (Sn[w] ^ (in.C[w] >> 5)) & M1;
-        if constexpr (kColour == 1) {
-            // unequal bonds, 2 per pair: the adder's sum and carry words
-            // (U^D^Lf, maj(U,D,Lf)) against the new spin count the unequal
-            // bonds to U, D, Lf once and twice (every bit of a byte above
-            // bit 0 repeats the "down" flag), R counts once
-            ue += ((s1 ^ Sn[w]) & M1) + ((c1 ^ Sn[w]) & 0x04040404u) + ((R ^ Sn[w]) & M1);
-            dn += (Sn[w] & M1) + (in.O[w] & M1);
-        }
-    }
-    store_words<4>(c.dS + oy, Sn);
-    if constexpr (kColour == 1) {
-        const int d2 = byte_sum(dn);
-        cnt.bond += 64 - byte_sum(ue);
-        cnt.mag += 32 - d2;
-        cnt.up += 32 - (d2 >> 1);
-        if constexpr (kRef) {
-            uint32_t R1[4], R0[4], dr = 0;
-            load_words<4>(c.r1 + oy, R1);
-            load_words<4>(c.r0 + oy, R0);
-#pragma unroll
-            for (int w = 0; w < 4; ++w) dr += ((Sn[w] ^ R1[w]) & M1) + ((in.O[w] ^ R0[w]) & M1);
-            cnt.acf += 32 - byte_sum(dr);
-        }
-    }
-    if constexpr (kFld) cnt.fld += 16 - byte_sum(ed);
-}
-
 constexpr int kPipeMinB = 2;   // CTAs per SM (the two chunks in flight need ~100 registers)
 
-// kFld: a 32-entry table, entries 16..31 built from the -h half of the full
-// table (t' = thr - 1 form, all ones = always), index sd << 3 | nd as for
-// entries 0..15.
-template <int kColour, bool kRef, bool kCpl = false, bool kFld = false>
-__global__ void __launch_bounds__(kThreads, kPipeMinB) k_wide_pipe(Geom g, int off)
+constexpr int kWalkMinB = 2;
+
+// 2D Ising, one colour.  kOne: a thread per chunk (the launch has one for
+// each); else a thread per (chunk column, band of consecutive rows), in one
+// wave of at least cpr threads.
+template <int kColour, bool kRef, int kDis, bool kSym, bool kAligned, bool kOne>
+__global__ void __launch_bounds__(kThreads, kWalkMinB) k_ising_walk(Geom g, SweepAt at)
 {
-    __shared__ uint32_t sthr[kFld ? 32 : 16];
+    __shared__ uint32_t sthr[16];
     __shared__ int red[kThreads / 32][5];
     if (threadIdx.x < 16) sthr[threadIdx.x] = g.thr16[threadIdx.x];
-    if constexpr (kFld) {
-        if (threadIdx.x >= 16 && threadIdx.x < 32) {
-            const int e = threadIdx.x - 16, nd = e & 7;
-            uint32_t t = 0u;
-            if (nd <= 4) {
-                const int ds = (e >> 3) ? 2 : -2, n = 4 - 2 * nd;
-                const TabEntry te = g.tab[(2 * g.dsmax + 1) * g.nn + (ds + g.dsmax) * g.nn + (n + g.nmax)];
-                t = te.always ? 0xFFFFFFFFu : te.thr - 1u;
-            }
-            sthr[threadIdx.x] = t;
-        }
-    }
     __syncthreads();
     dep_wait();
-    const unsigned long long sweep = g.ctrl->sweep + (unsigned long long)off;
+    const unsigned long long sweep = sweep_of(g.ctrl, at);
     const SweepView v = sweep_view(g);
-    const int8_t *old = (sweep & 1) ? v.s1 : v.s0;
-    int8_t *nw = (sweep & 1) ? v.s0 : v.s1;
     Counts cnt;
-    // thread -> (chunk column k, first row y); rs rows between visits.  The
-    // launch has at least cpr threads, and rs * cpr of them work.
-    const uint32_t cpr = g.half >> 4;
-    const uint32_t rs = (gridDim.x * blockDim.x) / cpr;
+    const uint32_t L = (uint32_t)g.L, cpr = (g.half + 15u) >> 4;
+    const uint32_t nb = kOne ? L : min((gridDim.x * blockDim.x) / cpr, L);
     const uint32_t gt = blockIdx.x * blockDim.x + threadIdx.x;
-    uint32_t y = gt / cpr;
-    const uint32_t k = gt - y * cpr;
-    if (y < rs && y < (uint32_t)g.L) {
-        PhiloxPre pp;
-        philox_prepare(pp, (uint32_t)sweep, (uint32_t)(sweep >> 32), g.key0, g.key1);
-        const ColWalk<kColour> c = col_walk<kColour>(v, old, nw, k);
-        const uint32_t L = (uint32_t)g.L;
-        // Two chunks in flight, in registers A and B in turn: each block
-        // loads and draws one chunk while the Metropolis step of the other
-        // runs (no copies between the two).
-        WideIn A, B;
-        U4 uA[4], uB[4];
-        col_load<kColour, kCpl>(c, y, A);
-        col_draws<kColour>(pp, c, y, uA);
-        for (;;) {
-            const uint32_t y1 = y + rs;
-            if (y1 >= L) {
-                col_step<kColour, kRef, kCpl, kFld>(c, sthr, y, A, uA, cnt);
-                break;
-            }
-            col_load<kColour, kCpl>(c, y1, B);
-            col_draws<kColour>(pp, c, y1, uB);
-            col_step<kColour, kRef, kCpl, kFld>(c, sthr, y, A, uA, cnt);
-            const uint32_t y2 = y1 + rs;
-            if (y2 >= L) {
-                col_step<kColour, kRef, kCpl, kFld>(c, sthr, y1, B, uB, cnt);
-                break;
-            }
-            col_load<kColour, kCpl>(c, y2, A);
-            col_draws<kColour>(pp, c, y2, uA);
-            col_step<kColour, kRef, kCpl, kFld>(c, sthr, y1, B, uB, cnt);
-            y = y2;
+    const uint32_t band = gt / cpr;
+    if (band < nb) {
+        const IsingPlanes<kColour> p = ising_planes<kColour>(v, sweep);
+        if constexpr (kOne) {
+            ising_one<kColour, kRef, kDis, kSym, kAligned>(p, g.acc, sthr, sweep, g.key0, g.key1, gt - band * cpr,
+                                                           band, cnt);
+        } else {
+            uint32_t y, y1;
+            band_rows(band, nb, L, y, y1);
+            ising_walk<kColour, kRef, kDis, kSym, kAligned>(p, g.acc, sthr, sweep, g.key0, g.key1, gt - band * cpr, y,
+                                                            y1, cnt);
         }
     }
     dep_launch();   // main work done: the next kernel may be scheduled
-    if constexpr (kColour == 1) flush(v, sweep, cnt, false, red);
-    if constexpr (kFld) flush_one(fld_slot(g.ctrl, sweep), cnt.fld, red);   // both colours
+    if constexpr (kColour == 1) {
+        if (gt == 0u) sweep_done(g.ctrl, at);
+        flush(v, sweep, cnt, false, red);
+    }
+    if constexpr (kDis == kFields) flush_one(fld_slot(g.ctrl, sweep), cnt.fld, red);   // both colours
 }
 
 // ---------------------------------------------------------------------
@@ -526,11 +316,7 @@ __global__ void __launch_bounds__(kThreads, kPipeMinB) k_wide_pipe(Geom g, int o
 // ---------------------------------------------------------------------
 constexpr int kNeSlots = 4 * 32;   // list entries per warp (4 groups per lane)
 
-// kCMode: the c-mode rates of §III.B depend on the move alone, not on the
-// neighbour sum (every neighbour-count entry of a row of the table is the
-// same), so the index skips the neighbour-count bits (colour 0 then needs no
-// neighbour adder at all; colour 1 keeps it for the bond count).
-template <int kColour, bool kRef, bool kCMode = false>
+template <int kColour, bool kRef>
 LAT_D void ne_col_step(bool act, const ColWalk<kColour> &c, const uint8_t *fl_c, const uint8_t *fl_o,
                        const uint32_t *sthr, uint32_t y, const WideIn &in, const PhiloxPre &pp,
                        uint32_t *gtab, uint4 *dq, Counts &cnt)
@@ -561,9 +347,8 @@ LAT_D void ne_col_step(bool act, const ColWalk<kColour> &c, const uint8_t *fl_c,
         // down: bit 6 of U | R set) indexes entries 16..31 of the table, all
         // t' = all ones, so it needs no draw; its flip is masked off below.
         locked[w] = Uw | R[w];
-        const uint32_t idx = kCMode ? (in.S[w] & 0x20202020u) | (locked[w] & 0x40404040u)
-                                    : (b0 & 0x04040404u) | (b1 & 0x08080808u) | (b2 & 0x10101010u) |
-                                          (in.S[w] & 0x20202020u) | (locked[w] & 0x40404040u);
+        const uint32_t idx = (b0 & 0x04040404u) | (b1 & 0x08080808u) | (b2 & 0x10101010u) |
+                             (in.S[w] & 0x20202020u) | (locked[w] & 0x40404040u);
         t[w][0] = *reinterpret_cast<const uint32_t *>(tb + (idx & 0xFFu));
         t[w][1] = *reinterpret_cast<const uint32_t *>(tb + ((idx >> 8) & 0xFFu));
         t[w][2] = *reinterpret_cast<const uint32_t *>(tb + ((idx >> 16) & 0xFFu));
@@ -638,7 +423,7 @@ LAT_D void ne_col_step(bool act, const ColWalk<kColour> &c, const uint8_t *fl_c,
     }
 }
 
-template <int kColour, bool kRef, bool kCMode = false>
+template <int kColour, bool kRef>
 __global__ void __launch_bounds__(kThreads, kPipeMinB) k_wide_pipe_ne(Geom g, int off)
 {
     __shared__ uint32_t sthr[32];   // entries 16..31: locked sites, always accepted (then masked)
@@ -676,12 +461,12 @@ __global__ void __launch_bounds__(kThreads, kPipeMinB) k_wide_pipe_ne(Geom g, in
         const uint32_t y1 = y + rs;
         const bool act1 = act && y1 < L;
         if (act1) col_load<kColour>(c, y1, B);
-        ne_col_step<kColour, kRef, kCMode>(act, c, fl_c, fl_o, sthr, y, A, pp, gtab[warp], dq[warp], cnt);
+        ne_col_step<kColour, kRef>(act, c, fl_c, fl_o, sthr, y, A, pp, gtab[warp], dq[warp], cnt);
         if (!__any_sync(0xffffffffu, act1)) break;
         const uint32_t y2 = y1 + rs;
         const bool act2 = act1 && y2 < L;
         if (act2) col_load<kColour>(c, y2, A);
-        ne_col_step<kColour, kRef, kCMode>(act1, c, fl_c, fl_o, sthr, y1, B, pp, gtab[warp], dq[warp], cnt);
+        ne_col_step<kColour, kRef>(act1, c, fl_c, fl_o, sthr, y1, B, pp, gtab[warp], dq[warp], cnt);
         y = y2;
         act = act2;
     }
@@ -700,60 +485,6 @@ __global__ void __launch_bounds__(kThreads, kPipeMinB) k_wide_pipe_ne(Geom g, in
 // k_wide_pipe (Ising: the next chunk's draws too) and, for the North-East
 // model, the warp-compacted draws of k_wide_pipe_ne.
 // ---------------------------------------------------------------------
-
-// Bytes p[0 .. nv) (1 <= nv <= 16) as four words, byte b = p[b], the bytes
-// from nv on unspecified; an aligned word that holds none of them is not
-// read (the spin buffers are multiples of 4 bytes, so every word read is in
-// bounds).  kAligned: p is 16-byte aligned and nv = 16 (every chunk of a
-// lattice with L % 32 == 0), one 16-byte load.
-template <bool kAligned = false>
-LAT_D void load16_any(const int8_t *p, uint32_t nv, uint32_t (&v)[4])
-{
-    if constexpr (kAligned) {
-        load_words<4>(p, v);
-        return;
-    }
-    const uintptr_t a = reinterpret_cast<uintptr_t>(p);
-    const uint32_t sh = (uint32_t)(a & 3u);
-    const uint32_t *w = reinterpret_cast<const uint32_t *>(a - sh);
-    uint32_t x[5];
-    x[0] = w[0];
-#pragma unroll
-    for (int i = 1; i < 5; ++i) x[i] = (4u * (uint32_t)i < nv + sh) ? w[i] : 0u;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) v[i] = __funnelshift_r(x[i], x[i + 1], 8u * sh);
-}
-
-// Write bytes [0, nv) of v to p (any alignment) and no other byte: whole
-// aligned words where the chunk covers them, single bytes at its ends.
-template <bool kAligned = false>
-LAT_D void store16_any(int8_t *p, uint32_t nv, const uint32_t (&v)[4])
-{
-    if constexpr (kAligned) {
-        store_words<4>(p, v);
-        return;
-    }
-    const uintptr_t a = reinterpret_cast<uintptr_t>(p);
-    const uint32_t sh = (uint32_t)(a & 3u);
-    uint32_t *w = reinterpret_cast<uint32_t *>(a - sh);
-    uint32_t o[5];   // o[i]: the chunk's bytes that fall in aligned word i
-    o[0] = __funnelshift_l(0u, v[0], 8u * sh);
-#pragma unroll
-    for (int i = 1; i < 4; ++i) o[i] = __funnelshift_l(v[i - 1], v[i], 8u * sh);
-    o[4] = __funnelshift_l(v[3], 0u, 8u * sh);
-#pragma unroll
-    for (int i = 0; i < 5; ++i) {
-        const int lo = i == 0 ? (int)sh : 0;
-        const int hi = min(4, (int)(nv + sh) - 4 * i);
-        if (hi <= lo) continue;
-        if (lo == 0 && hi == 4) {
-            w[i] = o[i];
-        } else {
-            int8_t *pb = reinterpret_cast<int8_t *>(w + i);
-            for (int j = lo; j < hi; ++j) pb[j] = (int8_t)(o[i] >> (8 * j));
-        }
-    }
-}
 
 struct AnyIn {
     uint32_t S[4], O[4], U[4], D[4];
@@ -897,61 +628,10 @@ LAT_D void any_step(const AnyWalk<kColour> &c, const uint32_t *sthr, uint32_t y,
     }
 }
 
-template <int kColour, bool kRef>
-__global__ void __launch_bounds__(kThreads, kPipeMinB) k_any_pipe(Geom g, int off)
-{
-    __shared__ uint32_t sthr[16];
-    __shared__ int red[kThreads / 32][5];
-    if (threadIdx.x < 16) sthr[threadIdx.x] = g.thr16[threadIdx.x];
-    __syncthreads();
-    dep_wait();
-    const unsigned long long sweep = g.ctrl->sweep + (unsigned long long)off;
-    const SweepView v = sweep_view(g);
-    const int8_t *old = (sweep & 1) ? v.s1 : v.s0;
-    int8_t *nw = (sweep & 1) ? v.s0 : v.s1;
-    Counts cnt;
-    const uint32_t cpr = (g.half + 15u) >> 4;   // chunks per plane row, the last partial
-    const uint32_t rs = (gridDim.x * blockDim.x) / cpr;
-    const uint32_t gt = blockIdx.x * blockDim.x + threadIdx.x;
-    uint32_t y = gt / cpr;
-    const uint32_t k = gt - y * cpr;
-    if (y < rs && y < (uint32_t)g.L) {
-        PhiloxPre pp;
-        philox_prepare(pp, (uint32_t)sweep, (uint32_t)(sweep >> 32), g.key0, g.key1);
-        const AnyWalk<kColour> c = any_walk<kColour>(v, old, nw, k);
-        const uint32_t L = (uint32_t)g.L;
-        AnyIn A, B;
-        U4 uA[4], uB[4];
-        any_load<kColour>(c, y, A);
-        any_draws<kColour>(pp, c, y, uA);
-        for (;;) {
-            const uint32_t y1 = y + rs;
-            if (y1 >= L) {
-                any_step<kColour, kRef>(c, sthr, y, A, uA, cnt);
-                break;
-            }
-            any_load<kColour>(c, y1, B);
-            any_draws<kColour>(pp, c, y1, uB);
-            any_step<kColour, kRef>(c, sthr, y, A, uA, cnt);
-            const uint32_t y2 = y1 + rs;
-            if (y2 >= L) {
-                any_step<kColour, kRef>(c, sthr, y1, B, uB, cnt);
-                break;
-            }
-            any_load<kColour>(c, y2, A);
-            any_draws<kColour>(pp, c, y2, uA);
-            any_step<kColour, kRef>(c, sthr, y1, B, uB, cnt);
-            y = y2;
-        }
-    }
-    dep_launch();   // main work done: the next kernel may be scheduled
-    if constexpr (kColour == 1) flush(v, sweep, cnt, false, red);
-}
-
 // North-East at any even L: the step of ne_col_step with any-alignment
 // loads and stores, per-byte persistence updates (the groups of a row need
 // not start on a word), and the warp-compacted draws.
-template <int kColour, bool kRef, bool kAligned = false, bool kCMode = false>
+template <int kColour, bool kRef, bool kAligned = false>
 LAT_D void any_ne_step(bool act, const AnyWalk<kColour> &c, uint8_t *fl_c, const uint8_t *fl_o,
                        const uint32_t *sthr, uint32_t y, const AnyIn &in, const PhiloxPre &pp, uint32_t *gtab,
                        uint4 *dq, Counts &cnt)
@@ -974,9 +654,8 @@ LAT_D void any_ne_step(bool act, const AnyWalk<kColour> &c, uint8_t *fl_c, const
         // §III.B: a locked site (north or east down) indexes the all-accept
         // entries 16..31; so do the bytes past the row (masked below)
         locked[w] = Uw | R[w] | ~c.vm[w];
-        const uint32_t idx = kCMode ? (in.S[w] & 0x20202020u) | (locked[w] & 0x40404040u)
-                                    : (b0 & 0x04040404u) | (b1 & 0x08080808u) | (b2 & 0x10101010u) |
-                                          (in.S[w] & 0x20202020u) | (locked[w] & 0x40404040u);
+        const uint32_t idx = (b0 & 0x04040404u) | (b1 & 0x08080808u) | (b2 & 0x10101010u) |
+                             (in.S[w] & 0x20202020u) | (locked[w] & 0x40404040u);
         t[w][0] = *reinterpret_cast<const uint32_t *>(tb + (idx & 0xFFu));
         t[w][1] = *reinterpret_cast<const uint32_t *>(tb + ((idx >> 8) & 0xFFu));
         t[w][2] = *reinterpret_cast<const uint32_t *>(tb + ((idx >> 16) & 0xFFu));
@@ -1059,7 +738,7 @@ LAT_D void any_ne_step(bool act, const AnyWalk<kColour> &c, uint8_t *fl_c, const
     }
 }
 
-template <int kColour, bool kRef, bool kCMode = false>
+template <int kColour, bool kRef>
 __global__ void __launch_bounds__(kThreads, kPipeMinB) k_any_pipe_ne(Geom g, int off)
 {
     __shared__ uint32_t sthr[32];   // entries 16..31: locked sites, always accepted (then masked)
@@ -1094,12 +773,12 @@ __global__ void __launch_bounds__(kThreads, kPipeMinB) k_any_pipe_ne(Geom g, int
         const uint32_t y1 = y + rs;
         const bool act1 = act && y1 < L;
         if (act1) any_load<kColour>(c, y1, B);
-        any_ne_step<kColour, kRef, false, kCMode>(act, c, fl_c, fl_o, sthr, y, A, pp, gtab[warp], dq[warp], cnt);
+        any_ne_step<kColour, kRef>(act, c, fl_c, fl_o, sthr, y, A, pp, gtab[warp], dq[warp], cnt);
         if (!__any_sync(0xffffffffu, act1)) break;
         const uint32_t y2 = y1 + rs;
         const bool act2 = act1 && y2 < L;
         if (act2) any_load<kColour>(c, y2, A);
-        any_ne_step<kColour, kRef, false, kCMode>(act1, c, fl_c, fl_o, sthr, y1, B, pp, gtab[warp], dq[warp], cnt);
+        any_ne_step<kColour, kRef>(act1, c, fl_c, fl_o, sthr, y1, B, pp, gtab[warp], dq[warp], cnt);
         y = y2;
         act = act2;
     }
@@ -1112,26 +791,7 @@ __global__ void __launch_bounds__(kThreads, kPipeMinB) k_any_pipe_ne(Geom g, int
 // rows of more than 256 chunks, a segment of 256 chunk columns; a thread
 // walks one chunk column down the band with two chunks in flight, as the
 // solo kernels do.
-struct AnyItemShape {
-    uint32_t cpr, nseg, rsb, br;   // chunks per row, column segments, rows per pass, rows per band
-};
-
-// Rows a thread visits per item (passes): given by the batch (its tuner),
-// or 0 for the default: 8 on large lattices (few items, long pipelines), 2
-// on small ones (enough items to spread a batch of small lattices over the
-// SMs).
-LAT_HD AnyItemShape any_item_shape(uint32_t half, uint32_t passes)
-{
-    AnyItemShape sh;
-    sh.cpr = (half + 15u) >> 4;
-    sh.nseg = (sh.cpr + kThreads - 1u) / kThreads;
-    sh.rsb = sh.cpr <= (uint32_t)kThreads ? (uint32_t)kThreads / sh.cpr : 1u;
-    if (passes == 0u) passes = half >= 512u ? 8u : 2u;
-    sh.br = passes * sh.rsb;
-    return sh;
-}
-
-template <int kColour, bool kNE, bool kAligned, bool kCMode>
+template <int kColour, bool kNE, bool kAligned>
 LAT_D void batch_any_item(const SweepView &v, const uint32_t *sthr, uint32_t item, uint32_t passes, uint32_t *gtab,
                           uint4 *dq, Counts &cnt)
 {
@@ -1196,23 +856,21 @@ LAT_D void batch_any_item(const SweepView &v, const uint32_t *sthr, uint32_t ite
             const uint32_t ya = y + sh.rsb;
             const bool act1 = act && ya < y1;
             if (act1) any_load<kColour, kAligned>(c, ya, B);
-            if (v.ref) any_ne_step<kColour, true, kAligned, kCMode>(act, c, fl_c, fl_o, sthr, y, A, pp, gtab, dq, cnt);
-            else any_ne_step<kColour, false, kAligned, kCMode>(act, c, fl_c, fl_o, sthr, y, A, pp, gtab, dq, cnt);
+            if (v.ref) any_ne_step<kColour, true, kAligned>(act, c, fl_c, fl_o, sthr, y, A, pp, gtab, dq, cnt);
+            else any_ne_step<kColour, false, kAligned>(act, c, fl_c, fl_o, sthr, y, A, pp, gtab, dq, cnt);
             if (!__any_sync(0xffffffffu, act1)) break;
             const uint32_t yb = ya + sh.rsb;
             const bool act2 = act1 && yb < y1;
             if (act2) any_load<kColour, kAligned>(c, yb, A);
-            if (v.ref) any_ne_step<kColour, true, kAligned, kCMode>(act1, c, fl_c, fl_o, sthr, ya, B, pp, gtab, dq, cnt);
-            else any_ne_step<kColour, false, kAligned, kCMode>(act1, c, fl_c, fl_o, sthr, ya, B, pp, gtab, dq, cnt);
+            if (v.ref) any_ne_step<kColour, true, kAligned>(act1, c, fl_c, fl_o, sthr, ya, B, pp, gtab, dq, cnt);
+            else any_ne_step<kColour, false, kAligned>(act1, c, fl_c, fl_o, sthr, ya, B, pp, gtab, dq, cnt);
             y = yb;
             act = act2;
         }
     }
 }
 
-// kCMode: a list of c-mode North-East lattices (their steps skip the
-// neighbour-count bits of the table index).
-template <bool kNE, bool kAligned, int kColour, bool kCMode = false>
+template <bool kNE, bool kAligned, int kColour>
 __global__ void __launch_bounds__(kThreads, kPipeMinB) k_batch_any(const Geom *geoms, const uint2 *items, int n_items,
                                                                   unsigned *next_item, uint32_t passes)
 {
@@ -1242,7 +900,7 @@ __global__ void __launch_bounds__(kThreads, kPipeMinB) k_batch_any(const Geom *g
         }
         const SweepView v = sweep_view(sg);
         Counts cnt;
-        batch_any_item<kColour, kNE, kAligned, kCMode>(v, sthr, w.y, passes, gtab[warp], dq[warp], cnt);
+        batch_any_item<kColour, kNE, kAligned>(v, sthr, w.y, passes, gtab[warp], dq[warp], cnt);
         if constexpr (kColour == 1) flush(v, v.ctrl->sweep, cnt, kNE, red);   // ends with __syncthreads()
         __syncthreads();
     }
@@ -1262,14 +920,13 @@ constexpr size_t kResMaxBytes = 220 * 1024;
 // memory (the batched kernel): the sweep loop reads only register copies.
 // advance: the CTA also moves the lattice's sweep counter on by n_sweeps.
 template <bool kNE, int W>
-LAT_D void resident_body(const Geom &g, int off, int n_sweeps, bool advance, uint4 *res_smem, uint32_t *sthr,
+LAT_D void resident_body(const Geom &g, unsigned long long sweep0, int n_sweeps, bool advance, uint4 *res_smem, uint32_t *sthr,
                          int (*red)[5])
 {
     int8_t *sp = reinterpret_cast<int8_t *>(res_smem);
     const uint64_t n16 = g.N >> 4;                       // N % 16 == 0 (L % 32 == 0)
     const uint64_t f16 = kNE ? ((uint64_t)2 * g.rows * g.G) >> 4 : 0;  // flag bytes / 16
     uint4 *fl4 = res_smem + n16;
-    const unsigned long long sweep0 = g.ctrl->sweep + (unsigned long long)off;
     {
         const uint4 *src = reinterpret_cast<const uint4 *>(g.s[sweep0 & 1]);
         for (uint64_t i = threadIdx.x; i < n16; i += blockDim.x) res_smem[i] = src[i];
@@ -1337,12 +994,12 @@ LAT_D void resident_body(const Geom &g, int off, int n_sweeps, bool advance, uin
 }
 
 template <bool kNE, int W>
-__global__ void __launch_bounds__(kResThreads, 1) k_resident(Geom g, int off, int n_sweeps)
+__global__ void __launch_bounds__(kResThreads, 1) k_resident(Geom g, SweepAt at, int n_sweeps)
 {
     extern __shared__ uint4 res_smem[];
     __shared__ uint32_t sthr[16];
     __shared__ int red[kResThreads / 32][5];
-    resident_body<kNE, W>(g, off, n_sweeps, false, res_smem, sthr, red);
+    resident_body<kNE, W>(g, sweep_of(g.ctrl, at), n_sweeps, at.known != 0, res_smem, sthr, red);
 }
 
 // Batched form: CTA i sweeps lattice i (descriptor geoms[i]) by
@@ -1363,11 +1020,11 @@ __global__ void __launch_bounds__(kResThreads, 1) k_batch_resident(const Geom *g
     __syncthreads();
     const bool narrow = (uint64_t)sg.L * (sg.half >> 2) <= (uint64_t)kResThreads;
     if (sg.model == LAT_NE) {
-        if (narrow) resident_body<true, 1>(sg, 0, m, true, res_smem, sthr, red);
-        else resident_body<true, 4>(sg, 0, m, true, res_smem, sthr, red);
+        if (narrow) resident_body<true, 1>(sg, sg.ctrl->sweep, m, true, res_smem, sthr, red);
+        else resident_body<true, 4>(sg, sg.ctrl->sweep, m, true, res_smem, sthr, red);
     } else {
-        if (narrow) resident_body<false, 1>(sg, 0, m, true, res_smem, sthr, red);
-        else resident_body<false, 4>(sg, 0, m, true, res_smem, sthr, red);
+        if (narrow) resident_body<false, 1>(sg, sg.ctrl->sweep, m, true, res_smem, sthr, red);
+        else resident_body<false, 4>(sg, sg.ctrl->sweep, m, true, res_smem, sthr, red);
     }
 }
 
@@ -1420,88 +1077,60 @@ int batch_any_grid(bool ne)
 }
 
 cudaError_t launch_batch_any(const Geom *geoms, const uint2 *items, int n_items, unsigned *next_item, int colour,
-                             bool ne, bool cmode, bool aligned, int passes, int grid, cudaStream_t st)
+                             bool ne, bool aligned, int passes, int grid, cudaStream_t st)
 {
     using K = void (*)(const Geom *, const uint2 *, int, unsigned *, uint32_t);
-    // [Ising, North-East at T, North-East in c-mode][aligned][colour]
-    static const K kern[3][2][2] = {
+    // [Ising, North-East at T][aligned][colour]
+    static const K kern[2][2][2] = {
         {{k_batch_any<false, false, 0>, k_batch_any<false, false, 1>},
          {k_batch_any<false, true, 0>, k_batch_any<false, true, 1>}},
         {{k_batch_any<true, false, 0>, k_batch_any<true, false, 1>},
-         {k_batch_any<true, true, 0>, k_batch_any<true, true, 1>}},
-        {{k_batch_any<true, false, 0, true>, k_batch_any<true, false, 1, true>},
-         {k_batch_any<true, true, 0, true>, k_batch_any<true, true, 1, true>}}};
-    const int m = ne ? (cmode ? 2 : 1) : 0;
-    return launch_pdl(kern[m][aligned ? 1 : 0][colour ? 1 : 0], (unsigned)grid, kThreads, st, geoms, items, n_items,
-                      next_item, (uint32_t)passes);
+         {k_batch_any<true, true, 0>, k_batch_any<true, true, 1>}}};
+    return launch_pdl(kern[ne ? 1 : 0][aligned ? 1 : 0][colour ? 1 : 0], (unsigned)grid, kThreads, st, geoms, items,
+                      n_items, next_item, (uint32_t)passes);
 }
 
-cudaError_t launch_sweep_wide(const Geom &g, bool fields, int off, cudaStream_t st)
+bool sweep_at_known(const Geom &g) { return g.model == LAT_ISING || ne_walk_supported(g); }
+
+cudaError_t launch_sweep_wide(const Geom &g, bool fields, SweepAt at, cudaStream_t st)
 {
+    if (ne_walk_supported(g)) return launch_sweep_ne(g, at, st);
     const Geom k = tiled_geom(g);  // compact table in t' = thr - 1 form
-    int dev = 0;
-    cudaGetDevice(&dev);
-    // one wave: SMs x resident CTAs per SM, queried once per kernel
-    auto wave = [dev](const void *fn, int &cache) {
-        if (cache == 0) {
-            int sms = 0, per = 0;
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, kThreads, 0);
-            cache = sms * (per > 0 ? per : 1);
-        }
-        return cache;
-    };
-    if (!wide_supported(g)) {   // L % 32 != 0: the any-L kernels, 16 sites per lane
-        static int res_any = 0;
-        const uint64_t chunks = (uint64_t)g.L * ((g.half + 15u) >> 4);
-        const unsigned gb = (unsigned)std::min<long long>(
-            (long long)((chunks + kThreads - 1) / kThreads),
-            wave(reinterpret_cast<const void *>(k_any_pipe_ne<1, true>), res_any));
-        using KG = void (*)(Geom, int);
-        const bool ne = g.model == LAT_NE, ref = k.ref != nullptr;
-        // North-East: [c-mode][reference][colour]
-        static const KG kne[2][2][2] = {
+    const int ref = k.ref != nullptr ? 1 : 0, al = g.L % 32 == 0 ? 1 : 0;
+    const uint64_t blocks = ((uint64_t)g.L * ((g.half + 15u) >> 4) + kThreads - 1) / kThreads;
+    if (g.model == LAT_NE) {   // North-East at temperature T
+        using K = void (*)(Geom, int);
+        static const K ne[2][2][2] = {
             {{k_any_pipe_ne<0, false>, k_any_pipe_ne<1, false>}, {k_any_pipe_ne<0, true>, k_any_pipe_ne<1, true>}},
-            {{k_any_pipe_ne<0, false, true>, k_any_pipe_ne<1, false, true>},
-             {k_any_pipe_ne<0, true, true>, k_any_pipe_ne<1, true, true>}}};
-        const int cm = g.cmode ? 1 : 0;
-        const KG c0 = ne ? kne[cm][ref][0] : (ref ? k_any_pipe<0, true> : k_any_pipe<0, false>);
-        const KG c1 = ne ? kne[cm][ref][1] : (ref ? k_any_pipe<1, true> : k_any_pipe<1, false>);
-        cudaError_t e = launch_pdl(c0, gb, kThreads, st, k, off);
-        return e == cudaSuccess ? launch_pdl(c1, gb, kThreads, st, k, off) : e;
+            {{k_wide_pipe_ne<0, false>, k_wide_pipe_ne<1, false>}, {k_wide_pipe_ne<0, true>, k_wide_pipe_ne<1, true>}}};
+        static const unsigned w[2] = {one_wave(reinterpret_cast<const void *>(ne[0][1][1])),
+                                      one_wave(reinterpret_cast<const void *>(ne[1][1][1]))};
+        const unsigned grid = (unsigned)std::min<uint64_t>(blocks, w[al]);
+        cudaError_t e = launch_pdl(ne[al][ref][0], grid, kThreads, st, k, at.off);
+        return e == cudaSuccess ? launch_pdl(ne[al][ref][1], grid, kThreads, st, k, at.off) : e;
     }
-    if (g.model == LAT_NE && g.cpl == nullptr) {   // North-East: pipelined, draws compacted per warp
-        static int res_ne = 0;
-        const unsigned pb = (unsigned)std::min<long long>(
-            wide_chunks(g), wave(reinterpret_cast<const void *>(k_wide_pipe_ne<1, true>), res_ne));
-        using KG = void (*)(Geom, int);
-        static const KG kne[2][2][2] = {
-            {{k_wide_pipe_ne<0, false>, k_wide_pipe_ne<1, false>}, {k_wide_pipe_ne<0, true>, k_wide_pipe_ne<1, true>}},
-            {{k_wide_pipe_ne<0, false, true>, k_wide_pipe_ne<1, false, true>},
-             {k_wide_pipe_ne<0, true, true>, k_wide_pipe_ne<1, true, true>}}};
-        const int cm = g.cmode ? 1 : 0, ref = k.ref != nullptr ? 1 : 0;
-        cudaError_t e = launch_pdl(kne[cm][ref][0], pb, kThreads, st, k, off);
-        return e == cudaSuccess ? launch_pdl(kne[cm][ref][1], pb, kThreads, st, k, off) : e;
-    }
-    // Ising, uniform or with per-bond couplings (and per-site field signs):
-    // the software-pipelined kernels
-    using KP = void (*)(Geom, int);
-    static const KP pipe[3][2][2] = {
-        {{k_wide_pipe<0, false>, k_wide_pipe<1, false>}, {k_wide_pipe<0, true>, k_wide_pipe<1, true>}},
-        {{k_wide_pipe<0, false, true, false>, k_wide_pipe<1, false, true, false>},
-         {k_wide_pipe<0, true, true, false>, k_wide_pipe<1, true, true, false>}},
-        {{k_wide_pipe<0, false, true, true>, k_wide_pipe<1, false, true, true>},
-         {k_wide_pipe<0, true, true, true>, k_wide_pipe<1, true, true, true>}}};
-    static int res_pipe[3] = {0, 0, 0};
-    const int m = g.cpl == nullptr ? 0 : (fields ? 2 : 1);
-    const int ref = k.ref != nullptr ? 1 : 0;
-    const unsigned pb = (unsigned)std::min<long long>(
-        wide_chunks(g), wave(reinterpret_cast<const void *>(pipe[m][1][1]), res_pipe[m]));
-    for (int colour = 0; colour < 2; ++colour) {
-        cudaError_t e = launch_pdl(pipe[m][ref][colour], pb, kThreads, st, k, off);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+    // kinds: uniform at any even L with a general or a symmetric table; then
+    // L % 32 == 0: the same, bonds with either table, fields
+    using K = void (*)(Geom, SweepAt);
+#define LAT_WALK(ref, dis, sym, al, one) {k_ising_walk<0, ref, dis, sym, al, one>, k_ising_walk<1, ref, dis, sym, al, one>}
+#define LAT_KIND(dis, sym, al)                                                              \
+    {{LAT_WALK(false, dis, sym, al, false), LAT_WALK(true, dis, sym, al, false)},           \
+     {LAT_WALK(false, dis, sym, al, true), LAT_WALK(true, dis, sym, al, true)}}
+    static const K is[7][2][2][2] = {LAT_KIND(kUniform, false, false), LAT_KIND(kUniform, true, false),
+                                     LAT_KIND(kUniform, false, true),  LAT_KIND(kUniform, true, true),
+                                     LAT_KIND(kBonds, false, true),    LAT_KIND(kBonds, true, true),
+                                     LAT_KIND(kFields, false, true)};
+#undef LAT_KIND
+#undef LAT_WALK
+    static const unsigned wave = one_wave(reinterpret_cast<const void *>(is[3][0][0][1]));   // all: kWalkMinB per SM
+    const int sym = k.acc_sym ? 1 : 0;
+    const int m = g.cpl != nullptr ? (fields ? 6 : 4 + sym) : 2 * al + sym;
+    // one chunk a thread up to two waves of them: up to there the row walk's
+    // start-up costs more than its register reuse saves
+    const int one = blocks <= 2u * wave ? 1 : 0;
+    const unsigned grid = one ? (unsigned)blocks : wave;
+    cudaError_t e = launch_pdl(is[m][one][ref][0], grid, kThreads, st, k, at);
+    return e == cudaSuccess ? launch_pdl(is[m][one][ref][1], grid, kThreads, st, k, at) : e;
 }
 
 }  // namespace lat
@@ -1513,7 +1142,7 @@ bool resident_supported(const Geom &g)
     return wide_supported(g) && g.cpl == nullptr && resident_bytes(g) <= kResMaxBytes;
 }
 
-cudaError_t launch_sweep_resident(const Geom &g, int off, int n_sweeps, cudaStream_t st)
+cudaError_t launch_sweep_resident(const Geom &g, SweepAt at, int n_sweeps, cudaStream_t st)
 {
     const Geom k = tiled_geom(g);
     const size_t smem = resident_bytes(g);
@@ -1521,14 +1150,14 @@ cudaError_t launch_sweep_resident(const Geom &g, int off, int n_sweeps, cudaStre
     const bool narrow = (uint64_t)g.L * (g.half >> 2) <= (uint64_t)kResThreads;
     const int m = (g.model == LAT_NE ? 2 : 0) + (narrow ? 1 : 0);
     static bool attr[4] = {false, false, false, false};
-    void (*fn[4])(Geom, int, int) = {k_resident<false, 4>, k_resident<false, 1>, k_resident<true, 4>,
+    void (*fn[4])(Geom, SweepAt, int) = {k_resident<false, 4>, k_resident<false, 1>, k_resident<true, 4>,
                                      k_resident<true, 1>};
     if (!attr[m]) {
         cudaError_t e = cudaFuncSetAttribute(fn[m], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResMaxBytes);
         if (e != cudaSuccess) return e;
         attr[m] = true;
     }
-    fn[m]<<<1, kResThreads, smem, st>>>(k, off, n_sweeps);
+    fn[m]<<<1, kResThreads, smem, st>>>(k, at, n_sweeps);
     return cudaGetLastError();
 }
 

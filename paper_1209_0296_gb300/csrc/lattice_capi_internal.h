@@ -28,6 +28,19 @@ int create_impl(struct ::lattice **out, int dims, int L, int two_S, int model, d
                 double T_or_c, uint64_t seed, int init, int layout, void *cuda_stream);
 int sweep_impl(struct ::lattice *lt, int64_t n);
 int choose_kernel(const struct ::lattice *lt);
+// A host-visible error word for band launches (one of a fixed page), zeroed.
+int *band_error_word();
+// Order a band launch on st after the last one on any stream: two of them
+// must not wait for each other's SMs.  Holds a lock until destroyed.
+class BandTurn {
+public:
+    explicit BandTurn(cudaStream_t st);
+    ~BandTurn();
+    cudaError_t status = cudaSuccess;
+
+private:
+    cudaStream_t st_;
+};
 int ensure_series(struct ::lattice *lt, unsigned long long need);
 bool tile_shape_ok(int tile_w, int tile_h);
 int default_tile_h();
@@ -74,9 +87,14 @@ struct lattice {
     std::vector<lat::TabEntry> host_tab;
     int64_t sweeps = 0;        // sweeps done (global index of the next sweep)
     int64_t series_first = 0;  // first sweep index recorded in the series buffer
+    int64_t unfl_base = 0;     // unflipped sites before that sweep (North-East)
     int kernel = 0, tile_w = 0, tile_h = 0, graph_sweeps = 0;
     int tuned_kernel = 0;      // autotuner's choice for LAT_KERNEL_AUTO (0 = not tuned)
     bool graph_pinned = false; // sweeps per graph set by lattice_set_kernel (the tuner keeps it)
     cudaGraphExec_t graph_exec = nullptr;
     bool graph_valid = false;
+    // band-resident sweeps (kernels_band.cu)
+    void *band_mail = nullptr;           // boundary-row packets
+    unsigned band_epoch = 0;             // at least every packet mark sent so far
+    int *band_err = nullptr;             // host-visible word: a bounded wait gave up
 };

@@ -140,6 +140,7 @@ struct Ctrl {
     unsigned long long series_cap;   // sweeps the series buffer can hold
     unsigned long long *acf;         // [series_cap] sum_i s_i(t) s_i(ref), same indexing
     unsigned long long *fld;         // [series_cap] sum_i eta_i s_i (per-site field signs), same indexing
+    unsigned long long unfl_base;    // unflipped sites before sweep series_base (North-East)
 };
 
 // Work items of the batched 8-site-chunk kernels (3D / spin-S, Potts): a
@@ -162,6 +163,15 @@ LAT_HD ColItemShape col_item_shape(uint32_t half, uint32_t rows, uint32_t passes
     sh.br = passes * sh.rsb;
     return sh;
 }
+
+// Which sweep a launch works on: `off` sweeps after the device counter (a
+// captured launch, which must replay unchanged), or, when known, sweep number
+// `sweep` from the host, whose last launch then moves the counter itself.
+struct SweepAt {
+    unsigned long long sweep;
+    int off;
+    int known;
+};
 
 #if defined(__CUDACC__)
 // Programmatic dependent launch.  The sweep kernels are launched so that the
@@ -207,6 +217,24 @@ LAT_D unsigned long long *series_slot(const Ctrl *c, unsigned long long sweep)
 LAT_D unsigned long long *acf_slot(const Ctrl *c, unsigned long long sweep)
 {
     return c->acf + (sweep - c->series_base);
+}
+
+LAT_D unsigned long long sweep_of(const Ctrl *c, const SweepAt &at)
+{
+    return at.known ? at.sweep : c->sweep + (unsigned long long)at.off;
+}
+
+// By one thread of a launch whose other threads do not read the counter.
+LAT_D void sweep_done(Ctrl *c, const SweepAt &at)
+{
+    if (at.known) c->sweep = at.sweep + 1ull;
+}
+
+// Unflipped sites before sweep `sweep`: the previous sweep's counter (its
+// kernels are done), or the count the series started from.
+LAT_D long long ne_unflipped_before(const Ctrl *c, unsigned long long sweep)
+{
+    return (long long)(sweep > c->series_base ? series_slot(c, sweep - 1ull)[3] : c->unfl_base);
 }
 
 // Field-sum slot of global sweep `sweep`: sum_i eta_i s_i over the state
@@ -261,6 +289,13 @@ struct Geom {
     // kernels): index (self down) << 3 | (# down neighbours).
     uint32_t thr16[16];
     uint32_t always16;
+    // The top 16 bits of the t' table as byte-permute operands, set by
+    // tiled_geom (accept16.cuh).  acc_sym: acc[0..1] = thresholds for 0, 1,
+    // 2, 3 or more unlike neighbours; else acc[0..7] = low bytes (two
+    // words: 0..3 and 4 down neighbours) and high bytes of an up spin, then
+    // of a down spin.
+    uint32_t acc[8];
+    uint32_t acc_sym;
     // 1 when no entry that a spin-1/2 or spin-1 move can reach is
     // never-accept (not always and thr = 0), so the table converts to the
     // t' = thr - 1 form of the byte-parallel 3D / spin-1 kernels.
@@ -353,7 +388,7 @@ cudaError_t launch_measure(const Geom &g, const int8_t *spins, unsigned long lon
 cudaError_t launch_advance(Ctrl *ctrl, unsigned long long k, cudaStream_t st);
 cudaError_t launch_set_ctrl(Ctrl *ctrl, unsigned long long sweep, unsigned long long *series,
                             unsigned long long base, unsigned long long cap, unsigned long long *acf,
-                            unsigned long long *fld, cudaStream_t st);
+                            unsigned long long *fld, unsigned long long unfl_base, cudaStream_t st);
 bool tiled_supported(const Geom &g);
 cudaError_t launch_sweep_tiled(const Geom &g, int tile_w, int tile_h, int off, cudaStream_t st);
 cudaError_t launch_pack_bits(const Geom &g, const int8_t *planar, uint32_t *bits, cudaStream_t st);
@@ -368,14 +403,18 @@ bool bitpacked_supported(const Geom &g);
 bool wide_supported(const Geom &g);
 // fields: per-site field signs are set (g.cpl bit 6; the -h table half
 // follows the first in g.tab, with no never-accept entry)
-cudaError_t launch_sweep_wide(const Geom &g, bool fields, int off, cudaStream_t st);
+// (with at.known: 2D Ising and c-mode North-East lattices only, which
+// sweep_at_known says)
+bool sweep_at_known(const Geom &g);
+cudaError_t launch_sweep_wide(const Geom &g, bool fields, SweepAt at, cudaStream_t st);
 // The paper's random-sub-lattice, random-site sweep (kernels_rsite.cu).
 // balanced: the balance-preserving variant (single-colour rounds, four launches)
 bool rsite_params_ok(const Geom &g, int b, int lambda, bool balanced);
 cudaError_t launch_sweep_rsite(const Geom &g, int8_t *scratch, int b, int lambda, bool balanced, int off,
                                cudaStream_t st);
 bool resident_supported(const Geom &g);
-cudaError_t launch_sweep_resident(const Geom &g, int off, int n_sweeps, cudaStream_t st);
+// at.known: the launch moves the sweep counter on by n_sweeps
+cudaError_t launch_sweep_resident(const Geom &g, SweepAt at, int n_sweeps, cudaStream_t st);
 size_t resident_smem_bytes(const Geom &g);
 // geoms: compact-table descriptors (tiled_geom); n[i]: sweeps for lattice i
 cudaError_t launch_batch_resident(const Geom *geoms, const long long *n, int n_lat, long long done, int chunk,
@@ -410,10 +449,27 @@ bool any_supported(const Geom &g);
 // per item (0: the size-based default)
 int any_items(const Geom &g, int passes);
 int batch_any_grid(bool ne);
-// aligned: every lattice of the items has L % 32 == 0 (16-byte aligned
-// rows); cmode (with ne): every lattice of the items is a c-mode North-East one
+// aligned: every lattice of the items has L % 32 == 0 (16-byte aligned rows)
 cudaError_t launch_batch_any(const Geom *geoms, const uint2 *items, int n_items, unsigned *next_item, int colour,
-                             bool ne, bool cmode, bool aligned, int passes, int grid, cudaStream_t st);
+                             bool ne, bool aligned, int passes, int grid, cudaStream_t st);
+// c-mode North-East lattices without disorder, any even L (kernels_ne.cu);
+// batch items as any_items
+bool ne_walk_supported(const Geom &g);
+cudaError_t launch_sweep_ne(const Geom &g, SweepAt at, cudaStream_t st);
+int batch_ne_grid();
+cudaError_t launch_batch_ne(const Geom *geoms, const uint2 *items, int n_items, unsigned *next_item, int colour,
+                            bool aligned, int passes, int grid, cudaStream_t st);
+// Many sweeps in one cooperative launch (kernels_band.cu): the CTAs hold
+// bands of rows in shared memory.  band_count_for: CTAs for one lattice on
+// the whole GPU (0: not supported or too large).  mail: band_mail_bytes() of
+// device memory, zeroed once; epoch: at least every packet mark sent through
+// it before, the launch marks up to epoch + 2 n; err: host-visible word set
+// when a bounded wait gave up (mail must then be zeroed again).  Advances
+// ctrl->sweep.
+int band_count_for(const Geom &g);
+size_t band_mail_bytes(const Geom &g, int bands);
+cudaError_t launch_sweep_band(const Geom &g, bool fields, int bands, unsigned long long sweep0, int n, void *mail,
+                              unsigned epoch, int *err, cudaStream_t st);
 // batched engine
 Geom tiled_geom(const Geom &g);
 int tiles_of(const Geom &g, int tile_h);

@@ -1,0 +1,134 @@
+// ne_walk.cuh -- the pieces of a c-mode North-East half-sweep shared by the
+// streaming kernels (kernels_ne.cu) and the band-resident ones
+// (kernels_band.cu): the constraint and the certain moves of a 16-site
+// chunk, the queued draws, counters.
+#pragma once
+
+#include "accept16.cuh"
+#include "wide_common.cuh"
+
+#if defined(__CUDACC__)
+namespace lat {
+namespace {
+
+constexpr int kNeQueue = 32 + 4 * 32; // jobs per warp: under 32 left over, 4 per lane new
+constexpr uint32_t kB1 = 0x02020202u; // one copy of a byte's "down" flag
+
+// A queued group: Philox group index, byte offset of its first site in the
+// colour's plane, flags of the sites whose draw decides, and the west (bit 1)
+// and south (bit 2) neighbours' flags (colour 1).
+struct __align__(16) NeJob {
+    uint32_t g, at, cand, ws;
+};
+
+// The draw threshold (accept iff u <= K), and the flag flip that marks the
+// state which draws (0: down spins, all ones: up spins).
+struct NeRate {
+    uint32_t K, inv;
+};
+
+LAT_D NeRate ne_rate(const uint32_t *thr16)
+{
+    // index sd << 3 | nd; in c-mode every nd has the same entry
+    const bool up_draws = thr16[8] == 0xFFFFFFFFu && thr16[0] != 0xFFFFFFFFu;
+    return NeRate{up_draws ? thr16[0] : thr16[8], up_draws ? 0xFFFFFFFFu : 0u};
+}
+
+// Where a queued move is applied: the colour's spins (row pitch `pitch`),
+// its persistence bytes (one per group, at a quarter of the spins' offset)
+// and the reference plane 1 (row pitch `half`, first row y0).
+struct NePlanes {
+    uint8_t *spins, *flags;
+    const int8_t *ref;
+    uint32_t y0, half, pitch;
+};
+
+// One queued group: draw, accept, apply.
+template <bool kRef>
+LAT_D void ne_job(const NePlanes &p, const PhiloxPre &pp, const NeRate rate, const NeJob job, uint32_t colour,
+                  Counts &cnt, uint32_t flag_at = 0xFFFFFFFFu)
+{
+    const U4 u = philox_item(pp, job.g, colour);
+    // all ones where u > K
+    auto above = [&](uint32_t x) {
+        uint32_t d, m;
+        asm("sub.cc.u32 %0, %2, %3;\n\tsubc.u32 %1, 0, 0;" : "=r"(d), "=r"(m) : "r"(rate.K), "r"(x));
+        return m;
+    };
+    const uint32_t m0 = above(u.x), m1 = above(u.y), m2 = above(u.z), m3 = above(u.w);
+    const uint32_t lo = (m0 & 0x000000FFu) | (m1 & 0xFFFFFF00u), hi = (m2 & 0x00FFFFFFu) | (m3 & 0xFF000000u);
+    const uint32_t rej = (lo & 0x0000FFFFu) | (hi & 0xFFFF0000u);
+    const uint32_t f = job.cand & ~rej & kB1;   // accepted moves
+    if (f == 0u) return;
+    const uint8_t now = rate.inv ? 0xFFu : 0x01u;   // the spin after the move
+    uint8_t *d = p.spins + job.at;
+#pragma unroll
+    for (int b = 0; b < 4; ++b)
+        if (f & (2u << (8 * b))) d[b] = now;
+    const uint32_t bits = (uint32_t)dot4(f, 0x08040201u, 0) >> 1;
+    uint8_t *fl = p.flags + (flag_at == 0xFFFFFFFFu ? job.at >> 2 : flag_at);
+    const uint32_t was = *fl;
+    *fl = (uint8_t)(was | bits);
+    cnt.unfl -= __popc(bits & ~was);
+    if (colour == 1u) {
+        // north and east are up, so a site's neighbour sum is 4 - 2 (west down + south down)
+        const int n = __popc(f), side = __popc(f & job.ws) + __popc((f << 1) & job.ws), sg = rate.inv ? -2 : 2;
+        cnt.mag += sg * n;
+        cnt.bond += sg * (4 * n - 2 * side);
+        if constexpr (kRef) {
+            const uint32_t row = job.at / p.pitch;
+            const int8_t *r = p.ref + (size_t)(p.y0 + row) * p.half + (job.at - row * p.pitch);
+#pragma unroll
+            for (int b = 0; b < 4; ++b)
+                if (f & (2u << (8 * b))) cnt.acf += sg * (int)r[b];
+        }
+    }
+}
+
+// The moves of a chunk that need no draw: north U, south D, east E, west W,
+// own spins S -> spins after the certain moves Sn, flags of those moves
+// (sure), of the sites whose draw decides (cand) and of their west and south
+// neighbours (ws), and which groups need a draw.
+template <bool kFull>
+LAT_D void ne_moves(const uint32_t (&U)[4], const uint32_t (&D)[4], const uint32_t (&E)[4], const uint32_t (&W)[4],
+                    const uint32_t (&S)[4], const uint32_t (&vm)[4], const NeRate rate, uint32_t (&cand)[4],
+                    uint32_t (&sure)[4], uint32_t (&ws)[4], uint32_t (&Sn)[4], bool (&need)[4])
+{
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+        const uint32_t open = kFull ? ~(U[w] | E[w]) : ~(U[w] | E[w]) & vm[w];
+        cand[w] = open & (S[w] ^ rate.inv);
+        sure[w] = open & ~(S[w] ^ rate.inv);
+        need[w] = (cand[w] & kB1) != 0u;
+        Sn[w] = S[w] ^ (sure[w] & 0xFEFEFEFEu);
+        ws[w] = (W[w] & kB1) | (D[w] & ~kB1);
+    }
+}
+
+// Persistence bits of the certain moves: byte w = group w, bit q = its site q.
+LAT_D uint32_t ne_changed(const uint32_t (&sure)[4])
+{
+    int c = dot4(sure[3] & kB1, 0x08040201u, 0);
+#pragma unroll
+    for (int w = 2; w >= 0; --w) c = dot4(sure[w] & kB1, 0x08040201u, c * 256);
+    return (uint32_t)c >> 1;
+}
+
+// Colour 1: bonds of the new spins, both planes' magnetisation.
+LAT_D void ne_count(const uint32_t (&Sn)[4], const uint32_t (&U)[4], const uint32_t (&D)[4], const uint32_t (&O)[4],
+                    const uint32_t (&X)[4], const uint32_t (&vm)[4], Counts &cnt)
+{
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+        const uint32_t Sv = Sn[w] & vm[w], one = 0x01010101u & vm[w];
+        cnt.bond = dot4(Sv, U[w], cnt.bond);
+        cnt.bond = dot4(Sv, D[w], cnt.bond);
+        cnt.bond = dot4(Sv, O[w], cnt.bond);
+        cnt.bond = dot4(Sv, X[w], cnt.bond);
+        cnt.mag = dot4(Sn[w], one, dot4(O[w], one, cnt.mag));
+    }
+}
+
+}  // namespace
+}  // namespace lat
+#endif

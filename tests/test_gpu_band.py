@@ -1,0 +1,77 @@
+"""The band-resident kernel (many sweeps per launch, rows of a lattice split
+over the SMs) against the CPU oracle, bit for bit: two bands to one per SM,
+bands of two rows, rows of any byte alignment, partial chunks and groups,
+odd and even sweep counts mixed with single sweeps (other kernels), every
+table kind, disorder, a reference state."""
+import numpy as np
+import pytest
+
+import oracle
+import paper_1209_0296_gb300 as lt
+
+pytestmark = pytest.mark.gpu
+
+
+def _run(args, seed, init, calls, reference=False, bonds=None, fields=None):
+    g = lt.Lattice(*args, seed=seed, init=init)
+    o = oracle.Lattice(*args, seed=seed, init=init)
+    g.set_kernel(lt.KERNEL_WIDE)
+    if bonds is not None:
+        g.set_couplings(bonds)
+        o.set_couplings(bonds)
+    if fields is not None:
+        g.set_fields(fields)
+        o.set_fields(fields)
+    if reference:
+        g.set_reference()
+        o.set_reference()
+    done = 0
+    for n in calls:
+        ser_o = o.sweep(n)
+        g.sweep(n)
+        ser = g.series(done, n)
+        for k in ("bond", "mag", "up") + (("unflipped",) if args[3] == lt.NE else ()):
+            assert np.array_equal(ser[k], ser_o[k]), (k, n)
+        if reference:
+            assert np.array_equal(g.autocorrelation(done, n, m=0.0)[0], ser_o["overlap"])
+        if fields is not None:
+            assert np.array_equal(g.field_series(done, n), ser_o["field"])
+        spins, flags, _ = g.get_state()
+        assert np.array_equal(spins, o.spins), n
+        if args[3] == lt.NE:
+            assert np.array_equal(flags, o.flags), n
+        done += n
+    g.close()
+
+
+CALLS = [5, 1, 4, 7]
+
+
+@pytest.mark.parametrize("L", [4, 6, 34, 62, 64, 100, 130, 250, 304, 306, 610])
+@pytest.mark.parametrize("J,h", [(1.0, 0.0), (1.0, 0.3), (-0.7, 0.0), (0.0, 0.0)])
+def test_ising(L, J, h):
+    _run((2, L, 1, lt.ISING, J, h, 2.3), 17 + L, lt.INIT_RANDOM, CALLS, reference=L in (6, 64, 250))
+
+
+@pytest.mark.parametrize("L,c", [(4, 0.4), (6, 0.3), (34, 0.7), (62, 0.1), (64, 0.5), (130, 0.3), (304, 0.05),
+                                 (306, 0.9), (510, 0.35)])
+def test_north_east(L, c):
+    _run((2, L, 1, lt.NE, 0.0, 0.0, c), 5 + L, lt.INIT_EQUILIBRIUM, CALLS, reference=L in (6, 64, 306))
+
+
+@pytest.mark.parametrize("model", [lt.ISING, lt.NE])
+@pytest.mark.parametrize("L", [1000, 2050])
+def test_large(L, model):
+    a = (0.0, 0.0, 0.25) if model == lt.NE else (1.0, 0.0, 2.269185)
+    _run((2, L, 1, model) + a, 3, lt.INIT_EQUILIBRIUM if model == lt.NE else lt.INIT_RANDOM, [4])
+
+
+@pytest.mark.parametrize("L", [32, 96, 320])
+@pytest.mark.parametrize("kind", ["bonds", "bonds_h", "fields", "both"])
+def test_disorder(L, kind):
+    rng = np.random.default_rng(L)
+    sign = lambda n: np.where(rng.random(n) < 0.5, -1, 1).astype(np.int8)
+    bonds = sign(2 * L * L) if kind != "fields" else None
+    fields = sign(L * L) if kind in ("fields", "both") else None
+    h = 0.0 if kind == "bonds" else 0.6
+    _run((2, L, 1, lt.ISING, 1.0, h, 1.7), 9, lt.INIT_RANDOM, CALLS, reference=L == 96, bonds=bonds, fields=fields)
