@@ -13,6 +13,7 @@
 // table and sweep counter, so its result is bit-identical to running it
 // alone.
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <map>
 #include <mutex>
@@ -40,6 +41,8 @@ struct BatchSlot {
     int res_geoms_cap = 0;
     long long *d_res_n = nullptr;
     int res_n_cap = 0;
+    Geom *d_band_geoms = nullptr;   // lattices of the band-resident launches
+    int band_geoms_cap = 0;
     char *h_pin = nullptr;     // pinned staging of the uploads
     size_t h_cap = 0;
     cudaEvent_t done = nullptr;
@@ -72,6 +75,10 @@ struct lattice_batch {
     unsigned *d_counters = nullptr;
     int grid_tiled_ising = 0, grid_tiled_ne = 0, grid_generic = 0, grid_wide[2] = {0, 0}, grid_potts = 0;
     int grid_any[3] = {0, 0, 0};  // 2D any-L: Ising, North-East at T, North-East in c-mode
+    // band-resident lattices: boundary-row packets (kernels_band_batch.cu)
+    void *d_mail = nullptr;
+    size_t mail_cap = 0;
+    unsigned mail_epoch = 0;
     // resident lattices
     cudaStream_t res_stream = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
@@ -318,6 +325,145 @@ int run_resident(lattice_batch *b, BatchSlot &sl, const std::vector<std::pair<la
     if (e == cudaSuccess) e = cudaEventRecord(b->ev_join, b->res_stream);
     if (e != cudaSuccess) return cuda_fail(e, "batch resident launch");
     return LAT_OK;
+}
+
+using Work = std::vector<std::pair<lattice *, int64_t>>;
+using BandList = std::vector<std::pair<const Geom *, long long>>;
+
+// Lattices that run together in one band-resident launch.
+struct BandGroup {
+    Work work;
+    std::vector<int> ctas;
+    double us;   // estimate
+};
+
+BandList band_list(const Work &w)
+{
+    BandList l;
+    for (auto &pr : w) l.emplace_back(&pr.first->geom, (long long)pr.second);
+    return l;
+}
+
+// Split `work` into groups for band-resident launches and the rest for the
+// step loop (in place).  A group's lattices share the SMs for all their
+// sweeps, so lattices of like work go together; the step loop keeps them all
+// when it is estimated to be done sooner (many lattices much smaller than an
+// SM's share).  Its estimate: 350 site updates per ns and 25 us a step, what
+// it measured on the served mix.
+// at_least: fewer such lattices stay on the step loop.  The server asks for
+// two: between the step loop's kernels a small request that arrives during a
+// lone lattice's round starts at once, a band launch keeps every SM until
+// the round is over.
+void plan_bands(Work &work, std::vector<BandGroup> &groups, size_t at_least)
+{
+    constexpr int64_t kMinSweeps = 4;   // below, the launch and the copies in and out are most of the time
+    Work fit, rest;
+    for (auto &pr : work) {
+        const lattice *lt = pr.first;
+        const bool ok = pr.second >= kMinSweeps && !lt->graph_pinned && choose_kernel(lt) == LAT_KERNEL_WIDE &&
+                        band_min_ctas(lt->geom) > 0;
+        (ok ? fit : rest).push_back(pr);
+    }
+    if (fit.size() < at_least) return;
+    std::stable_sort(fit.begin(), fit.end(), [](const auto &a, const auto &c) {
+        return (double)a.first->P.N * (double)a.second > (double)c.first->P.N * (double)c.second;
+    });
+    double updates = 0.0, band_us = 0.0;
+    int64_t steps = 0;
+    std::vector<BandGroup> out;
+    Work cur;
+    std::vector<int> ctas;
+    int used = 0;
+    auto close = [&]() {
+        if (cur.empty()) return;
+        BandGroup g{cur, {}, 0.0};
+        g.us = band_share(band_list(cur), g.ctas);
+        band_us += g.us + 10.0;
+        out.push_back(std::move(g));
+        cur.clear();
+        used = 0;
+    };
+    for (auto &pr : fit) {
+        const int c = band_min_ctas(pr.first->geom);
+        if (used + c > band_sms()) close();
+        cur.push_back(pr);
+        used += c;
+        updates += (double)pr.first->P.N * (double)pr.second;
+        steps = std::max(steps, pr.second);
+    }
+    close();
+    if (band_us > updates / 350e3 + 25.0 * (double)steps) return;
+    work.swap(rest);
+    groups.swap(out);
+}
+
+// Launch the groups one after another on the batch stream.
+int run_bands(lattice_batch *b, BatchSlot &sl, size_t at, std::vector<BandGroup> &groups)
+{
+    size_t n = 0, mail = 0;
+    for (auto &g : groups) {
+        n += g.work.size();
+        mail = std::max(mail, band_batch_mail_bytes(band_list(g.work), g.ctas));
+    }
+    std::vector<Geom> geoms;
+    geoms.reserve(n);
+    for (auto &g : groups)
+        for (auto &pr : g.work) {
+            if (pr.first->band_err == nullptr && (pr.first->band_err = band_error_word()) == nullptr) return LAT_ENOMEM;
+            geoms.push_back(tiled_geom(pr.first->geom));
+        }
+    int rc = grow(&sl.d_band_geoms, sl.band_geoms_cap, (int)n, b->stream);
+    if (rc != LAT_OK) return rc;
+    cudaError_t e = cudaSuccess;
+    if (mail > b->mail_cap) {
+        void *p = nullptr;
+        e = dev_alloc(&p, mail, b->stream);
+        if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? LAT_ENOMEM : cuda_fail(e, "batch packets");
+        dev_free(b->d_mail, b->stream);
+        b->d_mail = p;
+        b->mail_cap = mail;
+        b->mail_epoch = 1u << 30;   // clear below
+    }
+    if (sl.h_cap < at + n * sizeof(Geom) + 64) {
+        // growing frees staging that earlier uploads of this run may still read
+        e = cudaStreamSynchronize(b->stream);
+        if (e != cudaSuccess) return cuda_fail(e, "batch staging");
+        rc = ensure_pinned(sl, at + n * sizeof(Geom) + 64);
+        if (rc != LAT_OK) return rc;
+    }
+    stage(sl, at, sl.d_band_geoms, geoms.data(), n, b->stream, e);
+    size_t first = 0;
+    for (auto &g : groups) {
+        // launches of well under a second each: every lattice's sweeps in equal parts
+        const int parts = (int)std::max(1.0, std::ceil(g.us / 2.5e5));
+        for (int k = 0; k < parts && e == cudaSuccess; ++k) {
+            BandList l;
+            std::vector<unsigned long long> sweep0;
+            std::vector<int *> err;
+            long long most = 0;
+            for (auto &pr : g.work) {
+                const long long from = pr.second * k / parts, to = pr.second * (k + 1) / parts;
+                l.emplace_back(&pr.first->geom, to - from);
+                sweep0.push_back((unsigned long long)(pr.first->sweeps + from));
+                err.push_back(pr.first->band_err);
+                most = std::max(most, to - from);
+            }
+            if (b->mail_epoch >= 1u << 30) {
+                e = cudaMemsetAsync(b->d_mail, 0, b->mail_cap, b->stream);
+                b->mail_epoch = 0;
+            }
+            if (e == cudaSuccess) {
+                BandTurn turn(b->stream);
+                e = turn.status;
+                if (e == cudaSuccess)
+                    e = launch_batch_band(sl.d_band_geoms + first, l, sweep0, err, g.ctas, b->d_mail, b->mail_epoch,
+                                          b->stream);
+            }
+            b->mail_epoch += 2u * (unsigned)most;
+        }
+        first += g.work.size();
+    }
+    return e == cudaSuccess ? LAT_OK : cuda_fail(e, "batch band launch");
 }
 
 // The work lists of one phase (the first n_active lattices of `work`),
@@ -585,14 +731,30 @@ int lattice_batch_run(lattice_batch_t *b)
     }
     for (auto &pr : res) pr.first->sweeps += pr.second;
     work.swap(rest);
+    // Lattices that fit the chip's shared memory: all their sweeps in a few launches.
+    std::vector<BandGroup> groups;
+    plan_bands(work, groups, b->caller_orders ? 2 : 1);
+    // the resident and band lattices' uploads sit at the front of the staging
+    size_t res_bytes = res.empty() ? 0 : ((res.size() * (sizeof(Geom) + sizeof(long long)) + 64 + 15) & ~(size_t)15);
+    std::vector<std::pair<lattice *, int64_t>> banded;
+    if (!groups.empty()) {
+        mark_start();
+        int rc = run_bands(b, sl, res_bytes, groups);
+        if (rc != LAT_OK) return rc;
+        for (auto &g : groups)
+            for (auto &pr : g.work) {
+                pr.first->sweeps += pr.second;
+                banded.push_back(pr);
+            }
+        res_bytes = (res_bytes + banded.size() * sizeof(Geom) + 64 + 15) & ~(size_t)15;
+        b->last_passes = 0;
+        b->last_gsteps = kGraphSteps;
+    }
     // Run in phases: all lattices until the smallest remaining count is
     // done, then drop it, and so on.  Every phase's descriptors and items are
     // built first and uploaded together, so the phases are queued back to
     // back with no host synchronisation between them.
     std::sort(work.begin(), work.end(), [](const auto &a, const auto &c) { return a.second > c.second; });
-    // the resident lattices' uploads sit at the front of the staging
-    const size_t res_bytes =
-        res.empty() ? 0 : ((res.size() * (sizeof(Geom) + sizeof(long long)) + 64 + 15) & ~(size_t)15);
     BatchTune tune{0, kGraphSteps};
     if (!work.empty()) {
         const uint64_t key = composition_key(work);
@@ -663,7 +825,7 @@ int lattice_batch_run(lattice_batch_t *b)
     if (e == cudaSuccess) sl.used = true;
     if (!b->caller_orders) {
         streams.clear();
-        for (auto *list : {&work, &res})
+        for (auto *list : {&work, &res, &banded})
             for (auto &pr : *list) {
                 cudaStream_t ls = pr.first->stream;
                 if (ls != b->stream && std::find(streams.begin(), streams.end(), ls) == streams.end())
@@ -720,6 +882,7 @@ void lattice_batch_destroy(lattice_batch_t *b)
         dev_free(sl.d_ctrls, b->stream);
         dev_free(sl.d_res_geoms, b->stream);
         dev_free(sl.d_res_n, b->stream);
+        dev_free(sl.d_band_geoms, b->stream);
         if (sl.done) cudaEventDestroy(sl.done);
     }
     cudaStreamSynchronize(b->stream);
@@ -727,6 +890,7 @@ void lattice_batch_destroy(lattice_batch_t *b)
         if (sl.h_pin) cudaFreeHost(sl.h_pin);
     for (cudaEvent_t ev : b->ev_streams) cudaEventDestroy(ev);
     dev_free(b->d_counters, b->stream);
+    dev_free(b->d_mail, b->stream);
     if (b->res_stream) cudaStreamDestroy(b->res_stream);
     if (b->ev_fork) cudaEventDestroy(b->ev_fork);
     if (b->ev_join) cudaEventDestroy(b->ev_join);

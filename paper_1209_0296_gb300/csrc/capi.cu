@@ -262,7 +262,7 @@ int *band_error_word()
     static std::mutex mu;
     static int *page = nullptr;
     static unsigned next = 0;
-    constexpr unsigned kWords = 1024;
+    constexpr unsigned kWords = 16384;
     std::lock_guard<std::mutex> g(mu);
     if (page == nullptr && cudaHostAlloc((void **)&page, kWords * sizeof(int), cudaHostAllocPortable) != cudaSuccess) {
         (void)cudaGetLastError();

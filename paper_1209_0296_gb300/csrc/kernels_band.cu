@@ -1,608 +1,37 @@
-// kernels_band.cu -- many sweeps in one launch for 2D spin-1/2 lattices that
-// fit the chip's shared memory: every CTA keeps a band of rows resident and
-// neighbouring bands exchange their boundary rows.
-//
-// With two launches per sweep a lattice of a million sites spends most of
-// its time between kernels: a launch costs about 2.5 us of start-up, memory
-// latency and drain, its work 0.6 us.  Here one cooperative launch runs all
-// sweeps of a call.  CTA b holds rows [y0, y1) of both colour planes in
-// shared memory, rows at 16-byte alignment whatever L is, and updates a
-// colour in place.  The new values of its first and last row go to the two
-// neighbouring bands as packets of 4 data bytes and a 4-byte half-sweep
-// number in one 64-bit word; the reader polls the packets themselves, so a
-// row costs one trip through L2 and no fence or flag.  Interior rows come
-// first, so the neighbours' packets are usually there before they are asked
-// for, and the next half-sweep's first draws are made before that.
-// A packet is overwritten two half-sweeps later, after the reader's own
-// packet of the half-sweep in between has arrived.
-//
-// A wait is bounded: when it gives up the launch ends normally and the host
-// sees the error word (LAT_ETIMEOUT).
+// kernels_band.cu -- the band-resident kernel (band.cuh) of one lattice: a
+// grid of one CTA per SM, all sweeps of a call in one cooperative launch.
 #include <algorithm>
 #include <mutex>
 
-#include "ising_walk.cuh"
-#include "ne_walk.cuh"
+#include "band.cuh"
 
 namespace lat {
 
 namespace {
 
-constexpr int kBandThreads = 512;
-constexpr int kBandWarps = kBandThreads / 32;
-constexpr unsigned kSpinLimit = 1u << 24;   // polls of about half a microsecond: ten seconds
-constexpr uint32_t kAbortBytes = 128;       // the abort word's line, before a lattice's packets
-constexpr size_t kBandMaxSmem = 224 * 1024;
-
-// What a CTA runs: band `band` of `bands` of one lattice.
-struct BandPart {
-    uint32_t band, bands, epoch;
-    uint32_t pad;
-    unsigned long long sweep0;   // sweeps done before the launch
-    int n;                       // sweeps to run
-    int pad2;
-};
-
-struct BandShared {
-    uint32_t sthr[16];
-    int sum[2][5];   // a sweep's bond, mag, up, unflipped, overlap: two sweeps in turn
-    int fld;
-    int bad;         // a wait gave up
-    int unfl;        // unflipped sites of the band
-};
-
-// The launch's view of a band.
-struct Band {
-    uint32_t y0, nr, half, pitch, cpr, L, G;
-    bool al;                     // rows are 16-byte aligned in global memory
-    size_t plane;
-    const int8_t *src;           // spins before the launch
-    uint32_t up, dn;             // rows above and below the band
-    unsigned *abort;             // set when a wait of the launch gave up
-    // packet rows of colour 0 (colour 1: + cpr packet pairs): this band's
-    // first and last row, the last row of the band above, the first below
-    ulonglong2 *first, *last;
-    const ulonglong2 *above, *below;
-};
-
-LAT_D Band band_of(const Geom &g, const BandPart &p, uint8_t *mail)
-{
-    Band b;
-    uint32_t y1;
-    b.L = (uint32_t)g.L;
-    band_rows(p.band, p.bands, b.L, b.y0, y1);
-    b.nr = y1 - b.y0;
-    b.half = g.half;
-    b.cpr = (g.half + 15u) >> 4;
-    b.pitch = 16u * b.cpr;
-    b.G = g.G;
-    b.al = (g.half & 15u) == 0u;
-    b.plane = (size_t)g.plane;
-    b.src = (p.sweep0 & 1) ? g.s[1] : g.s[0];
-    b.up = b.y0 == 0u ? b.L - 1u : b.y0 - 1u;
-    b.dn = y1 == b.L ? 0u : y1;
-    b.abort = reinterpret_cast<unsigned *>(mail);
-    ulonglong2 *m = reinterpret_cast<ulonglong2 *>(mail + kAbortBytes);
-    const size_t row = 4u * b.cpr;   // both colours, two packet pairs a chunk
-    const uint32_t above = p.band == 0u ? p.bands - 1u : p.band - 1u, below = p.band + 1u == p.bands ? 0u : p.band + 1u;
-    b.first = m + (size_t)p.band * 2u * row;
-    b.last = b.first + row;
-    b.above = m + (size_t)above * 2u * row + row;
-    b.below = m + (size_t)below * 2u * row;
-    return b;
-}
-
-LAT_D ulonglong2 ld_pair(const ulonglong2 *q)
-{
-    ulonglong2 v;
-    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(q) : "memory");
-    return v;
-}
-
-// Send 16 bytes as packets marked `tag`.
-LAT_D void mail_put(ulonglong2 *q, uint32_t tag, const uint32_t (&v)[4])
-{
-    const unsigned long long t = (unsigned long long)tag << 32;
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-        asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(q + i), "l"(t | v[2 * i]), "l"(t | v[2 * i + 1])
-                     : "memory");
-}
-
-// Wait for the 16 bytes marked `tag`; false when the wait gave up.
-LAT_D bool mail_take(const ulonglong2 *q, uint32_t tag, unsigned *abort, uint32_t (&v)[4])
-{
-    for (unsigned i = 0;; ++i) {
-        const ulonglong2 a = ld_pair(q), b = ld_pair(q + 1);
-        v[0] = (uint32_t)a.x;
-        v[1] = (uint32_t)a.y;
-        v[2] = (uint32_t)b.x;
-        v[3] = (uint32_t)b.y;
-        if ((uint32_t)(a.x >> 32) == tag && (uint32_t)(a.y >> 32) == tag && (uint32_t)(b.x >> 32) == tag &&
-            (uint32_t)(b.y >> 32) == tag)
-            return true;
-        if ((i & 1023u) == 1023u && (i >= kSpinLimit || *reinterpret_cast<volatile unsigned *>(abort) != 0u)) {
-            *reinterpret_cast<volatile unsigned *>(abort) = 1u;
-            return false;
-        }
-    }
-}
-
-// Local rows in the order they are visited: interior first, then the first
-// and the last.
-LAT_D uint32_t band_row(uint32_t o, uint32_t nr) { return o + 2u < nr ? o + 1u : (o + 2u == nr ? 0u : nr - 1u); }
-
-// nr rows of half bytes, global (row pitch half) -> shared (row pitch
-// pitch, a multiple of 4), whole words at any alignment.
-LAT_D void rows_in(const int8_t *from, uint32_t half, uint32_t nr, uint8_t *to, uint32_t pitch)
-{
-    if ((half & 15u) == 0u && pitch == half) {
-        const uint4 *q = reinterpret_cast<const uint4 *>(from);
-        for (uint32_t i = threadIdx.x; i < nr * (half >> 4); i += blockDim.x) reinterpret_cast<uint4 *>(to)[i] = q[i];
-        return;
-    }
-    const uint32_t wpr = (half + 3u) >> 2;
-    for (uint32_t i = threadIdx.x; i < nr * wpr; i += blockDim.x) {
-        const uint32_t r = i / wpr, w = i - r * wpr;
-        const uintptr_t a = reinterpret_cast<uintptr_t>(from + (size_t)r * half + 4u * w);
-        const uint32_t sh = (uint32_t)(a & 3u), nv = min(4u, half - 4u * w);
-        const uint32_t *q = reinterpret_cast<const uint32_t *>(a - sh);
-        const uint32_t hi = nv + sh > 4u ? q[1] : 0u;
-        *reinterpret_cast<uint32_t *>(to + (size_t)r * pitch + 4u * w) = __funnelshift_r(q[0], hi, 8u * sh);
-    }
-}
-
-// The way back: only the rows' own bytes are written.
-LAT_D void rows_out(const uint8_t *from, uint32_t pitch, uint32_t nr, int8_t *to, uint32_t half)
-{
-    if ((half & 15u) == 0u && pitch == half) {
-        uint4 *q = reinterpret_cast<uint4 *>(to);
-        for (uint32_t i = threadIdx.x; i < nr * (half >> 4); i += blockDim.x)
-            q[i] = reinterpret_cast<const uint4 *>(from)[i];
-    } else if ((half & 3u) == 0u && (reinterpret_cast<uintptr_t>(to) & 3u) == 0u) {
-        const uint32_t wpr = half >> 2;
-        for (uint32_t i = threadIdx.x; i < nr * wpr; i += blockDim.x) {
-            const uint32_t r = i / wpr, w = i - r * wpr;
-            *reinterpret_cast<uint32_t *>(to + (size_t)r * half + 4u * w) =
-                *reinterpret_cast<const uint32_t *>(from + (size_t)r * pitch + 4u * w);
-        }
-    } else {
-        for (uint32_t i = threadIdx.x; i < nr * half; i += blockDim.x) {
-            const uint32_t r = i / half, x = i - r * half;
-            to[i] = (int8_t)from[(size_t)r * pitch + x];
-        }
-    }
-}
-
-LAT_D void smem_words(const uint8_t *q, uint32_t (&v)[4]) { load_words<4>(reinterpret_cast<const int8_t *>(q), v); }
-
-// The block's sweep counters: warp sums into sh.sum[par]; after the next
-// barrier warp 1 adds them to the sweep's slots and clears them.
-LAT_D void band_count(BandShared &sh, int par, const Counts &c, bool ne, bool ref)
-{
-    const int lane = threadIdx.x & 31;
-    const int v[5] = {c.bond, c.mag, c.up, c.unfl, c.acf};
-#pragma unroll
-    for (int i = 0; i < 5; ++i) {
-        if ((i == 3 && !ne) || (i == 4 && !ref)) continue;
-        const int s = __reduce_add_sync(0xffffffffu, v[i]);
-        if (lane == 0) atomicAdd(&sh.sum[par][i], s);
-    }
-}
-
-LAT_D void band_post(BandShared &sh, int par, const Geom &g, unsigned long long sweep, bool ne, bool ref)
-{
-    const int i = (int)threadIdx.x - 32;
-    if (i < 0 || i >= 5 || (i == 3 && !ne) || (i == 4 && !ref)) return;
-    long long v = sh.sum[par][i];
-    if (i == 3) {
-        sh.unfl += (int)v;   // newly flipped sites, negative
-        v = sh.unfl;
-    }
-    sh.sum[par][i] = 0;
-    add_counter(i < 4 ? series_slot(g.ctrl, sweep) + i : acf_slot(g.ctrl, sweep), v);
-}
-
-// Exact flips of one chunk from full 32-bit draws (rare; a call keeps it out
-// of the sweep's registers).
-struct Chunk16 {
-    Nbr n[4];
-    uint32_t S[4];
-};
-__device__ __noinline__ uint4 band_exact(const uint32_t *sthr, unsigned long long sweep, uint32_t key0, uint32_t key1,
-                                         uint32_t g0, uint32_t colour, const Chunk16 c)
-{
-    PhiloxPre pp;
-    philox_prepare(pp, (uint32_t)sweep, (uint32_t)(sweep >> 32), key0, key1);
-    uint32_t F[4];
-#pragma unroll 1
-    for (int w = 0; w < 4; ++w)
-        F[w] = ~reject4_exact(sthr, c.n[w], c.S[w], philox_item(pp, g0 + (uint32_t)w, colour)) & 0xFEFEFEFEu;
-    return make_uint4(F[0], F[1], F[2], F[3]);
-}
-
-// The other plane's row shifted towards the side neighbour that is not at the
-// same index (shifted_row), row and its wrap-around read from shared memory.
-template <bool kFull>
-LAT_D void band_shifted(const ChunkCol<kFull> &cc, bool odd, const uint8_t *row, const uint32_t (&O)[4], uint32_t (&X)[4])
-{
-    if constexpr (kFull) {   // whole words: the one after the chunk, or the one before it
-        const uint32_t nb = *reinterpret_cast<const uint32_t *>(row + (odd ? cc.jn : cc.jp - 3u));
-#pragma unroll
-        for (int w = 0; w < 4; ++w)
-            X[w] = odd ? __funnelshift_r(O[w], w == 3 ? nb : O[w + 1], 8)
-                       : __funnelshift_l(w == 0 ? nb : O[w - 1], O[w], 8);
-    } else {
-        shifted_row<false>(cc, odd, row[odd ? cc.jn : cc.jp], O, X);
-    }
-}
-
-// North and south neighbour words of local row r: from the band, or for its
-// first and last row from the neighbours (before the launch's first
-// half-sweep from the spins themselves).
-struct BandWait {
-    const int8_t *src;   // the other colour's plane before the launch
-    uint32_t tag;        // of the packets to wait for (0: read src)
-    uint32_t mail;       // packet index of the other colour's chunk in a packet row
-};
-
-LAT_D bool band_updown(const Band &b, const BandWait &wt, const uint8_t *other, uint32_t r, uint32_t j0, uint32_t nv,
-                       uint32_t (&U)[4], uint32_t (&D)[4])
-{
-    bool ok = true;
-    auto from = [&](const ulonglong2 *mail, uint32_t y, uint32_t (&v)[4]) {
-        if (wt.tag != 0u) ok = mail_take(mail + wt.mail, wt.tag, b.abort, v) && ok;
-        else if (b.al) load16_any<true>(wt.src + (size_t)y * b.half + j0, nv, v);
-        else load16_any<false>(wt.src + (size_t)y * b.half + j0, nv, v);
-    };
-    const uint8_t *at = other + r * b.pitch + j0;
-    if (r == 0u) from(b.above, b.up, U);
-    else smem_words(at - b.pitch, U);
-    if (r + 1u == b.nr) from(b.below, b.dn, D);
-    else smem_words(at + b.pitch, D);
-    return ok;
-}
-
-// Ising, uniform or with the disorder of Eq. 1.
-template <bool kRef, int kDis, bool kSym, bool kFull>
-LAT_D void band_ising(const Geom &g, const BandPart part, uint8_t *mail, BandShared &sh, uint8_t *smem)
-{
-    const Band b = band_of(g, part, mail);
-    const uint32_t tid = threadIdx.x, pb = b.nr * b.pitch;
-    uint8_t *dis = smem + 2u * pb;
-    for (int c = 0; c < 2; ++c) {
-        rows_in(b.src + c * b.plane + (size_t)b.y0 * b.half, b.half, b.nr, smem + c * pb, b.pitch);
-        if constexpr (kDis != kUniform)
-            rows_in(reinterpret_cast<const int8_t *>(g.cpl) + c * b.plane + (size_t)b.y0 * b.half, b.half, b.nr,
-                    dis + c * pb, b.pitch);
-    }
-    if (tid < 16) sh.sthr[tid] = g.thr16[tid];
-    if (tid < 10) (&sh.sum[0][0])[tid] = 0;
-    if (tid == 10) sh.bad = 0;
-    if (tid == 11) sh.fld = 0;
-    __syncthreads();
-    const uint32_t rsb = (uint32_t)kBandThreads / b.cpr, rr = tid / b.cpr, k = tid - rr * b.cpr;
-    const uint32_t o0 = rr < rsb ? rr : b.nr;   // first visited row ordinal (none: nr)
-    const ChunkCol<kFull> cc = chunk_col<kFull>(k, b.half);
-    const int last = 2 * part.n;
-    uint32_t p01[4], p23[4];
-    PhiloxPre pp;
-    philox_prepare(pp, (uint32_t)part.sweep0, (uint32_t)(part.sweep0 >> 32), g.key0, g.key1);
-    auto draw = [&](uint32_t y, uint32_t colour) {
-        const uint32_t g0 = y * b.G + 4u * k;
-#pragma unroll
-        for (int w = 0; w < 4; ++w) top_halves(philox_item(pp, g0 + (uint32_t)w, colour), p01[w], p23[w]);
-    };
-    if (o0 < b.nr) draw(b.y0 + band_row(o0, b.nr), 0u);
-    Counts cnt;
-    int bad = 0;   // a wait of this thread gave up
-    for (int h = 0; h < last; ++h) {
-        const uint32_t colour = (uint32_t)h & 1u;
-        const unsigned long long sweep = part.sweep0 + (unsigned long long)(h >> 1);
-        uint8_t *mine = smem + colour * pb;
-        const uint8_t *other = smem + (1u - colour) * pb;
-        const BandWait wt{b.src + (1u - colour) * b.plane, h > 0 ? part.epoch + (uint32_t)h : 0u,
-                          2u * ((1u - colour) * b.cpr + k)};
-        for (uint32_t o = o0; o < b.nr; o += rsb) {
-            const uint32_t r = band_row(o, b.nr), y = b.y0 + r, at = r * b.pitch + cc.j0;
-            const bool odd = ((colour + y) & 1u) != 0u;
-            IsingChunk c;
-            uint32_t C[4] = {0, 0, 0, 0}, O[4];
-            if (!band_updown(b, wt, other, r, cc.j0, cc.nv, c.U, c.D)) bad = 1;
-            smem_words(mine + at, c.S);
-            smem_words(other + at, O);
-            if constexpr (kDis != kUniform) smem_words(dis + colour * pb + at, C);
-            band_shifted<kFull>(cc, odd, other + r * b.pitch, O, c.X);
-#pragma unroll
-            for (int w = 0; w < 4; ++w) c.O[w] = O[w];
-            ising_neighbours<kDis>(c, C, odd);
-            uint32_t F[4], Sn[4];
-            if (flips16<kSym>(g.acc, c.n, c.St, p01, p23, F)) {
-                Chunk16 e;
-#pragma unroll
-                for (int w = 0; w < 4; ++w) {
-                    e.n[w] = c.n[w];
-                    e.S[w] = c.St[w];
-                }
-                const uint4 f = band_exact(sh.sthr, sweep, g.key0, g.key1, y * b.G + 4u * k, colour, e);
-                F[0] = f.x;
-                F[1] = f.y;
-                F[2] = f.z;
-                F[3] = f.w;
-            }
-#pragma unroll
-            for (int w = 0; w < 4; ++w) Sn[w] = c.S[w] ^ F[w];
-            store_words<4>(reinterpret_cast<int8_t *>(mine) + at, Sn);
-            const uint32_t box = 2u * (colour * b.cpr + k);
-            if (r == 0u) mail_put(b.first + box, part.epoch + (uint32_t)h + 1u, Sn);
-            if (r + 1u == b.nr) mail_put(b.last + box, part.epoch + (uint32_t)h + 1u, Sn);
-            // the next chunk's draws: this colour's next row, else the next half-sweep's first
-            if (o + rsb < b.nr) {
-                draw(b.y0 + band_row(o + rsb, b.nr), colour);
-            } else {
-                if (colour == 1u) {
-                    const unsigned long long s1 = sweep + 1ull;
-                    philox_prepare(pp, (uint32_t)s1, (uint32_t)(s1 >> 32), g.key0, g.key1);
-                }
-                draw(b.y0 + band_row(o0, b.nr), 1u - colour);
-            }
-            if (colour == 1u) {
-                ising_count<1, kDis, kFull>(c, Sn, cc.vm, cnt);
-#pragma unroll
-                for (int w = 0; w < 4; ++w) cnt.mag = dot4(O[w], 0x01010101u & cc.vm[w], cnt.mag);
-                if constexpr (kRef) {
-                    uint32_t R1[4], R0[4];
-                    const int8_t *r0 = g.ref + (size_t)y * b.half + cc.j0;
-                    load16_any<kFull>(r0 + b.plane, cc.nv, R1);
-                    load16_any<kFull>(r0, cc.nv, R0);
-#pragma unroll
-                    for (int w = 0; w < 4; ++w)
-                        cnt.acf = dot4(Sn[w] & cc.vm[w], R1[w], dot4(O[w] & cc.vm[w], R0[w], cnt.acf));
-                }
-                cnt.up += (int)cc.nv;
-            } else if constexpr (kDis == kFields) {
-                ising_count<0, kDis, kFull>(c, Sn, cc.vm, cnt);
-            }
-        }
-        if (colour == 1u) {
-            cnt.up += cnt.mag / 2;   // nv sites of each plane: up = nv + mag / 2
-            band_count(sh, h >> 1 & 1, cnt, false, kRef);
-            if constexpr (kDis == kFields) {
-                const int f = __reduce_add_sync(0xffffffffu, cnt.fld);
-                if ((tid & 31u) == 0u) atomicAdd(&sh.fld, f);
-            }
-            cnt = Counts();
-        }
-        const int stop = __syncthreads_or(bad);
-        if (colour == 1u) {
-            band_post(sh, h >> 1 & 1, g, sweep, false, kRef);
-            if constexpr (kDis == kFields) {
-                if (tid == 64u) {
-                    add_counter(fld_slot(g.ctrl, sweep), (long long)sh.fld);
-                    sh.fld = 0;   // next added to a barrier later
-                }
-            }
-        }
-        if (stop) {
-            sh.bad = 1;
-            break;
-        }
-    }
-    int8_t *fin = ((part.sweep0 + (unsigned long long)part.n) & 1) ? g.s[1] : g.s[0];
-    for (int c = 0; c < 2; ++c)
-        rows_out(smem + c * pb, b.pitch, b.nr, fin + c * b.plane + (size_t)b.y0 * b.half, b.half);
-}
-
-// North-East in c-mode: the main pass and the per-warp draw queue of
-// ne_walk.cuh on shared memory; boundary rows are sent once their queued
-// moves are done.
-template <bool kRef, bool kFull>
-LAT_D void band_ne(const Geom &g, const BandPart part, uint8_t *mail, BandShared &sh, uint8_t *smem)
-{
-    const Band b = band_of(g, part, mail);
-    const uint32_t tid = threadIdx.x, pb = b.nr * b.pitch, fp = b.pitch >> 2;   // flag bytes per row
-    uint8_t *fl = smem + 2u * pb;
-    NeJob *queue = reinterpret_cast<NeJob *>(smem + ((2u * pb + 2u * b.nr * fp + 15u) & ~15u)) + (tid >> 5) * kNeQueue;
-    int changed = 0;
-    for (int c = 0; c < 2; ++c) {
-        rows_in(b.src + c * b.plane + (size_t)b.y0 * b.half, b.half, b.nr, smem + c * pb, b.pitch);
-        const uint8_t *q = g.flags + ((size_t)c * g.rows + b.y0) * b.G;
-        for (uint32_t i = tid; i < b.nr * b.G; i += blockDim.x) {
-            const uint32_t r = i / b.G, m = i - r * b.G;
-            const uint8_t f = q[i];
-            fl[(c * b.nr + r) * fp + m] = f;
-            changed += __popc((uint32_t)f);
-        }
-    }
-    if (tid < 10) (&sh.sum[0][0])[tid] = 0;
-    if (tid == 10) sh.bad = 0;
-    if (tid == 11) sh.unfl = (int)(2u * b.nr * b.half);
-    __syncthreads();
-    changed = __reduce_add_sync(0xffffffffu, changed);
-    if ((tid & 31u) == 0u) atomicSub(&sh.unfl, changed);
-    __syncthreads();
-    const uint32_t rsb = (uint32_t)kBandThreads / b.cpr, rr = tid / b.cpr, k = tid - rr * b.cpr;
-    const ChunkCol<kFull> cc = chunk_col<kFull>(k, b.half);
-    const NeRate rate = ne_rate(g.thr16);
-    const int lane = (int)(tid & 31u);
-    const unsigned below = (1u << lane) - 1u;
-    const int last = 2 * part.n;
-    PhiloxPre pp;
-    Counts cnt;
-    int bad = 0;   // a wait of this thread gave up
-    for (int h = 0; h < last; ++h) {
-        const uint32_t colour = (uint32_t)h & 1u;
-        const unsigned long long sweep = part.sweep0 + (unsigned long long)(h >> 1);
-        if (colour == 0u) philox_prepare(pp, (uint32_t)sweep, (uint32_t)(sweep >> 32), g.key0, g.key1);
-        uint8_t *mine = smem + colour * pb;
-        const uint8_t *other = smem + (1u - colour) * pb;
-        uint8_t *flc = fl + (size_t)colour * b.nr * fp;
-        const BandWait wt{b.src + (1u - colour) * b.plane, h > 0 ? part.epoch + (uint32_t)h : 0u,
-                          2u * ((1u - colour) * b.cpr + k)};
-        unsigned queued = 0;
-        const NePlanes where{mine, flc, kRef ? g.ref + b.plane : nullptr, b.y0, b.half, b.pitch};
-        auto drain = [&](bool all) {
-            __syncwarp();
-            while (queued >= 32u) {
-                queued -= 32u;
-                ne_job<kRef>(where, pp, rate, queue[queued + lane], colour, cnt);
-            }
-            if (all && (unsigned)lane < queued) ne_job<kRef>(where, pp, rate, queue[lane], colour, cnt);
-            __syncwarp();
-        };
-        for (uint32_t o = rr;; o += rsb) {
-            const bool act = rr < rsb && o < b.nr;
-            if (!__any_sync(0xffffffffu, act)) break;
-            uint32_t cand[4], ws[4], g0 = 0, at = 0;
-            bool need[4] = {false, false, false, false};
-            if (act) {
-                const uint32_t r = band_row(o, b.nr), y = b.y0 + r;
-                const bool odd = ((colour + y) & 1u) != 0u;
-                at = r * b.pitch + cc.j0;
-                g0 = y * b.G + 4u * k;
-                uint32_t U[4], D[4], O[4], S[4], X[4], Sn[4], sure[4];
-                if (!band_updown(b, wt, other, r, cc.j0, cc.nv, U, D)) bad = 1;
-                smem_words(mine + at, S);
-                smem_words(other + at, O);
-                if (odd) {   // east is the shifted row
-                    band_shifted<kFull>(cc, true, other + r * b.pitch, O, X);
-                    ne_moves<kFull>(U, D, X, O, S, cc.vm, rate, cand, sure, ws, Sn, need);
-                } else {
-                    band_shifted<kFull>(cc, false, other + r * b.pitch, O, X);
-                    ne_moves<kFull>(U, D, O, X, S, cc.vm, rate, cand, sure, ws, Sn, need);
-                }
-                store_words<4>(reinterpret_cast<int8_t *>(mine) + at, Sn);
-                if (((sure[0] | sure[1] | sure[2] | sure[3]) & kB1) != 0u) {
-                    uint32_t *f4 = reinterpret_cast<uint32_t *>(flc + (at >> 2));
-                    const uint32_t chg = ne_changed(sure), was = *f4;
-                    *f4 = was | chg;
-                    cnt.unfl -= __popc(chg & ~was);
-                }
-                if (colour == 1u) {
-                    ne_count(Sn, U, D, O, X, cc.vm, cnt);
-                    cnt.up += (int)cc.nv;
-                    if constexpr (kRef) {
-                        uint32_t R1[4], R0[4];
-                        const int8_t *r0 = g.ref + (size_t)y * b.half + cc.j0;
-                        load16_any<kFull>(r0 + b.plane, cc.nv, R1);
-                        load16_any<kFull>(r0, cc.nv, R0);
-#pragma unroll
-                        for (int w = 0; w < 4; ++w)
-                            cnt.acf = dot4(Sn[w] & cc.vm[w], R1[w], dot4(O[w] & cc.vm[w], R0[w], cnt.acf));
-                    }
-                }
-            }
-#pragma unroll
-            for (int w = 0; w < 4; ++w) {
-                const unsigned bal = __ballot_sync(0xffffffffu, need[w]);
-                if (need[w])
-                    queue[queued + __popc(bal & below)] = NeJob{g0 + (uint32_t)w, at + 4u * (uint32_t)w, cand[w], ws[w]};
-                queued += __popc(bal);
-            }
-            if (queued >= 32u) drain(false);
-        }
-        drain(true);
-        if (colour == 1u) {
-            cnt.up += cnt.mag / 2;
-            band_count(sh, h >> 1 & 1, cnt, true, kRef);
-            cnt = Counts();
-        }
-        const int stop = __syncthreads_or(bad);
-        // send the boundary rows; all waits of this half-sweep are over
-        for (uint32_t i = tid; i < 2u * b.cpr; i += blockDim.x) {
-            const bool lo = i >= b.cpr;
-            const uint32_t q = lo ? i - b.cpr : i;
-            uint32_t v[4];
-            smem_words(mine + (lo ? b.nr - 1u : 0u) * b.pitch + 16u * q, v);
-            mail_put((lo ? b.last : b.first) + 2u * (colour * b.cpr + q), part.epoch + (uint32_t)h + 1u, v);
-        }
-        if (colour == 1u) band_post(sh, h >> 1 & 1, g, sweep, true, kRef);
-        if (stop) {
-            sh.bad = 1;
-            break;
-        }
-    }
-    int8_t *fin = ((part.sweep0 + (unsigned long long)part.n) & 1) ? g.s[1] : g.s[0];
-    for (int c = 0; c < 2; ++c) {
-        rows_out(smem + c * pb, b.pitch, b.nr, fin + c * b.plane + (size_t)b.y0 * b.half, b.half);
-        uint8_t *q = g.flags + ((size_t)c * g.rows + b.y0) * b.G;
-        for (uint32_t i = tid; i < b.nr * b.G; i += blockDim.x) {
-            const uint32_t r = i / b.G, m = i - r * b.G;
-            q[i] = fl[(c * b.nr + r) * fp + m];
-        }
-    }
-}
-
-// End of a CTA's run: tell the host if a wait gave up; band 0 moves the
-// lattice's sweep counter on.
-LAT_D void band_end(const Geom &g, const BandPart &p, const BandShared &sh, int *err)
-{
-    if (threadIdx.x != 0) return;
-    if (sh.bad) *reinterpret_cast<volatile int *>(err) = 1;
-    if (p.band == 0u) g.ctrl->sweep = p.sweep0 + (unsigned long long)p.n;
-}
-
-// Kinds: Ising with a general or a symmetric table and North-East, each with
-// a partial last chunk or without; without: bonds (either table), fields.
-enum BandKind { kBandGen = 0, kBandSym, kBandNe, kBandGenFull, kBandSymFull, kBandNeFull, kBandBondGen, kBandBondSym,
-                kBandFields, kBandKinds };
-
-template <int kKind, bool kRef>
-LAT_D void band_body(const Geom &g, const BandPart &part, uint8_t *mail, BandShared &sh, uint8_t *smem)
-{
-    if constexpr (kKind == kBandNe) band_ne<kRef, false>(g, part, mail, sh, smem);
-    else if constexpr (kKind == kBandNeFull) band_ne<kRef, true>(g, part, mail, sh, smem);
-    else if constexpr (kKind == kBandGen) band_ising<kRef, kUniform, false, false>(g, part, mail, sh, smem);
-    else if constexpr (kKind == kBandSym) band_ising<kRef, kUniform, true, false>(g, part, mail, sh, smem);
-    else if constexpr (kKind == kBandGenFull) band_ising<kRef, kUniform, false, true>(g, part, mail, sh, smem);
-    else if constexpr (kKind == kBandSymFull) band_ising<kRef, kUniform, true, true>(g, part, mail, sh, smem);
-    else if constexpr (kKind == kBandBondGen) band_ising<kRef, kBonds, false, true>(g, part, mail, sh, smem);
-    else if constexpr (kKind == kBandBondSym) band_ising<kRef, kBonds, true, true>(g, part, mail, sh, smem);
-    else band_ising<kRef, kFields, false, true>(g, part, mail, sh, smem);
-}
-
 // One lattice over the whole grid.
 template <int kKind, bool kRef>
-__global__ void __launch_bounds__(kBandThreads, 1) k_band(Geom g, BandPart part, uint8_t *mail, int *err)
+__global__ void __launch_bounds__(kBandThreads, 1) k_band(const __grid_constant__ Geom g,
+                                                          const __grid_constant__ BandPart part, uint8_t *mail)
 {
     extern __shared__ __align__(16) uint8_t band_smem[];
     __shared__ BandShared sh;
-    part.band = blockIdx.x;
-    part.bands = gridDim.x;
-    band_body<kKind, kRef>(g, part, mail, sh, band_smem);
-    band_end(g, part, sh, err);
+    band_body<kKind, kRef>(g, part, blockIdx.x, gridDim.x, mail, sh, band_smem);
+    band_end(g, part, blockIdx.x, sh);
 }
 
 }  // namespace
 
-// Rows per band are at least 2, so a lattice has at most L / 2 bands.
-static size_t band_smem_bytes(const Geom &g, int bands)
-{
-    const size_t nr = ((size_t)g.L + bands - 1) / bands, pitch = ((size_t)g.half + 15) & ~(size_t)15;
-    size_t b = 2 * nr * pitch;
-    if (g.cpl != nullptr) b *= 2;
-    if (g.model == LAT_NE) b = ((b + 2 * nr * (pitch / 4) + 15) & ~(size_t)15) + kBandWarps * kNeQueue * sizeof(NeJob);
-    return b;
-}
-
-static int band_sms()
+int band_sms()
 {
     static const int sms = [] {
         int dev = 0, n = 0, coop = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-        return coop ? n : 0;
+        return coop ? std::min(n, kBandMaxCtas) : 0;
     }();
     return sms;
-}
-
-static int band_kind(const Geom &k, bool fields)
-{
-    const int full = k.half % 16 == 0 ? kBandGenFull : kBandGen;
-    if (k.model == LAT_NE) return full + kBandNe;
-    if (k.cpl == nullptr) return full + (k.acc_sym ? kBandSym : kBandGen);
-    return fields ? kBandFields : (k.acc_sym ? kBandBondSym : kBandBondGen);
 }
 
 int band_count_for(const Geom &g)
@@ -615,13 +44,13 @@ int band_count_for(const Geom &g)
 
 size_t band_mail_bytes(const Geom &g, int bands)
 {
-    return kAbortBytes + (size_t)bands * 2 * 4 * ((g.half + 15) / 16) * sizeof(ulonglong2);
+    return kAbortBytes + band_mail_pairs(g, bands) * sizeof(ulonglong2);
 }
 
 cudaError_t launch_sweep_band(const Geom &g, bool fields, int bands, unsigned long long sweep0, int n, void *mail,
                               unsigned epoch, int *err, cudaStream_t st)
 {
-    using K = void (*)(Geom, BandPart, uint8_t *, int *);
+    using K = void (*)(Geom, BandPart, uint8_t *);
 #define LAT_BAND(k) {k_band<k, false>, k_band<k, true>}
     static const K kern[kBandKinds][2] = {LAT_BAND(kBandGen),     LAT_BAND(kBandSym),     LAT_BAND(kBandNe),
                                           LAT_BAND(kBandGenFull), LAT_BAND(kBandSymFull), LAT_BAND(kBandNeFull),
@@ -639,7 +68,7 @@ cudaError_t launch_sweep_band(const Geom &g, bool fields, int bands, unsigned lo
     });
     if (attr != cudaSuccess) return attr;
     const Geom k = tiled_geom(g);
-    BandPart part{0u, (uint32_t)bands, epoch, 0u, sweep0, n, 0};
+    const BandPart part = band_part(k, sweep0, n, epoch, err);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)bands);
     cfg.blockDim = dim3(kBandThreads);
@@ -650,7 +79,7 @@ cudaError_t launch_sweep_band(const Geom &g, bool fields, int bands, unsigned lo
     a[0].val.cooperative = 1;
     cfg.attrs = a;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern[band_kind(k, fields)][k.ref != nullptr ? 1 : 0], k, part, (uint8_t *)mail, err);
+    return cudaLaunchKernelEx(&cfg, kern[band_kind(k, fields)][k.ref != nullptr ? 1 : 0], k, part, (uint8_t *)mail);
 }
 
 }  // namespace lat

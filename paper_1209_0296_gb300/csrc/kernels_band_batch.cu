@@ -1,0 +1,152 @@
+// kernels_band_batch.cu -- the band-resident kernel (band.cuh) for a batch:
+// the SMs are shared out over uneven 2D lattices, each a ring of bands, and
+// every lattice runs all its sweeps in the one cooperative launch.
+#include <algorithm>
+#include <cmath>
+#include <mutex>
+
+#include "band.cuh"
+
+namespace lat {
+
+namespace {
+
+// A CTA's part is a kernel parameter (uniform loads), the lattice's
+// descriptor is read from memory once.
+struct BandParts {
+    BandPart p[kBandMaxCtas];
+};
+
+template <bool kRef>
+LAT_D void band_any(const Geom &g, const BandPart &part, uint8_t *mail, BandShared &sh, uint8_t *smem)
+{
+    switch (part.kind) {
+    case kBandGen: band_body<kBandGen, kRef>(g, part, part.band, part.bands, mail, sh, smem); break;
+    case kBandSym: band_body<kBandSym, kRef>(g, part, part.band, part.bands, mail, sh, smem); break;
+    case kBandNe: band_body<kBandNe, kRef>(g, part, part.band, part.bands, mail, sh, smem); break;
+    case kBandGenFull: band_body<kBandGenFull, kRef>(g, part, part.band, part.bands, mail, sh, smem); break;
+    case kBandSymFull: band_body<kBandSymFull, kRef>(g, part, part.band, part.bands, mail, sh, smem); break;
+    default: band_body<kBandNeFull, kRef>(g, part, part.band, part.bands, mail, sh, smem); break;
+    }
+}
+
+__global__ void __launch_bounds__(kBandThreads, 1) k_band_batch(const Geom *geoms, const __grid_constant__ BandParts parts,
+                                                                uint8_t *mail)
+{
+    extern __shared__ __align__(16) uint8_t band_smem[];
+    __shared__ BandShared sh;
+    __shared__ Geom sg;
+    const BandPart &part = parts.p[blockIdx.x];
+    if (threadIdx.x < sizeof(Geom) / 4)
+        reinterpret_cast<uint32_t *>(&sg)[threadIdx.x] =
+            reinterpret_cast<const uint32_t *>(&geoms[part.lat])[threadIdx.x];
+    __syncthreads();
+    if (part.ref) band_any<true>(sg, part, mail, sh, band_smem);
+    else band_any<false>(sg, part, mail, sh, band_smem);
+    band_end(sg, part, part.band, sh);
+}
+
+// Estimated us of n sweeps of a lattice on c CTAs: about 5 sites per ns and
+// SM in a half-sweep, and the exchange with the neighbours.
+double band_time(const Geom &g, long long n, int c)
+{
+    const double rate = g.model == LAT_NE ? 7.0e3 : 5.0e3;   // sites per us and SM
+    return (double)n * 2.0 * (0.5 * (double)g.N / c / rate + 1.2);
+}
+
+}  // namespace
+
+// The fewest CTAs that hold the lattice, 0 when it cannot run here.
+int band_min_ctas(const Geom &g)
+{
+    if (g.cpl != nullptr || (g.half + 15) / 16 > (uint32_t)kBandThreads) return 0;
+    if (!(g.model == LAT_NE ? ne_walk_supported(g) : (g.model == LAT_ISING && any_supported(g)))) return 0;
+    const int most = std::min(band_sms(), g.L / 2);
+    int lo = 1, hi = most;
+    if (hi < 1 || band_smem_bytes(g, hi) > kBandMaxSmem) return 0;
+    while (lo < hi) {   // fewer bands need more memory each
+        const int mid = (lo + hi) / 2;
+        if (band_smem_bytes(g, mid) <= kBandMaxSmem) hi = mid;
+        else lo = mid + 1;
+    }
+    return lo;
+}
+
+// CTAs for each of the lattices so that the slowest finishes soonest;
+// returns its estimated us (infinite: they do not fit together).
+double band_share(const std::vector<std::pair<const Geom *, long long>> &lats, std::vector<int> &ctas)
+{
+    const int sms = band_sms();
+    ctas.assign(lats.size(), 0);
+    int used = 0;
+    for (size_t i = 0; i < lats.size(); ++i) {
+        ctas[i] = band_min_ctas(*lats[i].first);
+        if (ctas[i] == 0) return INFINITY;
+        used += ctas[i];
+    }
+    if (used > sms) return INFINITY;
+    for (;;) {   // a CTA more for the slowest while there is one and it helps
+        size_t worst = 0;
+        double t = -1.0;
+        for (size_t i = 0; i < lats.size(); ++i) {
+            const double ti = band_time(*lats[i].first, lats[i].second, ctas[i]);
+            if (ti > t) {
+                t = ti;
+                worst = i;
+            }
+        }
+        if (used >= sms || ctas[worst] >= lats[worst].first->L / 2) return t;
+        ++ctas[worst];
+        ++used;
+    }
+}
+
+size_t band_batch_mail_bytes(const std::vector<std::pair<const Geom *, long long>> &lats, const std::vector<int> &ctas)
+{
+    size_t pairs = 0;
+    for (size_t i = 0; i < lats.size(); ++i) pairs += band_mail_pairs(*lats[i].first, ctas[i]);
+    return kAbortBytes + pairs * sizeof(ulonglong2);
+}
+
+cudaError_t launch_batch_band(const Geom *d_geoms, const std::vector<std::pair<const Geom *, long long>> &lats,
+                              const std::vector<unsigned long long> &sweep0, const std::vector<int *> &err,
+                              const std::vector<int> &ctas, void *mail, unsigned epoch, cudaStream_t st)
+{
+    static std::once_flag once;
+    static cudaError_t attr = cudaSuccess;
+    std::call_once(once, [] {
+        attr = cudaFuncSetAttribute(k_band_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBandMaxSmem);
+    });
+    if (attr != cudaSuccess) return attr;
+    auto parts = std::make_unique<BandParts>();
+    size_t smem = 0, pairs = 0;
+    int cta = 0;
+    for (size_t i = 0; i < lats.size(); ++i) {
+        const Geom k = tiled_geom(*lats[i].first);
+        BandPart p = band_part(k, sweep0[i], (int)lats[i].second, epoch, err[i]);
+        p.bands = (uint32_t)ctas[i];
+        p.lat = (uint32_t)i;
+        p.kind = (uint32_t)band_kind(k, false);
+        p.ref = k.ref != nullptr ? 1u : 0u;
+        p.mail = (uint32_t)pairs;
+        pairs += band_mail_pairs(k, ctas[i]);
+        smem = std::max(smem, band_smem_bytes(k, ctas[i]));
+        for (int b = 0; b < ctas[i]; ++b) {
+            p.band = (uint32_t)b;
+            parts->p[cta++] = p;
+        }
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)cta);
+    cfg.blockDim = dim3(kBandThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute a[1];
+    a[0].id = cudaLaunchAttributeCooperative;
+    a[0].val.cooperative = 1;
+    cfg.attrs = a;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_band_batch, d_geoms, *parts, (uint8_t *)mail);
+}
+
+}  // namespace lat

@@ -7,6 +7,9 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <utility>
+#include <vector>
+
 #include "lattice.h"
 
 #if defined(__CUDACC__)
@@ -466,10 +469,22 @@ cudaError_t launch_batch_ne(const Geom *geoms, const uint2 *items, int n_items, 
 // it before, the launch marks up to epoch + 2 n; err: host-visible word set
 // when a bounded wait gave up (mail must then be zeroed again).  Advances
 // ctrl->sweep.
+int band_sms();   // CTAs of a launch at most
 int band_count_for(const Geom &g);
 size_t band_mail_bytes(const Geom &g, int bands);
 cudaError_t launch_sweep_band(const Geom &g, bool fields, int bands, unsigned long long sweep0, int n, void *mail,
                               unsigned epoch, int *err, cudaStream_t st);
+// Batched form (2D Ising without disorder, c-mode North-East): band_min_ctas
+// = the fewest CTAs that hold a lattice (0: not here); band_share = CTAs for
+// (lattice, sweeps) pairs run together and the estimated us (infinite: they
+// do not fit); the launch runs them all.  d_geoms: tiled_geom descriptors in
+// the same order; mail: band_batch_mail_bytes(), zeroed once.
+int band_min_ctas(const Geom &g);
+double band_share(const std::vector<std::pair<const Geom *, long long>> &lats, std::vector<int> &ctas);
+size_t band_batch_mail_bytes(const std::vector<std::pair<const Geom *, long long>> &lats, const std::vector<int> &ctas);
+cudaError_t launch_batch_band(const Geom *d_geoms, const std::vector<std::pair<const Geom *, long long>> &lats,
+                              const std::vector<unsigned long long> &sweep0, const std::vector<int *> &err,
+                              const std::vector<int> &ctas, void *mail, unsigned epoch, cudaStream_t st);
 // batched engine
 Geom tiled_geom(const Geom &g);
 int tiles_of(const Geom &g, int tile_h);
