@@ -21,6 +21,7 @@
 #pragma once
 
 #include <memory>
+#include <type_traits>
 #include <vector>
 
 #include "ising_walk.cuh"
@@ -291,19 +292,30 @@ LAT_D void band_ising(const Geom &g, const BandPart &part, uint32_t band, uint32
     if (tid == 10) sh.bad = 0;
     if (tid == 11) sh.fld = 0;
     __syncthreads();
+    // Interior rows 1 .. nr - 2: thread (rr, k) takes chunk k of rows 1 + rr,
+    // 1 + rr + rsb, ...  The two boundary rows' chunks are the last threads',
+    // which have an interior row less where the rows do not divide.
     const uint32_t rsb = (uint32_t)kBandThreads / b.cpr, rr = tid / b.cpr, k = tid - rr * b.cpr;
-    const uint32_t o0 = rr < rsb ? rr : b.nr;   // first visited row ordinal (none: nr)
+    const uint32_t r0 = rr < rsb ? 1u + rr : b.nr, rend = b.nr - 1u;
+    const uint32_t edge0 = (uint32_t)kBandThreads - 1u - tid, edges = 2u * b.cpr;   // (nr >= 2)
     const ChunkCol<kFull> cc = chunk_col<kFull>(k, b.half);
+    const uint32_t at0 = r0 * b.pitch + cc.j0, at_step = rsb * b.pitch;
+    const uint32_t g00 = (b.y0 + r0) * b.G + 4u * k, g_step = rsb * b.G;
+    // The group a thread draws for first in a half-sweep.
+    auto edge_row = [&](uint32_t e) { return e < b.cpr ? rend : 0u; };
+    auto edge_col = [&](uint32_t e) { return e < b.cpr ? e : e - b.cpr; };
+    auto edge_group = [&](uint32_t e) { return (b.y0 + edge_row(e)) * b.G + 4u * edge_col(e); };
+    const bool has_in = r0 < rend, has_edge = edge0 < edges;
+    const uint32_t g_first = has_in ? g00 : (has_edge ? edge_group(edge0) : 0u);
     const int last = 2 * part.n;
     uint32_t p01[4], p23[4];
     PhiloxPre pp;
     philox_prepare(pp, (uint32_t)part.sweep0, (uint32_t)(part.sweep0 >> 32), part.key0, part.key1);
-    auto draw = [&](uint32_t y, uint32_t colour) {
-        const uint32_t g0 = y * b.G + 4u * k;
+    auto draw = [&](const PhiloxPre &q, uint32_t g0, uint32_t colour, uint32_t (&d01)[4], uint32_t (&d23)[4]) {
 #pragma unroll
-        for (int w = 0; w < 4; ++w) top_halves(philox_item(pp, g0 + (uint32_t)w, colour), p01[w], p23[w]);
+        for (int w = 0; w < 4; ++w) top_halves(philox_item(q, g0 + (uint32_t)w, colour), d01[w], d23[w]);
     };
-    if (o0 < b.nr) draw(b.y0 + band_row(o0, b.nr), 0u);
+    if (has_in || has_edge) draw(pp, g_first, 0u, p01, p23);
     Counts cnt;
     int bad = 0;   // a wait of this thread gave up
     for (int h = 0; h < last; ++h) {
@@ -311,22 +323,33 @@ LAT_D void band_ising(const Geom &g, const BandPart &part, uint32_t band, uint32
         const unsigned long long sweep = part.sweep0 + (unsigned long long)(h >> 1);
         uint8_t *mine = smem + colour * pb;
         const uint8_t *other = smem + (1u - colour) * pb;
-        const BandWait wt{b.src + (1u - colour) * b.plane, h > 0 ? part.epoch + (uint32_t)h : 0u,
-                          2u * ((1u - colour) * b.cpr + k)};
-        for (uint32_t o = o0; o < b.nr; o += rsb) {
-            const uint32_t r = band_row(o, b.nr), y = b.y0 + r, at = r * b.pitch + cc.j0;
+        PhiloxPre pn = pp;   // of the next half-sweep's draws
+        if (colour == 1u)
+            philox_prepare(pn, (uint32_t)(sweep + 1ull), (uint32_t)((sweep + 1ull) >> 32), part.key0, part.key1);
+        // The draws of group gn, of the next half-sweep when `over`.
+        auto draw_next = [&](uint32_t gn, bool over, uint32_t (&d01)[4], uint32_t (&d23)[4]) {
+            PhiloxPre q = pp;
+            q.A = over ? pn.A : pp.A;
+            q.B = over ? pn.B : pp.B;
+            q.H2 = over ? pn.H2 : pp.H2;
+            q.L2 = over ? pn.L2 : pp.L2;
+            draw(q, gn, over ? 1u - colour : colour, d01, d23);
+        };
+        // One chunk whose neighbour rows are loaded: group g0, shared offset
+        // at.  Interior: the next chunk's draws share its instruction block;
+        // boundary: they wait until the neighbour has been served.
+        auto chunk = [&](auto interior, IsingChunk &c, const ChunkCol<kFull> &col, uint32_t at, uint32_t y, uint32_t g0,
+                         uint32_t gn, bool over, uint32_t (&Sn)[4]) {
+            uint32_t C[4] = {0, 0, 0, 0}, O[4], F[4], d01[4], d23[4];
             const bool odd = ((colour + y) & 1u) != 0u;
-            IsingChunk c;
-            uint32_t C[4] = {0, 0, 0, 0}, O[4];
-            if (!band_updown(b, wt, other, r, cc.j0, cc.nv, c.U, c.D)) bad = 1;
             smem_words(mine + at, c.S);
             smem_words(other + at, O);
             if constexpr (kDis != kUniform) smem_words(dis + colour * pb + at, C);
-            band_shifted<kFull>(cc, odd, other + r * b.pitch, O, c.X);
+            band_shifted<kFull>(col, odd, other + (at - col.j0), O, c.X);
 #pragma unroll
             for (int w = 0; w < 4; ++w) c.O[w] = O[w];
+            if constexpr (interior.value) draw_next(gn, over, d01, d23);
             ising_neighbours<kDis>(c, C, odd);
-            uint32_t F[4], Sn[4];
             if (flips16<kSym>(part.acc, c.n, c.St, p01, p23, F)) {
                 Chunk16 e;
 #pragma unroll
@@ -334,46 +357,74 @@ LAT_D void band_ising(const Geom &g, const BandPart &part, uint32_t band, uint32
                     e.n[w] = c.n[w];
                     e.S[w] = c.St[w];
                 }
-                const uint4 f = band_exact(sh.sthr, sweep, part.key0, part.key1, y * b.G + 4u * k, colour, e);
+                const uint4 f = band_exact(sh.sthr, sweep, part.key0, part.key1, g0, colour, e);
                 F[0] = f.x;
                 F[1] = f.y;
                 F[2] = f.z;
                 F[3] = f.w;
             }
 #pragma unroll
-            for (int w = 0; w < 4; ++w) Sn[w] = c.S[w] ^ F[w];
-            store_words<4>(reinterpret_cast<int8_t *>(mine) + at, Sn);
-            const uint32_t box = 2u * (colour * b.cpr + k);
-            if (r == 0u) mail_put(b.first + box, part.epoch + (uint32_t)h + 1u, Sn);
-            if (r + 1u == b.nr) mail_put(b.last + box, part.epoch + (uint32_t)h + 1u, Sn);
-            // the next chunk's draws: this colour's next row, else the next half-sweep's first
-            if (o + rsb < b.nr) {
-                draw(b.y0 + band_row(o + rsb, b.nr), colour);
-            } else {
-                if (colour == 1u) {
-                    const unsigned long long s1 = sweep + 1ull;
-                    philox_prepare(pp, (uint32_t)s1, (uint32_t)(s1 >> 32), part.key0, part.key1);
+            for (int w = 0; w < 4; ++w) {
+                Sn[w] = c.S[w] ^ F[w];
+                if constexpr (interior.value) {
+                    p01[w] = d01[w];
+                    p23[w] = d23[w];
                 }
-                draw(b.y0 + band_row(o0, b.nr), 1u - colour);
+            }
+            store_words<4>(reinterpret_cast<int8_t *>(mine) + at, Sn);
+            if constexpr (!interior.value) {
+                const uint32_t box = 2u * (colour * b.cpr + (col.j0 >> 4));
+                mail_put((y == b.y0 ? b.first : b.last) + box, part.epoch + (uint32_t)h + 1u, Sn);
+                draw_next(gn, over, p01, p23);
             }
             if (colour == 1u) {
-                ising_count<1, kDis, kFull>(c, Sn, cc.vm, cnt);
+                ising_count<1, kDis, kFull>(c, Sn, col.vm, cnt);
 #pragma unroll
-                for (int w = 0; w < 4; ++w) cnt.mag = dot4(O[w], 0x01010101u & cc.vm[w], cnt.mag);
+                for (int w = 0; w < 4; ++w) cnt.mag = dot4(O[w], 0x01010101u & col.vm[w], cnt.mag);
                 if constexpr (kRef) {
                     uint32_t R1[4], R0[4];
-                    const int8_t *r0 = g.ref + (size_t)y * b.half + cc.j0;
-                    load16_any<kFull>(r0 + b.plane, cc.nv, R1);
-                    load16_any<kFull>(r0, cc.nv, R0);
+                    const int8_t *rp = g.ref + (size_t)y * b.half + col.j0;
+                    load16_any<kFull>(rp + b.plane, col.nv, R1);
+                    load16_any<kFull>(rp, col.nv, R0);
 #pragma unroll
                     for (int w = 0; w < 4; ++w)
-                        cnt.acf = dot4(Sn[w] & cc.vm[w], R1[w], dot4(O[w] & cc.vm[w], R0[w], cnt.acf));
+                        cnt.acf = dot4(Sn[w] & col.vm[w], R1[w], dot4(O[w] & col.vm[w], R0[w], cnt.acf));
                 }
-                cnt.up += (int)cc.nv;
+                cnt.up += (int)col.nv;
             } else if constexpr (kDis == kFields) {
-                ising_count<0, kDis, kFull>(c, Sn, cc.vm, cnt);
+                ising_count<0, kDis, kFull>(c, Sn, col.vm, cnt);
+            }
+        };
+        {
+            uint32_t at = at0, g0 = g00;
+#pragma unroll 1
+            for (uint32_t r = r0; r < rend; r += rsb) {
+                IsingChunk c;
+                uint32_t Sn[4];
+                smem_words(other + at - b.pitch, c.U);
+                smem_words(other + at + b.pitch, c.D);
+                const bool more = r + rsb < rend;
+                const uint32_t gn = more ? g0 + g_step : (has_edge ? edge_group(edge0) : g_first);
+                chunk(std::true_type(), c, cc, at, b.y0 + r, g0, gn, !more && !has_edge, Sn);
+                at += at_step;
+                g0 += g_step;
             }
         }
+#pragma unroll 1
+        for (uint32_t e = edge0; e < edges; e += (uint32_t)kBandThreads) {
+            const uint32_t r = edge_row(e), q = edge_col(e), y = b.y0 + r;
+            const ChunkCol<kFull> col = chunk_col<kFull>(q, b.half);
+            const uint32_t at = r * b.pitch + col.j0;
+            const BandWait wt{b.src + (1u - colour) * b.plane, h > 0 ? part.epoch + (uint32_t)h : 0u,
+                              2u * ((1u - colour) * b.cpr + q)};
+            IsingChunk c;
+            uint32_t Sn[4];
+            if (!band_updown(b, wt, other, r, col.j0, col.nv, c.U, c.D)) bad = 1;
+            const bool more = e + (uint32_t)kBandThreads < edges;
+            chunk(std::false_type(), c, col, at, y, edge_group(e),
+                  more ? edge_group(e + (uint32_t)kBandThreads) : g_first, !more, Sn);
+        }
+        pp = pn;
         if (colour == 1u) {
             cnt.up += cnt.mag / 2;   // nv sites of each plane: up = nv + mag / 2
             band_count(sh, h >> 1 & 1, cnt, false, kRef);
@@ -544,6 +595,183 @@ LAT_D void band_ne(const Geom &g, const BandPart &part, uint32_t band, uint32_t 
     }
 }
 
+// Lattices with no more than one chunk a thread and colour, Ising or c-mode
+// North-East: a half-sweep is one pass whose length is the latency from a
+// neighbour's packet to this band's own, so everything else is taken off
+// that path.  A thread keeps its chunk of both colours (and disorder bytes,
+// reference, persistence bits) in registers; its draws of the next half-sweep
+// are made after its packet has left -- all of them for North-East too,
+// reduced to rejection masks, since with most threads idle a draw that is
+// not needed costs nothing.  A row is a warp's where it fits, so that the two
+// boundary rows wait side by side.
+LAT_HD bool band_is_small(uint32_t L, uint32_t half, uint32_t bands)
+{
+    const uint32_t nr = (L + bands - 1u) / bands, cpr = (half + 15u) >> 4;
+    return cpr <= 32u ? nr <= (uint32_t)kBandWarps : nr * cpr <= (uint32_t)kBandThreads;
+}
+
+template <bool kNe, bool kRef, int kDis, bool kSym, bool kFull>
+LAT_D void band_small(const Geom &g, const BandPart &part, uint32_t band, uint32_t bands, uint8_t *mail,
+                      BandShared &sh, uint8_t *smem)
+{
+    const Band b = band_of(g, part, band, bands, mail);
+    const uint32_t tid = threadIdx.x, pb = b.nr * b.pitch;
+    for (int c = 0; c < 2; ++c)
+        rows_in(b.src + c * b.plane + (size_t)b.y0 * b.half, b.half, b.nr, smem + c * pb, b.pitch);
+    if (tid < 16) sh.sthr[tid] = g.thr16[tid];
+    if (tid < 10) (&sh.sum[0][0])[tid] = 0;
+    if (tid == 10) sh.bad = 0;
+    if (tid == 11) sh.fld = 0;
+    if (tid == 12) sh.unfl = (int)(2u * b.nr * b.half);
+    __syncthreads();
+    const uint32_t r = b.cpr <= 32u ? tid >> 5 : tid / b.cpr, k = b.cpr <= 32u ? tid & 31u : tid - r * b.cpr;
+    const bool mine = r < b.nr && k < b.cpr, top = r == 0u, bottom = r + 1u == b.nr;
+    const ChunkCol<kFull> cc = chunk_col<kFull>(mine ? k : 0u, b.half);
+    const uint32_t at = r * b.pitch + cc.j0, y = b.y0 + r, g0 = y * b.G + 4u * k;
+    const NeRate rate = ne_rate(g.thr16);
+    uint32_t S[2][4], C[2][4] = {}, Rf[2][4] = {}, was[2] = {0u, 0u};
+    if (mine) {
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            smem_words(smem + c * pb + at, S[c]);
+            const size_t ga = c * b.plane + (size_t)y * b.half + cc.j0;
+            if constexpr (kDis != kUniform) load_words<4>(reinterpret_cast<const int8_t *>(g.cpl) + ga, C[c]);
+            if constexpr (kRef) load16_any<kFull>(g.ref + ga, cc.nv, Rf[c]);
+            if constexpr (kNe)
+                for (uint32_t w = 0; w < 4u && 4u * k + w < b.G; ++w)
+                    was[c] |= (uint32_t)g.flags[((size_t)c * g.rows + y) * b.G + 4u * k + w] << (8u * w);
+        }
+    }
+    if constexpr (kNe) {
+        const int n = __reduce_add_sync(0xffffffffu, __popc(was[0]) + __popc(was[1]));
+        if ((tid & 31u) == 0u) atomicSub(&sh.unfl, n);
+        __syncthreads();
+    }
+    uint32_t p01[4], p23[4];   // draws of the next half-sweep (North-East: p01 = rejections)
+    auto draw = [&](unsigned long long sweep, uint32_t colour) {
+        PhiloxPre pp;
+        philox_prepare(pp, (uint32_t)sweep, (uint32_t)(sweep >> 32), part.key0, part.key1);
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+            const U4 u = philox_item(pp, g0 + (uint32_t)w, colour);
+            if constexpr (kNe) p01[w] = ne_rejected(u, rate.K);
+            else top_halves(u, p01[w], p23[w]);
+        }
+    };
+    if (mine) draw(part.sweep0, 0u);
+    Counts cnt;
+    int bad = 0;   // a wait of this thread gave up
+    auto half_sweep = [&](auto which, int h, unsigned long long sweep) {
+        constexpr uint32_t colour = decltype(which)::value;
+        uint8_t *own = smem + colour * pb;
+        const uint8_t *other = smem + (1u - colour) * pb;
+        if (mine) {
+            const bool odd = ((colour + y) & 1u) != 0u;
+            IsingChunk c;
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+                c.S[w] = S[colour][w];
+                c.O[w] = S[1u - colour][w];
+            }
+            band_shifted<kFull>(cc, odd, other + (at - cc.j0), S[1u - colour], c.X);
+            const BandWait wt{b.src + (1u - colour) * b.plane, h > 0 ? part.epoch + (uint32_t)h : 0u,
+                              2u * ((1u - colour) * b.cpr + k)};
+            if (!band_updown(b, wt, other, r, cc.j0, cc.nv, c.U, c.D)) bad = 1;
+            uint32_t F[4], Sn[4];
+            [[maybe_unused]] uint32_t moved[4];
+            if constexpr (kNe) {
+                uint32_t cand[4], sure[4], ws[4], Sm[4];
+                bool need[4];
+                if (odd) ne_moves<kFull>(c.U, c.D, c.X, c.O, c.S, cc.vm, rate, cand, sure, ws, Sm, need);
+                else ne_moves<kFull>(c.U, c.D, c.O, c.X, c.S, cc.vm, rate, cand, sure, ws, Sm, need);
+#pragma unroll
+                for (int w = 0; w < 4; ++w) {
+                    moved[w] = sure[w] | (cand[w] & ~p01[w]);
+                    F[w] = moved[w] & 0xFEFEFEFEu;
+                }
+            } else {
+                ising_neighbours<kDis>(c, C[colour], odd);
+                if (flips16<kSym>(part.acc, c.n, c.St, p01, p23, F)) {
+                    Chunk16 e;
+#pragma unroll
+                    for (int w = 0; w < 4; ++w) {
+                        e.n[w] = c.n[w];
+                        e.S[w] = c.St[w];
+                    }
+                    const uint4 f = band_exact(sh.sthr, sweep, part.key0, part.key1, g0, colour, e);
+                    F[0] = f.x;
+                    F[1] = f.y;
+                    F[2] = f.z;
+                    F[3] = f.w;
+                }
+            }
+#pragma unroll
+            for (int w = 0; w < 4; ++w) Sn[w] = c.S[w] ^ F[w];
+            const uint32_t box = 2u * (colour * b.cpr + k), tag = part.epoch + (uint32_t)h + 1u;
+            if (top) mail_put(b.first + box, tag, Sn);
+            if (bottom) mail_put(b.last + box, tag, Sn);
+            store_words<4>(reinterpret_cast<int8_t *>(own) + at, Sn);
+            draw(sweep + (colour == 1u ? 1ull : 0ull), 1u - colour);
+            if constexpr (kNe) {
+                const uint32_t chg = ne_changed(moved);
+                cnt.unfl -= __popc(chg & ~was[colour]);
+                was[colour] |= chg;
+            }
+            if constexpr (colour == 1u) {
+                ising_count<1, kDis, kFull>(c, Sn, cc.vm, cnt);
+#pragma unroll
+                for (int w = 0; w < 4; ++w) {
+                    cnt.mag = dot4(S[0][w], 0x01010101u & cc.vm[w], cnt.mag);
+                    if constexpr (kRef)
+                        cnt.acf = dot4(Sn[w] & cc.vm[w], Rf[1][w], dot4(S[0][w] & cc.vm[w], Rf[0][w], cnt.acf));
+                }
+                cnt.up = (int)cc.nv + cnt.mag / 2;   // nv sites of each plane
+            } else if constexpr (kDis == kFields) {
+                ising_count<0, kDis, kFull>(c, Sn, cc.vm, cnt);
+            }
+#pragma unroll
+            for (int w = 0; w < 4; ++w) S[colour][w] = Sn[w];
+        }
+        if constexpr (colour == 1u) {
+            band_count(sh, h >> 1 & 1, cnt, kNe, kRef);
+            if constexpr (kDis == kFields) {
+                const int f = __reduce_add_sync(0xffffffffu, cnt.fld);
+                if ((tid & 31u) == 0u) atomicAdd(&sh.fld, f);
+            }
+            cnt = Counts();
+        }
+        const int stop = __syncthreads_or(bad);
+        if constexpr (colour == 1u) {
+            band_post(sh, h >> 1 & 1, g, sweep, kNe, kRef);
+            if constexpr (kDis == kFields) {
+                if (tid == 0u) {
+                    add_counter(fld_slot(g.ctrl, sweep), (long long)sh.fld);
+                    sh.fld = 0;   // next added to a barrier later
+                }
+            }
+        }
+        return stop;
+    };
+    for (int n = 0; n < part.n; ++n) {
+        const unsigned long long sweep = part.sweep0 + (unsigned long long)n;
+        int stop = half_sweep(std::integral_constant<uint32_t, 0>(), 2 * n, sweep);
+        if (!stop) stop = half_sweep(std::integral_constant<uint32_t, 1>(), 2 * n + 1, sweep);
+        if (stop) {
+            sh.bad = 1;
+            break;
+        }
+    }
+    int8_t *fin = ((part.sweep0 + (unsigned long long)part.n) & 1) ? g.s[1] : g.s[0];
+    for (int c = 0; c < 2; ++c)
+        rows_out(smem + c * pb, b.pitch, b.nr, fin + c * b.plane + (size_t)b.y0 * b.half, b.half);
+    if constexpr (kNe) {
+        if (mine)
+            for (int c = 0; c < 2; ++c)
+                for (uint32_t w = 0; w < 4u && 4u * k + w < b.G; ++w)
+                    g.flags[((size_t)c * g.rows + y) * b.G + 4u * k + w] = (uint8_t)(was[c] >> (8u * w));
+    }
+}
+
 // End of a CTA's run: tell the host if a wait gave up; band 0 moves the
 // lattice's sweep counter on.
 LAT_D void band_end(const Geom &g, const BandPart &p, uint32_t band, const BandShared &sh)
@@ -558,19 +786,39 @@ LAT_D void band_end(const Geom &g, const BandPart &p, uint32_t band, const BandS
 enum BandKind { kBandGen = 0, kBandSym, kBandNe, kBandGenFull, kBandSymFull, kBandNeFull, kBandBondGen, kBandBondSym,
                 kBandFields, kBandKinds };
 
+template <bool kRef, int kDis, bool kSym, bool kFull>
+LAT_D void band_ising_any(const Geom &g, const BandPart &part, uint32_t band, uint32_t bands, uint8_t *mail,
+                          BandShared &sh, uint8_t *smem)
+{
+    if (band_is_small((uint32_t)g.L, g.half, bands))
+        band_small<false, kRef, kDis, kSym, kFull>(g, part, band, bands, mail, sh, smem);
+    else
+        band_ising<kRef, kDis, kSym, kFull>(g, part, band, bands, mail, sh, smem);
+}
+
+template <bool kRef, bool kFull>
+LAT_D void band_ne_any(const Geom &g, const BandPart &part, uint32_t band, uint32_t bands, uint8_t *mail,
+                       BandShared &sh, uint8_t *smem)
+{
+    if (band_is_small((uint32_t)g.L, g.half, bands))
+        band_small<true, kRef, kUniform, false, kFull>(g, part, band, bands, mail, sh, smem);
+    else
+        band_ne<kRef, kFull>(g, part, band, bands, mail, sh, smem);
+}
+
 template <int kKind, bool kRef>
 LAT_D void band_body(const Geom &g, const BandPart &part, uint32_t band, uint32_t bands, uint8_t *mail,
                      BandShared &sh, uint8_t *smem)
 {
-    if constexpr (kKind == kBandNe) band_ne<kRef, false>(g, part, band, bands, mail, sh, smem);
-    else if constexpr (kKind == kBandNeFull) band_ne<kRef, true>(g, part, band, bands, mail, sh, smem);
-    else if constexpr (kKind == kBandGen) band_ising<kRef, kUniform, false, false>(g, part, band, bands, mail, sh, smem);
-    else if constexpr (kKind == kBandSym) band_ising<kRef, kUniform, true, false>(g, part, band, bands, mail, sh, smem);
-    else if constexpr (kKind == kBandGenFull) band_ising<kRef, kUniform, false, true>(g, part, band, bands, mail, sh, smem);
-    else if constexpr (kKind == kBandSymFull) band_ising<kRef, kUniform, true, true>(g, part, band, bands, mail, sh, smem);
-    else if constexpr (kKind == kBandBondGen) band_ising<kRef, kBonds, false, true>(g, part, band, bands, mail, sh, smem);
-    else if constexpr (kKind == kBandBondSym) band_ising<kRef, kBonds, true, true>(g, part, band, bands, mail, sh, smem);
-    else band_ising<kRef, kFields, false, true>(g, part, band, bands, mail, sh, smem);
+    if constexpr (kKind == kBandNe) band_ne_any<kRef, false>(g, part, band, bands, mail, sh, smem);
+    else if constexpr (kKind == kBandNeFull) band_ne_any<kRef, true>(g, part, band, bands, mail, sh, smem);
+    else if constexpr (kKind == kBandGen) band_ising_any<kRef, kUniform, false, false>(g, part, band, bands, mail, sh, smem);
+    else if constexpr (kKind == kBandSym) band_ising_any<kRef, kUniform, true, false>(g, part, band, bands, mail, sh, smem);
+    else if constexpr (kKind == kBandGenFull) band_ising_any<kRef, kUniform, false, true>(g, part, band, bands, mail, sh, smem);
+    else if constexpr (kKind == kBandSymFull) band_ising_any<kRef, kUniform, true, true>(g, part, band, bands, mail, sh, smem);
+    else if constexpr (kKind == kBandBondGen) band_ising_any<kRef, kBonds, false, true>(g, part, band, bands, mail, sh, smem);
+    else if constexpr (kKind == kBandBondSym) band_ising_any<kRef, kBonds, true, true>(g, part, band, bands, mail, sh, smem);
+    else band_ising_any<kRef, kFields, false, true>(g, part, band, bands, mail, sh, smem);
 }
 
 // Rows per band are at least 2, so a lattice has at most L / 2 bands.

@@ -71,7 +71,11 @@ cudaError_t launch_sweep_band(const Geom &g, bool fields, int bands, unsigned lo
     const BandPart part = band_part(k, sweep0, n, epoch, err);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)bands);
-    cfg.blockDim = dim3(kBandThreads);
+    // one chunk a thread: just the warps that have one (a row is a warp's when it fits)
+    const uint32_t nr = ((uint32_t)k.L + bands - 1) / bands, cpr = (k.half + 15) / 16;
+    const bool small = band_is_small((uint32_t)k.L, k.half, (uint32_t)bands);
+    cfg.blockDim = dim3(!small ? (uint32_t)kBandThreads
+                               : std::max(64u, cpr <= 32 ? 32u * nr : (nr * cpr + 31u) / 32u * 32u));
     cfg.dynamicSmemBytes = band_smem_bytes(k, bands);
     cfg.stream = st;
     cudaLaunchAttribute a[1];

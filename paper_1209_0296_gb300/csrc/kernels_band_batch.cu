@@ -30,6 +30,8 @@ LAT_D void band_any(const Geom &g, const BandPart &part, uint8_t *mail, BandShar
     }
 }
 
+// kRefs: some lattice of the launch has a reference state.
+template <bool kRefs>
 __global__ void __launch_bounds__(kBandThreads, 1) k_band_batch(const Geom *geoms, const __grid_constant__ BandParts parts,
                                                                 uint8_t *mail)
 {
@@ -41,17 +43,19 @@ __global__ void __launch_bounds__(kBandThreads, 1) k_band_batch(const Geom *geom
         reinterpret_cast<uint32_t *>(&sg)[threadIdx.x] =
             reinterpret_cast<const uint32_t *>(&geoms[part.lat])[threadIdx.x];
     __syncthreads();
-    if (part.ref) band_any<true>(sg, part, mail, sh, band_smem);
+    if (kRefs && part.ref) band_any<kRefs>(sg, part, mail, sh, band_smem);
     else band_any<false>(sg, part, mail, sh, band_smem);
     band_end(sg, part, part.band, sh);
 }
 
-// Estimated us of n sweeps of a lattice on c CTAs: about 5 sites per ns and
-// SM in a half-sweep, and the exchange with the neighbours.
+// Estimated us of n sweeps of a lattice on c CTAs: a half-sweep's exchange
+// with the neighbours and its sites at an SM's rate (measured: L = 1024, 2048
+// and 4096 on 152 SMs, 1.15, 2.9 and 8.8 us a half-sweep; rows with a partial
+// chunk L = 5000, 14.9; North-East at c = 0.3 L = 4096, 6.7).
 double band_time(const Geom &g, long long n, int c)
 {
-    const double rate = g.model == LAT_NE ? 7.0e3 : 5.0e3;   // sites per us and SM
-    return (double)n * 2.0 * (0.5 * (double)g.N / c / rate + 1.2);
+    const double rate = g.model == LAT_NE ? 9.0e3 : (g.half % 16 == 0 ? 6.6e3 : 5.8e3);   // sites per us and SM
+    return (double)n * 2.0 * (0.5 * (double)g.N / c / rate + 0.7);
 }
 
 }  // namespace
@@ -115,7 +119,9 @@ cudaError_t launch_batch_band(const Geom *d_geoms, const std::vector<std::pair<c
     static std::once_flag once;
     static cudaError_t attr = cudaSuccess;
     std::call_once(once, [] {
-        attr = cudaFuncSetAttribute(k_band_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBandMaxSmem);
+        for (auto f : {k_band_batch<false>, k_band_batch<true>})
+            if (attr == cudaSuccess)
+                attr = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBandMaxSmem);
     });
     if (attr != cudaSuccess) return attr;
     auto parts = std::make_unique<BandParts>();
@@ -146,7 +152,9 @@ cudaError_t launch_batch_band(const Geom *d_geoms, const std::vector<std::pair<c
     a[0].val.cooperative = 1;
     cfg.attrs = a;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_band_batch, d_geoms, *parts, (uint8_t *)mail);
+    bool refs = false;
+    for (const auto &l : lats) refs = refs || l.first->ref != nullptr;
+    return cudaLaunchKernelEx(&cfg, refs ? k_band_batch<true> : k_band_batch<false>, d_geoms, *parts, (uint8_t *)mail);
 }
 
 }  // namespace lat

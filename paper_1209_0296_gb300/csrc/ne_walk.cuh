@@ -43,21 +43,27 @@ struct NePlanes {
     uint32_t y0, half, pitch;
 };
 
+// 0xFF at the sites whose draw is above K.
+LAT_D uint32_t ne_rejected(const U4 &u, uint32_t K)
+{
+    auto above = [&](uint32_t x) {   // all ones where x > K: the borrow of K - x
+        uint32_t d, m;
+        asm("sub.cc.u32 %0, %2, %3;\n\tsubc.u32 %1, 0, 0;" : "=r"(d), "=r"(m) : "r"(K), "r"(x));
+        (void)d;
+        return m;
+    };
+    const uint32_t m0 = above(u.x), m1 = above(u.y), m2 = above(u.z), m3 = above(u.w);
+    const uint32_t lo = (m0 & 0x000000FFu) | (m1 & 0xFFFFFF00u), hi = (m2 & 0x00FFFFFFu) | (m3 & 0xFF000000u);
+    return (lo & 0x0000FFFFu) | (hi & 0xFFFF0000u);
+}
+
 // One queued group: draw, accept, apply.
 template <bool kRef>
 LAT_D void ne_job(const NePlanes &p, const PhiloxPre &pp, const NeRate rate, const NeJob job, uint32_t colour,
                   Counts &cnt, uint32_t flag_at = 0xFFFFFFFFu)
 {
     const U4 u = philox_item(pp, job.g, colour);
-    // all ones where u > K
-    auto above = [&](uint32_t x) {
-        uint32_t d, m;
-        asm("sub.cc.u32 %0, %2, %3;\n\tsubc.u32 %1, 0, 0;" : "=r"(d), "=r"(m) : "r"(rate.K), "r"(x));
-        return m;
-    };
-    const uint32_t m0 = above(u.x), m1 = above(u.y), m2 = above(u.z), m3 = above(u.w);
-    const uint32_t lo = (m0 & 0x000000FFu) | (m1 & 0xFFFFFF00u), hi = (m2 & 0x00FFFFFFu) | (m3 & 0xFF000000u);
-    const uint32_t rej = (lo & 0x0000FFFFu) | (hi & 0xFFFF0000u);
+    const uint32_t rej = ne_rejected(u, rate.K);
     const uint32_t f = job.cand & ~rej & kB1;   // accepted moves
     if (f == 0u) return;
     const uint8_t now = rate.inv ? 0xFFu : 0x01u;   // the spin after the move
