@@ -138,6 +138,26 @@ LAT_D bool mail_take(const ulonglong2 *q, uint32_t tag, unsigned *abort, uint32_
     }
 }
 
+// The same for one word.
+LAT_D void mail_put_word(unsigned long long *q, uint32_t tag, uint32_t v)
+{
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(q), "l"((unsigned long long)tag << 32 | v) : "memory");
+}
+
+LAT_D bool mail_take_word(const unsigned long long *q, uint32_t tag, unsigned *abort, uint32_t &v)
+{
+    for (unsigned i = 0;; ++i) {
+        unsigned long long a;
+        asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(a) : "l"(q) : "memory");
+        v = (uint32_t)a;
+        if ((uint32_t)(a >> 32) == tag) return true;
+        if ((i & 1023u) == 1023u && (i >= kSpinLimit || *reinterpret_cast<volatile unsigned *>(abort) != 0u)) {
+            *reinterpret_cast<volatile unsigned *>(abort) = 1u;
+            return false;
+        }
+    }
+}
+
 // Local rows in the order they are visited: interior first, then the first
 // and the last.
 LAT_D uint32_t band_row(uint32_t o, uint32_t nr) { return o + 2u < nr ? o + 1u : (o + 2u == nr ? 0u : nr - 1u); }

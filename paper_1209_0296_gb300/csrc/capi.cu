@@ -47,6 +47,59 @@ void dev_free(void *p, cudaStream_t st)
     if (p != nullptr) cudaFreeAsync(p, st);
 }
 
+// Pinned bounce buffers for counter read-backs: a copy of a few kilobytes to
+// pageable memory costs the host twice what one to pinned memory does (20 us
+// and 10 for a read of 200 sweeps' counters).  Up to kBounceMost are kept,
+// taken by one read at a time.
+namespace {
+constexpr size_t kBounceBytes = 64 * 1024;
+constexpr size_t kBounceMost = 16;
+std::mutex g_bounce_mu;
+std::vector<void *> g_bounce_free;
+size_t g_bounce_made = 0;
+
+class Bounce {
+public:
+    explicit Bounce(size_t bytes)
+    {
+        if (bytes > kBounceBytes) return;
+        std::lock_guard<std::mutex> g(g_bounce_mu);
+        if (!g_bounce_free.empty()) {
+            p_ = g_bounce_free.back();
+            g_bounce_free.pop_back();
+        } else if (g_bounce_made < kBounceMost) {
+            if (cudaHostAlloc(&p_, kBounceBytes, cudaHostAllocPortable) == cudaSuccess) {
+                ++g_bounce_made;
+                g_bounce_free.reserve(kBounceMost);
+            } else {
+                (void)cudaGetLastError();
+                p_ = nullptr;
+            }
+        }
+    }
+    ~Bounce()
+    {
+        if (p_ == nullptr) return;
+        std::lock_guard<std::mutex> g(g_bounce_mu);
+        g_bounce_free.push_back(p_);
+    }
+    void *get() const { return p_; }
+
+private:
+    void *p_ = nullptr;
+};
+
+// Copy device memory to the host and wait for the stream.
+cudaError_t read_back(void *dst, const void *src, size_t bytes, cudaStream_t st)
+{
+    const Bounce b(bytes);
+    cudaError_t e = cudaMemcpyAsync(b.get() ? b.get() : dst, src, bytes, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e == cudaSuccess && b.get()) memcpy(dst, b.get(), bytes);
+    return e;
+}
+}  // namespace
+
 // ---------------------------------------------------------------------------
 // Acceptance table (§III.A: P_acc = min[1, exp(-dH/T)]; §III.B: rates at
 // concentration c).  Built on the host in double precision:
@@ -331,9 +384,8 @@ static bool not_capturing(cudaStream_t st)
 // launch carries the host's sweep number, so it cannot be replayed).
 static int band_bands(const lattice *lt, int64_t n)
 {
-    if (n < band_min_sweeps(lt) || lt->graph_pinned || lt->P.layout != LAT_INT8 ||
-        lt->dynamics != LAT_DYNAMICS_CHECKERBOARD || choose_kernel(lt) != LAT_KERNEL_WIDE)
-        return 0;
+    if (n < band_min_sweeps(lt) || lt->graph_pinned || lt->dynamics != LAT_DYNAMICS_CHECKERBOARD) return 0;
+    if (lt->P.layout == LAT_INT8 && choose_kernel(lt) != LAT_KERNEL_WIDE) return 0;
     const int bands = band_count_for(lt->geom);
     if (bands == 0) return 0;
     return not_capturing(lt->stream) ? bands : 0;
@@ -973,11 +1025,8 @@ int lattice_series(lattice_t *lt, int64_t first, int64_t count, int64_t *bond, i
     if (first < lt->series_first || first + count > lt->sweeps) return LAT_ERANGE;
     if (count == 0) return LAT_OK;
     std::vector<long long> buf((size_t)count * 4);
-    cudaError_t e = cudaMemcpyAsync(buf.data(),
-                                    lt->series + 4ull * (unsigned long long)(first - lt->series_first),
-                                    (size_t)count * 4 * sizeof(long long), cudaMemcpyDeviceToHost,
-                                    lt->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(lt->stream);
+    const cudaError_t e = read_back(buf.data(), lt->series + 4ull * (unsigned long long)(first - lt->series_first),
+                                    (size_t)count * 4 * sizeof(long long), lt->stream);
     if (e != cudaSuccess) return cuda_fail(e, "series copy");
     for (int64_t k = 0; k < count; ++k) {
         if (bond) bond[k] = buf[4 * k + 0];
@@ -1180,10 +1229,9 @@ int lattice_field_series(lattice_t *lt, int64_t first, int64_t count, int64_t *f
     if (!lt->has_fields) return LAT_ENOENT;
     if (first < lt->series_first || first < lt->fields_from || first + count > lt->sweeps) return LAT_ERANGE;
     if (count == 0 || field == nullptr) return LAT_OK;
-    cudaError_t e = cudaMemcpyAsync(field,
-                                    lt->series + 5 * lt->series_cap + (unsigned long long)(first - lt->series_first),
-                                    (size_t)count * sizeof(int64_t), cudaMemcpyDeviceToHost, lt->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(lt->stream);
+    const cudaError_t e =
+        read_back(field, lt->series + 5 * lt->series_cap + (unsigned long long)(first - lt->series_first),
+                  (size_t)count * sizeof(int64_t), lt->stream);
     if (e != cudaSuccess) return cuda_fail(e, "field series copy");
     return band_status(lt);
 }
@@ -1217,10 +1265,9 @@ int lattice_autocorrelation(lattice_t *lt, int64_t first, int64_t count, double 
     if (first < lt->series_first || first < lt->ref_sweep || first + count > lt->sweeps) return LAT_ERANGE;
     if (count == 0) return LAT_OK;
     std::vector<long long> buf((size_t)count);
-    cudaError_t e = cudaMemcpyAsync(buf.data(),
-                                    lt->series + 4 * lt->series_cap + (unsigned long long)(first - lt->series_first),
-                                    (size_t)count * sizeof(long long), cudaMemcpyDeviceToHost, lt->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(lt->stream);
+    const cudaError_t e =
+        read_back(buf.data(), lt->series + 4 * lt->series_cap + (unsigned long long)(first - lt->series_first),
+                  (size_t)count * sizeof(long long), lt->stream);
     if (e != cudaSuccess) return cuda_fail(e, "autocorrelation copy");
     const double N = (double)lt->P.N, m2 = m * m;
     for (int64_t k = 0; k < count; ++k) {

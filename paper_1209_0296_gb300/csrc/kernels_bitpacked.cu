@@ -7,13 +7,12 @@
 // spin (+1).  Words per row bw = ceil((L/2) / 32).
 #include <algorithm>
 
-#include "lattice_internal.cuh"
+#include "bits_step.cuh"
+#include "wide_common.cuh"
 
 namespace lat {
 
 namespace {
-
-constexpr int kThreads = 256;
 
 // planar int8 -> bits: word k of plane c row y holds sites j = 32k .. 32k+31.
 __global__ void k_pack(Geom g, const int8_t *planar, uint32_t *bits)
@@ -215,6 +214,65 @@ __global__ void __launch_bounds__(kThreads, 3) k_bits_pipe(Geom g, int off)
     }
 }
 
+// One colour: a thread per (word column, band of consecutive rows), the
+// other plane's three rows rolling through registers.
+template <int kColour, bool kRef>
+__global__ void __launch_bounds__(kThreads, 3) k_bits_walk(Geom g, int off)
+{
+    __shared__ int red[kThreads / 32][5];
+    dep_wait();
+    const unsigned long long sweep = g.ctrl->sweep + (unsigned long long)off;
+    const uint32_t *old = g.bits[sweep & 1];
+    uint32_t *nw = g.bits[(sweep + 1) & 1];
+    const uint32_t L = (uint32_t)g.L, bw = g.bw;
+    const uint32_t *pS = old + (size_t)kColour * L * bw;
+    const uint32_t *pO = (kColour == 0 ? old : nw) + (size_t)(1 - kColour) * L * bw;
+    uint32_t *dS = nw + (size_t)kColour * L * bw;
+    const uint32_t nb = min((gridDim.x * blockDim.x) / bw, L);
+    const uint32_t gt = blockIdx.x * blockDim.x + threadIdx.x, band = gt / bw, k = gt - band * bw;
+    Counts cnt;
+    if (band < nb) {
+        const uint32_t km = k == 0 ? bw - 1 : k - 1, kp = k == bw - 1 ? 0 : k + 1;
+        PhiloxPre pp;
+        philox_prepare(pp, (uint32_t)sweep, (uint32_t)(sweep >> 32), g.key0, g.key1);
+        const SymK sk = bits_sym(g.thr16);
+        uint32_t y, y1;
+        band_rows(band, nb, L, y, y1);
+        const uint32_t rows = y1 - y;
+        uint32_t U = pO[(size_t)(y == 0 ? L - 1 : y - 1) * bw + k], O = pO[(size_t)y * bw + k];
+        uint32_t nD = pO[(size_t)(y + 1 == L ? 0 : y + 1) * bw + k], nS = pS[(size_t)y * bw + k];
+        uint32_t nN = pO[(size_t)y * bw + (((kColour + y) & 1) ? kp : km)];
+        int downs = 0, uneq = 0, diff = 0;
+        for (; y < y1; ++y) {
+            const uint32_t at = y * bw + k, S = nS, D = nD, N = nN;
+            if (y + 1 < y1) {
+                nS = pS[at + bw];
+                nD = pO[(size_t)(y + 2 >= L ? y + 2 - L : y + 2) * bw + k];
+                nN = pO[(size_t)(y + 1) * bw + (((kColour + y + 1) & 1) ? kp : km)];
+            }
+            const Nbr n = nbr_sum(U, D, O, bits_shifted(((kColour + y) & 1) != 0, O, N));
+            const uint32_t Sn = bits_step(sk, g.thr16, pp, sweep, g.key0, g.key1, y * g.G + 8u * k, (uint32_t)kColour,
+                                          n, S);
+            dS[at] = Sn;
+            if constexpr (kColour == 1) {
+                uneq += bits_unlike(n, Sn);
+                downs += __popc(~Sn) + __popc(~O);
+                if constexpr (kRef)
+                    diff += __popc(Sn ^ g.ref_bits[(size_t)L * bw + at]) + __popc(O ^ g.ref_bits[at]);
+            }
+            U = O;
+            O = D;
+        }
+        cnt.bond = 128 * (int)rows - 2 * uneq;
+        cnt.mag = 64 * (int)rows - 2 * downs;
+        cnt.up = 64 * (int)rows - downs;
+        cnt.acf = 64 * (int)rows - 2 * diff;
+    }
+    dep_launch();   // main work done: the next kernel may be scheduled
+    if constexpr (kColour == 1)
+        flush_slot(series_slot(g.ctrl, sweep), kRef ? acf_slot(g.ctrl, sweep) : nullptr, cnt, false, red);
+}
+
 }  // namespace
 
 cudaError_t launch_pack_bits(const Geom &g, const int8_t *planar, uint32_t *bits, cudaStream_t st)
@@ -234,23 +292,20 @@ cudaError_t launch_sweep_bitpacked(const Geom &g, int off, cudaStream_t st)
 {
     const Geom k = tiled_geom(g);  // compact table in t' = thr - 1 form
     using K = void (*)(Geom, int);
-    const bool ne = g.model == LAT_NE;
-    const K c0 = ne ? k_bits_pipe<true, 0> : k_bits_pipe<false, 0>;
-    const K c1 = ne ? k_bits_pipe<true, 1> : k_bits_pipe<false, 1>;
-    // one wave: SMs x resident CTAs per SM (queried once per model)
-    static int wave[2] = {0, 0};
-    int &w = wave[ne ? 1 : 0];
-    if (w == 0) {
-        int dev = 0, sms = 0, per = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, reinterpret_cast<const void *>(c1), kThreads, 0);
-        w = sms * (per > 0 ? per : 1);
-    }
+    // Ising without a reference, with one; any table; North-East
+    static const K kern[4][2] = {{k_bits_walk<0, false>, k_bits_walk<1, false>},
+                                 {k_bits_walk<0, true>, k_bits_walk<1, true>},
+                                 {k_bits_pipe<false, 0>, k_bits_pipe<false, 1>},
+                                 {k_bits_pipe<true, 0>, k_bits_pipe<true, 1>}};
+    static const unsigned wave[4] = {one_wave(reinterpret_cast<const void *>(kern[0][1])),
+                                     one_wave(reinterpret_cast<const void *>(kern[1][1])),
+                                     one_wave(reinterpret_cast<const void *>(kern[2][1])),
+                                     one_wave(reinterpret_cast<const void *>(kern[3][1]))};
+    const int m = g.model == LAT_NE ? 3 : (k.acc_sym ? (g.ref_bits != nullptr ? 1 : 0) : 2);
     const uint64_t words = (uint64_t)g.L * g.bw;
-    const unsigned blocks = (unsigned)std::min<uint64_t>((words + kThreads - 1) / kThreads, (uint64_t)w);
-    cudaError_t e = launch_pdl(c0, blocks, kThreads, st, k, off);
-    return e == cudaSuccess ? launch_pdl(c1, blocks, kThreads, st, k, off) : e;
+    const unsigned blocks = (unsigned)std::min<uint64_t>((words + kThreads - 1) / kThreads, wave[m]);
+    cudaError_t e = launch_pdl(kern[m][0], blocks, kThreads, st, k, off);
+    return e == cudaSuccess ? launch_pdl(kern[m][1], blocks, kThreads, st, k, off) : e;
 }
 
 bool bitpacked_supported(const Geom &g)

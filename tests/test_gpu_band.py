@@ -75,3 +75,25 @@ def test_disorder(L, kind):
     fields = sign(L * L) if kind in ("fields", "both") else None
     h = 0.0 if kind == "bonds" else 0.6
     _run((2, L, 1, lt.ISING, 1.0, h, 1.7), 9, lt.INIT_RANDOM, CALLS, reference=L == 96, bonds=bonds, fields=fields)
+
+
+@pytest.mark.parametrize("L", [64, 128, 320, 704, 2112])
+def test_bit_packed(L):
+    a = (2, L, 1, lt.ISING, 1.0, 0.0, 2.269185)
+    g = lt.Lattice(*a, seed=L, init=lt.INIT_RANDOM, layout=lt.BITPACKED)
+    o = oracle.Lattice(*a, seed=L, init=lt.INIT_RANDOM)
+    if L in (128, 704):
+        g.set_reference()
+        o.set_reference()
+    done = 0
+    for n in ([17, 1, 16, 5] if L < 1000 else [5]):
+        ser_o = o.sweep(n)
+        g.sweep(n)
+        ser = g.series(done, n)
+        for k in ("bond", "mag", "up"):
+            assert np.array_equal(ser[k], ser_o[k]), (k, n)
+        if L in (128, 704):
+            assert np.array_equal(g.autocorrelation(done, n, m=0.0)[0], ser_o["overlap"])
+        assert np.array_equal(g.get_spins(), o.spins), n
+        done += n
+    g.close()
