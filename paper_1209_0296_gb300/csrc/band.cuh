@@ -293,7 +293,7 @@ LAT_D bool band_updown(const Band &b, const BandWait &wt, const uint8_t *other, 
     return ok;
 }
 
-// Ising, uniform or with the disorder of Eq. 1.
+// Ising with a general table (uniform, bonds, fields), int8 on the chip.
 template <bool kRef, int kDis, bool kSym, bool kFull>
 LAT_D void band_ising(const Geom &g, const BandPart &part, uint32_t band, uint32_t bands, uint8_t *mail,
                      BandShared &sh, uint8_t *smem)
@@ -474,147 +474,6 @@ LAT_D void band_ising(const Geom &g, const BandPart &part, uint32_t band, uint32
         rows_out(smem + c * pb, b.pitch, b.nr, fin + c * b.plane + (size_t)b.y0 * b.half, b.half);
 }
 
-// North-East in c-mode: the main pass and the per-warp draw queue of
-// ne_walk.cuh on shared memory; boundary rows are sent once their queued
-// moves are done.
-template <bool kRef, bool kFull>
-LAT_D void band_ne(const Geom &g, const BandPart &part, uint32_t band, uint32_t bands, uint8_t *mail,
-                     BandShared &sh, uint8_t *smem)
-{
-    const Band b = band_of(g, part, band, bands, mail);
-    const uint32_t tid = threadIdx.x, pb = b.nr * b.pitch, fp = b.pitch >> 2;   // flag bytes per row
-    uint8_t *fl = smem + 2u * pb;
-    NeJob *queue = reinterpret_cast<NeJob *>(smem + ((2u * pb + 2u * b.nr * fp + 15u) & ~15u)) + (tid >> 5) * kNeQueue;
-    int changed = 0;
-    for (int c = 0; c < 2; ++c) {
-        rows_in(b.src + c * b.plane + (size_t)b.y0 * b.half, b.half, b.nr, smem + c * pb, b.pitch);
-        const uint8_t *q = g.flags + ((size_t)c * g.rows + b.y0) * b.G;
-        for (uint32_t i = tid; i < b.nr * b.G; i += blockDim.x) {
-            const uint32_t r = i / b.G, m = i - r * b.G;
-            const uint8_t f = q[i];
-            fl[(c * b.nr + r) * fp + m] = f;
-            changed += __popc((uint32_t)f);
-        }
-    }
-    if (tid < 10) (&sh.sum[0][0])[tid] = 0;
-    if (tid == 10) sh.bad = 0;
-    if (tid == 11) sh.unfl = (int)(2u * b.nr * b.half);
-    __syncthreads();
-    changed = __reduce_add_sync(0xffffffffu, changed);
-    if ((tid & 31u) == 0u) atomicSub(&sh.unfl, changed);
-    __syncthreads();
-    const uint32_t rsb = (uint32_t)kBandThreads / b.cpr, rr = tid / b.cpr, k = tid - rr * b.cpr;
-    const ChunkCol<kFull> cc = chunk_col<kFull>(k, b.half);
-    const NeRate rate = ne_rate(g.thr16);
-    const int lane = (int)(tid & 31u);
-    const unsigned below = (1u << lane) - 1u;
-    const int last = 2 * part.n;
-    PhiloxPre pp;
-    Counts cnt;
-    int bad = 0;   // a wait of this thread gave up
-    for (int h = 0; h < last; ++h) {
-        const uint32_t colour = (uint32_t)h & 1u;
-        const unsigned long long sweep = part.sweep0 + (unsigned long long)(h >> 1);
-        if (colour == 0u) philox_prepare(pp, (uint32_t)sweep, (uint32_t)(sweep >> 32), part.key0, part.key1);
-        uint8_t *mine = smem + colour * pb;
-        const uint8_t *other = smem + (1u - colour) * pb;
-        uint8_t *flc = fl + (size_t)colour * b.nr * fp;
-        const BandWait wt{b.src + (1u - colour) * b.plane, h > 0 ? part.epoch + (uint32_t)h : 0u,
-                          2u * ((1u - colour) * b.cpr + k)};
-        unsigned queued = 0;
-        const NePlanes where{mine, flc, kRef ? g.ref + b.plane : nullptr, b.y0, b.half, b.pitch};
-        auto drain = [&](bool all) {
-            __syncwarp();
-            while (queued >= 32u) {
-                queued -= 32u;
-                ne_job<kRef>(where, pp, rate, queue[queued + lane], colour, cnt);
-            }
-            if (all && (unsigned)lane < queued) ne_job<kRef>(where, pp, rate, queue[lane], colour, cnt);
-            __syncwarp();
-        };
-        for (uint32_t o = rr;; o += rsb) {
-            const bool act = rr < rsb && o < b.nr;
-            if (!__any_sync(0xffffffffu, act)) break;
-            uint32_t cand[4], ws[4], g0 = 0, at = 0;
-            bool need[4] = {false, false, false, false};
-            if (act) {
-                const uint32_t r = band_row(o, b.nr), y = b.y0 + r;
-                const bool odd = ((colour + y) & 1u) != 0u;
-                at = r * b.pitch + cc.j0;
-                g0 = y * b.G + 4u * k;
-                uint32_t U[4], D[4], O[4], S[4], X[4], Sn[4], sure[4];
-                if (!band_updown(b, wt, other, r, cc.j0, cc.nv, U, D)) bad = 1;
-                smem_words(mine + at, S);
-                smem_words(other + at, O);
-                if (odd) {   // east is the shifted row
-                    band_shifted<kFull>(cc, true, other + r * b.pitch, O, X);
-                    ne_moves<kFull>(U, D, X, O, S, cc.vm, rate, cand, sure, ws, Sn, need);
-                } else {
-                    band_shifted<kFull>(cc, false, other + r * b.pitch, O, X);
-                    ne_moves<kFull>(U, D, O, X, S, cc.vm, rate, cand, sure, ws, Sn, need);
-                }
-                store_words<4>(reinterpret_cast<int8_t *>(mine) + at, Sn);
-                if (((sure[0] | sure[1] | sure[2] | sure[3]) & kB1) != 0u) {
-                    uint32_t *f4 = reinterpret_cast<uint32_t *>(flc + (at >> 2));
-                    const uint32_t chg = ne_changed(sure), was = *f4;
-                    *f4 = was | chg;
-                    cnt.unfl -= __popc(chg & ~was);
-                }
-                if (colour == 1u) {
-                    ne_count(Sn, U, D, O, X, cc.vm, cnt);
-                    cnt.up += (int)cc.nv;
-                    if constexpr (kRef) {
-                        uint32_t R1[4], R0[4];
-                        const int8_t *r0 = g.ref + (size_t)y * b.half + cc.j0;
-                        load16_any<kFull>(r0 + b.plane, cc.nv, R1);
-                        load16_any<kFull>(r0, cc.nv, R0);
-#pragma unroll
-                        for (int w = 0; w < 4; ++w)
-                            cnt.acf = dot4(Sn[w] & cc.vm[w], R1[w], dot4(O[w] & cc.vm[w], R0[w], cnt.acf));
-                    }
-                }
-            }
-#pragma unroll
-            for (int w = 0; w < 4; ++w) {
-                const unsigned bal = __ballot_sync(0xffffffffu, need[w]);
-                if (need[w])
-                    queue[queued + __popc(bal & below)] = NeJob{g0 + (uint32_t)w, at + 4u * (uint32_t)w, cand[w], ws[w]};
-                queued += __popc(bal);
-            }
-            if (queued >= 32u) drain(false);
-        }
-        drain(true);
-        if (colour == 1u) {
-            cnt.up += cnt.mag / 2;
-            band_count(sh, h >> 1 & 1, cnt, true, kRef);
-            cnt = Counts();
-        }
-        const int stop = __syncthreads_or(bad);
-        // send the boundary rows; all waits of this half-sweep are over
-        for (uint32_t i = tid; i < 2u * b.cpr; i += blockDim.x) {
-            const bool lo = i >= b.cpr;
-            const uint32_t q = lo ? i - b.cpr : i;
-            uint32_t v[4];
-            smem_words(mine + (lo ? b.nr - 1u : 0u) * b.pitch + 16u * q, v);
-            mail_put((lo ? b.last : b.first) + 2u * (colour * b.cpr + q), part.epoch + (uint32_t)h + 1u, v);
-        }
-        if (colour == 1u) band_post(sh, h >> 1 & 1, g, sweep, true, kRef);
-        if (stop) {
-            sh.bad = 1;
-            break;
-        }
-    }
-    int8_t *fin = ((part.sweep0 + (unsigned long long)part.n) & 1) ? g.s[1] : g.s[0];
-    for (int c = 0; c < 2; ++c) {
-        rows_out(smem + c * pb, b.pitch, b.nr, fin + c * b.plane + (size_t)b.y0 * b.half, b.half);
-        uint8_t *q = g.flags + ((size_t)c * g.rows + b.y0) * b.G;
-        for (uint32_t i = tid; i < b.nr * b.G; i += blockDim.x) {
-            const uint32_t r = i / b.G, m = i - r * b.G;
-            q[i] = fl[(c * b.nr + r) * fp + m];
-        }
-    }
-}
-
 // Lattices with no more than one chunk a thread and colour, Ising or c-mode
 // North-East: a half-sweep is one pass whose length is the latency from a
 // neighbour's packet to this band's own, so everything else is taken off
@@ -790,89 +649,6 @@ LAT_D void band_small(const Geom &g, const BandPart &part, uint32_t band, uint32
                 for (uint32_t w = 0; w < 4u && 4u * k + w < b.G; ++w)
                     g.flags[((size_t)c * g.rows + y) * b.G + 4u * k + w] = (uint8_t)(was[c] >> (8u * w));
     }
-}
-
-// End of a CTA's run: tell the host if a wait gave up; band 0 moves the
-// lattice's sweep counter on.
-LAT_D void band_end(const Geom &g, const BandPart &p, uint32_t band, const BandShared &sh)
-{
-    if (threadIdx.x != 0) return;
-    if (sh.bad) *reinterpret_cast<volatile int *>(p.err) = 1;
-    if (band == 0u) g.ctrl->sweep = p.sweep0 + (unsigned long long)p.n;
-}
-
-// Kinds: Ising with a general or a symmetric table and North-East, each with
-// a partial last chunk or without; without: bonds (either table), fields.
-enum BandKind { kBandGen = 0, kBandSym, kBandNe, kBandGenFull, kBandSymFull, kBandNeFull, kBandBondGen, kBandBondSym,
-                kBandFields, kBandKinds };
-
-template <bool kRef, int kDis, bool kSym, bool kFull>
-LAT_D void band_ising_any(const Geom &g, const BandPart &part, uint32_t band, uint32_t bands, uint8_t *mail,
-                          BandShared &sh, uint8_t *smem)
-{
-    if (band_is_small((uint32_t)g.L, g.half, bands))
-        band_small<false, kRef, kDis, kSym, kFull>(g, part, band, bands, mail, sh, smem);
-    else
-        band_ising<kRef, kDis, kSym, kFull>(g, part, band, bands, mail, sh, smem);
-}
-
-template <bool kRef, bool kFull>
-LAT_D void band_ne_any(const Geom &g, const BandPart &part, uint32_t band, uint32_t bands, uint8_t *mail,
-                       BandShared &sh, uint8_t *smem)
-{
-    if (band_is_small((uint32_t)g.L, g.half, bands))
-        band_small<true, kRef, kUniform, false, kFull>(g, part, band, bands, mail, sh, smem);
-    else
-        band_ne<kRef, kFull>(g, part, band, bands, mail, sh, smem);
-}
-
-template <int kKind, bool kRef>
-LAT_D void band_body(const Geom &g, const BandPart &part, uint32_t band, uint32_t bands, uint8_t *mail,
-                     BandShared &sh, uint8_t *smem)
-{
-    if constexpr (kKind == kBandNe) band_ne_any<kRef, false>(g, part, band, bands, mail, sh, smem);
-    else if constexpr (kKind == kBandNeFull) band_ne_any<kRef, true>(g, part, band, bands, mail, sh, smem);
-    else if constexpr (kKind == kBandGen) band_ising_any<kRef, kUniform, false, false>(g, part, band, bands, mail, sh, smem);
-    else if constexpr (kKind == kBandSym) band_ising_any<kRef, kUniform, true, false>(g, part, band, bands, mail, sh, smem);
-    else if constexpr (kKind == kBandGenFull) band_ising_any<kRef, kUniform, false, true>(g, part, band, bands, mail, sh, smem);
-    else if constexpr (kKind == kBandSymFull) band_ising_any<kRef, kUniform, true, true>(g, part, band, bands, mail, sh, smem);
-    else if constexpr (kKind == kBandBondGen) band_ising_any<kRef, kBonds, false, true>(g, part, band, bands, mail, sh, smem);
-    else if constexpr (kKind == kBandBondSym) band_ising_any<kRef, kBonds, true, true>(g, part, band, bands, mail, sh, smem);
-    else band_ising_any<kRef, kFields, false, true>(g, part, band, bands, mail, sh, smem);
-}
-
-// Rows per band are at least 2, so a lattice has at most L / 2 bands.
-inline size_t band_smem_bytes(const Geom &g, int bands)
-{
-    const size_t nr = ((size_t)g.L + bands - 1) / bands, pitch = ((size_t)g.half + 15) & ~(size_t)15;
-    size_t b = 2 * nr * pitch;
-    if (g.cpl != nullptr) b *= 2;
-    if (g.model == LAT_NE) b = ((b + 2 * nr * (pitch / 4) + 15) & ~(size_t)15) + kBandWarps * kNeQueue * sizeof(NeJob);
-    return b;
-}
-
-// Packet pairs of a lattice in `bands` bands.
-inline size_t band_mail_pairs(const Geom &g, int bands) { return (size_t)bands * 2 * 4 * ((g.half + 15) / 16); }
-
-inline int band_kind(const Geom &k, bool fields)
-{
-    const int full = k.half % 16 == 0 ? kBandGenFull : kBandGen;
-    if (k.model == LAT_NE) return full + kBandNe;
-    if (k.cpl == nullptr) return full + (k.acc_sym ? kBandSym : kBandGen);
-    return fields ? kBandFields : (k.acc_sym ? kBandBondSym : kBandBondGen);
-}
-
-inline BandPart band_part(const Geom &k, unsigned long long sweep0, int n, unsigned epoch, int *err)
-{
-    BandPart p = {};
-    p.epoch = epoch;
-    p.sweep0 = sweep0;
-    p.err = err;
-    p.n = n;
-    p.key0 = k.key0;
-    p.key1 = k.key1;
-    for (int i = 0; i < 8; ++i) p.acc[i] = k.acc[i];
-    return p;
 }
 
 }  // namespace

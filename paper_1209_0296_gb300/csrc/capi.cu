@@ -386,7 +386,7 @@ static int band_bands(const lattice *lt, int64_t n)
 {
     if (n < band_min_sweeps(lt) || lt->graph_pinned || lt->dynamics != LAT_DYNAMICS_CHECKERBOARD) return 0;
     if (lt->P.layout == LAT_INT8 && choose_kernel(lt) != LAT_KERNEL_WIDE) return 0;
-    const int bands = band_count_for(lt->geom);
+    const int bands = band_count_for(lt->geom, lt->has_fields);
     if (bands == 0) return 0;
     return not_capturing(lt->stream) ? bands : 0;
 }
@@ -398,7 +398,7 @@ static int band_sweeps(lattice *lt, int bands, int64_t n, int64_t *done)
 {
     *done = 0;
     if (lt->band_err == nullptr && (lt->band_err = band_error_word()) == nullptr) return LAT_OK;
-    const size_t bytes = band_mail_bytes(lt->geom, bands);
+    const size_t bytes = band_mail_bytes(lt->geom, lt->has_fields, bands);
     if (lt->band_mail == nullptr) {
         if (dev_alloc(&lt->band_mail, bytes, lt->stream) != cudaSuccess) {
             (void)cudaGetLastError();

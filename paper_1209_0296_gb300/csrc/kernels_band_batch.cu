@@ -5,7 +5,7 @@
 #include <cmath>
 #include <mutex>
 
-#include "band.cuh"
+#include "band_kinds.cuh"
 
 namespace lat {
 
@@ -49,13 +49,14 @@ __global__ void __launch_bounds__(kBandThreads, 1) k_band_batch(const Geom *geom
 }
 
 // Estimated us of n sweeps of a lattice on c CTAs: a half-sweep's exchange
-// with the neighbours and its sites at an SM's rate (measured: L = 1024, 2048
-// and 4096 on 152 SMs, 1.15, 2.9 and 8.8 us a half-sweep; rows with a partial
-// chunk L = 5000, 14.9; North-East at c = 0.3 L = 4096, 6.7).
-double band_time(const Geom &g, long long n, int c)
+// with the neighbours and its sites at an SM's rate (from L = 1024 .. 4096 on
+// 152 SMs).
+double band_time(const Geom &k, int kind, long long n, int c)
 {
-    const double rate = g.model == LAT_NE ? 9.0e3 : (g.half % 16 == 0 ? 6.6e3 : 5.8e3);   // sites per us and SM
-    return (double)n * 2.0 * (0.5 * (double)g.N / c / rate + 0.7);
+    // sites per us and SM: int8, bits
+    double rate = 5.8e3;
+    if (band_on_bits(k, kind, c)) rate = k.model == LAT_NE ? 20e3 : 8.5e3;
+    return (double)n * 2.0 * (0.5 * (double)k.N / c / rate + 0.7);
 }
 
 }  // namespace
@@ -63,14 +64,15 @@ double band_time(const Geom &g, long long n, int c)
 // The fewest CTAs that hold the lattice, 0 when it cannot run here.
 int band_min_ctas(const Geom &g)
 {
-    if (g.cpl != nullptr || (g.half + 15) / 16 > (uint32_t)kBandThreads) return 0;
-    if (!(g.model == LAT_NE ? ne_walk_supported(g) : (g.model == LAT_ISING && any_supported(g)))) return 0;
+    const Geom k = tiled_geom(g);
+    const int kind = band_kind(k, false);
+    if (g.cpl != nullptr || kind >= kBandPacked || !band_kind_ok(g, kind)) return 0;
     const int most = std::min(band_sms(), g.L / 2);
     int lo = 1, hi = most;
-    if (hi < 1 || band_smem_bytes(g, hi) > kBandMaxSmem) return 0;
+    if (hi < 1 || !band_fits(k, kind, hi)) return 0;
     while (lo < hi) {   // fewer bands need more memory each
         const int mid = (lo + hi) / 2;
-        if (band_smem_bytes(g, mid) <= kBandMaxSmem) hi = mid;
+        if (band_fits(k, kind, mid)) hi = mid;
         else lo = mid + 1;
     }
     return lo;
@@ -83,7 +85,11 @@ double band_share(const std::vector<std::pair<const Geom *, long long>> &lats, s
     const int sms = band_sms();
     ctas.assign(lats.size(), 0);
     int used = 0;
+    std::vector<Geom> k;
+    std::vector<int> kind;
     for (size_t i = 0; i < lats.size(); ++i) {
+        k.push_back(tiled_geom(*lats[i].first));
+        kind.push_back(band_kind(k.back(), false));
         ctas[i] = band_min_ctas(*lats[i].first);
         if (ctas[i] == 0) return INFINITY;
         used += ctas[i];
@@ -93,7 +99,7 @@ double band_share(const std::vector<std::pair<const Geom *, long long>> &lats, s
         size_t worst = 0;
         double t = -1.0;
         for (size_t i = 0; i < lats.size(); ++i) {
-            const double ti = band_time(*lats[i].first, lats[i].second, ctas[i]);
+            const double ti = band_time(k[i], kind[i], lats[i].second, ctas[i]);
             if (ti > t) {
                 t = ti;
                 worst = i;
@@ -108,7 +114,10 @@ double band_share(const std::vector<std::pair<const Geom *, long long>> &lats, s
 size_t band_batch_mail_bytes(const std::vector<std::pair<const Geom *, long long>> &lats, const std::vector<int> &ctas)
 {
     size_t pairs = 0;
-    for (size_t i = 0; i < lats.size(); ++i) pairs += band_mail_pairs(*lats[i].first, ctas[i]);
+    for (size_t i = 0; i < lats.size(); ++i) {
+        const Geom k = tiled_geom(*lats[i].first);
+        pairs += band_mail_pairs(k, band_kind(k, false), ctas[i]);
+    }
     return kAbortBytes + pairs * sizeof(ulonglong2);
 }
 
@@ -135,8 +144,8 @@ cudaError_t launch_batch_band(const Geom *d_geoms, const std::vector<std::pair<c
         p.kind = (uint32_t)band_kind(k, false);
         p.ref = k.ref != nullptr ? 1u : 0u;
         p.mail = (uint32_t)pairs;
-        pairs += band_mail_pairs(k, ctas[i]);
-        smem = std::max(smem, band_smem_bytes(k, ctas[i]));
+        pairs += band_mail_pairs(k, (int)p.kind, ctas[i]);
+        smem = std::max(smem, band_smem_bytes(k, (int)p.kind, ctas[i]));
         for (int b = 0; b < ctas[i]; ++b) {
             p.band = (uint32_t)b;
             parts->p[cta++] = p;

@@ -470,8 +470,8 @@ cudaError_t launch_batch_ne(const Geom *geoms, const uint2 *items, int n_items, 
 // when a bounded wait gave up (mail must then be zeroed again).  Advances
 // ctrl->sweep.
 int band_sms();   // CTAs of a launch at most
-int band_count_for(const Geom &g);
-size_t band_mail_bytes(const Geom &g, int bands);
+int band_count_for(const Geom &g, bool fields);
+size_t band_mail_bytes(const Geom &g, bool fields, int bands);
 cudaError_t launch_sweep_band(const Geom &g, bool fields, int bands, unsigned long long sweep0, int n, void *mail,
                               unsigned epoch, int *err, cudaStream_t st);
 // Batched form (2D Ising without disorder, c-mode North-East): band_min_ctas

@@ -97,3 +97,38 @@ def test_bit_packed(L):
         assert np.array_equal(g.get_spins(), o.spins), n
         done += n
     g.close()
+
+
+# bands of more than one 16-site chunk a thread hold one bit a site: rows that
+# end inside a word, both directions of the certain move, references, bonds
+@pytest.mark.parametrize("L,ne,par,ref", [(1630, False, 2.3, True), (1602, False, 2.0, False), (1664, False, 2.5, False),
+                                          (1630, True, 0.3, True), (1602, True, 0.8, False), (1664, True, 0.1, True),
+                                          (1700, True, 0.5, False)])
+def test_bits_on_chip(L, ne, par, ref):
+    a = (2, L, 1, lt.NE, 0.0, 0.0, par) if ne else (2, L, 1, lt.ISING, 1.0, 0.0, par)
+    _run(a, 3 + L, lt.INIT_EQUILIBRIUM if ne else lt.INIT_RANDOM, [3, 1, 4], reference=ref)
+
+
+def test_bits_on_chip_with_bonds():
+    rng = np.random.default_rng(8)
+    L = 1632
+    bonds = np.where(rng.random(2 * L * L) < 0.5, -1, 1).astype(np.int8)
+    _run((2, L, 1, lt.ISING, 1.0, 0.0, 1.2), 4, lt.INIT_RANDOM, [5, 6], reference=True, bonds=bonds)
+
+
+@pytest.mark.parametrize("L,c", [(64, 0.3), (320, 0.7), (1728, 0.15)])
+def test_bit_packed_north_east(L, c):
+    a = (2, L, 1, lt.NE, 0.0, 0.0, c)
+    g = lt.Lattice(*a, seed=L, init=lt.INIT_EQUILIBRIUM, layout=lt.BITPACKED)
+    o = oracle.Lattice(*a, seed=L, init=lt.INIT_EQUILIBRIUM)
+    done = 0
+    for n in ([17, 1, 18] if L < 1000 else [3, 2, 4]):
+        ser_o = o.sweep(n)
+        g.sweep(n)
+        ser = g.series(done, n)
+        for k in ("bond", "mag", "up", "unflipped"):
+            assert np.array_equal(ser[k], ser_o[k]), (k, n)
+        spins, flags, _ = g.get_state()
+        assert np.array_equal(spins, o.spins) and np.array_equal(flags, o.flags)
+        done += n
+    g.close()
