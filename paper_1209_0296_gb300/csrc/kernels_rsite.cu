@@ -34,8 +34,8 @@
 //
 // GPU mapping.  lambda <= 32: a group of lambda lanes owns one sub-lattice,
 // a warp holds 32/lambda groups (fewer when shared memory is short) and
-// a CTA several independent warps; collisions are resolved in the warp
-// with match_any (lowest lane wins).  lambda > 32: one CTA of lambda
+// a CTA several independent warps; collisions (lowest lane wins) are found
+// through a byte per site and settled with match_any.  lambda > 32: one CTA of lambda
 // threads per sub-lattice, collisions through an atomicMin owner array.
 // The staged sub-lattice is x-fastest with a one-site halo ring, so a
 // pick's four neighbours are plain loads at +-1 and +-pitch; rows move
@@ -73,6 +73,8 @@ struct Tile {
 
 LAT_HD size_t grid_bytes_of(int b) { return (((size_t)(b + 2) * (size_t)(b + 8)) + 15) & ~(size_t)15; }
 LAT_HD size_t tile_bytes_of(int b) { return grid_bytes_of(b) + (size_t)b * b / 4; }
+// lambda <= 32: one byte per site (modulo this many) for the collision check.
+LAT_HD size_t own_bytes_of(int b) { return (size_t)b * b < 1024 ? (size_t)b * b : 1024; }
 
 LAT_D Tile tile_at(unsigned char *base, int b)
 {
@@ -120,13 +122,17 @@ LAT_D void load_row(const Geom &g, const int8_t *src, const Tile &t, int x0, int
     d[1] = hi;
 }
 
+// (The loops' global loads are independent; unrolled, several are in flight
+// at a time.  A tile is a few kilobytes, so one load after the other the
+// staging took longer than a third of the rounds.)
 template <bool kNE>
-LAT_D void load_tile(const Geom &g, const int8_t *src, const Tile &t, int x0, int y0, int b, bool whole, int tid,
+LAT_D void load_tile(const Geom &g, const int8_t *src, const Tile &t, int x0, int y0, int logb, bool whole, int tid,
                      int nthr)
 {
-    const int L = g.L, groups = b >> 3;   // 8-site groups per row
+    const int L = g.L, b = 1 << logb, lg = logb - 3, groups = b >> 3;   // 8-site groups per row
+#pragma unroll 4
     for (int v = tid; v < b * groups; v += nthr) {
-        const int ly = v / groups, k = v - ly * groups;
+        const int ly = v >> lg, k = v & (groups - 1);
         load_row(g, src, t, x0, y0 + ly, ly + 1, k);
     }
     if (!whole) {
@@ -136,16 +142,21 @@ LAT_D void load_tile(const Geom &g, const int8_t *src, const Tile &t, int x0, in
             load_row(g, src, t, x0, side ? ys : yn, side ? b + 1 : 0, k);
         }
         const int xw = wrapi(x0 - 1, L), xe = wrapi(x0 + b, L);
+#pragma unroll 2
         for (int v = tid; v < 2 * b; v += nthr) {
             const int side = v >= b, ly = v - side * b;
             t.g[(ly + 1) * t.pitch + (side ? b + 4 : 3)] = src[pidx(g, side ? xe : xw, y0 + ly)];
         }
     }
-    if constexpr (kNE) {
-        const int fpr = b >> 3;
-        for (int v = tid; v < 2 * b * fpr; v += nthr) {
-            const int row = v / fpr, m = v - row * fpr, c = row >= b, ly = row - c * b;
-            t.fl[v] = g.flags[((uint64_t)c * g.rows + (uint64_t)(y0 + ly)) * g.G + (uint64_t)((x0 >> 3) + m)];
+    if constexpr (kNE) {   // rows of b / 8 bytes, as words where they are whole ones
+        const bool words = b >= 32 && (g.G & 3u) == 0u;
+        const int lf = words ? logb - 5 : logb - 3, fpr = 1 << lf, n = 2 << (logb + lf);
+#pragma unroll 4
+        for (int v = tid; v < n; v += nthr) {
+            const int row = v >> lf, m = v & (fpr - 1), c = row >> logb, ly = row & (b - 1);
+            const uint8_t *q = g.flags + ((uint64_t)c * g.rows + (uint64_t)(y0 + ly)) * g.G + (uint64_t)(x0 >> 3);
+            if (words) reinterpret_cast<uint32_t *>(t.fl)[v] = reinterpret_cast<const uint32_t *>(q)[m];
+            else t.fl[v] = q[m];
         }
     }
 }
@@ -164,11 +175,12 @@ LAT_D void wrap_halo(const Tile &t, int b, int tid, int nthr)
 }
 
 template <bool kNE>
-LAT_D void store_tile(const Geom &g, int8_t *dst, const Tile &t, int x0, int y0, int b, int tid, int nthr)
+LAT_D void store_tile(const Geom &g, int8_t *dst, const Tile &t, int x0, int y0, int logb, int tid, int nthr)
 {
-    const int groups = b >> 3;
+    const int b = 1 << logb, lg = logb - 3, groups = b >> 3;
+#pragma unroll 4
     for (int v = tid; v < b * groups; v += nthr) {
-        const int ly = v / groups, k = v - ly * groups, y = y0 + ly;
+        const int ly = v >> lg, k = v & (groups - 1), y = y0 + ly;
         const uint32_t *s = reinterpret_cast<const uint32_t *>(t.g + (ly + 1) * t.pitch + 4 + 8 * k);
         uint32_t A, B;
         deinterleave(s[0], s[1], (y & 1) != 0, A, B);
@@ -177,10 +189,14 @@ LAT_D void store_tile(const Geom &g, int8_t *dst, const Tile &t, int x0, int y0,
         *reinterpret_cast<uint32_t *>(dst + g.plane + o) = B;
     }
     if constexpr (kNE) {
-        const int fpr = b >> 3;
-        for (int v = tid; v < 2 * b * fpr; v += nthr) {
-            const int row = v / fpr, m = v - row * fpr, c = row >= b, ly = row - c * b;
-            g.flags[((uint64_t)c * g.rows + (uint64_t)(y0 + ly)) * g.G + (uint64_t)((x0 >> 3) + m)] = t.fl[v];
+        const bool words = b >= 32 && (g.G & 3u) == 0u;
+        const int lf = words ? logb - 5 : logb - 3, fpr = 1 << lf, n = 2 << (logb + lf);
+#pragma unroll 4
+        for (int v = tid; v < n; v += nthr) {
+            const int row = v >> lf, m = v & (fpr - 1), c = row >> logb, ly = row & (b - 1);
+            uint8_t *q = g.flags + ((uint64_t)c * g.rows + (uint64_t)(y0 + ly)) * g.G + (uint64_t)(x0 >> 3);
+            if (words) reinterpret_cast<uint32_t *>(q)[m] = reinterpret_cast<const uint32_t *>(t.fl)[v];
+            else q[m] = t.fl[v];
         }
     }
 }
@@ -191,12 +207,12 @@ LAT_D void store_tile(const Geom &g, int8_t *dst, const Tile &t, int x0, int y0,
 // colour (the balance-preserving variant).
 template <bool kNE>
 LAT_D void decide(const Geom &g, const Tile &t, const TabEntry *stab, int b, int logb, int colour,
-                  uint32_t w_site, uint32_t w_acc, int &site, int8_t &nv, bool &chg)
+                  uint32_t w_site, uint32_t w_acc, int &site, int8_t &nv, bool &allowed, bool &chg)
 {
     if (colour < 0) {
-        site = (int)(((uint64_t)w_site * (uint64_t)(b * b)) >> 32);
+        site = (int)(w_site >> (32 - 2 * logb));   // floor(w * b^2 / 2^32), b a power of two
     } else {
-        const int m = (int)(((uint64_t)w_site * (uint64_t)(b * b / 2)) >> 32);
+        const int m = (int)(w_site >> (33 - 2 * logb));
         const int row = m >> (logb - 1);
         site = (row << logb) + 2 * (m & ((b >> 1) - 1)) + ((row + colour) & 1);
     }
@@ -204,7 +220,7 @@ LAT_D void decide(const Geom &g, const Tile &t, const TabEntry *stab, int b, int
     const int8_t *c = t.g + (ly + 1) * t.pitch + 4 + lx;
     const int s_old = c[0];
     const int nN = c[-t.pitch], nS = c[t.pitch], nW = c[-1], nE = c[1];
-    bool allowed = true;
+    allowed = true;
     if constexpr (kNE) allowed = nN == 1 && nE == 1;   // §III.B: north and east up
     chg = false;
     if (allowed) {
@@ -268,7 +284,7 @@ __global__ void __launch_bounds__(32 * kMaxWarpsPerCta) k_rsite_warp(RsArgs a)
     for (int k = 0; k < S && T0 + k < Q; ++k) {
         int x0, y0;
         tile_origin(T0 + k, nt, logb, x0, y0);
-        load_tile<kNE>(g, src, tile_at(wbase + (size_t)k * a.tile_bytes, b), x0, y0, b, whole, lane, 32);
+        load_tile<kNE>(g, src, tile_at(wbase + (size_t)k * a.tile_bytes, b), x0, y0, logb, whole, lane, 32);
     }
     __syncwarp();
     if (whole) {   // one sub-lattice: its halo is its own periodic image
@@ -286,31 +302,46 @@ __global__ void __launch_bounds__(32 * kMaxWarpsPerCta) k_rsite_warp(RsArgs a)
     const uint32_t calls = (uint32_t)((q + 1) >> 1) << a.loglam;   // Philox calls per sub-lattice
     const uint32_t base = (uint32_t)T * calls + (uint32_t)me;
     const uint32_t tag = 4u + (uint32_t)a.launch;
+    // Collisions: a pick that may move writes its lane to its site's byte; if
+    // some lane reads another's number back the warp settles the round with
+    // match_any.  That instruction alone took 280 of a round's cycles per
+    // scheduler when every round used it; with a 32 x 32 sub-lattice and 16
+    // picks a round, one North-East round in 140 needs it (locked picks
+    // cannot collide with others: they share their site's lock).
+    uint8_t *own = reinterpret_cast<uint8_t *>(t.fl) + (size_t)b * b / 4;
+    const int own_mask = (int)own_bytes_of(b) - 1;
     auto round = [&](uint32_t w_site, uint32_t w_acc, int colour) {
-        int key = -1 - lane;   // distinct for idle lanes
         int site = 0;
         int8_t nv = 0;
-        bool chg = false;
+        bool part = false, chg = false;
         if (act) {
-            decide<kNE>(g, t, stab, b, logb, colour, w_site, w_acc, site, nv, chg);
-            key = grp * P + site;
+            decide<kNE>(g, t, stab, b, logb, colour, w_site, w_acc, site, nv, part, chg);
+            if (part) own[site & own_mask] = (uint8_t)lane;
         }
         __syncwarp();                        // every read of the round is done
-        const unsigned m = __match_any_sync(0xffffffffu, key);
-        if (act && chg && (__ffs(m) - 1) == lane) commit<kNE>(t, b, logb, whole, site, nv);
+        const bool lost = part && own[site & own_mask] != (uint8_t)lane;
+        bool first = true;
+        if (__any_sync(0xffffffffu, lost)) {
+            const unsigned m = __match_any_sync(0xffffffffu, part ? grp * P + site : -1 - lane);
+            first = (__ffs(m) - 1) == lane;
+        }
+        if (chg && first) commit<kNE>(t, b, logb, whole, site, nv);
         __syncwarp();
     };
+    U4 w = act ? philox_item(pp, base, tag) : U4{0u, 0u, 0u, 0u};
     for (int r = 0; r < q; r += 2) {
-        U4 w = U4{0u, 0u, 0u, 0u};
-        if (act) w = philox_item(pp, base + ((uint32_t)(r >> 1) << a.loglam), tag);
+        // the next two rounds' call overlaps this pair's shared-memory latency
+        const U4 next = act && r + 2 < q ? philox_item(pp, base + ((uint32_t)((r >> 1) + 1) << a.loglam), tag)
+                                         : U4{0u, 0u, 0u, 0u};
         round(w.x, w.y, a.balanced ? 0 : -1);
         if (r + 1 < q) round(w.z, w.w, a.balanced ? 1 : -1);
+        w = next;
     }
 
     for (int k = 0; k < S && T0 + k < Q; ++k) {
         int xk, yk;
         tile_origin(T0 + k, nt, logb, xk, yk);
-        store_tile<kNE>(g, dst, tile_at(wbase + (size_t)k * a.tile_bytes, b), xk, yk, b, lane, 32);
+        store_tile<kNE>(g, dst, tile_at(wbase + (size_t)k * a.tile_bytes, b), xk, yk, logb, lane, 32);
     }
 }
 
@@ -336,7 +367,7 @@ __global__ void __launch_bounds__(1024) k_rsite_block(RsArgs a)
     uint32_t *own = reinterpret_cast<uint32_t *>(sm + a.tile_bytes);   // P entries
 
     for (int i = threadIdx.x; i < g.tab_n && i < kMaxTab; i += blockDim.x) stab[i] = g.tab[i];
-    load_tile<kNE>(g, src, t, x0, y0, b, whole, threadIdx.x, blockDim.x);
+    load_tile<kNE>(g, src, t, x0, y0, logb, whole, threadIdx.x, blockDim.x);
     for (int i = threadIdx.x; i < P; i += blockDim.x) own[i] = 0xFFFFFFFFu;
     __syncthreads();
     if (whole) {
@@ -355,7 +386,8 @@ __global__ void __launch_bounds__(1024) k_rsite_block(RsArgs a)
         int site;
         int8_t nv;
         bool chg;
-        decide<kNE>(g, t, stab, b, logb, colour, w_site, w_acc, site, nv, chg);
+        bool part;
+        decide<kNE>(g, t, stab, b, logb, colour, w_site, w_acc, site, nv, part, chg);
         __syncthreads();                     // every read of the round is done
         atomicMin(&own[site], (uint32_t)me);
         __syncthreads();
@@ -369,7 +401,7 @@ __global__ void __launch_bounds__(1024) k_rsite_block(RsArgs a)
         if (r + 1 < q) round(w.z, w.w, a.balanced ? 1 : -1);
     }
     __syncthreads();
-    store_tile<kNE>(g, dst, t, x0, y0, b, threadIdx.x, blockDim.x);
+    store_tile<kNE>(g, dst, t, x0, y0, logb, threadIdx.x, blockDim.x);
 }
 
 // Counters of the state after the sweep (the sub-lattices of launch 1 cannot
@@ -394,9 +426,9 @@ __global__ void __launch_bounds__(kMeasThreads) k_rsite_measure(Geom g, int off)
     const int8_t *sp = g.s[(sweep + 1) & 1];
     const uint32_t nwr = g.half >> 2;              // words per plane row
     const uint32_t cpr = nwr / W;                  // chunks per plane row
-    const uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;   // L^2 < 2^32, so chunks are too
     long long bond = 0, mag = 0, up = 0, unfl = 0, acf = 0;
-    if (t < (uint64_t)g.L * cpr) {
+    if (t < (uint32_t)g.L * cpr) {
         const int L = g.L;
         const int y = (int)(t / cpr), k = (int)(t % cpr);
         const int ym = y == 0 ? L - 1 : y - 1, yp = y == L - 1 ? 0 : y + 1;
@@ -482,7 +514,7 @@ struct RsPlan {
 RsPlan plan(int L, int b, int lambda)
 {
     RsPlan p;
-    const size_t tb = tile_bytes_of(b);
+    const size_t tb = tile_bytes_of(b) + (lambda <= 32 ? own_bytes_of(b) : 0);
     const int Q = (L / b) * (L / b);
     if (lambda <= 32) {
         int S = 32 / lambda;
@@ -535,7 +567,7 @@ cudaError_t launch_sweep_rsite(const Geom &g, int8_t *scratch, int b, int lambda
     a.off = off;
     a.per_warp = p.per_warp;
     a.warps = p.warps;
-    a.tile_bytes = (int)tile_bytes_of(b);
+    a.tile_bytes = (int)(tile_bytes_of(b) + (lambda <= 32 ? own_bytes_of(b) : 0));
     a.balanced = balanced ? 1 : 0;
     const int q = (b * b / 2) / lambda;
     a.rounds = balanced ? q / 2 : q;
