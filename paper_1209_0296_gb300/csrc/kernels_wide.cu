@@ -44,12 +44,10 @@ LAT_D int byte_sum(uint32_t x)
 
 // Sweep colour `colour` of the chunk k (4W sites, W Philox groups) of plane
 // row y of the resident kernel's shared-memory lattice, in place (both
-// buffer pointers of g are that array).  W = 4 is 16 sites per thread;
-// smaller W on small lattices gives more threads with shorter dependency
-// chains.  kPre: the chunk's draws come from the caller (upre).
-template <bool kNE, int W = 4, bool kPre = false>
+// buffer pointers of g are that array).
+template <bool kNE, int W = 4>
 LAT_D void wide_chunk(const SweepView g, const uint32_t *sthr, int colour, unsigned long long sweep,
-                      const PhiloxPre &pp, int y, int k, Counts &cnt, const U4 *upre = nullptr)
+                      const PhiloxPre &pp, int y, int k, Counts &cnt)
 {
     const int8_t *src = g.s0;
     int8_t *dst = g.s0;
@@ -114,10 +112,7 @@ LAT_D void wide_chunk(const SweepView g, const uint32_t *sthr, int colour, unsig
     }
     // An item that needs no draw has t' = all ones at every site, so any u
     // accepts exactly as "no draw" would.
-    if constexpr (kPre) {   // draws made by the caller (same groups, same counters)
-#pragma unroll
-        for (int w = 0; w < W; ++w) u[w] = upre[w];
-    } else if (need) {
+    if (need) {
         const uint32_t g0 = (uint32_t)y * g.G + (uint32_t)(W * k);
 #pragma unroll
         for (int w = 0; w < W; ++w) u[w] = philox_item(pp, g0 + (uint32_t)w, (uint32_t)colour);
@@ -919,7 +914,7 @@ constexpr size_t kResMaxBytes = 220 * 1024;
 // One lattice, n_sweeps sweeps, by the whole CTA.  g may live in shared
 // memory (the batched kernel): the sweep loop reads only register copies.
 // advance: the CTA also moves the lattice's sweep counter on by n_sweeps.
-template <bool kNE, int W>
+template <bool kNE>
 LAT_D void resident_body(const Geom &g, unsigned long long sweep0, int n_sweeps, bool advance, uint4 *res_smem, uint32_t *sthr,
                          int (*red)[5])
 {
@@ -941,42 +936,20 @@ LAT_D void resident_body(const Geom &g, unsigned long long sweep0, int n_sweeps,
     v.s0 = sp;
     v.s1 = sp;
     v.flags = reinterpret_cast<uint8_t *>(fl4);
-    const uint32_t cpr = g.half / (4 * W);
+    const uint32_t cpr = g.half >> 4;
     const uint32_t total = (uint32_t)g.L * cpr;
     unsigned long long *slot0 = series_slot(g.ctrl, sweep0);  // slots of consecutive sweeps are contiguous
     unsigned long long *acf0 = g.ref ? acf_slot(g.ctrl, sweep0) : nullptr;
-    // With at most one chunk per thread and colour, a thread draws both
-    // colours' numbers at the start of the sweep: the colour-1 draws do not
-    // depend on the colour-0 result, so their Philox chain leaves the
-    // critical path.
-    const bool one = W == 1 && total <= blockDim.x;   // (register budget: narrow chunks only)
-    const int y1 = (int)(threadIdx.x / cpr), k1 = (int)(threadIdx.x % cpr);
     for (int s = 0; s < n_sweeps; ++s) {
         const unsigned long long sweep = sweep0 + (unsigned long long)s;
         PhiloxPre pp;
         philox_prepare(pp, (uint32_t)sweep, (uint32_t)(sweep >> 32), g.key0, g.key1);
         Counts cnt;
-        if (W == 1 && one) {
-            const bool act = threadIdx.x < total;
-            U4 u0[W], u1[W];
-            if (act) {
-                const uint32_t g0 = (uint32_t)y1 * g.G + (uint32_t)(W * k1);
-#pragma unroll
-                for (int w = 0; w < W; ++w) {
-                    u0[w] = philox_item(pp, g0 + (uint32_t)w, 0u);
-                    u1[w] = philox_item(pp, g0 + (uint32_t)w, 1u);
-                }
-                wide_chunk<kNE, W, true>(v, sthr, 0, sweep, pp, y1, k1, cnt, u0);
-            }
-            __syncthreads();
-            if (act) wide_chunk<kNE, W, true>(v, sthr, 1, sweep, pp, y1, k1, cnt, u1);
-        } else {
-            for (uint32_t t = threadIdx.x; t < total; t += blockDim.x)
-                wide_chunk<kNE, W>(v, sthr, 0, sweep, pp, (int)(t / cpr), (int)(t % cpr), cnt);
-            __syncthreads();
-            for (uint32_t t = threadIdx.x; t < total; t += blockDim.x)
-                wide_chunk<kNE, W>(v, sthr, 1, sweep, pp, (int)(t / cpr), (int)(t % cpr), cnt);
-        }
+        for (uint32_t t = threadIdx.x; t < total; t += blockDim.x)
+            wide_chunk<kNE>(v, sthr, 0, sweep, pp, (int)(t / cpr), (int)(t % cpr), cnt);
+        __syncthreads();
+        for (uint32_t t = threadIdx.x; t < total; t += blockDim.x)
+            wide_chunk<kNE>(v, sthr, 1, sweep, pp, (int)(t / cpr), (int)(t % cpr), cnt);
         flush_slot(slot0 + 4ull * (unsigned)s, acf0 ? acf0 + (unsigned)s : nullptr, cnt, kNE, red);  // ends with __syncthreads()
     }
     {
@@ -993,13 +966,133 @@ LAT_D void resident_body(const Geom &g, unsigned long long sweep0, int n_sweeps,
     }
 }
 
-template <bool kNE, int W>
-__global__ void __launch_bounds__(kResThreads, 1) k_resident(Geom g, SweepAt at, int n_sweeps)
+// Lattices of at most one four-site word a thread and colour (L = 32, 64). A
+// sweep is then two short dependent steps, so what does not depend on the
+// other colour is taken out of them: a thread keeps its words of both
+// colours (and their persistence bits) in registers, draws for the next
+// half-sweep once its new word is stored, decides by the 16-bit compare, and
+// the counters are summed through shared memory and posted a barrier later.
+// L = 64: 0.93 us a sweep (1.06 with table look-ups, draws and three counter
+// barriers in line); four warps a scheduler, bound by their instruction issue.
+template <bool kNE, bool kSym>
+LAT_D void resident_words(const Geom &g, unsigned long long sweep0, int n_sweeps, bool advance, uint4 *res_smem,
+                          uint32_t *sthr, int (*sum)[5])
+{
+    uint32_t *pl = reinterpret_cast<uint32_t *>(res_smem);   // two planes of words
+    const uint32_t tid = threadIdx.x, wpr = g.half >> 2, words = (uint32_t)g.L * wpr;
+    const uint32_t y = tid / wpr, k = tid - y * wpr;
+    const bool mine = tid < words;
+    const uint32_t *src = reinterpret_cast<const uint32_t *>(g.s[sweep0 & 1]);
+    uint32_t S[2] = {0u, 0u}, was[2] = {0u, 0u}, rw[2] = {0u, 0u};
+    int unfl = 0;
+    if (mine)
+        for (int c = 0; c < 2; ++c) {
+            S[c] = src[c * words + tid];
+            pl[c * words + tid] = S[c];
+            if constexpr (kNE) was[c] = g.flags[c * words + tid];   // G = wpr groups a row
+            if (g.ref) rw[c] = reinterpret_cast<const uint32_t *>(g.ref)[c * words + tid];
+        }
+    if (tid < 16) sthr[tid] = g.thr16[tid];
+    if (tid >= 32 && tid < 42) (&sum[0][0])[tid - 32] = 0;
+    if constexpr (kNE) unfl = mine ? 8 - __popc(was[0]) - __popc(was[1]) : 0;
+    __syncthreads();
+    // shared word indices of the neighbours (the other plane's base is added)
+    const uint32_t iU = (y == 0u ? (uint32_t)g.L - 1u : y - 1u) * wpr + k, iD = (y + 1u == (uint32_t)g.L ? 0u : y + 1u) * wpr + k;
+    const uint32_t iW = y * wpr + (k == 0u ? wpr - 1u : k - 1u), iE = y * wpr + (k + 1u == wpr ? 0u : k + 1u);
+    unsigned long long *slot0 = series_slot(g.ctrl, sweep0);   // consecutive sweeps are contiguous
+    unsigned long long *acf0 = g.ref ? acf_slot(g.ctrl, sweep0) : nullptr;
+    const uint32_t g0 = y * g.G + k;
+    uint32_t p01 = 0, p23 = 0;
+    auto draw = [&](unsigned long long sweep, uint32_t colour) {
+        PhiloxPre pp;
+        philox_prepare(pp, (uint32_t)sweep, (uint32_t)(sweep >> 32), g.key0, g.key1);
+        top_halves(philox_item(pp, g0, colour), p01, p23);
+    };
+    draw(sweep0, 0u);
+    int bond = 0, mag = 0, acf = 0;
+    auto half_sweep = [&](auto which, unsigned long long sweep) {
+        constexpr uint32_t c = decltype(which)::value;
+        if (mine) {
+            const uint32_t *o = pl + (1u - c) * words;
+            const bool odd = ((c + y) & 1u) != 0u;
+            const uint32_t U = o[iU], D = o[iD], O = S[1u - c], nb = o[odd ? iE : iW];
+            const uint32_t X = odd ? __funnelshift_r(O, nb, 8) : __funnelshift_l(nb, O, 8);
+            const Nbr n = nbr_sum(U, D, O, X);
+            uint32_t t01[2], t23[2], tie = kNoTie;
+            if constexpr (kSym) sym_thresholds(g.acc, n, S[c], t01[0], t23[0]);
+            else gen_thresholds2(g.acc, n, n, S[c], S[c], t01, t23);
+            uint32_t rej = reject4(t01[0], t23[0], p01, p23, tie);
+            if (tie_hit(tie)) {
+                PhiloxPre pp;
+                philox_prepare(pp, (uint32_t)sweep, (uint32_t)(sweep >> 32), g.key0, g.key1);
+                rej = reject4_exact(sthr, n, S[c], philox_item(pp, g0, c));
+            }
+            uint32_t F = ~rej & 0xFEFEFEFEu;
+            if constexpr (kNE) F &= ~(U | (odd ? X : O));   // §III.B: north and east must be up
+            S[c] ^= F;
+            pl[c * words + tid] = S[c];
+            draw(sweep + (c == 1u ? 1ull : 0ull), 1u - c);
+            if constexpr (kNE) {
+                const uint32_t bits = (uint32_t)dot4(F & 0x02020202u, 0x08040201u, 0) >> 1;
+                unfl -= __popc(bits & ~was[c]);
+                was[c] |= bits;
+            }
+            if constexpr (c == 1u) {
+                bond = dot4(S[1], X, dot4(S[1], O, dot4(S[1], D, dot4(S[1], U, 0))));
+                mag = dot4(S[1], 0x01010101u, dot4(O, 0x01010101u, 0));
+                if (g.ref) acf = dot4(S[1], rw[1], dot4(O, rw[0], 0));
+            }
+        }
+        if constexpr (c == 1u) {
+            const int par = (int)(sweep & 1ull);
+            const int b = __reduce_add_sync(0xffffffffu, bond), m = __reduce_add_sync(0xffffffffu, mag);
+            [[maybe_unused]] const int f = kNE ? __reduce_add_sync(0xffffffffu, unfl) : 0;
+            const int a = g.ref ? __reduce_add_sync(0xffffffffu, acf) : 0;
+            if ((tid & 31u) == 0u) {
+                atomicAdd(&sum[par][0], b);
+                atomicAdd(&sum[par][1], m);
+                if constexpr (kNE) atomicAdd(&sum[par][3], f);
+                if (g.ref) atomicAdd(&sum[par][4], a);
+            }
+        }
+        __syncthreads();
+        if constexpr (c == 1u) {   // posted while the next half-sweep runs; cleared two barriers before its next use
+            if (tid == 0u) {
+                const int par = (int)(sweep & 1ull);
+                unsigned long long *slot = slot0 + 4ull * (sweep - sweep0);
+                const long long m = sum[par][1];
+                add_counter(slot + 0, sum[par][0]);
+                add_counter(slot + 1, m);
+                add_counter(slot + 2, (m + (long long)g.N) / 2);
+                if constexpr (kNE) add_counter(slot + 3, sum[par][3]);
+                if (g.ref) add_counter(acf0 + (sweep - sweep0), sum[par][4]);
+                for (int i = 0; i < 5; ++i) sum[par][i] = 0;
+            }
+        }
+    };
+    for (int s = 0; s < n_sweeps; ++s) {
+        half_sweep(std::integral_constant<uint32_t, 0>(), sweep0 + (unsigned long long)s);
+        half_sweep(std::integral_constant<uint32_t, 1>(), sweep0 + (unsigned long long)s);
+    }
+    uint32_t *dst = reinterpret_cast<uint32_t *>(g.s[(sweep0 + (unsigned long long)n_sweeps) & 1]);
+    if (mine)
+        for (int c = 0; c < 2; ++c) {
+            dst[c * words + tid] = S[c];
+            if constexpr (kNE) g.flags[c * words + tid] = (uint8_t)was[c];
+        }
+    if (advance && tid == 0) g.ctrl->sweep = sweep0 + (unsigned long long)n_sweeps;   // read by all before the first barrier
+}
+
+// kind 0: the general body; 1, 2: at most one word a thread, general or
+// symmetric table.
+template <bool kNE, int kKind>
+__global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_constant__ Geom g, SweepAt at, int n_sweeps)
 {
     extern __shared__ uint4 res_smem[];
     __shared__ uint32_t sthr[16];
     __shared__ int red[kResThreads / 32][5];
-    resident_body<kNE, W>(g, sweep_of(g.ctrl, at), n_sweeps, at.known != 0, res_smem, sthr, red);
+    if constexpr (kKind == 0) resident_body<kNE>(g, sweep_of(g.ctrl, at), n_sweeps, at.known != 0, res_smem, sthr, red);
+    else resident_words<kNE, kKind == 2>(g, sweep_of(g.ctrl, at), n_sweeps, at.known != 0, res_smem, sthr, red);
 }
 
 // Batched form: CTA i sweeps lattice i (descriptor geoms[i]) by
@@ -1020,11 +1113,12 @@ __global__ void __launch_bounds__(kResThreads, 1) k_batch_resident(const Geom *g
     __syncthreads();
     const bool narrow = (uint64_t)sg.L * (sg.half >> 2) <= (uint64_t)kResThreads;
     if (sg.model == LAT_NE) {
-        if (narrow) resident_body<true, 1>(sg, sg.ctrl->sweep, m, true, res_smem, sthr, red);
-        else resident_body<true, 4>(sg, sg.ctrl->sweep, m, true, res_smem, sthr, red);
+        if (narrow) resident_words<true, false>(sg, sg.ctrl->sweep, m, true, res_smem, sthr, red);
+        else resident_body<true>(sg, sg.ctrl->sweep, m, true, res_smem, sthr, red);
     } else {
-        if (narrow) resident_body<false, 1>(sg, sg.ctrl->sweep, m, true, res_smem, sthr, red);
-        else resident_body<false, 4>(sg, sg.ctrl->sweep, m, true, res_smem, sthr, red);
+        if (narrow && sg.acc_sym) resident_words<false, true>(sg, sg.ctrl->sweep, m, true, res_smem, sthr, red);
+        else if (narrow) resident_words<false, false>(sg, sg.ctrl->sweep, m, true, res_smem, sthr, red);
+        else resident_body<false>(sg, sg.ctrl->sweep, m, true, res_smem, sthr, red);
     }
 }
 
@@ -1146,18 +1240,21 @@ cudaError_t launch_sweep_resident(const Geom &g, SweepAt at, int n_sweeps, cudaS
 {
     const Geom k = tiled_geom(g);
     const size_t smem = resident_bytes(g);
-    // Sites per thread: 4 (W = 1) while that keeps every thread busy, else 16.
     const bool narrow = (uint64_t)g.L * (g.half >> 2) <= (uint64_t)kResThreads;
-    const int m = (g.model == LAT_NE ? 2 : 0) + (narrow ? 1 : 0);
-    static bool attr[4] = {false, false, false, false};
-    void (*fn[4])(Geom, SweepAt, int) = {k_resident<false, 4>, k_resident<false, 1>, k_resident<true, 4>,
-                                     k_resident<true, 1>};
-    if (!attr[m]) {
-        cudaError_t e = cudaFuncSetAttribute(fn[m], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResMaxBytes);
-        if (e != cudaSuccess) return e;
-        attr[m] = true;
-    }
-    fn[m]<<<1, kResThreads, smem, st>>>(k, at, n_sweeps);
+    using K = void (*)(Geom, SweepAt, int);
+    static const K fn[2][3] = {{k_resident<false, 0>, k_resident<false, 1>, k_resident<false, 2>},
+                               {k_resident<true, 0>, k_resident<true, 1>, k_resident<true, 1>}};
+    static const cudaError_t attr = [] {
+        cudaError_t e = cudaSuccess;
+        for (const auto &row : fn)
+            for (K f : row)
+                if (e == cudaSuccess)
+                    e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResMaxBytes);
+        return e;
+    }();
+    if (attr != cudaSuccess) return attr;
+    const unsigned threads = narrow ? std::max(64u, ((unsigned)(g.N / 8) + 31u) / 32u * 32u) : (unsigned)kResThreads;
+    fn[g.model == LAT_NE ? 1 : 0][narrow ? (k.acc_sym ? 2 : 1) : 0]<<<1, threads, smem, st>>>(k, at, n_sweeps);
     return cudaGetLastError();
 }
 
