@@ -58,12 +58,9 @@ LAT_D uint32_t pack32(const int8_t *q, uint32_t nv, bool al, uint32_t vm)
     return ~gather32(w, 7) & vm;
 }
 
-// The way back: 32 int8 spins, only the nv that exist.
-LAT_D void unpack32(uint32_t v, int8_t *q, uint32_t nv, bool al)
+// The way back: 32 bytes to q, only the nv that exist.
+LAT_D void store32(const uint32_t (&w)[8], int8_t *q, uint32_t nv, bool al)
 {
-    uint32_t w[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) w[i] = ~((((v >> (4 * i)) & 0xFu) * 0x00204081u & 0x01010101u) * 0xFEu);
     if (al) {
         reinterpret_cast<uint4 *>(q)[0] = make_uint4(w[0], w[1], w[2], w[3]);
         reinterpret_cast<uint4 *>(q)[1] = make_uint4(w[4], w[5], w[6], w[7]);
@@ -78,6 +75,14 @@ LAT_D void unpack32(uint32_t v, int8_t *q, uint32_t nv, bool al)
             for (int b = 0; b < 4; ++b)
                 if (4u * (uint32_t)i + (uint32_t)b < nv) q[4 * i + b] = (int8_t)(w[i] >> (8 * b));
     }
+}
+
+LAT_D void unpack32(uint32_t v, int8_t *q, uint32_t nv, bool al)
+{
+    uint32_t w[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) w[i] = ~((((v >> (4 * i)) & 0xFu) * 0x00204081u & 0x01010101u) * 0xFEu);
+    store32(w, q, nv, al);
 }
 
 // One row of the other plane as words: its word k shifted towards the side

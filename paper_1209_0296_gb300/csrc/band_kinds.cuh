@@ -3,6 +3,7 @@
 #pragma once
 
 #include "band_bits.cuh"
+#include "band_potts.cuh"
 
 #if defined(__CUDACC__)
 namespace lat {
@@ -19,9 +20,9 @@ LAT_D void band_end(const Geom &g, const BandPart &p, uint32_t band, const BandS
 
 // Kinds: Ising with a general or a symmetric table and North-East, each with
 // a partial last chunk or without; without: bonds (either table), fields;
-// bit-packed layout: Ising (symmetric table), North-East.
+// bit-packed layout: Ising (symmetric table), North-East; 3-state Potts.
 enum BandKind { kBandGen = 0, kBandSym, kBandNe, kBandGenFull, kBandSymFull, kBandNeFull, kBandBondGen, kBandBondSym,
-                kBandFields, kBandPacked, kBandPackedNe, kBandKinds };
+                kBandFields, kBandPacked, kBandPackedNe, kBandPotts3, kBandKinds };
 
 // Kinds that have one bit a site on the chip unless the bands are small.
 LAT_HD bool band_kind_bits(int kind)
@@ -39,7 +40,9 @@ LAT_D void band_body(const Geom &g, const BandPart &part, uint32_t band, uint32_
     constexpr bool kSym = kKind == kBandSym || kKind == kBandSymFull || kKind == kBandBondSym;
     constexpr int kDis = kKind == kBandBondGen || kKind == kBandBondSym ? kBonds : (kKind == kBandFields ? kFields : kUniform);
     constexpr bool kPacked = kKind == kBandPacked || kKind == kBandPackedNe;
-    if constexpr (kPacked) {
+    if constexpr (kKind == kBandPotts3) {
+        band_potts<kRef>(g, part, band, bands, mail, sh, smem);
+    } else if constexpr (kPacked) {
         band_bits<kNe, kRef, false, true>(g, part, band, bands, mail, sh, smem);
     } else {
         if (band_is_small((uint32_t)g.L, g.half, bands))
@@ -54,6 +57,7 @@ LAT_D void band_body(const Geom &g, const BandPart &part, uint32_t band, uint32_
 inline int band_kind(const Geom &k, bool fields)
 {
     if (k.bits[0] != nullptr) return k.model == LAT_NE ? kBandPackedNe : kBandPacked;
+    if (k.model == LAT_POTTS) return kBandPotts3;
     const int full = k.half % 16 == 0 ? kBandGenFull : kBandGen;
     if (k.model == LAT_NE) return full + kBandNe;
     if (k.cpl == nullptr) return full + (k.acc_sym ? kBandSym : kBandGen);
@@ -72,6 +76,7 @@ inline size_t band_smem_bytes(const Geom &k, int kind, int bands)
     const size_t nr = ((size_t)k.L + bands - 1) / bands, ref = k.ref != nullptr || k.ref_bits != nullptr ? 1 : 0;
     if (band_on_bits(k, kind, bands)) {
         const size_t bw = ((size_t)k.half + 31) / 32;
+        if (kind == kBandPotts3) return 4 * nr * bw * (1 + ref) * 4;
         size_t words = 2 * (nr + 2) * bw + 2 * nr * bw * ref;
         if (kind == kBandBondSym) words += 8 * nr * bw;
         if (k.model == LAT_NE) words += 2 * nr * bw + kBandWarps * kBitQueue;
@@ -84,7 +89,7 @@ inline size_t band_smem_bytes(const Geom &k, int kind, int bands)
 // Packet pairs of a lattice.
 inline size_t band_mail_pairs(const Geom &k, int kind, int bands)
 {
-    if (band_on_bits(k, kind, bands)) return (size_t)bands * 2 * ((k.half + 31) / 32);
+    if (band_on_bits(k, kind, bands)) return (size_t)bands * (kind == kBandPotts3 ? 4 : 2) * ((k.half + 31) / 32);
     return (size_t)bands * 2 * 4 * ((k.half + 15) / 16);
 }
 
@@ -101,6 +106,7 @@ inline bool band_kind_ok(const Geom &g, int kind)
 {
     if (kind == kBandPacked) return bitpacked_supported(g) && tiled_geom(g).acc_sym != 0;
     if (kind == kBandPackedNe) return bitpacked_supported(g) && g.cmode != 0;
+    if (kind == kBandPotts3) return g.potts3_ok != 0 && g.cpl == nullptr;
     if (g.model == LAT_NE) return ne_walk_supported(g);
     if (g.model != LAT_ISING) return false;
     return g.cpl == nullptr ? any_supported(g) : wide_supported(g);
@@ -115,7 +121,7 @@ inline BandPart band_part(const Geom &k, unsigned long long sweep0, int n, unsig
     p.n = n;
     p.key0 = k.key0;
     p.key1 = k.key1;
-    for (int i = 0; i < 8; ++i) p.acc[i] = k.acc[i];
+    for (int i = 0; i < 8; ++i) p.acc[i] = k.model == LAT_POTTS ? (i < 4 ? k.potts3[i] : 0u) : k.acc[i];
     return p;
 }
 

@@ -273,6 +273,19 @@ void compact_table(Geom &g, const TabEntry *host_tab)
             }
         }
     }
+    g.potts3_ok = 0;
+    if (g.model == LAT_POTTS && g.dims == 2 && g.two_S == 2) {
+        g.potts3_ok = 1;
+        for (int dn = -g.nmax; dn <= g.nmax; ++dn) {
+            const TabEntry e = host_tab[g.nn + dn + g.nmax];   // df = 0
+            for (int df = 0; df < 3; ++df) {
+                const TabEntry f = host_tab[df * g.nn + dn + g.nmax];
+                if (f.always != e.always || f.thr != e.thr) g.potts3_ok = 0;
+            }
+            if (dn >= 0 ? !e.always : (!e.always && e.thr == 0u)) g.potts3_ok = 0;
+            if (dn < 0) g.potts3[-dn - 1] = e.always ? 0xFFFFFFFFu : e.thr - 1u;
+        }
+    }
     if (g.dims != 2 || g.two_S != 1) return;
     for (int k = 0; k < 16; ++k) {
         const int sd = k >> 3, nd = k & 7;
@@ -385,7 +398,10 @@ static bool not_capturing(cudaStream_t st)
 static int band_bands(const lattice *lt, int64_t n)
 {
     if (n < band_min_sweeps(lt) || lt->graph_pinned || lt->dynamics != LAT_DYNAMICS_CHECKERBOARD) return 0;
-    if (lt->P.layout == LAT_INT8 && choose_kernel(lt) != LAT_KERNEL_WIDE) return 0;
+    // (3-state Potts at sizes without a wide kernel too, unless the generic one was asked for)
+    if (lt->P.layout == LAT_INT8 && choose_kernel(lt) != LAT_KERNEL_WIDE &&
+        !(lt->P.model == LAT_POTTS && lt->kernel != LAT_KERNEL_GENERIC))
+        return 0;
     const int bands = band_count_for(lt->geom, lt->has_fields);
     if (bands == 0) return 0;
     return not_capturing(lt->stream) ? bands : 0;

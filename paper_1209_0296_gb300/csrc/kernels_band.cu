@@ -55,7 +55,7 @@ cudaError_t launch_sweep_band(const Geom &g, bool fields, int bands, unsigned lo
     static const K kern[kBandKinds][2] = {LAT_BAND(kBandGen),      LAT_BAND(kBandSym),     LAT_BAND(kBandNe),
                                           LAT_BAND(kBandGenFull),  LAT_BAND(kBandSymFull), LAT_BAND(kBandNeFull),
                                           LAT_BAND(kBandBondGen),  LAT_BAND(kBandBondSym), LAT_BAND(kBandFields),
-                                          LAT_BAND(kBandPacked),   LAT_BAND(kBandPackedNe)};
+                                          LAT_BAND(kBandPacked),   LAT_BAND(kBandPackedNe), LAT_BAND(kBandPotts3)};
 #undef LAT_BAND
     static std::once_flag once;
     static cudaError_t attr = cudaSuccess;

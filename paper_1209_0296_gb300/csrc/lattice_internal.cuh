@@ -303,6 +303,10 @@ struct Geom {
     // never-accept (not always and thr = 0), so the table converts to the
     // t' = thr - 1 form of the byte-parallel 3D / spin-1 kernels.
     uint32_t tab_strict;
+    // 2D 3-state Potts without field and J >= 0: t' of a move that makes m = 1
+    // .. 4 more neighbours unlike (every other move is certain).
+    uint32_t potts3[4];
+    uint32_t potts3_ok;
 };
 
 // The fields of a Geom that the 2D spin-1/2 sweep kernels read, small

@@ -132,3 +132,28 @@ def test_bit_packed_north_east(L, c):
         assert np.array_equal(spins, o.spins) and np.array_equal(flags, o.flags)
         done += n
     g.close()
+
+
+# words of 32 sites, partial last words, two-row bands, dE = 0 and infinite-T moves, references
+@pytest.mark.parametrize("L,J,T", [(4, 1.0, 0.9), (6, 1.0, 1.5), (62, 1.0, 0.995), (64, 0.0, 1.0), (66, 1.0, 0.3),
+                                   (130, 0.7, 0.7), (306, 1.0, 0.995), (610, 1.0, 2.0), (1632, 1.0, 0.995)])
+def test_potts3(L, J, T):
+    a = (2, L, 2, lt.POTTS, J, 0.0, T)
+    g = lt.Lattice(*a, seed=L, init=lt.INIT_RANDOM)
+    o = oracle.Lattice(*a, seed=L, init=lt.INIT_RANDOM)
+    ref = L in (62, 64, 306)
+    if ref:
+        g.set_reference()
+        o.set_reference()
+    done = 0
+    for n in ([17, 1, 16, 5] if L < 1000 else [4, 3]):
+        ser_o = o.sweep(n)
+        g.sweep(n)
+        ser = g.series(done, n)
+        for k in ("bond", "mag", "up"):
+            assert np.array_equal(ser[k], ser_o[k]), (k, n)
+        if ref:
+            assert np.array_equal(g.autocorrelation(done, n, m=0.0)[0], ser_o["overlap"])
+        assert np.array_equal(g.get_spins(), o.spins), n
+        done += n
+    g.close()
