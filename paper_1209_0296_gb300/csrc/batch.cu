@@ -1,5 +1,7 @@
 // batch.cu -- the batched engine behind lattice_batch_*: many lattices of
-// any sizes and models advanced together.  Each sweep step is a set of
+// any sizes and models advanced together.  2D spin-1/2 lattices whose bands
+// fit the SMs side by side share one cooperative launch for all their sweeps
+// (kernels_band_batch.cu); for the others each sweep step is a set of
 // persistent-grid launches over work lists: two (colour 0, colour 1) per
 // model over (lattice, item) pairs of the 2D spin-1/2 wide kernel, one over
 // (lattice, tile) items of lattices set to the fused tiled kernel, two over
@@ -8,10 +10,9 @@
 // advances every lattice's sweep counter.  Small 2D spin-1/2 lattices
 // instead run as resident CTAs (one CTA per lattice holding it in shared
 // memory for all its sweeps) on a side stream, concurrently with the step
-// loop of the others.  Steps with the same set of lattices are captured
-// once in a CUDA graph and replayed.  Every lattice keeps its own seed,
-// table and sweep counter, so its result is bit-identical to running it
-// alone.
+// loop of the others.  Steps with the same set of lattices are captured once
+// in a CUDA graph and replayed.  Every lattice keeps its own seed, table and
+// sweep counter, so its result is bit-identical to running it alone.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -397,7 +398,10 @@ void plan_bands(Work &work, std::vector<BandGroup> &groups, size_t at_least)
     groups.swap(out);
 }
 
-// Launch the groups one after another on the batch stream.
+// Launch the groups one after another on the batch stream. kBandsRefused:
+// nothing was launched (no memory for the packets, or fewer SMs than the
+// device reports), the step loop takes the lattices.
+constexpr int kBandsRefused = 1;
 int run_bands(lattice_batch *b, BatchSlot &sl, size_t at, std::vector<BandGroup> &groups)
 {
     size_t n = 0, mail = 0;
@@ -409,16 +413,18 @@ int run_bands(lattice_batch *b, BatchSlot &sl, size_t at, std::vector<BandGroup>
     geoms.reserve(n);
     for (auto &g : groups)
         for (auto &pr : g.work) {
-            if (pr.first->band_err == nullptr && (pr.first->band_err = band_error_word()) == nullptr) return LAT_ENOMEM;
+            if (pr.first->band_err == nullptr && (pr.first->band_err = band_error_word()) == nullptr) return kBandsRefused;
             geoms.push_back(tiled_geom(pr.first->geom));
         }
     int rc = grow(&sl.d_band_geoms, sl.band_geoms_cap, (int)n, b->stream);
+    if (rc == LAT_ENOMEM) return kBandsRefused;
     if (rc != LAT_OK) return rc;
     cudaError_t e = cudaSuccess;
     if (mail > b->mail_cap) {
         void *p = nullptr;
         e = dev_alloc(&p, mail, b->stream);
-        if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? LAT_ENOMEM : cuda_fail(e, "batch packets");
+        if (e == cudaErrorMemoryAllocation) return kBandsRefused;
+        if (e != cudaSuccess) return cuda_fail(e, "batch packets");
         dev_free(b->d_mail, b->stream);
         b->d_mail = p;
         b->mail_cap = mail;
@@ -458,6 +464,7 @@ int run_bands(lattice_batch *b, BatchSlot &sl, size_t at, std::vector<BandGroup>
                 if (e == cudaSuccess)
                     e = launch_batch_band(sl.d_band_geoms + first, l, sweep0, err, g.ctas, b->d_mail, b->mail_epoch,
                                           b->stream);
+                if (e == cudaErrorCooperativeLaunchTooLarge && first == 0 && k == 0) return kBandsRefused;
             }
             b->mail_epoch += 2u * (unsigned)most;
         }
@@ -733,14 +740,26 @@ int lattice_batch_run(lattice_batch_t *b)
     work.swap(rest);
     // Lattices that fit the chip's shared memory: all their sweeps in a few launches.
     std::vector<BandGroup> groups;
-    plan_bands(work, groups, b->caller_orders ? 2 : 1);
+    const auto unplanned = work;
+    // (the launches carry the host's sweep numbers: not while the caller captures the stream)
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(b->stream, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone)
+        plan_bands(work, groups, b->caller_orders ? 2 : 1);
     // the resident and band lattices' uploads sit at the front of the staging
     size_t res_bytes = res.empty() ? 0 : ((res.size() * (sizeof(Geom) + sizeof(long long)) + 64 + 15) & ~(size_t)15);
     std::vector<std::pair<lattice *, int64_t>> banded;
     if (!groups.empty()) {
         mark_start();
         int rc = run_bands(b, sl, res_bytes, groups);
-        if (rc != LAT_OK) return rc;
+        if (rc == kBandsRefused) {
+            (void)cudaGetLastError();
+            work = unplanned;
+            groups.clear();
+        } else if (rc != LAT_OK) {
+            return rc;
+        }
+    }
+    if (!groups.empty()) {
         for (auto &g : groups)
             for (auto &pr : g.work) {
                 pr.first->sweeps += pr.second;

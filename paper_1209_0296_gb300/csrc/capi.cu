@@ -375,6 +375,11 @@ BandTurn::~BandTurn()
 // resident kernel is made for it saves little more than nothing.
 static int64_t band_min_sweeps(const lattice *lt)
 {
+    // 3-state Potts: the half-sweep of a small lattice is the chain of one
+    // word's draws and its packets, 2.6 us, longer than a launch (16 sweeps, L =
+    // 768: 98 us in bands, 90 in launches; 896: 100 and 115; 4 sweeps 31 and 31).
+    // L no multiple of 16 has the generic kernel to beat (L = 100: 182 us, 84).
+    if (lt->P.model == LAT_POTTS) return !potts_supported(lt->geom) || lt->P.N >= 750000u ? 4 : INT64_MAX;
     if (lt->P.L <= 128) return 16;
     return lt->P.N * (lt->geom.cpl != nullptr ? 2u : 1u) > 6000000u ? 5 : 3;
 }
@@ -415,12 +420,16 @@ static int band_sweeps(lattice *lt, int bands, int64_t n, int64_t *done)
     *done = 0;
     if (lt->band_err == nullptr && (lt->band_err = band_error_word()) == nullptr) return LAT_OK;
     const size_t bytes = band_mail_bytes(lt->geom, lt->has_fields, bands);
-    if (lt->band_mail == nullptr) {
+    if (bytes > lt->band_mail_cap) {
+        dev_free(lt->band_mail, lt->stream);
+        lt->band_mail = nullptr;
+        lt->band_mail_cap = 0;
         if (dev_alloc(&lt->band_mail, bytes, lt->stream) != cudaSuccess) {
             (void)cudaGetLastError();
             lt->band_mail = nullptr;
             return LAT_OK;
         }
+        lt->band_mail_cap = bytes;
         lt->band_epoch = 1u << 30;   // clear below
     }
     const int64_t most = std::max<int64_t>(8, std::min<int64_t>(1 << 16, (int64_t)(1e11 / (double)lt->P.N)));
@@ -428,7 +437,7 @@ static int band_sweeps(lattice *lt, int bands, int64_t n, int64_t *done)
         const int k = (int)std::min<int64_t>(most, n - *done);
         cudaError_t e = cudaSuccess;
         if (lt->band_epoch >= 1u << 30) {
-            e = cudaMemsetAsync(lt->band_mail, 0, bytes, lt->stream);
+            e = cudaMemsetAsync(lt->band_mail, 0, lt->band_mail_cap, lt->stream);
             lt->band_epoch = 0;
         }
         if (e == cudaSuccess) {
@@ -437,6 +446,10 @@ static int band_sweeps(lattice *lt, int bands, int64_t n, int64_t *done)
             if (e == cudaSuccess)
                 e = launch_sweep_band(lt->geom, lt->has_fields, bands, (unsigned long long)(lt->sweeps + *done), k,
                                       lt->band_mail, lt->band_epoch, lt->band_err, lt->stream);
+        }
+        if (e == cudaErrorCooperativeLaunchTooLarge) {   // fewer SMs than the device reports: the launches go on
+            (void)cudaGetLastError();
+            return LAT_OK;
         }
         if (e != cudaSuccess) return cuda_fail(e, "band sweep launch");
         lt->band_epoch += 2u * (unsigned)k;

@@ -477,8 +477,9 @@ Geom tiled_geom(const Geom &g)
     for (int i = 0; i < 16; ++i)
         k.thr16[i] = ((g.always16 >> i) & 1u) ? 0xFFFFFFFFu : g.thr16[i] - 1u;
     // sd << 3 | nd indexes thr16: unlike neighbours of an up spin are the
-    // down ones, of a down spin the others
-    k.acc_sym = 1;
+    // down ones, of a down spin the others.  Field signs (a second table half,
+    // for -h) take the general form even at h = 0.
+    k.acc_sym = g.tab_n > (2 * g.dsmax + 1) * g.nn ? 0 : 1;
     for (int nd = 0; nd <= 4; ++nd)
         if (k.thr16[nd] != k.thr16[8 + 4 - nd] || (nd >= 2 && k.thr16[nd] != 0xFFFFFFFFu)) k.acc_sym = 0;
     for (uint32_t &w : k.acc) w = 0;

@@ -95,6 +95,7 @@ struct lattice {
     bool graph_valid = false;
     // band-resident sweeps (kernels_band.cu)
     void *band_mail = nullptr;           // boundary-row packets
+    size_t band_mail_cap = 0;            // its bytes: the kinds of a lattice's life differ (disorder set or dropped)
     unsigned band_epoch = 0;             // at least every packet mark sent so far
     int *band_err = nullptr;             // host-visible word: a bounded wait gave up
 };

@@ -136,12 +136,12 @@ def test_bit_packed_north_east(L, c):
 
 # words of 32 sites, partial last words, two-row bands, dE = 0 and infinite-T moves, references
 @pytest.mark.parametrize("L,J,T", [(4, 1.0, 0.9), (6, 1.0, 1.5), (62, 1.0, 0.995), (64, 0.0, 1.0), (66, 1.0, 0.3),
-                                   (130, 0.7, 0.7), (306, 1.0, 0.995), (610, 1.0, 2.0), (1632, 1.0, 0.995)])
+                                   (130, 0.7, 0.7), (306, 1.0, 0.995), (610, 1.0, 2.0), (896, 0.0, 1.0), (1632, 1.0, 0.995)])
 def test_potts3(L, J, T):
     a = (2, L, 2, lt.POTTS, J, 0.0, T)
     g = lt.Lattice(*a, seed=L, init=lt.INIT_RANDOM)
     o = oracle.Lattice(*a, seed=L, init=lt.INIT_RANDOM)
-    ref = L in (62, 64, 306)
+    ref = L in (62, 306, 896)
     if ref:
         g.set_reference()
         o.set_reference()
@@ -156,4 +156,27 @@ def test_potts3(L, J, T):
             assert np.array_equal(g.autocorrelation(done, n, m=0.0)[0], ser_o["overlap"])
         assert np.array_equal(g.get_spins(), o.spins), n
         done += n
+    g.close()
+
+
+# one lattice through kinds with packets of different sizes: bits, then fields (int8; h = 0, so that they are not
+# felt), bonds (bits), uniform again; in bands and, one sweep, in launches
+def test_kinds_of_one_lattice():
+    rng = np.random.default_rng(1)
+    L, n = 1632, 4
+    a = (2, L, 1, lt.ISING, 1.0, 0.0, 1.6)
+    g = lt.Lattice(*a, seed=2, init=lt.INIT_RANDOM)
+    o = oracle.Lattice(*a, seed=2, init=lt.INIT_RANDOM)
+    g.set_kernel(lt.KERNEL_WIDE)
+    sign = lambda m: np.where(rng.random(m) < 0.5, -1, 1).astype(np.int8)
+    for step in ("uniform", "fields", "bonds", "none"):
+        fields = sign(L * L) if step == "fields" else None
+        bonds = sign(2 * L * L) if step == "bonds" else None
+        for x in (g, o):
+            x.set_fields(fields)
+            x.set_couplings(bonds)
+        for m in (n, 1):
+            g.sweep(m)
+            o.sweep(m)
+            assert np.array_equal(g.get_spins(), o.spins), (step, m)
     g.close()
