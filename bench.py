@@ -238,17 +238,24 @@ def run_gpu(args):
     updates = world * args.steps * n_lat * S * L * L
     value = replica_value(args.steps * n_lat * S * L * L, world, total_ms * 1e-3)
 
-    # Kernel launches per step: per int8 lattice, S sweeps (one launch each
-    # for the tiled kernel, two for the wide one); per bit-packed lattice two
-    # launches per sweep; plus one counter-advance kernel per graph replay
-    # and per direct remainder.
+    # Kernel launches per step.  A call of S sweeps on the wide kernel or the
+    # bit-packed layout is one launch (the band-resident kernel; up to 1e11
+    # site updates each) unless a graph size was asked for.  Else, per int8
+    # lattice, S sweeps (one launch each for the tiled kernel, two for the
+    # wide one), per bit-packed lattice two launches per sweep; plus one
+    # counter-advance kernel per graph replay and per direct remainder.
     kinfo = lats["int8"][0].get_kernel()
     gk = kinfo["sweeps_per_graph"]
     gkb = lats["bitpacked"][0].get_kernel()["sweeps_per_graph"]
+    calls = lambda cap: -(-S // cap)
+    band_cap = max(8, min(1 << 16, int(1e11 / (L * L))))
+    int8_band = kinfo["kernel"] == lt.KERNEL_WIDE and args.graph == 0 and S >= 5
+    bits_band = S >= 5
     per_sweep = 1 if kinfo["kernel"] == lt.KERNEL_TILED else 2
-    adv = lambda g_: S // g_ + (1 if S % g_ else 0)
-    launches = args.steps * len(TEMPS) * (per_sweep * S + adv(gk) + 2 * S + adv(gkb))
-    sweep_launches = args.steps * len(TEMPS) * (per_sweep + 2) * S
+    sweeps_of = lambda band, per: calls(band_cap) if band else per * S
+    sweep_launches = args.steps * len(TEMPS) * (sweeps_of(int8_band, per_sweep) + sweeps_of(bits_band, 2))
+    launches = sweep_launches + args.steps * len(TEMPS) * ((0 if int8_band else calls(gk)) +
+                                                           (0 if bits_band else calls(gkb)))
     # average duration of one sweep of one lattice (all its launches, the
     # tiny advance kernels and launch gaps: this under-reports kernel rates)
     avg_kernel_us = ms_int8 * 1e3 / (args.steps * len(TEMPS) * S)
@@ -261,7 +268,9 @@ def run_gpu(args):
     prof = load_profile_numbers(kname)
     roofline = {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s",
                 "frac": achieved / hbm, "traffic": prof.get("traffic_bytes_per_sweep"),
-                "kernel": "k_sweep_tiled<Ising>" if kname == "tiled" else "k_wide_pipe<colour 0, colour 1>",
+                "kernel": "k_sweep_tiled<Ising>" if kname == "tiled" else
+                          ("k_band<symmetric table, one bit a site on the chip>" if int8_band else
+                           "k_ising_walk<colour 0, colour 1>"),
                 "peak_kind": peak_kind + " (copy bandwidth)",
                 "bytes_per_sweep": alg_bytes,
                 "avg_sweep_us": avg_kernel_us}
@@ -269,7 +278,7 @@ def run_gpu(args):
     bbytes = 0.25 * L * L  # one bit read + one bit written per site per sweep
     bach = bbytes / (avg_bits_us * 1e-6) / 1e9
     roofline_bits = {"bound": "hbm", "achieved": bach, "peak": hbm, "unit": "GB/s", "frac": bach / hbm,
-                     "traffic": bprof.get("traffic_bytes_per_sweep"), "kernel": "k_bits_pipe<colour 0, colour 1>",
+                     "traffic": bprof.get("traffic_bytes_per_sweep"), "kernel": "k_band<bit-packed>" if bits_band else "k_bits_walk<colour 0, colour 1>",
                      "bytes_per_sweep": bbytes, "avg_sweep_us": avg_bits_us,
                      "updates_per_ns": L * L / (avg_bits_us * 1e3)}
     sm_clk = (clk.summary().get("sm_mhz") or 2070.0) * 1e6
@@ -694,7 +703,7 @@ def hbm_sized_run(dev, hbm, L5=32768, n=100):
     out = {"workload": "2D Ising spin-1/2, L=%d, T=2.269185, random start (seed 7), int8" % L5,
            "sweeps": n, "updates_per_ns": N5 * n / t / 1e9, "achieved": ach, "peak": hbm, "unit": "GB/s",
            "frac": ach / hbm, "bytes_per_sweep": 2.0 * N5, "avg_sweep_us": t / n * 1e6,
-           "kernel": {lt.KERNEL_WIDE: "k_wide_pipe<colour 0, colour 1>", lt.KERNEL_TILED: "k_sweep_tiled<Ising>"}.get(
+           "kernel": {lt.KERNEL_WIDE: "k_ising_walk<colour 0, colour 1>", lt.KERNEL_TILED: "k_sweep_tiled<Ising>"}.get(
                g.get_kernel()["kernel"], "?")}
     g.close()
     return out

@@ -66,7 +66,10 @@ enum lattice_status {
     LAT_EINVAL = -1,   /* invalid argument */
     LAT_ENOMEM = -2,   /* device or host allocation failed */
     LAT_ECUDA = -3,    /* a CUDA call failed (see lattice_last_cuda_error) */
-    LAT_ETIMEOUT = -4, /* a bounded device-side wait gave up */
+    LAT_ETIMEOUT = -4, /* a bounded wait gave up: lattice_server_drain's limit, or (about
+                          ten seconds) a band of a band-resident launch waiting for its
+                          neighbour's rows; after the latter the lattice's state is
+                          undefined and every call on it returns this */
     LAT_EBUSY = -5,    /* result not ready yet (server poll) */
     LAT_ENOTSUP = -6,  /* valid but unsupported combination */
     LAT_ERANGE = -7,   /* index or size out of range */
@@ -101,9 +104,13 @@ enum lattice_kernel {
     LAT_KERNEL_TILED = 2,   /* one launch per sweep, shared-memory tiles with halo
                                recompute; 2D spin-1/2 (Ising and North-East), L % 32 == 0 */
     LAT_KERNEL_WIDE = 3,    /* two launches per sweep, several sites per thread: 2D
-                               spin-1/2 (Ising and North-East, L % 32 == 0; with
-                               coupling and field signs too), Ising in 3D / with
-                               spin S > 1/2 (L % 16 == 0), or Potts (L % 16 == 0) */
+                               spin-1/2 (Ising and North-East at any even L; with
+                               coupling and field signs for L % 32 == 0), Ising in 3D /
+                               with spin S > 1/2 (L % 16 == 0), or Potts (L % 16 == 0).
+                               Calls of a few sweeps or more on 2D spin-1/2 and 3-state
+                               Potts lattices that fit the SMs' shared memory run in
+                               one cooperative launch instead (every SM holds a band of
+                               rows), unless lattice_set_kernel gave a graph size */
     LAT_KERNEL_RESIDENT = 4 /* one launch for many sweeps: one CTA holds the whole
                                lattice in shared memory; 2D spin-1/2 (Ising and
                                North-East), L % 32 == 0, L^2 (+ L^2/4 for North-East)
@@ -325,8 +332,10 @@ int lattice_synchronize(lattice_t *lat);
 void lattice_destroy(lattice_t *lat);
 
 /* ------------------------------------------------------------------ */
-/* Batch: many lattices (any sizes and models) advanced by one          */
-/* persistent-kernel launch per sweep step, replayed from a CUDA graph. */
+/* Batch: many lattices (any sizes and models) advanced together: 2D    */
+/* spin-1/2 ones that fit the SMs side by side by one cooperative       */
+/* launch for all their sweeps, the others by one set of persistent     */
+/* launches per sweep step, replayed from a CUDA graph.                 */
 /* Results are bit-exact with running each lattice alone.               */
 /* ------------------------------------------------------------------ */
 

@@ -158,10 +158,6 @@ LAT_D bool mail_take_word(const unsigned long long *q, uint32_t tag, unsigned *a
     }
 }
 
-// Local rows in the order they are visited: interior first, then the first
-// and the last.
-LAT_D uint32_t band_row(uint32_t o, uint32_t nr) { return o + 2u < nr ? o + 1u : (o + 2u == nr ? 0u : nr - 1u); }
-
 // nr rows of half bytes, global (row pitch half) -> shared (row pitch
 // pitch, a multiple of 4), whole words at any alignment.
 LAT_D void rows_in(const int8_t *from, uint32_t half, uint32_t nr, uint8_t *to, uint32_t pitch)

@@ -10,15 +10,15 @@
 // writes.  Neighbour counts, thresholds and acceptance are those of the
 // tiled kernel (bytes 0x01 / 0xFF, bit-sliced adder, t' = thr - 1 table).
 //
-// The solo kernels (k_wide_pipe for Ising, uniform or with per-bond and
-// per-site disorder; k_wide_pipe_ne for the North-East model; k_any_pipe*
-// for any even L) walk one chunk column per thread down the rows with two
-// chunks in flight, so the Philox draws of one chunk (wide multiplies) and
-// the Metropolis step of the other (logic) share each instruction block.
-// They read s[sweep & 1] and write s[(sweep+1) & 1] without copying a
-// plane: colour 1 takes the new colour-0 sites from the new buffer.  The
-// resident kernels (wide_chunk, in place) keep the whole lattice in one
-// CTA's shared memory.
+// The solo kernels (k_ising_walk for Ising at any even L, uniform or with
+// per-bond and per-site disorder: ising_walk.cuh; k_wide_pipe_ne and
+// k_any_pipe_ne for North-East rates that are not of the c-mode form, which
+// kernels_ne.cu has) walk one chunk column per thread down the rows. They
+// read s[sweep & 1] and write s[(sweep+1) & 1] without copying a plane:
+// colour 1 takes the new colour-0 sites from the new buffer. Calls of
+// several sweeps on lattices that fit the SMs' shared memory run in bands
+// instead (kernels_band.cu). The resident kernels (wide_chunk or one word a
+// thread, in place) keep the whole lattice in one CTA's shared memory.
 #include <algorithm>
 
 #include "ising_walk.cuh"
@@ -42,13 +42,14 @@ LAT_D int byte_sum(uint32_t x)
     return (int)((s & 0xFFFFu) + (s >> 16));
 }
 
-// Sweep colour `colour` of the chunk k (4W sites, W Philox groups) of plane
+// Sweep colour `colour` of the chunk k (16 sites, four Philox groups) of plane
 // row y of the resident kernel's shared-memory lattice, in place (both
 // buffer pointers of g are that array).
-template <bool kNE, int W = 4>
+template <bool kNE>
 LAT_D void wide_chunk(const SweepView g, const uint32_t *sthr, int colour, unsigned long long sweep,
                       const PhiloxPre &pp, int y, int k, Counts &cnt)
 {
+    constexpr int W = 4;
     const int8_t *src = g.s0;
     int8_t *dst = g.s0;
     const int L = g.L;
@@ -143,23 +144,10 @@ LAT_D void wide_chunk(const SweepView g, const uint32_t *sthr, int colour, unsig
         // persistence bytes of the W groups (bit q = site 4m+q)
         uint8_t *fb = g.flags + ((uint64_t)colour * L + y) * g.G + (uint64_t)(W * k);
         const uint8_t *fob = g.flags + ((uint64_t)oc * L + y) * g.G + (uint64_t)(W * k);
-        uint32_t f, fo = 0;
-        if constexpr (W == 4) {
-            uint32_t *fp = reinterpret_cast<uint32_t *>(fb);
-            f = *fp | chg;
-            *fp = f;
-            if (colour == 1) fo = *reinterpret_cast<const uint32_t *>(fob);
-        } else if constexpr (W == 2) {
-            uint16_t *fp = reinterpret_cast<uint16_t *>(fb);
-            f = (uint32_t)*fp | chg;
-            *fp = (uint16_t)f;
-            if (colour == 1) fo = *reinterpret_cast<const uint16_t *>(fob);
-        } else {
-            f = (uint32_t)*fb | chg;
-            *fb = (uint8_t)f;
-            if (colour == 1) fo = *fob;
-        }
-        if (colour == 1) unfl = 8 * W - __popc(f) - __popc(fo);
+        uint32_t *fp = reinterpret_cast<uint32_t *>(fb);
+        const uint32_t f = *fp | chg;
+        *fp = f;
+        if (colour == 1) unfl = 8 * W - __popc(f) - __popc(*reinterpret_cast<const uint32_t *>(fob));
     }
     if (colour == 1) {
         const int d2 = byte_sum(dn);
@@ -181,20 +169,13 @@ LAT_D void wide_chunk(const SweepView g, const uint32_t *sthr, int colour, unsig
 }
 
 // ---------------------------------------------------------------------
-// Software-pipelined two-launch Ising sweep, uniform or with per-bond
-// coupling signs (kCpl) and per-site field signs (kFld).  Same chunks,
-// draws, table and bits as the resident kernel's wide_chunk; the difference
-// is the schedule.  A chunk costs two kinds of work that load
-// different pipes: its four Philox4x32-10 calls (wide multiplies on the
-// FMA pipe) and the Metropolis step (logic on the ALU pipe).  Done one
-// after the other they keep one pipe idle while the other works, so each
-// iteration here loads and draws chunk i+1 in the same straight-line block
-// as the Metropolis step of chunk i, and the two streams interleave.
+// One 16-site chunk of a North-East column walk: the kernels that take any
+// rate table and the general step (k_wide_pipe_ne) load chunk i + 1 in the
+// same straight-line block as the step of chunk i.
 // ---------------------------------------------------------------------
 struct WideIn {
     uint32_t S[4], O[4], U[4], D[4];
     uint32_t adj;
-    uint32_t C[4];   // disorder bytes of the chunk's sites (kCpl only)
 };
 
 // What one thread needs to walk its chunk column k (16 sites) down the
@@ -208,7 +189,6 @@ struct ColWalk {
     const int8_t *pOrow;   // the other colour's current sites (row starts)
     int8_t *dS;            // this colour's plane in the new buffer, + 16k
     const int8_t *r1, *r0; // reference planes 1 and 0, + 16k (or null)
-    const int8_t *pC;      // this colour's disorder bytes, + 16k (or null)
     uint32_t half, L, G, k;
     uint32_t adjb0, adjb1; // byte offset in the row of the neighbour word past the chunk end, x parity 0 / 1
 };
@@ -229,7 +209,6 @@ LAT_D ColWalk<kColour> col_walk(const SweepView &g, const int8_t *old, int8_t *n
     c.dS = nw + (size_t)kColour * plane + 16 * k;
     c.r1 = g.ref ? g.ref + (size_t)plane + 16 * k : nullptr;
     c.r0 = g.ref ? g.ref + 16 * k : nullptr;
-    c.pC = g.cpl ? reinterpret_cast<const int8_t *>(g.cpl) + (size_t)kColour * plane + 16 * k : nullptr;
     c.half = g.half;
     c.L = (uint32_t)g.L;
     c.G = g.G;
@@ -240,8 +219,8 @@ LAT_D ColWalk<kColour> col_walk(const SweepView &g, const int8_t *old, int8_t *n
     return c;
 }
 
-// Loads of the walk's chunk in plane row y (and its disorder bytes when kCpl).
-template <int kColour, bool kCpl = false>
+// Loads of the walk's chunk in plane row y.
+template <int kColour>
 LAT_D void col_load(const ColWalk<kColour> &c, uint32_t y, WideIn &in)
 {
     const uint32_t oy = y * c.half;
@@ -252,12 +231,10 @@ LAT_D void col_load(const ColWalk<kColour> &c, uint32_t y, WideIn &in)
     load_words<4>(c.pO + oym, in.U);   // north
     load_words<4>(c.pO + oyp, in.D);   // south
     in.adj = *reinterpret_cast<const uint32_t *>(c.pOrow + oy + (((kColour + y) & 1) ? c.adjb1 : c.adjb0));
-    if constexpr (kCpl) load_words<4>(c.pC + oy, in.C);
 }
 
 constexpr int kPipeMinB = 2;   // CTAs per SM (the two chunks in flight need ~100 registers)
-
-constexpr int kWalkMinB = 2;
+constexpr int kWalkMinB = 2;   // (3, with fewer registers: 24 us a sweep at L = 4096 for 20.5)
 
 // 2D Ising, one colour.  kOne: a thread per chunk (the launch has one for
 // each); else a thread per (chunk column, band of consecutive rows), in one
@@ -476,9 +453,9 @@ __global__ void __launch_bounds__(kThreads, kPipeMinB) k_wide_pipe_ne(Geom g, in
 // L/2 % 16 sites (its bytes past the row are masked, its neighbour past the
 // row end is the row's first byte); stores write whole aligned words inside
 // the chunk and single bytes at its two ends, so no byte of another lane's
-// chunk is touched.  Column walk with two chunks in flight as in
-// k_wide_pipe (Ising: the next chunk's draws too) and, for the North-East
-// model, the warp-compacted draws of k_wide_pipe_ne.
+// chunk is touched.  Column walk with two chunks in flight (Ising: the next
+// chunk's draws too) and, for the North-East model, the warp-compacted draws
+// of k_wide_pipe_ne.  Ising in batches' step loop, North-East at any rates.
 // ---------------------------------------------------------------------
 
 struct AnyIn {
@@ -1139,8 +1116,6 @@ bool wide_supported(const Geom &g)
     }
     return true;
 }
-
-int wide_chunks(const Geom &g) { return (int)(((uint64_t)g.L * (g.half >> 4) + kThreads - 1) / kThreads); }
 
 bool any_supported(const Geom &g)
 {

@@ -447,7 +447,6 @@ int batch_item_passes(uint64_t chunk_rows);
 int batch_wide3_grid(bool swar);
 cudaError_t launch_batch_wide3(const Geom *geoms, const uint2 *items, int n_items, unsigned *next_item,
                                int colour, bool swar, int passes, int grid, cudaStream_t st);
-int wide_chunks(const Geom &g);
 // 2D spin-1/2 Ising / North-East with uniform couplings at any even L (the
 // wide kernel's sweep on rows at any byte alignment; launch_sweep_wide takes
 // these lattices when L % 32 != 0), and its batched form

@@ -47,9 +47,8 @@ struct NePlanes {
 LAT_D uint32_t ne_rejected(const U4 &u, uint32_t K)
 {
     auto above = [&](uint32_t x) {   // all ones where x > K: the borrow of K - x
-        uint32_t d, m;
-        asm("sub.cc.u32 %0, %2, %3;\n\tsubc.u32 %1, 0, 0;" : "=r"(d), "=r"(m) : "r"(K), "r"(x));
-        (void)d;
+        uint32_t m;
+        asm("{\n\t.reg .u32 d;\n\tsub.cc.u32 d, %1, %2;\n\tsubc.u32 %0, 0, 0;\n\t}" : "=r"(m) : "r"(K), "r"(x));
         return m;
     };
     const uint32_t m0 = above(u.x), m1 = above(u.y), m2 = above(u.z), m3 = above(u.w);
