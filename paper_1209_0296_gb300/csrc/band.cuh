@@ -33,6 +33,7 @@ namespace {
 
 constexpr int kBandThreads = 512;
 constexpr int kBandWarps = kBandThreads / 32;
+constexpr int kBandNeThreads = 1024;        // North-East on bits, alone on the GPU, bands of more than 1024 words
 constexpr int kBandMaxCtas = 160;           // a batched launch's parts are kernel parameters
 constexpr unsigned kSpinLimit = 1u << 24;   // polls of about half a microsecond: ten seconds
 constexpr uint32_t kAbortBytes = 128;       // the abort word's line, before a lattice's packets

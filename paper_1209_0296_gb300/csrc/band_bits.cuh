@@ -100,7 +100,8 @@ LAT_D uint32_t bit_side(const uint32_t *row, uint32_t k, uint32_t bw, uint32_t n
     return __funnelshift_l(prev, O, 1);
 }
 
-template <bool kNe, bool kRef, bool kBonds, bool kPacked>
+// kT: threads of the CTA.
+template <bool kNe, bool kRef, bool kBonds, bool kPacked, int kT>
 LAT_D void band_bits(const Geom &g, const BandPart &part, uint32_t band, uint32_t bands, uint8_t *mail,
                      BandShared &sh, uint8_t *smem)
 {
@@ -131,7 +132,7 @@ LAT_D void band_bits(const Geom &g, const BandPart &part, uint32_t band, uint32_
     __syncthreads();
     int changed = 0;
     for (uint32_t c = 0; c < 2u; ++c)
-        for (uint32_t i = tid; i < fw; i += kBandThreads) {
+        for (uint32_t i = tid; i < fw; i += kT) {
             const uint32_t r = i / bw, k = i - r * bw, y = y0 + r;
             sm[c * pw + bw + i] = spins_at(c, y, k);
             if constexpr (kRef) {
@@ -177,8 +178,8 @@ LAT_D void band_bits(const Geom &g, const BandPart &part, uint32_t band, uint32_
     const uint32_t lane = tid & 31u;
     // interior rows 1 .. nr - 2: thread (rr, k); the boundary rows' words are
     // the last threads'
-    const uint32_t rsb = (uint32_t)kBandThreads / bw, rr = tid / bw, kc = tid - rr * bw;
-    const uint32_t r0 = rr < rsb ? 1u + rr : nr, edge0 = (uint32_t)kBandThreads - 1u - tid, edges = 2u * bw;
+    const uint32_t rsb = (uint32_t)kT / bw, rr = tid / bw, kc = tid - rr * bw;
+    const uint32_t r0 = rr < rsb ? 1u + rr : nr, edge0 = (uint32_t)kT - 1u - tid, edges = 2u * bw;
     Counts cnt;   // mag counts up spins
     int bad = 0, sites = 0;
     for (int h = 0; h < 2 * part.n; ++h) {
@@ -293,7 +294,7 @@ LAT_D void band_bits(const Geom &g, const BandPart &part, uint32_t band, uint32_
 #pragma unroll 1
             for (uint32_t r = r0; r < rend; r += rsb) word(r, kc, other[r * bw + kc], other[(r + 2u) * bw + kc], none);
         }
-        for (uint32_t e = edge0;; e += (uint32_t)kBandThreads) {
+        for (uint32_t e = edge0;; e += (uint32_t)kT) {
             const bool act = e < edges;
             if (!__any_sync(0xffffffffu, act)) break;
             uint32_t cand = 0, k = 0, r = 0;
@@ -327,7 +328,7 @@ LAT_D void band_bits(const Geom &g, const BandPart &part, uint32_t band, uint32_
         }
         const int stop = __syncthreads_or(bad);
         if constexpr (kNe) {   // boundary rows out, their queued moves done
-            for (uint32_t i = tid; i < edges; i += kBandThreads) {
+            for (uint32_t i = tid; i < edges; i += kT) {
                 const bool lo = i < bw;
                 const uint32_t k = lo ? i : i - bw;
                 mail_put_word((lo ? last_row : first) + colour * bw + k, part.epoch + (uint32_t)h + 1u,
@@ -344,7 +345,7 @@ LAT_D void band_bits(const Geom &g, const BandPart &part, uint32_t band, uint32_
     int8_t *fin = fin_odd ? g.s[1] : g.s[0];
     uint32_t *bfin = fin_odd ? g.bits[1] : g.bits[0];
     for (uint32_t c = 0; c < 2u; ++c)
-        for (uint32_t i = tid; i < fw; i += kBandThreads) {
+        for (uint32_t i = tid; i < fw; i += kT) {
             const uint32_t r = i / bw, k = i - r * bw, y = y0 + r;
             const uint32_t v = sm[c * pw + bw + i];
             if constexpr (kPacked) bfin[((size_t)c * L + y) * bw + k] = v;

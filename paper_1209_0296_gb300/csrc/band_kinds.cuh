@@ -31,7 +31,8 @@ LAT_HD bool band_kind_bits(int kind)
            kind >= kBandPacked;
 }
 
-template <int kKind, bool kRef>
+// kT: threads of the CTA; kForm: small bands (0), the others (1), either (2).
+template <int kKind, bool kRef, int kT, int kForm>
 LAT_D void band_body(const Geom &g, const BandPart &part, uint32_t band, uint32_t bands, uint8_t *mail,
                      BandShared &sh, uint8_t *smem)
 {
@@ -43,14 +44,14 @@ LAT_D void band_body(const Geom &g, const BandPart &part, uint32_t band, uint32_
     if constexpr (kKind == kBandPotts3) {
         band_potts<kRef>(g, part, band, bands, mail, sh, smem);
     } else if constexpr (kPacked) {
-        band_bits<kNe, kRef, false, true>(g, part, band, bands, mail, sh, smem);
+        band_bits<kNe, kRef, false, true, kT>(g, part, band, bands, mail, sh, smem);
     } else {
-        if (band_is_small((uint32_t)g.L, g.half, bands))
+        if (kForm == 0 || (kForm == 2 && band_is_small((uint32_t)g.L, g.half, bands))) {
             band_small<kNe, kRef, kDis, kSym, kFull>(g, part, band, bands, mail, sh, smem);
-        else if constexpr (kNe || kSym)
-            band_bits<kNe, kRef, kDis == kBonds, false>(g, part, band, bands, mail, sh, smem);
-        else
-            band_ising<kRef, kDis, kSym, kFull>(g, part, band, bands, mail, sh, smem);
+        } else if constexpr (kForm != 0) {
+            if constexpr (kNe || kSym) band_bits<kNe, kRef, kDis == kBonds, false, kT>(g, part, band, bands, mail, sh, smem);
+            else band_ising<kRef, kDis, kSym, kFull>(g, part, band, bands, mail, sh, smem);
+        }
     }
 }
 
@@ -71,7 +72,7 @@ inline bool band_on_bits(const Geom &k, int kind, int bands)
 
 // k: a tiled_geom descriptor.  Rows per band are at least 2, so a lattice has
 // at most L / 2 bands.
-inline size_t band_smem_bytes(const Geom &k, int kind, int bands)
+inline size_t band_smem_bytes(const Geom &k, int kind, int bands, int threads = kBandThreads)
 {
     const size_t nr = ((size_t)k.L + bands - 1) / bands, ref = k.ref != nullptr || k.ref_bits != nullptr ? 1 : 0;
     if (band_on_bits(k, kind, bands)) {
@@ -79,7 +80,7 @@ inline size_t band_smem_bytes(const Geom &k, int kind, int bands)
         if (kind == kBandPotts3) return 4 * nr * bw * (1 + ref) * 4;
         size_t words = 2 * (nr + 2) * bw + 2 * nr * bw * ref;
         if (kind == kBandBondSym) words += 8 * nr * bw;
-        if (k.model == LAT_NE) words += 2 * nr * bw + kBandWarps * kBitQueue;
+        if (k.model == LAT_NE) words += 2 * nr * bw + (size_t)threads / 32 * kBitQueue;
         return words * 4;
     }
     const size_t pitch = ((size_t)k.half + 15) & ~(size_t)15;

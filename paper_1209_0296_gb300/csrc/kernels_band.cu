@@ -9,15 +9,34 @@ namespace lat {
 
 namespace {
 
-// One lattice over the whole grid.
-template <int kKind, bool kRef>
-__global__ void __launch_bounds__(kBandThreads, 1) k_band(const __grid_constant__ Geom g,
-                                                          const __grid_constant__ BandPart part, uint8_t *mail)
+// One lattice over the whole grid. kForm as in band_body.
+template <int kKind, bool kRef, int kT, int kForm>
+__global__ void __launch_bounds__(kT, 1) k_band(const __grid_constant__ Geom g, const __grid_constant__ BandPart part,
+                                                uint8_t *mail)
 {
     extern __shared__ __align__(16) uint8_t band_smem[];
     __shared__ BandShared sh;
-    band_body<kKind, kRef>(g, part, blockIdx.x, gridDim.x, mail, sh, band_smem);
+    band_body<kKind, kRef, kT, kForm>(g, part, blockIdx.x, gridDim.x, mail, sh, band_smem);
     band_end(g, part, blockIdx.x, sh);
+}
+
+using BandKernel = void (*)(Geom, BandPart, uint8_t *);
+
+// Kernels of a kind by reference set and form: small bands, the others, and
+// for North-East the others with more threads.
+template <int kKind, bool kRef, int kVar>
+constexpr BandKernel band_kernel()
+{
+    constexpr bool kNe = kKind == kBandNe || kKind == kBandNeFull || kKind == kBandPackedNe;
+    if constexpr (kVar == 0) {
+        if constexpr (kKind >= kBandPacked) return nullptr;
+        else return k_band<kKind, kRef, kBandThreads, 0>;
+    } else if constexpr (kVar == 1) {
+        return k_band<kKind, kRef, kBandThreads, 1>;
+    } else {
+        if constexpr (kNe) return k_band<kKind, kRef, kBandNeThreads, 1>;
+        else return nullptr;
+    }
 }
 
 }  // namespace
@@ -50,22 +69,25 @@ size_t band_mail_bytes(const Geom &g, bool fields, int bands)
 cudaError_t launch_sweep_band(const Geom &g, bool fields, int bands, unsigned long long sweep0, int n, void *mail,
                               unsigned epoch, int *err, cudaStream_t st)
 {
-    using K = void (*)(Geom, BandPart, uint8_t *);
-#define LAT_BAND(k) {k_band<k, false>, k_band<k, true>}
-    static const K kern[kBandKinds][2] = {LAT_BAND(kBandGen),      LAT_BAND(kBandSym),     LAT_BAND(kBandNe),
-                                          LAT_BAND(kBandGenFull),  LAT_BAND(kBandSymFull), LAT_BAND(kBandNeFull),
-                                          LAT_BAND(kBandBondGen),  LAT_BAND(kBandBondSym), LAT_BAND(kBandFields),
-                                          LAT_BAND(kBandPacked),   LAT_BAND(kBandPackedNe), LAT_BAND(kBandPotts3)};
+#define LAT_VAR(k, ref) {band_kernel<k, ref, 0>(), band_kernel<k, ref, 1>(), band_kernel<k, ref, 2>()}
+#define LAT_BAND(k) {LAT_VAR(k, false), LAT_VAR(k, true)}
+    static const BandKernel kern[kBandKinds][2][3] = {
+        LAT_BAND(kBandGen),     LAT_BAND(kBandSym),     LAT_BAND(kBandNe),     LAT_BAND(kBandGenFull),
+        LAT_BAND(kBandSymFull), LAT_BAND(kBandNeFull),  LAT_BAND(kBandBondGen), LAT_BAND(kBandBondSym),
+        LAT_BAND(kBandFields),  LAT_BAND(kBandPacked),  LAT_BAND(kBandPackedNe), LAT_BAND(kBandPotts3)};
 #undef LAT_BAND
+#undef LAT_VAR
     static std::once_flag once;
     static cudaError_t attr = cudaSuccess;
     std::call_once(once, [] {
-        for (const auto &row : kern)
-            for (K f : row) {
-                const cudaError_t e =
-                    cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBandMaxSmem);
-                if (e != cudaSuccess) attr = e;
-            }
+        for (const auto &kind : kern)
+            for (const auto &ref : kind)
+                for (BandKernel f : ref) {
+                    const cudaError_t e = f == nullptr ? cudaSuccess
+                                                       : cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                                              (int)kBandMaxSmem);
+                    if (e != cudaSuccess) attr = e;
+                }
     });
     if (attr != cudaSuccess) return attr;
     const Geom k = tiled_geom(g);
@@ -76,9 +98,17 @@ cudaError_t launch_sweep_band(const Geom &g, bool fields, int bands, unsigned lo
     const int kind = band_kind(k, fields);
     const uint32_t nr = ((uint32_t)k.L + bands - 1) / bands, cpr = (k.half + 15) / 16;
     const bool small = kind < kBandPacked && band_is_small((uint32_t)k.L, k.half, (uint32_t)bands);
-    cfg.blockDim = dim3(!small ? (uint32_t)kBandThreads
+    // North-East waits on shared memory and warp scans more than on a pipe: bands
+    // of several words a thread run with twice the threads, where their queues
+    // fit (L = 8192, c = 0.3: 38.7 us a sweep with 512 threads, 32.0 with 768,
+    // 31.5 with 1024; 4096: 12.1, 11.3, 10.0; at L = 2048 the idle warps cost: 4.6,
+    // 4.9, 5.0)
+    const bool more = !small && nr * ((k.half + 31u) / 32u) > 1024u && (kind == kBandNe || kind == kBandNeFull || kind == kBandPackedNe) &&
+                      band_smem_bytes(k, kind, bands, kBandNeThreads) <= kBandMaxSmem;
+    const int threads = more ? kBandNeThreads : kBandThreads;
+    cfg.blockDim = dim3(!small ? (uint32_t)threads
                                : std::max(64u, cpr <= 32 ? 32u * nr : (nr * cpr + 31u) / 32u * 32u));
-    cfg.dynamicSmemBytes = band_smem_bytes(k, kind, bands);
+    cfg.dynamicSmemBytes = band_smem_bytes(k, kind, bands, threads);
     cfg.stream = st;
     cudaLaunchAttribute a[1];
     a[0].id = cudaLaunchAttributeCooperative;
@@ -86,7 +116,7 @@ cudaError_t launch_sweep_band(const Geom &g, bool fields, int bands, unsigned lo
     cfg.attrs = a;
     cfg.numAttrs = 1;
     const int ref = k.ref != nullptr || k.ref_bits != nullptr ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kern[kind][ref], k, part, (uint8_t *)mail);
+    return cudaLaunchKernelEx(&cfg, kern[kind][ref][small ? 0 : more ? 2 : 1], k, part, (uint8_t *)mail);
 }
 
 }  // namespace lat

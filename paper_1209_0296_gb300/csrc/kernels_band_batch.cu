@@ -21,12 +21,12 @@ template <bool kRef>
 LAT_D void band_any(const Geom &g, const BandPart &part, uint8_t *mail, BandShared &sh, uint8_t *smem)
 {
     switch (part.kind) {
-    case kBandGen: band_body<kBandGen, kRef>(g, part, part.band, part.bands, mail, sh, smem); break;
-    case kBandSym: band_body<kBandSym, kRef>(g, part, part.band, part.bands, mail, sh, smem); break;
-    case kBandNe: band_body<kBandNe, kRef>(g, part, part.band, part.bands, mail, sh, smem); break;
-    case kBandGenFull: band_body<kBandGenFull, kRef>(g, part, part.band, part.bands, mail, sh, smem); break;
-    case kBandSymFull: band_body<kBandSymFull, kRef>(g, part, part.band, part.bands, mail, sh, smem); break;
-    default: band_body<kBandNeFull, kRef>(g, part, part.band, part.bands, mail, sh, smem); break;
+    case kBandGen: band_body<kBandGen, kRef, kBandThreads, 2>(g, part, part.band, part.bands, mail, sh, smem); break;
+    case kBandSym: band_body<kBandSym, kRef, kBandThreads, 2>(g, part, part.band, part.bands, mail, sh, smem); break;
+    case kBandNe: band_body<kBandNe, kRef, kBandThreads, 2>(g, part, part.band, part.bands, mail, sh, smem); break;
+    case kBandGenFull: band_body<kBandGenFull, kRef, kBandThreads, 2>(g, part, part.band, part.bands, mail, sh, smem); break;
+    case kBandSymFull: band_body<kBandSymFull, kRef, kBandThreads, 2>(g, part, part.band, part.bands, mail, sh, smem); break;
+    default: band_body<kBandNeFull, kRef, kBandThreads, 2>(g, part, part.band, part.bands, mail, sh, smem); break;
     }
 }
 

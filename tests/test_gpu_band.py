@@ -180,3 +180,8 @@ def test_kinds_of_one_lattice():
             o.sweep(m)
             assert np.array_equal(g.get_spins(), o.spins), (step, m)
     g.close()
+
+
+# bands of more than 1024 words: North-East with twice the threads, rows ending inside a word
+def test_north_east_more_threads():
+    _run((2, 3202, 1, lt.NE, 0.0, 0.0, 0.3), 6, lt.INIT_EQUILIBRIUM, [5, 6], reference=True)
