@@ -488,7 +488,7 @@ int enqueue_sweeps(lattice *lt, int64_t k, cudaStream_t st, bool direct = false)
     int kern = choose_kernel(lt);
     // Under AUTO a short call on a small lattice takes the kernel that is
     // cheaper for it, tuned or not: two launches for one sweep (L = 64: 4.0
-    // us, resident 5.8), one resident launch for more (1.1 us a sweep on top).
+    // us, resident 5.8), one resident launch for more (0.8 us a sweep on top).
     if (direct && lt->kernel == LAT_KERNEL_AUTO && lt->P.L <= 128 && resident_supported(lt->geom) &&
         lt->geom.cpl == nullptr && (kern == LAT_KERNEL_WIDE || kern == LAT_KERNEL_RESIDENT) && sweep_at_known(lt->geom))
         kern = k == 1 ? LAT_KERNEL_WIDE : LAT_KERNEL_RESIDENT;

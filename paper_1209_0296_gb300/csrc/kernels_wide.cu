@@ -950,7 +950,7 @@ LAT_D void resident_body(const Geom &g, unsigned long long sweep0, int n_sweeps,
 // half-sweep once its new word is stored, decides by the 16-bit compare, and
 // the counters are summed through shared memory and posted a barrier later.
 // L = 64: 0.93 us a sweep (1.06 with table look-ups, draws and three counter
-// barriers in line); four warps a scheduler, bound by their instruction issue.
+// barriers in line). Batches; a lattice alone has k_resident_pair.
 template <bool kNE, bool kSym>
 LAT_D void resident_words(const Geom &g, unsigned long long sweep0, int n_sweeps, bool advance, uint4 *res_smem,
                           uint32_t *sthr, int (*sum)[5])
@@ -1060,16 +1060,149 @@ LAT_D void resident_words(const Geom &g, unsigned long long sweep0, int n_sweeps
     if (advance && tid == 0) g.ctrl->sweep = sweep0 + (unsigned long long)n_sweeps;   // read by all before the first barrier
 }
 
-// kind 0: the general body; 1, 2: at most one word a thread, general or
-// symmetric table.
-template <bool kNE, int kKind>
-__global__ void __launch_bounds__(kResThreads, 1) k_resident(const __grid_constant__ Geom g, SweepAt at, int n_sweeps)
+__global__ void __launch_bounds__(kResThreads, 1) k_resident_ising(const __grid_constant__ Geom g, SweepAt at, int n_sweeps)
 {
     extern __shared__ uint4 res_smem[];
     __shared__ uint32_t sthr[16];
     __shared__ int red[kResThreads / 32][5];
-    if constexpr (kKind == 0) resident_body<kNE>(g, sweep_of(g.ctrl, at), n_sweeps, at.known != 0, res_smem, sthr, red);
-    else resident_words<kNE, kKind == 2>(g, sweep_of(g.ctrl, at), n_sweeps, at.known != 0, res_smem, sthr, red);
+    resident_body<false>(g, sweep_of(g.ctrl, at), n_sweeps, at.known != 0, res_smem, sthr, red);
+}
+
+__global__ void __launch_bounds__(kResThreads, 1) k_resident_ne(const __grid_constant__ Geom g, SweepAt at, int n_sweeps)
+{
+    extern __shared__ uint4 res_smem[];
+    __shared__ uint32_t sthr[16];
+    __shared__ int red[kResThreads / 32][5];
+    resident_body<true>(g, sweep_of(g.ctrl, at), n_sweeps, at.known != 0, res_smem, sthr, red);
+}
+
+// L = 32 or 64 alone on the GPU: as resident_words, with threads of their own
+// for either colour. While one colour steps, the other draws and sums its
+// counters, so a half-sweep takes the longer of the two and not their sum.
+// L = 64: 0.93 us a sweep with one thread for both colours, 0.81 here; 64% of
+// issue on its one SM, waiting for the draws' multiply pipe.
+template <bool kNE, bool kSym>
+__global__ void __launch_bounds__(2 * kResThreads, 1) k_resident_pair(const __grid_constant__ Geom g, SweepAt at,
+                                                                      int n_sweeps)
+{
+    __shared__ uint32_t pl[2 * kResThreads], sthr[16];
+    __shared__ int sum[2][5];   // a sweep's counters: two sweeps in turn
+    const unsigned long long sweep0 = sweep_of(g.ctrl, at);
+    const uint32_t wpr = g.half >> 2, words = (uint32_t)g.L * wpr;   // a multiple of 32
+    const uint32_t c = threadIdx.x >= words ? 1u : 0u, i = threadIdx.x - c * words;
+    const uint32_t y = i / wpr, k = i - y * wpr;
+    const uint32_t *src = reinterpret_cast<const uint32_t *>(g.s[sweep0 & 1]);
+    uint32_t S = src[c * words + i], was = 0, rw[2] = {0u, 0u};
+    pl[c * words + i] = S;
+    if constexpr (kNE) was = g.flags[c * words + i];   // G = wpr groups a row
+    if (g.ref != nullptr && c == 1u)
+        for (int p = 0; p < 2; ++p) rw[p] = reinterpret_cast<const uint32_t *>(g.ref)[p * words + i];
+    int unfl = 4 - __popc(was);
+    if (threadIdx.x < 16) sthr[threadIdx.x] = g.thr16[threadIdx.x];
+    if (threadIdx.x >= 32 && threadIdx.x < 42) (&sum[0][0])[threadIdx.x - 32] = 0;
+    __syncthreads();
+    // the other plane's words around this one
+    const uint32_t *o = pl + (1u - c) * words;
+    const bool odd = ((c + y) & 1u) != 0u;
+    const uint32_t *pU = o + (y == 0u ? (uint32_t)g.L - 1u : y - 1u) * wpr + k;
+    const uint32_t *pD = o + (y + 1u == (uint32_t)g.L ? 0u : y + 1u) * wpr + k;
+    const uint32_t *pN = o + y * wpr + (odd ? (k + 1u == wpr ? 0u : k + 1u) : (k == 0u ? wpr - 1u : k - 1u));
+    unsigned long long *slot0 = series_slot(g.ctrl, sweep0);   // consecutive sweeps are contiguous
+    unsigned long long *acf0 = g.ref ? acf_slot(g.ctrl, sweep0) : nullptr;
+    const uint32_t g0 = y * g.G + k;
+    uint32_t p01 = 0, p23 = 0;
+    int bond = 0, mag = 0, acf = 0;
+    auto draw = [&](int s) {
+        const unsigned long long sweep = sweep0 + (unsigned long long)s;
+        PhiloxPre pp;
+        philox_prepare(pp, (uint32_t)sweep, (uint32_t)(sweep >> 32), g.key0, g.key1);
+        top_halves(philox_item(pp, g0, c), p01, p23);
+    };
+    auto step = [&](int s) {
+        const uint32_t U = *pU, D = *pD, O = o[i], nb = *pN;
+        const uint32_t X = odd ? __funnelshift_r(O, nb, 8) : __funnelshift_l(nb, O, 8);
+        const Nbr n = nbr_sum(U, D, O, X);
+        uint32_t t01[2], t23[2], tie = kNoTie;
+        if constexpr (kSym) sym_thresholds(g.acc, n, S, t01[0], t23[0]);
+        else gen_thresholds2(g.acc, n, n, S, S, t01, t23);
+        uint32_t rej = reject4(t01[0], t23[0], p01, p23, tie);
+        if (tie_hit(tie)) {
+            const unsigned long long sweep = sweep0 + (unsigned long long)s;
+            PhiloxPre pp;
+            philox_prepare(pp, (uint32_t)sweep, (uint32_t)(sweep >> 32), g.key0, g.key1);
+            rej = reject4_exact(sthr, n, S, philox_item(pp, g0, c));
+        }
+        uint32_t F = ~rej & 0xFEFEFEFEu;
+        if constexpr (kNE) F &= ~(U | (odd ? X : O));   // §III.B: north and east must be up
+        S ^= F;
+        pl[c * words + i] = S;
+        if constexpr (kNE) {
+            const uint32_t bits = (uint32_t)dot4(F & 0x02020202u, 0x08040201u, 0) >> 1;
+            unfl -= __popc(bits & ~was);
+            was |= bits;
+        }
+        if (c == 1u) {
+            bond = dot4(S, X, dot4(S, O, dot4(S, D, dot4(S, U, 0))));
+            mag = dot4(S, 0x01010101u, dot4(O, 0x01010101u, 0));
+            if (g.ref) acf = dot4(S, rw[1], dot4(O, rw[0], 0));
+        }
+    };
+    // this colour's share of sweep s's counters, after its step
+    auto reduce = [&](int s) {
+        int *t = sum[s & 1];
+        const bool first = (threadIdx.x & 31u) == 0u;
+        if constexpr (kNE) {
+            const int f = __reduce_add_sync(0xffffffffu, unfl);
+            if (first) atomicAdd(&t[3], f);
+        }
+        if (c == 0u) return;
+        const int b = __reduce_add_sync(0xffffffffu, bond), m = __reduce_add_sync(0xffffffffu, mag);
+        const int a = g.ref ? __reduce_add_sync(0xffffffffu, acf) : 0;
+        if (first) {
+            atomicAdd(&t[0], b);
+            atomicAdd(&t[1], m);
+            if (g.ref) atomicAdd(&t[4], a);
+        }
+    };
+    // a sweep's counters go out once both colours have summed theirs; cleared
+    // two barriers before their next use
+    auto post = [&](int s) {
+        if (threadIdx.x != 0u || s < 0) return;
+        int *t = sum[s & 1];
+        unsigned long long *slot = slot0 + 4ull * (unsigned)s;
+        const long long m = t[1];
+        add_counter(slot + 0, t[0]);
+        add_counter(slot + 1, m);
+        add_counter(slot + 2, (m + (long long)g.N) / 2);
+        if constexpr (kNE) add_counter(slot + 3, t[3]);
+        if (g.ref) add_counter(acf0 + (unsigned)s, t[4]);
+        for (int j = 0; j < 5; ++j) t[j] = 0;
+    };
+    if (c == 0u) {
+        draw(0);
+        for (int s = 0; s < n_sweeps; ++s) {
+            step(s);
+            __syncthreads();
+            post(s - 1);
+            reduce(s);
+            if (s + 1 < n_sweeps) draw(s + 1);
+            __syncthreads();
+        }
+    } else {
+        for (int s = 0; s < n_sweeps; ++s) {
+            if (s > 0) reduce(s - 1);
+            draw(s);
+            __syncthreads();
+            step(s);
+            __syncthreads();
+        }
+        reduce(n_sweeps - 1);
+    }
+    __syncthreads();
+    post(n_sweeps - 1);
+    reinterpret_cast<uint32_t *>(g.s[(sweep0 + (unsigned long long)n_sweeps) & 1])[c * words + i] = S;
+    if constexpr (kNE) g.flags[c * words + i] = (uint8_t)was;
+    if (at.known != 0 && threadIdx.x == 0) g.ctrl->sweep = sweep0 + (unsigned long long)n_sweeps;
 }
 
 // Batched form: CTA i sweeps lattice i (descriptor geoms[i]) by
@@ -1217,19 +1350,22 @@ cudaError_t launch_sweep_resident(const Geom &g, SweepAt at, int n_sweeps, cudaS
     const size_t smem = resident_bytes(g);
     const bool narrow = (uint64_t)g.L * (g.half >> 2) <= (uint64_t)kResThreads;
     using K = void (*)(Geom, SweepAt, int);
-    static const K fn[2][3] = {{k_resident<false, 0>, k_resident<false, 1>, k_resident<false, 2>},
-                               {k_resident<true, 0>, k_resident<true, 1>, k_resident<true, 1>}};
+    const bool ne = g.model == LAT_NE;
+    if (narrow) {   // L = 32, 64
+        static const K pair[3] = {k_resident_pair<false, false>, k_resident_pair<false, true>, k_resident_pair<true, false>};
+        pair[ne ? 2 : (k.acc_sym ? 1 : 0)]<<<1, (unsigned)(g.N / 4), 0, st>>>(k, at, n_sweeps);
+        return cudaGetLastError();
+    }
+    static const K fn[2] = {k_resident_ising, k_resident_ne};
     static const cudaError_t attr = [] {
         cudaError_t e = cudaSuccess;
-        for (const auto &row : fn)
-            for (K f : row)
-                if (e == cudaSuccess)
-                    e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResMaxBytes);
+        for (K f : fn)
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResMaxBytes);
         return e;
     }();
     if (attr != cudaSuccess) return attr;
-    const unsigned threads = narrow ? std::max(64u, ((unsigned)(g.N / 8) + 31u) / 32u * 32u) : (unsigned)kResThreads;
-    fn[g.model == LAT_NE ? 1 : 0][narrow ? (k.acc_sym ? 2 : 1) : 0]<<<1, threads, smem, st>>>(k, at, n_sweeps);
+    fn[ne ? 1 : 0]<<<1, kResThreads, smem, st>>>(k, at, n_sweeps);
     return cudaGetLastError();
 }
 

@@ -185,3 +185,34 @@ def test_kinds_of_one_lattice():
 # bands of more than 1024 words: North-East with twice the threads, rows ending inside a word
 def test_north_east_more_threads():
     _run((2, 3202, 1, lt.NE, 0.0, 0.0, 0.3), 6, lt.INIT_EQUILIBRIUM, [5, 6], reference=True)
+
+
+# the one-CTA kernel for L = 32 and 64: runs of one, two and many sweeps, every table kind, references
+@pytest.mark.parametrize("L", [32, 64])
+@pytest.mark.parametrize("model,J,h,par", [(lt.ISING, 1.0, 0.0, 2.3), (lt.ISING, 1.0, 0.3, 2.0), (lt.ISING, -0.7, 0.0, 1.5),
+                                           (lt.NE, 0.0, 0.0, 0.3), (lt.NE, 0.0, 0.0, 0.7)])
+@pytest.mark.parametrize("ref", [False, True])
+def test_resident_words(L, model, J, h, par, ref):
+    a = (2, L, 1, model, J, h, par)
+    init = lt.INIT_EQUILIBRIUM if model == lt.NE else lt.INIT_RANDOM
+    g = lt.Lattice(*a, seed=L, init=init)
+    o = oracle.Lattice(*a, seed=L, init=init)
+    g.set_kernel(lt.KERNEL_RESIDENT)
+    if ref:
+        g.set_reference()
+        o.set_reference()
+    done = 0
+    for n in (1, 2, 3, 40):
+        ser_o = o.sweep(n)
+        g.sweep(n)
+        ser = g.series(done, n)
+        for k in ("bond", "mag", "up") + (("unflipped",) if model == lt.NE else ()):
+            assert np.array_equal(ser[k], ser_o[k]), (k, n)
+        if ref:
+            assert np.array_equal(g.autocorrelation(done, n, m=0.0)[0], ser_o["overlap"])
+        spins, flags, _ = g.get_state()
+        assert np.array_equal(spins, o.spins), n
+        if model == lt.NE:
+            assert np.array_equal(flags, o.flags), n
+        done += n
+    g.close()
