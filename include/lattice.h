@@ -67,7 +67,7 @@ enum lattice_status {
     LAT_ENOMEM = -2,   /* device or host allocation failed */
     LAT_ECUDA = -3,    /* a CUDA call failed (see lattice_last_cuda_error) */
     LAT_ETIMEOUT = -4, /* a bounded wait gave up: lattice_server_drain's limit, or (about
-                          ten seconds) a band of a band-resident launch waiting for its
+                          four seconds) a band of a band-resident launch waiting for its
                           neighbour's rows; after the latter the lattice's state is
                           undefined and every call on it returns this */
     LAT_EBUSY = -5,    /* result not ready yet (server poll) */

@@ -88,6 +88,7 @@ SIGNATURES = {
 # Entry points outside include/lattice.h used only by the tests.
 TEST_SIGNATURES = {
     "lattice_test_fail_alloc": (c_int, [c_int]),
+    "lattice_test_band_wait": (c_int, [ctypes.c_uint, c_int]),
 }
 
 

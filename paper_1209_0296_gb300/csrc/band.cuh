@@ -17,7 +17,9 @@
 // packet of the half-sweep in between has arrived.
 //
 // A wait is bounded: when it gives up the launch ends normally and the host
-// sees the error word (LAT_ETIMEOUT).
+// sees the error word (LAT_ETIMEOUT).  It also leaves the launch's own mark in
+// the abort word, which ends the launch's other waits early; the next launch
+// on the same packets has another mark, so nothing needs to be cleared.
 #pragma once
 
 #include <memory>
@@ -35,7 +37,6 @@ constexpr int kBandThreads = 512;
 constexpr int kBandWarps = kBandThreads / 32;
 constexpr int kBandNeThreads = 1024;        // North-East on bits, alone on the GPU, bands of more than 1024 words
 constexpr int kBandMaxCtas = 160;           // a batched launch's parts are kernel parameters
-constexpr unsigned kSpinLimit = 1u << 24;   // polls of about half a microsecond: ten seconds
 constexpr uint32_t kAbortBytes = 128;       // the abort word's line, before a lattice's packets
 constexpr size_t kBandMaxSmem = 224 * 1024;
 
@@ -48,6 +49,8 @@ struct BandPart {
     uint32_t epoch;              // packets are marked epoch + 1 .. epoch + 2 n
     unsigned long long sweep0;   // sweeps done before the launch
     int *err;                    // host-visible error word of the lattice
+    uint32_t limit;              // polls after which a wait gives up
+    uint32_t mute;               // solo: 1 + the band that sends nothing (0: none), by which tests let waits run out
     uint32_t mail;               // batched: packet rows start at this pair
     int n;                       // sweeps to run
     uint32_t key0, key1;
@@ -69,7 +72,7 @@ struct Band {
     size_t plane;
     const int8_t *src;           // spins before the launch
     uint32_t up, dn;             // rows above and below the band
-    unsigned *abort;             // set when a wait of the launch gave up
+    unsigned *abort;             // the launch's mark when a wait of it gave up
     // packet rows of colour 0 (colour 1: + cpr packet pairs): this band's
     // first and last row, the last row of the band above, the first below
     ulonglong2 *first, *last;
@@ -120,8 +123,19 @@ LAT_D void mail_put(ulonglong2 *q, uint32_t tag, const uint32_t (&v)[4])
                      : "memory");
 }
 
+// After poll i: whether the wait gives up, at its limit or because another
+// wait of the launch did.
+LAT_D bool mail_over(unsigned i, const BandPart &p, unsigned *abort)
+{
+    if ((i & 1023u) != 1023u) return false;
+    const uint32_t mark = p.epoch + 1u;   // no other launch on these packets has it
+    if (i < p.limit && *reinterpret_cast<volatile unsigned *>(abort) != mark) return false;
+    *reinterpret_cast<volatile unsigned *>(abort) = mark;
+    return true;
+}
+
 // Wait for the 16 bytes marked `tag`; false when the wait gave up.
-LAT_D bool mail_take(const ulonglong2 *q, uint32_t tag, unsigned *abort, uint32_t (&v)[4])
+LAT_D bool mail_take(const ulonglong2 *q, uint32_t tag, const BandPart &p, unsigned *abort, uint32_t (&v)[4])
 {
     for (unsigned i = 0;; ++i) {
         const ulonglong2 a = ld_pair(q), b = ld_pair(q + 1);
@@ -132,10 +146,7 @@ LAT_D bool mail_take(const ulonglong2 *q, uint32_t tag, unsigned *abort, uint32_
         if ((uint32_t)(a.x >> 32) == tag && (uint32_t)(a.y >> 32) == tag && (uint32_t)(b.x >> 32) == tag &&
             (uint32_t)(b.y >> 32) == tag)
             return true;
-        if ((i & 1023u) == 1023u && (i >= kSpinLimit || *reinterpret_cast<volatile unsigned *>(abort) != 0u)) {
-            *reinterpret_cast<volatile unsigned *>(abort) = 1u;
-            return false;
-        }
+        if (mail_over(i, p, abort)) return false;
     }
 }
 
@@ -145,17 +156,14 @@ LAT_D void mail_put_word(unsigned long long *q, uint32_t tag, uint32_t v)
     asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(q), "l"((unsigned long long)tag << 32 | v) : "memory");
 }
 
-LAT_D bool mail_take_word(const unsigned long long *q, uint32_t tag, unsigned *abort, uint32_t &v)
+LAT_D bool mail_take_word(const unsigned long long *q, uint32_t tag, const BandPart &p, unsigned *abort, uint32_t &v)
 {
     for (unsigned i = 0;; ++i) {
         unsigned long long a;
         asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(a) : "l"(q) : "memory");
         v = (uint32_t)a;
         if ((uint32_t)(a >> 32) == tag) return true;
-        if ((i & 1023u) == 1023u && (i >= kSpinLimit || *reinterpret_cast<volatile unsigned *>(abort) != 0u)) {
-            *reinterpret_cast<volatile unsigned *>(abort) = 1u;
-            return false;
-        }
+        if (mail_over(i, p, abort)) return false;
     }
 }
 
@@ -273,12 +281,12 @@ struct BandWait {
     uint32_t mail;       // packet index of the other colour's chunk in a packet row
 };
 
-LAT_D bool band_updown(const Band &b, const BandWait &wt, const uint8_t *other, uint32_t r, uint32_t j0, uint32_t nv,
-                       uint32_t (&U)[4], uint32_t (&D)[4])
+LAT_D bool band_updown(const Band &b, const BandPart &part, const BandWait &wt, const uint8_t *other, uint32_t r,
+                       uint32_t j0, uint32_t nv, uint32_t (&U)[4], uint32_t (&D)[4])
 {
     bool ok = true;
     auto from = [&](const ulonglong2 *mail, uint32_t y, uint32_t (&v)[4]) {
-        if (wt.tag != 0u) ok = mail_take(mail + wt.mail, wt.tag, b.abort, v) && ok;
+        if (wt.tag != 0u) ok = mail_take(mail + wt.mail, wt.tag, part, b.abort, v) && ok;
         else if (b.al) load16_any<true>(wt.src + (size_t)y * b.half + j0, nv, v);
         else load16_any<false>(wt.src + (size_t)y * b.half + j0, nv, v);
     };
@@ -436,7 +444,7 @@ LAT_D void band_ising(const Geom &g, const BandPart &part, uint32_t band, uint32
                               2u * ((1u - colour) * b.cpr + q)};
             IsingChunk c;
             uint32_t Sn[4];
-            if (!band_updown(b, wt, other, r, col.j0, col.nv, c.U, c.D)) bad = 1;
+            if (!band_updown(b, part, wt, other, r, col.j0, col.nv, c.U, c.D)) bad = 1;
             const bool more = e + (uint32_t)kBandThreads < edges;
             chunk(std::false_type(), c, col, at, y, edge_group(e),
                   more ? edge_group(e + (uint32_t)kBandThreads) : g_first, !more, Sn);
@@ -552,7 +560,7 @@ LAT_D void band_small(const Geom &g, const BandPart &part, uint32_t band, uint32
             band_shifted<kFull>(cc, odd, other + (at - cc.j0), S[1u - colour], c.X);
             const BandWait wt{b.src + (1u - colour) * b.plane, h > 0 ? part.epoch + (uint32_t)h : 0u,
                               2u * ((1u - colour) * b.cpr + k)};
-            if (!band_updown(b, wt, other, r, cc.j0, cc.nv, c.U, c.D)) bad = 1;
+            if (!band_updown(b, part, wt, other, r, cc.j0, cc.nv, c.U, c.D)) bad = 1;
             uint32_t F[4], Sn[4];
             [[maybe_unused]] uint32_t moved[4];
             if constexpr (kNe) {

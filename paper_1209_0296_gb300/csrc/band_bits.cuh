@@ -304,7 +304,7 @@ LAT_D void band_bits(const Geom &g, const BandPart &part, uint32_t band, uint32_
                 r = lo ? rend : 0u;
                 uint32_t far = 0;
                 if (h == 0) far = spins_at(1u - colour, lo ? dn : up, k);
-                else if (!mail_take_word((lo ? below : above) + (1u - colour) * bw + k, part.epoch + (uint32_t)h, abort, far))
+                else if (!mail_take_word((lo ? below : above) + (1u - colour) * bw + k, part.epoch + (uint32_t)h, part, abort, far))
                     bad = 1;
                 const uint32_t near = other[(lo ? rend : 2u) * bw + k];   // row rend - 1, row 1
                 if constexpr (kNe) {

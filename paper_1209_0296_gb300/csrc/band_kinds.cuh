@@ -119,6 +119,7 @@ inline BandPart band_part(const Geom &k, unsigned long long sweep0, int n, unsig
     p.epoch = epoch;
     p.sweep0 = sweep0;
     p.err = err;
+    p.limit = band_test().limit;
     p.n = n;
     p.key0 = k.key0;
     p.key1 = k.key1;

@@ -190,8 +190,8 @@ LAT_D void band_potts(const Geom &g, const BandPart &part, uint32_t band, uint32
             } else {
                 const unsigned long long *box =
                     reinterpret_cast<const unsigned long long *>((lo ? below : above) + (1u - colour) * bw + k);
-                if (!mail_take_word(box, part.epoch + (uint32_t)h, abort, far.a) ||
-                    !mail_take_word(box + 1, part.epoch + (uint32_t)h, abort, far.b))
+                if (!mail_take_word(box, part.epoch + (uint32_t)h, part, abort, far.a) ||
+                    !mail_take_word(box + 1, part.epoch + (uint32_t)h, part, abort, far.b))
                     bad = 1;
             }
             const Lab near = row_lab(lo ? rend - 1u : 1u, k);

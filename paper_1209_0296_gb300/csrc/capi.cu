@@ -1591,4 +1591,14 @@ int lattice_test_fail_alloc(int countdown)
     return LAT_OK;
 }
 
+// Test hook: waits of band launches give up after `polls` polls (0: the
+// default), and CTA `mute` - 1 of the next band launch sends nothing (0:
+// none), so that its neighbours' waits run out.
+int lattice_test_band_wait(unsigned polls, int mute)
+{
+    band_test().limit.store(polls != 0u ? polls : 1u << 24);
+    band_test().mute.store(mute > 0 ? (uint32_t)mute : 0u);
+    return LAT_OK;
+}
+
 }  // extern "C"

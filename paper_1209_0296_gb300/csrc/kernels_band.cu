@@ -16,6 +16,7 @@ __global__ void __launch_bounds__(kT, 1) k_band(const __grid_constant__ Geom g, 
 {
     extern __shared__ __align__(16) uint8_t band_smem[];
     __shared__ BandShared sh;
+    if (blockIdx.x + 1u == part.mute) return;
     band_body<kKind, kRef, kT, kForm>(g, part, blockIdx.x, gridDim.x, mail, sh, band_smem);
     band_end(g, part, blockIdx.x, sh);
 }
@@ -40,6 +41,12 @@ constexpr BandKernel band_kernel()
 }
 
 }  // namespace
+
+BandTest &band_test()
+{
+    static BandTest t;
+    return t;
+}
 
 int band_sms()
 {
@@ -91,7 +98,8 @@ cudaError_t launch_sweep_band(const Geom &g, bool fields, int bands, unsigned lo
     });
     if (attr != cudaSuccess) return attr;
     const Geom k = tiled_geom(g);
-    const BandPart part = band_part(k, sweep0, n, epoch, err);
+    BandPart part = band_part(k, sweep0, n, epoch, err);
+    part.mute = band_test().mute.exchange(0);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)bands);
     // one chunk a thread: just the warps that have one (a row is a warp's when it fits)

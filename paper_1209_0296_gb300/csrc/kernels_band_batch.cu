@@ -134,6 +134,7 @@ cudaError_t launch_batch_band(const Geom *d_geoms, const std::vector<std::pair<c
     });
     if (attr != cudaSuccess) return attr;
     auto parts = std::make_unique<BandParts>();
+    const int mute = (int)band_test().mute.exchange(0) - 1;
     size_t smem = 0, pairs = 0;
     int cta = 0;
     for (size_t i = 0; i < lats.size(); ++i) {
@@ -148,7 +149,9 @@ cudaError_t launch_batch_band(const Geom *d_geoms, const std::vector<std::pair<c
         smem = std::max(smem, band_smem_bytes(k, (int)p.kind, ctas[i]));
         for (int b = 0; b < ctas[i]; ++b) {
             p.band = (uint32_t)b;
-            parts->p[cta++] = p;
+            parts->p[cta] = p;
+            if (cta == mute) parts->p[cta].n = 0;   // it leaves its rows alone and sends nothing
+            ++cta;
         }
     }
     cudaLaunchConfig_t cfg = {};

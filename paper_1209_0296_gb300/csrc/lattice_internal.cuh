@@ -7,6 +7,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <utility>
 #include <vector>
 
@@ -470,8 +471,14 @@ cudaError_t launch_batch_ne(const Geom *geoms, const uint2 *items, int n_items, 
 // the whole GPU (0: not supported or too large).  mail: band_mail_bytes() of
 // device memory, zeroed once; epoch: at least every packet mark sent through
 // it before, the launch marks up to epoch + 2 n; err: host-visible word set
-// when a bounded wait gave up (mail must then be zeroed again).  Advances
-// ctrl->sweep.
+// when a bounded wait gave up.  Advances ctrl->sweep.
+// Test settings of band launches: polls after which a wait gives up (about a quarter of a
+// microsecond each: four seconds), 1 + the CTA of the next launch that sends
+// nothing (0: none).
+struct BandTest {
+    std::atomic<uint32_t> limit{1u << 24}, mute{0};
+};
+BandTest &band_test();
 int band_sms();   // CTAs of a launch at most
 int band_count_for(const Geom &g, bool fields);
 size_t band_mail_bytes(const Geom &g, bool fields, int bands);
