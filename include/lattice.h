@@ -69,7 +69,8 @@ enum lattice_status {
     LAT_ETIMEOUT = -4, /* a bounded wait gave up: lattice_server_drain's limit, or (about
                           four seconds) a band of a band-resident launch waiting for its
                           neighbour's rows; after the latter the lattice's state is
-                          undefined and every call on it returns this */
+                          undefined, and every call that reads, advances or refers to it
+                          (in a batch too) returns this until lattice_set_state */
     LAT_EBUSY = -5,    /* result not ready yet (server poll) */
     LAT_ENOTSUP = -6,  /* valid but unsupported combination */
     LAT_ERANGE = -7,   /* index or size out of range */
@@ -352,6 +353,8 @@ int lattice_batch_add(lattice_batch_t *b, lattice_t *lat, int64_t n);
  * set to LAT_KERNEL_RESIDENT run as resident CTAs, one per lattice, for all
  * their sweeps, concurrently with the others. */
 int lattice_batch_run(lattice_batch_t *b);
+/* Wait for the runs queued so far; LAT_ETIMEOUT when a wait of one of them
+ * gave up since the last call (the lattices concerned return it too). */
 int lattice_batch_synchronize(lattice_batch_t *b);
 /* The batch engine's two tunables as its last run used them: the rows a
  * thread visits per item of the pipelined 2D spin-1/2 kernel

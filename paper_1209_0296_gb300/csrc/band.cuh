@@ -48,7 +48,7 @@ struct BandPart {
     uint32_t lat, kind, ref;     // batched: descriptor index, BandKind, reference set
     uint32_t epoch;              // packets are marked epoch + 1 .. epoch + 2 n
     unsigned long long sweep0;   // sweeps done before the launch
-    int *err;                    // host-visible error word of the lattice
+    int *err, *err_all;          // host-visible error words of the lattice and (or null) of its batch
     uint32_t limit;              // polls after which a wait gives up
     uint32_t mute;               // solo: 1 + the band that sends nothing (0: none), by which tests let waits run out
     uint32_t mail;               // batched: packet rows start at this pair

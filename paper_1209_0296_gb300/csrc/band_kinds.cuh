@@ -14,7 +14,10 @@ namespace {
 LAT_D void band_end(const Geom &g, const BandPart &p, uint32_t band, const BandShared &sh)
 {
     if (threadIdx.x != 0) return;
-    if (sh.bad) *reinterpret_cast<volatile int *>(p.err) = 1;
+    if (sh.bad) {
+        *reinterpret_cast<volatile int *>(p.err) = 1;
+        if (p.err_all != nullptr) *reinterpret_cast<volatile int *>(p.err_all) = 1;
+    }
     if (band == 0u) g.ctrl->sweep = p.sweep0 + (unsigned long long)p.n;
 }
 

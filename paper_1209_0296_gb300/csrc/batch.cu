@@ -80,6 +80,7 @@ struct lattice_batch {
     void *d_mail = nullptr;
     size_t mail_cap = 0;
     unsigned mail_epoch = 0;
+    int *band_err = nullptr;   // host-visible: a wait of a run gave up since the last synchronise
     // resident lattices
     cudaStream_t res_stream = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
@@ -409,6 +410,7 @@ int run_bands(lattice_batch *b, BatchSlot &sl, size_t at, std::vector<BandGroup>
         n += g.work.size();
         mail = std::max(mail, band_batch_mail_bytes(band_list(g.work), g.ctas));
     }
+    if (b->band_err == nullptr && (b->band_err = band_error_word()) == nullptr) return kBandsRefused;
     std::vector<Geom> geoms;
     geoms.reserve(n);
     for (auto &g : groups)
@@ -462,8 +464,8 @@ int run_bands(lattice_batch *b, BatchSlot &sl, size_t at, std::vector<BandGroup>
                 BandTurn turn(b->stream);
                 e = turn.status;
                 if (e == cudaSuccess)
-                    e = launch_batch_band(sl.d_band_geoms + first, l, sweep0, err, g.ctas, b->d_mail, b->mail_epoch,
-                                          b->stream);
+                    e = launch_batch_band(sl.d_band_geoms + first, l, sweep0, err, b->band_err, g.ctas, b->d_mail,
+                                          b->mail_epoch, b->stream);
                 if (e == cudaErrorCooperativeLaunchTooLarge && first == 0 && k == 0) return kBandsRefused;
             }
             b->mail_epoch += 2u * (unsigned)most;
@@ -682,6 +684,8 @@ int lattice_batch_add(lattice_batch_t *b, lattice_t *lt, int64_t n)
     if (b == nullptr || lt == nullptr || n < 0) return LAT_EINVAL;
     if (lt->P.layout == LAT_BITPACKED || lt->dynamics != LAT_DYNAMICS_CHECKERBOARD) return LAT_ENOTSUP;
     if (n == 0) return LAT_OK;
+    const int rc = band_status(lt);
+    if (rc != LAT_OK) return rc;
     for (auto &pr : b->pending)
         if (pr.first == lt) {
             pr.second += n;
@@ -697,6 +701,13 @@ int lattice_batch_run(lattice_batch_t *b)
     std::vector<std::pair<lattice *, int64_t>> work;
     work.swap(b->pending);
     if (work.empty()) return LAT_OK;
+    // (The server's requests end one by one: each sees its own status when it
+    // is added to the next round or read back.)
+    if (!b->caller_orders)
+        for (auto &pr : work) {
+            const int rc = band_status(pr.first);
+            if (rc != LAT_OK) return rc;
+        }
     // Counter space for every sweep of the run (queued on each lattice's own
     // stream), then the batch stream waits for the work queued so far on
     // each distinct lattice stream (lattices often share one): an event
@@ -887,6 +898,10 @@ int lattice_batch_synchronize(lattice_batch_t *b)
     cudaError_t e = cudaStreamSynchronize(b->stream);
     if (e == cudaSuccess && b->res_stream) e = cudaStreamSynchronize(b->res_stream);
     if (e != cudaSuccess) return cuda_fail(e, "batch synchronize");
+    if (b->band_err != nullptr && *(volatile int *)b->band_err != 0) {
+        *b->band_err = 0;
+        return LAT_ETIMEOUT;
+    }
     return LAT_OK;
 }
 

@@ -458,8 +458,7 @@ static int band_sweeps(lattice *lt, int bands, int64_t n, int64_t *done)
     return LAT_OK;
 }
 
-// Whether a bounded wait of an earlier launch gave up (after a synchronise).
-static int band_status(const lattice *lt)
+int band_status(const lattice *lt)
 {
     return lt->band_err != nullptr && *(volatile int *)lt->band_err != 0 ? LAT_ETIMEOUT : LAT_OK;
 }
@@ -1069,6 +1068,8 @@ int lattice_series(lattice_t *lt, int64_t first, int64_t count, int64_t *bond, i
 int lattice_set_reference(lattice_t *lt, int64_t *ref_sweep)
 {
     if (lt == nullptr) return LAT_EINVAL;
+    const int rc = band_status(lt);
+    if (rc != LAT_OK) return rc;
     cudaStream_t st = lt->stream;
     cudaError_t e = cudaSuccess;
     if (lt->P.layout == LAT_BITPACKED) {
@@ -1403,6 +1404,8 @@ int lattice_set_spins(lattice_t *lt, const int8_t *host_in)
         e = cudaMemcpyAsync(&bad, lt->scratch4, sizeof bad, cudaMemcpyDeviceToHost, lt->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(lt->stream);   // the caller may reuse host_in now
     if (e != cudaSuccess) return cuda_fail(e, "set spins");
+    const int rc = band_status(lt);   // the flags and counters would stay undefined
+    if (rc != LAT_OK) return rc;
     if (bad != 0) return LAT_EINVAL;
     e = launch_to_planar(lt->geom, lin, dst, lt->stream);
     if (e == cudaSuccess && lt->P.layout == LAT_BITPACKED) e = launch_pack_bits(lt->geom, dst, lt->bits[par], lt->stream);
@@ -1431,7 +1434,7 @@ int lattice_get_state(lattice_t *lt, int8_t *spins, uint8_t *flags, int64_t *swe
         }
     }
     if (sweeps) *sweeps = lt->sweeps;
-    return LAT_OK;
+    return band_status(lt);
 }
 
 int lattice_set_state(lattice_t *lt, const int8_t *spins, const uint8_t *flags, int64_t sweeps)
@@ -1489,6 +1492,8 @@ int lattice_info(lattice_t *lt, int64_t *sweeps, int64_t *n_sites, int64_t *devi
 int lattice_device_spins(lattice_t *lt, void **dev_ptr, size_t *bytes)
 {
     if (lt == nullptr || dev_ptr == nullptr) return LAT_EINVAL;
+    const int rc = band_status(lt);
+    if (rc != LAT_OK) return rc;
     const int par = (int)(lt->sweeps & 1);
     if (lt->P.layout == LAT_BITPACKED) {
         *dev_ptr = lt->bits[par];

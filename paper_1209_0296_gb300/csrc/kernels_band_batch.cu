@@ -123,7 +123,7 @@ size_t band_batch_mail_bytes(const std::vector<std::pair<const Geom *, long long
 
 cudaError_t launch_batch_band(const Geom *d_geoms, const std::vector<std::pair<const Geom *, long long>> &lats,
                               const std::vector<unsigned long long> &sweep0, const std::vector<int *> &err,
-                              const std::vector<int> &ctas, void *mail, unsigned epoch, cudaStream_t st)
+                              int *err_all, const std::vector<int> &ctas, void *mail, unsigned epoch, cudaStream_t st)
 {
     static std::once_flag once;
     static cudaError_t attr = cudaSuccess;
@@ -140,6 +140,7 @@ cudaError_t launch_batch_band(const Geom *d_geoms, const std::vector<std::pair<c
     for (size_t i = 0; i < lats.size(); ++i) {
         const Geom k = tiled_geom(*lats[i].first);
         BandPart p = band_part(k, sweep0[i], (int)lats[i].second, epoch, err[i]);
+        p.err_all = err_all;
         p.bands = (uint32_t)ctas[i];
         p.lat = (uint32_t)i;
         p.kind = (uint32_t)band_kind(k, false);

@@ -30,6 +30,9 @@ int sweep_impl(struct ::lattice *lt, int64_t n);
 int choose_kernel(const struct ::lattice *lt);
 // A host-visible error word for band launches (one of a fixed page), zeroed.
 int *band_error_word();
+// Whether a bounded wait of an earlier launch gave up, as far as the host has
+// seen (after a synchronise: all of them).
+int band_status(const struct ::lattice *lt);
 // Order a band launch on st after the last one on any stream: two of them
 // must not wait for each other's SMs.  Holds a lock until destroyed.
 class BandTurn {

@@ -488,13 +488,14 @@ cudaError_t launch_sweep_band(const Geom &g, bool fields, int bands, unsigned lo
 // = the fewest CTAs that hold a lattice (0: not here); band_share = CTAs for
 // (lattice, sweeps) pairs run together and the estimated us (infinite: they
 // do not fit); the launch runs them all.  d_geoms: tiled_geom descriptors in
-// the same order; mail: band_batch_mail_bytes(), zeroed once.
+// the same order; mail: band_batch_mail_bytes(), zeroed once; err, err_all: set
+// when a wait of that lattice, of any lattice gave up.
 int band_min_ctas(const Geom &g);
 double band_share(const std::vector<std::pair<const Geom *, long long>> &lats, std::vector<int> &ctas);
 size_t band_batch_mail_bytes(const std::vector<std::pair<const Geom *, long long>> &lats, const std::vector<int> &ctas);
 cudaError_t launch_batch_band(const Geom *d_geoms, const std::vector<std::pair<const Geom *, long long>> &lats,
                               const std::vector<unsigned long long> &sweep0, const std::vector<int *> &err,
-                              const std::vector<int> &ctas, void *mail, unsigned epoch, cudaStream_t st);
+                              int *err_all, const std::vector<int> &ctas, void *mail, unsigned epoch, cudaStream_t st);
 // batched engine
 Geom tiled_geom(const Geom &g);
 int tiles_of(const Geom &g, int tile_h);

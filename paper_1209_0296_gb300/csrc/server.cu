@@ -45,6 +45,7 @@ struct Req {
     size_t bytes;          // device footprint charged against the budget
     lattice *lt = nullptr;
     int64_t planned = 0;   // sweeps queued so far
+    int rc = LAT_OK;       // why it ends early, with rounds of it still running
     lattice_result_t res{};
     std::vector<int8_t> spins;
 };
@@ -123,8 +124,8 @@ void fail(lattice_server *s, Req *q, int status)
 // which the batch never makes wait on later rounds.
 void retire(lattice_server *s, Req *q)
 {
-    int rc = LAT_OK;
-    if (q->r.sweeps > 0) {
+    int rc = q->rc;
+    if (rc == LAT_OK && q->r.sweeps > 0) {
         int64_t b, m, u, f;
         rc = lattice_series(q->lt, q->r.sweeps - 1, 1, &b, &m, &u, &f);
         if (rc == LAT_OK) {
@@ -247,7 +248,12 @@ void scheduler(lattice_server *s)
             if (k > 0) {
                 const int rc = lattice_batch_add(s->batch, q->lt, k);
                 if (rc != LAT_OK) {   // this request alone
-                    fail(s, q, rc);
+                    if (q->planned == 0) {
+                        fail(s, q, rc);
+                    } else {   // freed with this round: the rounds before it may still use the lattice
+                        q->rc = rc;
+                        rd.retiring.push_back(q);
+                    }
                     continue;
                 }
                 q->planned += k;
