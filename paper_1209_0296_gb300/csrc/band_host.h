@@ -1,0 +1,72 @@
+// band_host.h -- host-side bookkeeping of band launches that needs no CUDA
+// call of its own (plain C++, tested without a GPU).
+#pragma once
+
+#include <cstddef>
+#include <mutex>
+#include <utility>
+#include <vector>
+
+namespace lat {
+
+// Words that kernels write and the host reads (an error word per lattice).  A
+// word given back is handed out again only when the work that may still write
+// it is complete, so no two live owners ever share one.
+class WordPool {
+public:
+    using Page = int *(*)(size_t words);   // new words, or null
+    using Done = bool (*)(void *event);    // the work recorded in event is complete (then the event is freed)
+
+    WordPool(Page page, Done done, size_t words) : page_(page), done_(done), words_(words) {}
+
+    // A zeroed word, or null when there is no memory.
+    int *take()
+    {
+        std::lock_guard<std::mutex> g(mu_);
+        try {
+            for (size_t i = 0; i < pending_.size();) {
+                if (done_(pending_[i].second)) {
+                    int *w = pending_[i].first;
+                    pending_[i] = pending_.back();
+                    pending_.pop_back();
+                    free_.push_back(w);
+                } else {
+                    ++i;
+                }
+            }
+            if (free_.empty()) {
+                free_.reserve(words_);
+                int *p = page_(words_);
+                if (p == nullptr) return nullptr;
+                for (size_t i = words_; i-- > 0;) free_.push_back(p + i);
+            }
+        } catch (...) {   // a word that cannot be listed is lost, never shared
+            return nullptr;
+        }
+        int *w = free_.back();
+        free_.pop_back();
+        *w = 0;
+        return w;
+    }
+
+    // Give w back, free once event is complete (null: at once).
+    void give(int *w, void *event)
+    {
+        std::lock_guard<std::mutex> g(mu_);
+        try {
+            if (event == nullptr) free_.push_back(w);
+            else pending_.emplace_back(w, event);
+        } catch (...) {
+        }
+    }
+
+private:
+    const Page page_;
+    const Done done_;
+    const size_t words_;
+    std::mutex mu_;
+    std::vector<int *> free_;
+    std::vector<std::pair<int *, void *>> pending_;
+};
+
+}  // namespace lat

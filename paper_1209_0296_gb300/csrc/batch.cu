@@ -925,6 +925,7 @@ void lattice_batch_destroy(lattice_batch_t *b)
     for (cudaEvent_t ev : b->ev_streams) cudaEventDestroy(ev);
     dev_free(b->d_counters, b->stream);
     dev_free(b->d_mail, b->stream);
+    band_error_word_back(b->band_err, b->stream, false);
     if (b->res_stream) cudaStreamDestroy(b->res_stream);
     if (b->ev_fork) cudaEventDestroy(b->ev_fork);
     if (b->ev_join) cudaEventDestroy(b->ev_join);

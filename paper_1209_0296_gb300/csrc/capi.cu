@@ -13,6 +13,7 @@
 #include <string>
 #include <vector>
 
+#include "band_host.h"
 #include "lattice_capi_internal.h"
 
 namespace lat {
@@ -323,21 +324,40 @@ int choose_kernel(const lattice *lt)
     return LAT_KERNEL_GENERIC;
 }
 
-int *band_error_word()
+static WordPool &error_words()
 {
-    static std::mutex mu;
-    static int *page = nullptr;
-    static unsigned next = 0;
-    constexpr unsigned kWords = 16384;
-    std::lock_guard<std::mutex> g(mu);
-    if (page == nullptr && cudaHostAlloc((void **)&page, kWords * sizeof(int), cudaHostAllocPortable) != cudaSuccess) {
-        (void)cudaGetLastError();
-        page = nullptr;
-        return nullptr;
+    static WordPool *pool = new WordPool(   // (never destroyed: lattices may outlive static objects)
+        [](size_t words) {
+            void *p = nullptr;
+            if (cudaHostAlloc(&p, words * sizeof(int), cudaHostAllocPortable) == cudaSuccess) return (int *)p;
+            (void)cudaGetLastError();
+            return (int *)nullptr;
+        },
+        [](void *ev) {
+            if (cudaEventQuery((cudaEvent_t)ev) != cudaSuccess) {
+                (void)cudaGetLastError();   // not ready
+                return false;
+            }
+            cudaEventDestroy((cudaEvent_t)ev);
+            return true;
+        },
+        4096);
+    return *pool;
+}
+
+int *band_error_word() { return error_words().take(); }
+
+void band_error_word_back(int *w, cudaStream_t st, bool busy)
+{
+    if (w == nullptr) return;
+    cudaEvent_t ev = nullptr;
+    if (busy && (cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess ||
+                 cudaEventRecord(ev, st) != cudaSuccess)) {
+        (void)cudaGetLastError();   // the word is not used again
+        if (ev != nullptr) cudaEventDestroy(ev);
+        return;
     }
-    int *w = page + next++ % kWords;
-    *w = 0;
-    return w;
+    error_words().give(w, ev);
 }
 
 // One event per device, recorded after every band launch.
@@ -859,6 +879,7 @@ static void release(lattice *lt)
     dev_free(lt->rs_scratch, st);
     dev_free(lt->cpl, st);
     dev_free(lt->band_mail, st);
+    band_error_word_back(lt->band_err, st, true);
     delete lt;
 }
 

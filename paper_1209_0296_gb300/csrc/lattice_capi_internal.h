@@ -28,8 +28,10 @@ int create_impl(struct ::lattice **out, int dims, int L, int two_S, int model, d
                 double T_or_c, uint64_t seed, int init, int layout, void *cuda_stream);
 int sweep_impl(struct ::lattice *lt, int64_t n);
 int choose_kernel(const struct ::lattice *lt);
-// A host-visible error word for band launches (one of a fixed page), zeroed.
+// A host-visible error word for band launches, zeroed (null: no memory), the
+// owner's until it is given back; busy: launches on st may still write it.
 int *band_error_word();
+void band_error_word_back(int *w, cudaStream_t st, bool busy);
 // Whether a bounded wait of an earlier launch gave up, as far as the host has
 // seen (after a synchronise: all of them).
 int band_status(const struct ::lattice *lt);
