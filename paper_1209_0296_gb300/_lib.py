@@ -89,6 +89,8 @@ SIGNATURES = {
 TEST_SIGNATURES = {
     "lattice_test_fail_alloc": (c_int, [c_int]),
     "lattice_test_band_wait": (c_int, [ctypes.c_uint, c_int]),
+    "lattice_test_band_refuse": (c_int, [c_int]),
+    "lattice_test_band_launches": (c_int64, []),
 }
 
 

@@ -667,26 +667,18 @@ bool tune_choice_ok(const lattice *lt, const TuneChoice &c)
     }
 }
 
-// n sweeps of the band-resident kernel, `ahead` sweeps after the lattice's
-// count (the tuner moves the count on after a candidate).
-int band_candidate(lattice *lt, int bands, int ahead, int n)
-{
-    int64_t done = 0;
-    lt->sweeps += ahead;
-    const int rc = band_sweeps(lt, bands, n, &done);
-    lt->sweeps -= ahead;
-    return rc != LAT_OK || done == n ? rc : LAT_ENOMEM;
-}
-
 // Time one replay of a graph of n sweeps after one untimed replay (the
 // resident and band-resident kernels: two launches of n sweeps, the second
-// timed); 2n sweeps are enqueued on the lattice's stream.  graph_only: as a
-// graph whichever way the sweep loop would run them.
-int time_candidate(lattice *lt, int n, cudaEvent_t ev0, cudaEvent_t ev1, float &ms, bool graph_only = false)
+// timed); 2n sweeps are enqueued on the lattice's stream, counted and taken
+// off `left` as they are queued.  Where the bands are refused the launches do
+// their sweeps, as in the sweep loop.  graph_only: as a graph whichever way
+// the sweep loop would run them.
+int time_candidate(lattice *lt, int n, cudaEvent_t ev0, cudaEvent_t ev1, float &ms, int64_t &left,
+                   bool graph_only = false)
 {
     cudaGraphExec_t exec = nullptr;
     int rc = LAT_OK;
-    const int bands = graph_only ? 0 : band_bands(lt, n);
+    int bands = graph_only ? 0 : band_bands(lt, n);
     const bool graphed = choose_kernel(lt) != LAT_KERNEL_RESIDENT && bands == 0;
     if (graphed) {
         if (lt->cap_stream == nullptr &&
@@ -704,10 +696,20 @@ int time_candidate(lattice *lt, int n, cudaEvent_t ev0, cudaEvent_t ev1, float &
     }
     for (int rep = 0; rep < 2 && rc == LAT_OK; ++rep) {
         if (rep == 1 && cudaEventRecord(ev0, lt->stream) != cudaSuccess) rc = LAT_ECUDA;
-        if (rc == LAT_OK) {
+        int64_t done = 0;
+        if (rc == LAT_OK && bands > 0) {
+            rc = band_sweeps(lt, bands, n, &done);
+            if (done < n) bands = 0;
+            lt->sweeps += done;
+            left -= done;
+        }
+        if (rc == LAT_OK && done < n) {
             if (graphed) rc = cudaGraphLaunch(exec, lt->stream) == cudaSuccess ? LAT_OK : LAT_ECUDA;
-            else if (bands > 0) rc = band_candidate(lt, bands, rep * n, n);
-            else rc = enqueue_sweeps(lt, n, lt->stream);
+            else rc = enqueue_sweeps(lt, n - done, lt->stream);
+            if (rc == LAT_OK) {
+                lt->sweeps += n - done;
+                left -= n - done;
+            }
         }
     }
     if (rc == LAT_OK && cudaEventRecord(ev1, lt->stream) != cudaSuccess) rc = LAT_ECUDA;
@@ -773,10 +775,8 @@ static int autotune(lattice *lt, int64_t &left)
             lt->tuned_kernel = cand[(size_t)c].kernel;
             lt->tile_h = cand[(size_t)c].tile_h;
             float ms = 0.f;
-            rc = time_candidate(lt, kTuneSweeps, ev[0], ev[1], ms);
+            rc = time_candidate(lt, kTuneSweeps, ev[0], ev[1], ms, left);
             if (rc != LAT_OK) break;
-            lt->sweeps += 2 * kTuneSweeps;
-            left -= 2 * kTuneSweeps;
             if (ms < best) {
                 best = ms;
                 pick = cand[(size_t)c];
@@ -792,10 +792,8 @@ static int autotune(lattice *lt, int64_t &left)
             const int gs = std::max(2, g0 * f / 2);
             if (left < 2 * (int64_t)gs) break;
             float ms = 0.f;
-            rc = time_candidate(lt, gs, ev[0], ev[1], ms, true);
+            rc = time_candidate(lt, gs, ev[0], ev[1], ms, left, true);
             if (rc != LAT_OK) break;
-            lt->sweeps += 2 * gs;
-            left -= 2 * gs;
             if (ms / gs < best) {
                 best = ms / gs;
                 pick.graph = gs;
@@ -1626,5 +1624,16 @@ int lattice_test_band_wait(unsigned polls, int mute)
     band_test().mute.store(mute > 0 ? (uint32_t)mute : 0u);
     return LAT_OK;
 }
+
+// Test hook: the countdown-th next band launch is refused as too large for the
+// device (0: none).
+int lattice_test_band_refuse(int countdown)
+{
+    band_test().refuse.store(countdown < 0 ? 0 : countdown);
+    return LAT_OK;
+}
+
+// Test hook: band launches of this process so far.
+int64_t lattice_test_band_launches(void) { return band_test().launches.load(); }
 
 }  // extern "C"

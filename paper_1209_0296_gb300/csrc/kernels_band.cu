@@ -97,6 +97,7 @@ cudaError_t launch_sweep_band(const Geom &g, bool fields, int bands, unsigned lo
                 }
     });
     if (attr != cudaSuccess) return attr;
+    if (band_test().launch()) return cudaErrorCooperativeLaunchTooLarge;
     const Geom k = tiled_geom(g);
     BandPart part = band_part(k, sweep0, n, epoch, err);
     part.mute = band_test().mute.exchange(0);

@@ -133,6 +133,7 @@ cudaError_t launch_batch_band(const Geom *d_geoms, const std::vector<std::pair<c
                 attr = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBandMaxSmem);
     });
     if (attr != cudaSuccess) return attr;
+    if (band_test().launch()) return cudaErrorCooperativeLaunchTooLarge;
     auto parts = std::make_unique<BandParts>();
     const int mute = (int)band_test().mute.exchange(0) - 1;
     size_t smem = 0, pairs = 0;

@@ -474,9 +474,20 @@ cudaError_t launch_batch_ne(const Geom *geoms, const uint2 *items, int n_items, 
 // when a bounded wait gave up.  Advances ctrl->sweep.
 // Test settings of band launches: polls after which a wait gives up (about a quarter of a
 // microsecond each: four seconds), 1 + the CTA of the next launch that sends
-// nothing (0: none).
+// nothing (0: none), launches until one is refused (1: the next; 0: none); and
+// the launches so far.
 struct BandTest {
     std::atomic<uint32_t> limit{1u << 24}, mute{0};
+    std::atomic<int> refuse{0};
+    std::atomic<long long> launches{0};
+    // At each launch: true when it is to be refused as too large.
+    bool launch()
+    {
+        int r = refuse.load();
+        if (r > 0 && (r = refuse.fetch_sub(1)) == 1) return true;
+        ++launches;
+        return false;
+    }
 };
 BandTest &band_test();
 int band_sms();   // CTAs of a launch at most
