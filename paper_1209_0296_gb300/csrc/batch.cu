@@ -337,6 +337,7 @@ struct BandGroup {
     Work work;
     std::vector<int> ctas;
     double us;   // estimate
+    std::vector<int64_t> ran;   // sweeps of each lattice queued by run_bands
 };
 
 BandList band_list(const Work &w)
@@ -378,7 +379,7 @@ void plan_bands(Work &work, std::vector<BandGroup> &groups, size_t at_least)
     int used = 0;
     auto close = [&]() {
         if (cur.empty()) return;
-        BandGroup g{cur, {}, 0.0};
+        BandGroup g{cur, {}, 0.0, std::vector<int64_t>(cur.size(), 0)};
         g.us = band_share(band_list(cur), g.ctas);
         band_us += g.us + 10.0;
         out.push_back(std::move(g));
@@ -399,10 +400,10 @@ void plan_bands(Work &work, std::vector<BandGroup> &groups, size_t at_least)
     groups.swap(out);
 }
 
-// Launch the groups one after another on the batch stream. kBandsRefused:
-// nothing was launched (no memory for the packets, or fewer SMs than the
-// device reports), the step loop takes the lattices.
-constexpr int kBandsRefused = 1;
+// Launch the groups one after another on the batch stream; their `ran` says
+// what was queued: less than all when the bands are refused (no memory for the
+// packets, or fewer SMs than the device reports), and then the step loop takes
+// the rest.
 int run_bands(lattice_batch *b, BatchSlot &sl, size_t at, std::vector<BandGroup> &groups)
 {
     size_t n = 0, mail = 0;
@@ -410,22 +411,28 @@ int run_bands(lattice_batch *b, BatchSlot &sl, size_t at, std::vector<BandGroup>
         n += g.work.size();
         mail = std::max(mail, band_batch_mail_bytes(band_list(g.work), g.ctas));
     }
-    if (b->band_err == nullptr && (b->band_err = band_error_word()) == nullptr) return kBandsRefused;
+    if (b->band_err == nullptr && (b->band_err = band_error_word()) == nullptr) return LAT_OK;
     std::vector<Geom> geoms;
     geoms.reserve(n);
     for (auto &g : groups)
         for (auto &pr : g.work) {
-            if (pr.first->band_err == nullptr && (pr.first->band_err = band_error_word()) == nullptr) return kBandsRefused;
+            if (pr.first->band_err == nullptr && (pr.first->band_err = band_error_word()) == nullptr) return LAT_OK;
             geoms.push_back(tiled_geom(pr.first->geom));
         }
     int rc = grow(&sl.d_band_geoms, sl.band_geoms_cap, (int)n, b->stream);
-    if (rc == LAT_ENOMEM) return kBandsRefused;
+    if (rc == LAT_ENOMEM) {
+        (void)cudaGetLastError();
+        return LAT_OK;
+    }
     if (rc != LAT_OK) return rc;
     cudaError_t e = cudaSuccess;
     if (mail > b->mail_cap) {
         void *p = nullptr;
         e = dev_alloc(&p, mail, b->stream);
-        if (e == cudaErrorMemoryAllocation) return kBandsRefused;
+        if (e == cudaErrorMemoryAllocation) {
+            (void)cudaGetLastError();
+            return LAT_OK;
+        }
         if (e != cudaSuccess) return cuda_fail(e, "batch packets");
         dev_free(b->d_mail, b->stream);
         b->d_mail = p;
@@ -466,9 +473,13 @@ int run_bands(lattice_batch *b, BatchSlot &sl, size_t at, std::vector<BandGroup>
                 if (e == cudaSuccess)
                     e = launch_batch_band(sl.d_band_geoms + first, l, sweep0, err, b->band_err, g.ctas, b->d_mail,
                                           b->mail_epoch, b->stream);
-                if (e == cudaErrorCooperativeLaunchTooLarge && first == 0 && k == 0) return kBandsRefused;
+                if (e == cudaErrorCooperativeLaunchTooLarge) {
+                    (void)cudaGetLastError();
+                    return LAT_OK;
+                }
             }
             b->mail_epoch += 2u * (unsigned)most;
+            for (size_t i = 0; i < l.size() && e == cudaSuccess; ++i) g.ran[i] += l[i].second;
         }
         first += g.work.size();
     }
@@ -751,7 +762,6 @@ int lattice_batch_run(lattice_batch_t *b)
     work.swap(rest);
     // Lattices that fit the chip's shared memory: all their sweeps in a few launches.
     std::vector<BandGroup> groups;
-    const auto unplanned = work;
     // (the launches carry the host's sweep numbers: not while the caller captures the stream)
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(b->stream, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone)
@@ -761,21 +771,15 @@ int lattice_batch_run(lattice_batch_t *b)
     std::vector<std::pair<lattice *, int64_t>> banded;
     if (!groups.empty()) {
         mark_start();
-        int rc = run_bands(b, sl, res_bytes, groups);
-        if (rc == kBandsRefused) {
-            (void)cudaGetLastError();
-            work = unplanned;
-            groups.clear();
-        } else if (rc != LAT_OK) {
-            return rc;
-        }
-    }
-    if (!groups.empty()) {
+        const int rc = run_bands(b, sl, res_bytes, groups);
         for (auto &g : groups)
-            for (auto &pr : g.work) {
-                pr.first->sweeps += pr.second;
-                banded.push_back(pr);
+            for (size_t i = 0; i < g.work.size(); ++i) {
+                lattice *lt = g.work[i].first;
+                lt->sweeps += g.ran[i];
+                banded.push_back(g.work[i]);
+                if (g.ran[i] < g.work[i].second) work.emplace_back(lt, g.work[i].second - g.ran[i]);
             }
+        if (rc != LAT_OK) return rc;
         res_bytes = (res_bytes + banded.size() * sizeof(Geom) + 64 + 15) & ~(size_t)15;
         b->last_passes = 0;
         b->last_gsteps = kGraphSteps;

@@ -48,3 +48,38 @@ def test_tuning_call(lib, L, how, at):
     if L % 32:                                            # (else the tuner may have found another kernel)
         assert lib.lattice_test_band_launches() > before  # bands again
     g.close()
+
+
+# 170 lattices go in two band launches or more: none, the second or a later one is refused
+@pytest.mark.parametrize("at", [1, 2])
+def test_batch(lib, at):
+    pairs = [_make(130 + 2 * (i % 9), 700 + i, i % 4 == 1) for i in range(170)]
+    b = lt.Batch()
+    for rep in range(2):                 # the second run follows on what both forms left
+        lib.lattice_test_band_refuse(at if rep == 0 else 0)
+        before = lib.lattice_test_band_launches()
+        for i, (g, _) in enumerate(pairs):
+            b.add(g, 20 + i % 3)
+        b.run()
+        b.synchronize()
+        assert (lib.lattice_test_band_launches() - before) == (at - 1) or rep == 1
+        for i in range(0, 170, 11):
+            g, o = pairs[i]
+            n = 20 + i % 3
+            _check(g, o, o.sweep(n), rep * n, n)
+    b.close()
+
+
+def test_batch_without_memory_for_the_packets(lib):
+    b = lt.Batch()
+    pairs = [_make(L, L) for L in (300, 512, 610)]
+    for g, _ in pairs:
+        g.sweep(1)
+        b.add(g, 12)
+    lib.lattice_test_fail_alloc(2)       # the band descriptors, then the packets
+    b.run()
+    lib.lattice_test_fail_alloc(0)
+    for g, o in pairs:
+        o.sweep(1)
+        _check(g, o, o.sweep(12), 1, 12)
+    b.close()
