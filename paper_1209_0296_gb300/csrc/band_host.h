@@ -69,4 +69,23 @@ private:
     std::vector<std::pair<int *, void *>> pending_;
 };
 
+// A value found once per device (function attributes and SM counts belong to
+// one); devices past kMax are asked every time.
+template <typename T>
+class PerDevice {
+public:
+    template <typename F>
+    T get(int device, F find)
+    {
+        if (device < 0 || device >= kMax) return find();
+        std::call_once(once_[device], [&] { value_[device] = find(); });
+        return value_[device];
+    }
+
+private:
+    static constexpr int kMax = 64;
+    std::once_flag once_[kMax];
+    T value_[kMax] = {};
+};
+
 }  // namespace lat

@@ -1,8 +1,8 @@
 // kernels_band.cu -- the band-resident kernel (band.cuh) of one lattice: a
 // grid of one CTA per SM, all sweeps of a call in one cooperative launch.
 #include <algorithm>
-#include <mutex>
 
+#include "band_host.h"
 #include "band_kinds.cuh"
 
 namespace lat {
@@ -50,14 +50,15 @@ BandTest &band_test()
 
 int band_sms()
 {
-    static const int sms = [] {
-        int dev = 0, n = 0, coop = 0;
-        cudaGetDevice(&dev);
+    static PerDevice<int> sms;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    return sms.get(dev, [dev] {
+        int n = 0, coop = 0;
         cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
         return coop ? std::min(n, kBandMaxCtas) : 0;
-    }();
-    return sms;
+    });
 }
 
 int band_count_for(const Geom &g, bool fields)
@@ -84,17 +85,21 @@ cudaError_t launch_sweep_band(const Geom &g, bool fields, int bands, unsigned lo
         LAT_BAND(kBandFields),  LAT_BAND(kBandPacked),  LAT_BAND(kBandPackedNe), LAT_BAND(kBandPotts3)};
 #undef LAT_BAND
 #undef LAT_VAR
-    static std::once_flag once;
-    static cudaError_t attr = cudaSuccess;
-    std::call_once(once, [] {
+    static PerDevice<cudaError_t> attrs;
+    int dev = 0;
+    cudaError_t attr = cudaGetDevice(&dev);
+    if (attr != cudaSuccess) return attr;
+    attr = attrs.get(dev, [] {
+        cudaError_t bad = cudaSuccess;
         for (const auto &kind : kern)
             for (const auto &ref : kind)
                 for (BandKernel f : ref) {
                     const cudaError_t e = f == nullptr ? cudaSuccess
                                                        : cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                                               (int)kBandMaxSmem);
-                    if (e != cudaSuccess) attr = e;
+                    if (e != cudaSuccess) bad = e;
                 }
+        return bad;
     });
     if (attr != cudaSuccess) return attr;
     if (band_test().launch()) return cudaErrorCooperativeLaunchTooLarge;

@@ -3,8 +3,8 @@
 // every lattice runs all its sweeps in the one cooperative launch.
 #include <algorithm>
 #include <cmath>
-#include <mutex>
 
+#include "band_host.h"
 #include "band_kinds.cuh"
 
 namespace lat {
@@ -125,12 +125,16 @@ cudaError_t launch_batch_band(const Geom *d_geoms, const std::vector<std::pair<c
                               const std::vector<unsigned long long> &sweep0, const std::vector<int *> &err,
                               int *err_all, const std::vector<int> &ctas, void *mail, unsigned epoch, cudaStream_t st)
 {
-    static std::once_flag once;
-    static cudaError_t attr = cudaSuccess;
-    std::call_once(once, [] {
+    static PerDevice<cudaError_t> attrs;
+    int dev = 0;
+    cudaError_t attr = cudaGetDevice(&dev);
+    if (attr != cudaSuccess) return attr;
+    attr = attrs.get(dev, [] {
+        cudaError_t bad = cudaSuccess;
         for (auto f : {k_band_batch<false>, k_band_batch<true>})
-            if (attr == cudaSuccess)
-                attr = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBandMaxSmem);
+            if (bad == cudaSuccess)
+                bad = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBandMaxSmem);
+        return bad;
     });
     if (attr != cudaSuccess) return attr;
     if (band_test().launch()) return cudaErrorCooperativeLaunchTooLarge;

@@ -65,3 +65,28 @@ int main()
     return 0;
 }
 """)
+
+
+# function attributes and SM counts belong to a device: found once for each, not once for all
+@pytest.mark.skipif(CXX is None, reason="no C++ compiler")
+def test_found_once_per_device(tmp_path):
+    _run(tmp_path, r"""
+#include <atomic>
+int main()
+{
+    PerDevice<int> v;
+    std::atomic<int> found[66] = {};
+    std::vector<std::thread> t;
+    for (int k = 0; k < 8; ++k)
+        t.emplace_back([&] {
+            for (int dev = 0; dev < 64; ++dev)
+                for (int rep = 0; rep < 3; ++rep)
+                    CHECK(v.get(dev, [&, dev] { ++found[dev]; return 100 + dev; }) == 100 + dev);
+        });
+    for (auto &x : t) x.join();
+    for (int dev = 0; dev < 64; ++dev) CHECK(found[dev] == 1);
+    CHECK(v.get(65, [&] { ++found[65]; return 5; }) == 5 && v.get(65, [&] { ++found[65]; return 6; }) == 6);
+    CHECK(v.get(-1, [] { return 3; }) == 3);
+    return 0;
+}
+""")
