@@ -111,7 +111,14 @@ enum lattice_kernel {
                                Calls of a few sweeps or more on 2D spin-1/2 and 3-state
                                Potts lattices that fit the SMs' shared memory run in
                                one cooperative launch instead (every SM holds a band of
-                               rows), unless lattice_set_kernel gave a graph size */
+                               rows), unless lattice_set_kernel gave a graph size.  Such a
+                               launch needs every SM at once, so it starts when other
+                               streams' kernels leave them: give a graph size to a
+                               lattice that shares the GPU with kernels that run for
+                               long.  Lattices on streams of their own use it while they
+                               do not meet; where small ones do, they go back to
+                               launches, which overlap, and none ever waits for work of
+                               another stream other than such launches of large lattices */
     LAT_KERNEL_RESIDENT = 4 /* one launch for many sweeps: one CTA holds the whole
                                lattice in shared memory; 2D spin-1/2 (Ising and
                                North-East), L % 32 == 0, L^2 (+ L^2/4 for North-East)

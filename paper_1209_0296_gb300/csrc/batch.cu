@@ -80,6 +80,7 @@ struct lattice_batch {
     void *d_mail = nullptr;
     size_t mail_cap = 0;
     unsigned mail_epoch = 0;
+    lat::BandShare band_share;
     int *band_err = nullptr;   // host-visible: a wait of a run gave up since the last synchronise
     // resident lattices
     cudaStream_t res_stream = nullptr;
@@ -402,9 +403,9 @@ void plan_bands(Work &work, std::vector<BandGroup> &groups, size_t at_least)
 
 // Launch the groups one after another on the batch stream; their `ran` says
 // what was queued: less than all when the bands are refused (no memory for the
-// packets, or fewer SMs than the device reports), and then the step loop takes
-// the rest.
-int run_bands(lattice_batch *b, BatchSlot &sl, size_t at, std::vector<BandGroup> &groups)
+// packets, fewer SMs than the device reports, another stream's band launch in
+// flight), and then the step loop takes the rest.
+int run_bands(lattice_batch *b, BatchSlot &sl, size_t at, std::vector<BandGroup> &groups, bool clear)
 {
     size_t n = 0, mail = 0;
     for (auto &g : groups) {
@@ -449,6 +450,8 @@ int run_bands(lattice_batch *b, BatchSlot &sl, size_t at, std::vector<BandGroup>
     stage(sl, at, sl.d_band_geoms, geoms.data(), n, b->stream, e);
     size_t first = 0;
     for (auto &g : groups) {
+        uint64_t sites = 0;
+        for (auto &pr : g.work) sites += pr.first->P.N;
         // launches of well under a second each: every lattice's sweeps in equal parts
         const int parts = (int)std::max(1.0, std::ceil(g.us / 2.5e5));
         for (int k = 0; k < parts && e == cudaSuccess; ++k) {
@@ -468,7 +471,8 @@ int run_bands(lattice_batch *b, BatchSlot &sl, size_t at, std::vector<BandGroup>
                 b->mail_epoch = 0;
             }
             if (e == cudaSuccess) {
-                BandTurn turn(b->stream);
+                BandTurn turn(b->stream, &b->band_share, sites, clear);
+                if (!turn.go) return LAT_OK;
                 e = turn.status;
                 if (e == cudaSuccess)
                     e = launch_batch_band(sl.d_band_geoms + first, l, sweep0, err, b->band_err, g.ctas, b->d_mail,
@@ -724,7 +728,11 @@ int lattice_batch_run(lattice_batch_t *b)
     // each distinct lattice stream (lattices often share one): an event
     // wait, so the host does not block.
     std::vector<cudaStream_t> streams;
+    bool clear = idle_stream(b->stream);   // the run waits for nothing queued before it
     for (auto &pr : work) {
+        clear = clear && (pr.first->stream == b->stream ||
+                          std::find(streams.begin(), streams.end(), pr.first->stream) != streams.end() ||
+                          idle_stream(pr.first->stream));
         int rc = ensure_series(pr.first, (unsigned long long)(pr.first->sweeps + pr.second));
         if (rc != LAT_OK) return rc;
         cudaStream_t ls = pr.first->stream;
@@ -764,14 +772,15 @@ int lattice_batch_run(lattice_batch_t *b)
     std::vector<BandGroup> groups;
     // (the launches carry the host's sweep numbers: not while the caller captures the stream)
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(b->stream, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone)
+    if (cudaStreamIsCapturing(b->stream, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone &&
+        band_may(b->stream, &b->band_share))
         plan_bands(work, groups, b->caller_orders ? 2 : 1);
     // the resident and band lattices' uploads sit at the front of the staging
     size_t res_bytes = res.empty() ? 0 : ((res.size() * (sizeof(Geom) + sizeof(long long)) + 64 + 15) & ~(size_t)15);
     std::vector<std::pair<lattice *, int64_t>> banded;
     if (!groups.empty()) {
         mark_start();
-        const int rc = run_bands(b, sl, res_bytes, groups);
+        const int rc = run_bands(b, sl, res_bytes, groups, clear);
         for (auto &g : groups)
             for (size_t i = 0; i < g.work.size(); ++i) {
                 lattice *lt = g.work[i].first;
@@ -930,6 +939,7 @@ void lattice_batch_destroy(lattice_batch_t *b)
     dev_free(b->d_counters, b->stream);
     dev_free(b->d_mail, b->stream);
     band_error_word_back(b->band_err, b->stream, false);
+    band_forget(&b->band_share);
     if (b->res_stream) cudaStreamDestroy(b->res_stream);
     if (b->ev_fork) cudaEventDestroy(b->ev_fork);
     if (b->ev_join) cudaEventDestroy(b->ev_join);

@@ -360,29 +360,106 @@ void band_error_word_back(int *w, cudaStream_t st, bool busy)
     error_words().give(w, ev);
 }
 
-// One event per device, recorded after every band launch.
-static std::mutex g_band_mu;
-static std::map<int, cudaEvent_t> g_band_last;
+// The last band launch on each device.
+namespace {
+struct BandLast {
+    cudaEvent_t ev = nullptr;        // recorded after it
+    unsigned long long stream = 0;   // cudaStreamGetId: a handle may be used again, an id is not
+    bool clear = false;
+    int depth = 0;                   // band launches of other streams it waits for
+    uint64_t sites = 0;
+    BandShare *owner = nullptr;
+};
+constexpr int kBandDevices = 64;
+std::mutex g_band_mu;
+BandLast g_band_last[kBandDevices];
 
-BandTurn::BandTurn(cudaStream_t st) : st_(st)
+// The last band launch of another stream than `id` is still queued or running.
+bool in_flight(const BandLast &l, unsigned long long id)
+{
+    if (l.ev == nullptr || l.stream == id) return false;
+    if (cudaEventQuery(l.ev) == cudaSuccess) return false;
+    (void)cudaGetLastError();
+    return true;
+}
+
+bool band_place(cudaStream_t st, int &dev, unsigned long long &id)
+{
+    if (cudaGetDevice(&dev) == cudaSuccess && dev < kBandDevices && cudaStreamGetId(st, &id) == cudaSuccess) return true;
+    (void)cudaGetLastError();
+    return false;
+}
+
+}  // namespace
+
+bool idle_stream(cudaStream_t st)
+{
+    unsigned flags = 0;
+    const bool idle = cudaStreamGetFlags(st, &flags) == cudaSuccess && (flags & cudaStreamNonBlocking) != 0u &&
+                      cudaStreamQuery(st) == cudaSuccess;
+    if (!idle) (void)cudaGetLastError();
+    return idle;
+}
+
+bool band_may(cudaStream_t st, BandShare *me)
+{
+    int dev = 0;
+    unsigned long long id = 0;
+    if (!band_place(st, dev, id)) return false;
+    std::lock_guard<std::mutex> g(g_band_mu);
+    if (me->yield == 0) return true;
+    --me->yield;
+    const BandLast &l = g_band_last[dev];
+    if (in_flight(l, id)) {
+        me->yield = kBandYield;
+        if (l.owner != nullptr) l.owner->yield = kBandYield;
+    }
+    return false;
+}
+
+void band_forget(BandShare *me)
+{
+    std::lock_guard<std::mutex> g(g_band_mu);
+    for (BandLast &l : g_band_last)
+        if (l.owner == me) l.owner = nullptr;
+}
+
+BandTurn::BandTurn(cudaStream_t st, BandShare *me, uint64_t sites, bool clear)
+    : st_(st), me_(me), clear_(clear), sites_(sites)
 {
     g_band_mu.lock();
-    int dev = 0;
-    status = cudaGetDevice(&dev);
-    auto it = g_band_last.find(dev);
-    if (status == cudaSuccess && it != g_band_last.end()) status = cudaStreamWaitEvent(st, it->second, 0);
+    if (!band_place(st, dev_, id_)) {
+        dev_ = -1;
+        return;
+    }
+    BandLast &l = g_band_last[dev_];
+    go = true;
+    if (in_flight(l, id_)) {
+        const uint64_t least = std::min(sites, l.sites);
+        if (l.clear && (least >= kBandLarge || (least >= kBandTwo && l.depth == 0))) {
+            status = cudaStreamWaitEvent(st, l.ev, 0);
+            depth_ = l.depth + 1;
+        } else {
+            go = false;
+            if (least < kBandLarge) {
+                me->yield = kBandYield;
+                if (l.owner != nullptr) l.owner->yield = kBandYield;
+            }
+        }
+    }
+    if (go && status == cudaSuccess && l.ev == nullptr) status = cudaEventCreateWithFlags(&l.ev, cudaEventDisableTiming);
 }
 
 BandTurn::~BandTurn()
 {
-    int dev = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess) {
-        auto it = g_band_last.find(dev);
-        if (it == g_band_last.end()) {
-            cudaEvent_t ev = nullptr;
-            if (cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) == cudaSuccess) it = g_band_last.emplace(dev, ev).first;
-        }
-        if (it != g_band_last.end()) cudaEventRecord(it->second, st_);
+    if (go && status == cudaSuccess) {
+        BandLast &l = g_band_last[dev_];
+        cudaEventRecord(l.ev, st_);
+        l.stream = id_;
+        l.clear = clear_;
+        l.depth = depth_;
+        l.sites = sites_;
+        l.owner = me_;
     }
     g_band_mu.unlock();
 }
@@ -420,7 +497,7 @@ static bool not_capturing(cudaStream_t st)
 // the wide kernel that fit the chip's shared memory, unless the caller chose
 // a graph size (which asks for launches) or is capturing the stream (the
 // launch carries the host's sweep number, so it cannot be replayed).
-static int band_bands(const lattice *lt, int64_t n)
+static int band_bands(lattice *lt, int64_t n)
 {
     if (n < band_min_sweeps(lt) || lt->graph_pinned || lt->dynamics != LAT_DYNAMICS_CHECKERBOARD) return 0;
     // (3-state Potts at sizes without a wide kernel too, unless the generic one was asked for)
@@ -429,13 +506,14 @@ static int band_bands(const lattice *lt, int64_t n)
         return 0;
     const int bands = band_count_for(lt->geom, lt->has_fields);
     if (bands == 0) return 0;
-    return not_capturing(lt->stream) ? bands : 0;
+    return not_capturing(lt->stream) && band_may(lt->stream, &lt->band_share) ? bands : 0;
 }
 
 // Queue n sweeps on the band-resident kernel (sets *done to the sweeps
-// queued, 0 when its packet buffer cannot be allocated: the launches take over).
-// Each launch is kept well under a second.
-static int band_sweeps(lattice *lt, int bands, int64_t n, int64_t *done)
+// queued, less than n when its packet buffer cannot be allocated or a launch
+// is refused: the launches take over).  clear: the stream was idle when the call
+// began.  Each launch is kept well under a second.
+static int band_sweeps(lattice *lt, int bands, int64_t n, bool clear, int64_t *done)
 {
     *done = 0;
     if (lt->band_err == nullptr && (lt->band_err = band_error_word()) == nullptr) return LAT_OK;
@@ -461,7 +539,8 @@ static int band_sweeps(lattice *lt, int bands, int64_t n, int64_t *done)
             lt->band_epoch = 0;
         }
         if (e == cudaSuccess) {
-            BandTurn turn(lt->stream);
+            BandTurn turn(lt->stream, &lt->band_share, lt->P.N, clear);
+            if (!turn.go) return LAT_OK;
             e = turn.status;
             if (e == cudaSuccess)
                 e = launch_sweep_band(lt->geom, lt->has_fields, bands, (unsigned long long)(lt->sweeps + *done), k,
@@ -698,7 +777,7 @@ int time_candidate(lattice *lt, int n, cudaEvent_t ev0, cudaEvent_t ev1, float &
         if (rep == 1 && cudaEventRecord(ev0, lt->stream) != cudaSuccess) rc = LAT_ECUDA;
         int64_t done = 0;
         if (rc == LAT_OK && bands > 0) {
-            rc = band_sweeps(lt, bands, n, &done);
+            rc = band_sweeps(lt, bands, n, false, &done);
             if (done < n) bands = 0;
             lt->sweeps += done;
             left -= done;
@@ -816,6 +895,7 @@ int sweep_impl(lattice *lt, int64_t n)
     if (n < 0) return LAT_EINVAL;
     if (n == 0) return LAT_OK;
     int rc = band_status(lt);
+    const bool clear = n >= band_min_sweeps(lt) && idle_stream(lt->stream);
     if (rc == LAT_OK) rc = ensure_series(lt, (unsigned long long)(lt->sweeps + n));
     if (rc != LAT_OK) return rc;
     int64_t left = n;
@@ -829,7 +909,7 @@ int sweep_impl(lattice *lt, int64_t n)
     }
     if (const int bands = band_bands(lt, left)) {
         int64_t done = 0;
-        rc = band_sweeps(lt, bands, left, &done);
+        rc = band_sweeps(lt, bands, left, clear, &done);
         lt->sweeps += done;
         if (rc != LAT_OK || done == left) return rc;
         left -= done;
@@ -878,6 +958,7 @@ static void release(lattice *lt)
     dev_free(lt->cpl, st);
     dev_free(lt->band_mail, st);
     band_error_word_back(lt->band_err, st, true);
+    band_forget(&lt->band_share);
     delete lt;
 }
 

@@ -35,16 +35,50 @@ void band_error_word_back(int *w, cudaStream_t st, bool busy);
 // Whether a bounded wait of an earlier launch gave up, as far as the host has
 // seen (after a synchronise: all of them).
 int band_status(const struct ::lattice *lt);
-// Order a band launch on st after the last one on any stream: two of them
-// must not wait for each other's SMs.  Holds a lock until destroyed.
+// Band launches of several streams.  A band launch takes every SM, so two of
+// them must not wait for each other's, and work that would have run beside it
+// waits.  A launch on one stream therefore never waits for another stream's
+// band launch that may itself wait for something (it is refused, and its
+// caller queues the two-launch sweeps, which run beside whatever there is); it
+// does wait where that one was queued on an idle stream of its own and both
+// lattices are large (or, less large, only two of them meet), which is sooner
+// done than their launches side by side.  Otherwise both owners leave the
+// bands alone for their next kBandYield calls: small lattices on streams of
+// their own overlap their launches.  Launches side by side and bands in turn,
+// ms: 16 x L = 256, 100 sweeps 1.0 and 3.7; 2 x L = 512 0.42 and 0.47; 2, 4, 8 x
+// L = 1000 0.76 and 0.52, 0.97 and 1.02, 1.45 and 2.02; 4 x L = 2048, 20 sweeps
+// 0.49 and 0.43.
+struct BandShare {
+    int yield = 0;   // calls that still do without bands
+};
+constexpr int kBandYield = 32;
+constexpr uint64_t kBandLarge = 2000000, kBandTwo = 800000;   // sites from which bands in turn win, for any number and for two
+// At the start of a call that could use bands on st: whether it may.
+bool band_may(cudaStream_t st, BandShare *me);
+// Whether work queued on st now would start when the GPU has room: st is idle,
+// and no other stream's work is implicitly ordered before it (as a blocking
+// stream's or the legacy stream's is).
+bool idle_stream(cudaStream_t st);
+// Before *me is freed.
+void band_forget(BandShare *me);
+
+// Held while one band launch is queued on st.
 class BandTurn {
 public:
-    explicit BandTurn(cudaStream_t st);
+    // clear: the launch waits for no other work than this call's and bands like it.
+    BandTurn(cudaStream_t st, BandShare *me, uint64_t sites, bool clear);
     ~BandTurn();
+    bool go = false;      // launch (else: refused)
     cudaError_t status = cudaSuccess;
 
 private:
     cudaStream_t st_;
+    BandShare *me_;
+    int dev_ = -1;
+    unsigned long long id_ = 0;
+    bool clear_;
+    int depth_ = 0;
+    uint64_t sites_;
 };
 int ensure_series(struct ::lattice *lt, unsigned long long need);
 bool tile_shape_ok(int tile_w, int tile_h);
@@ -103,4 +137,5 @@ struct lattice {
     size_t band_mail_cap = 0;            // its bytes: the kinds of a lattice's life differ (disorder set or dropped)
     unsigned band_epoch = 0;             // at least every packet mark sent so far
     int *band_err = nullptr;             // host-visible word: a bounded wait gave up
+    lat::BandShare band_share;
 };
