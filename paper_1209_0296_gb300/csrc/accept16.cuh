@@ -93,13 +93,14 @@ LAT_D void gen_thresholds2(const uint32_t (&acc)[8], const Nbr &n0, const Nbr &n
     }
 }
 
-// The exact rejections of one word from full 32-bit draws and the t' table.
-LAT_D uint32_t reject4_exact(const uint32_t *sthr, const Nbr &n, uint32_t S, const U4 &u)
+// The exact rejections of one word from full 32-bit draws and the t' table;
+// far: 0x40 at the sites whose entries are 16 on.
+LAT_D uint32_t reject4_exact(const uint32_t *sthr, const Nbr &n, uint32_t S, const U4 &u, uint32_t far = 0u)
 {
     const uint32_t b0 = n.s1 ^ n.R, b1 = n.c1 ^ (n.s1 & n.R), b2 = n.c1 & n.s1 & n.R;
-    const uint32_t idx = ((b0 & 0x04040404u) | (b1 & 0x08080808u) | (b2 & 0x10101010u) | (S & 0x20202020u)) >> 2;
-    return (u.x > sthr[idx & 0xFu] ? 0xFFu : 0u) | (u.y > sthr[(idx >> 8) & 0xFu] ? 0xFF00u : 0u) |
-           (u.z > sthr[(idx >> 16) & 0xFu] ? 0xFF0000u : 0u) | (u.w > sthr[(idx >> 24) & 0xFu] ? 0xFF000000u : 0u);
+    const uint32_t idx = ((b0 & 0x04040404u) | (b1 & 0x08080808u) | (b2 & 0x10101010u) | (S & 0x20202020u) | far) >> 2;
+    return (u.x > sthr[idx & 0x1Fu] ? 0xFFu : 0u) | (u.y > sthr[(idx >> 8) & 0x1Fu] ? 0xFF00u : 0u) |
+           (u.z > sthr[(idx >> 16) & 0x1Fu] ? 0xFF0000u : 0u) | (u.w > sthr[idx >> 24] ? 0xFF000000u : 0u);
 }
 
 // Top halves of a Philox call's four words, in pairs.

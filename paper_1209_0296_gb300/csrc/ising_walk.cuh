@@ -10,6 +10,8 @@
 // done again exactly, from memory, after the walk (one chunk in 2700).
 #pragma once
 
+#include <type_traits>
+
 #include "accept16.cuh"
 #include "wide_common.cuh"
 
@@ -59,8 +61,9 @@ struct IsingChunk {
     uint32_t St[4];   // the spins as the table sees them
 };
 
-// C: the chunk's disorder bytes; odd: x = 2j + 1 in this row.
-template <int kDis>
+// C: the chunk's disorder bytes; odd: x = 2j + 1 in this row.  kFold: field
+// signs go into the neighbours and spins (else into the table index).
+template <int kDis, bool kFold = true>
 LAT_D void ising_neighbours(IsingChunk &c, const uint32_t (&C)[4], bool odd)
 {
     if constexpr (kDis != kUniform) {
@@ -80,10 +83,10 @@ LAT_D void ising_neighbours(IsingChunk &c, const uint32_t (&C)[4], bool odd)
     for (int w = 0; w < 4; ++w) {
         c.n[w] = nbr_sum(c.U[w], c.D[w], c.O[w], c.X[w]);
         c.St[w] = c.S[w];
-        if constexpr (kDis == kFields) {
+        if constexpr (kDis == kFields) c.E[w] = ((C[w] >> 6) & 0x01010101u) * 0xFEu;
+        if constexpr (kDis == kFields && kFold) {
             // eta_i = -1: the move has the energy of the flipped spin among
             // flipped neighbours at eta_i = +1 (sum and carry are self-dual)
-            c.E[w] = ((C[w] >> 6) & 0x01010101u) * 0xFEu;
             c.n[w].s1 ^= c.E[w];
             c.n[w].c1 ^= c.E[w];
             c.n[w].R ^= c.E[w];
@@ -161,9 +164,37 @@ __device__ __noinline__ Counts ising_redo(const IsingPlanes<kColour> p, const ui
     return cnt;
 }
 
+template <bool kTop>
 struct IsingDraws {
     uint32_t p01[4], p23[4];   // top halves of the chunk's draws
 };
+template <>
+struct IsingDraws<false> {
+    U4 u[4];
+};
+
+// The table of ising_flips: the t' table, and with field signs a second half
+// for eta_i = -1 (the energy of the flipped spin among flipped neighbours).
+template <int kDis>
+LAT_D void ising_table(const uint32_t *thr16, uint32_t *sthr)
+{
+    const uint32_t i = threadIdx.x;
+    if (i < 16u) sthr[i] = thr16[i];
+    if constexpr (kDis == kFields)
+        if (i >= 16u && i < 32u && (i & 7u) <= 4u) sthr[i] = thr16[((i & 8u) ^ 8u) | (4u - (i & 7u))];
+}
+
+// 0xFE at the chunk's flipped sites, from full 32-bit draws.
+template <int kDis>
+LAT_D void ising_flips(const IsingChunk &c, const uint32_t *sthr, const U4 (&u)[4], uint32_t (&F)[4])
+{
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+        uint32_t far = 0;   // bit 6 of a byte: the second half
+        if constexpr (kDis == kFields) far = c.E[w] & 0x40404040u;
+        F[w] = ~reject4_exact(sthr, c.n[w], c.St[w], u[w], far) & 0xFEFEFEFEu;
+    }
+}
 
 // Rows [y, y1), y < y1, of chunk column k.
 template <int kColour, bool kRef, int kDis, bool kSym, bool kAligned>
@@ -178,7 +209,7 @@ LAT_D void ising_walk(const IsingPlanes<kColour> &p, const uint32_t (&acc)[8], c
     uint32_t R[4][4];   // rows of the other plane, row y - 1 + i in R[(s + i) & 3] at step s
     Row16<kAligned> nS, nD;
     uint32_t nC[4] = {0, 0, 0, 0}, nb_next;
-    IsingDraws draws[2];
+    IsingDraws<kSym> draws[2];
     auto other_row = [&](uint32_t r) { return p.pO + (size_t)r * p.half + cc.j0; };
     auto fetch = [&](uint32_t r) {   // row r's own sites and neighbour byte, row r + 1 of the other plane
         const size_t at = (size_t)r * p.half;
@@ -187,11 +218,14 @@ LAT_D void ising_walk(const IsingPlanes<kColour> &p, const uint32_t (&acc)[8], c
         nb_next = (uint32_t)(uint8_t)p.pO[at + (((kColour + r) & 1u) ? cc.jn : cc.jp)];
         if constexpr (kDis != kUniform) load_words<4>(p.pC + at + cc.j0, nC);
     };
-    auto draw = [&](uint32_t r, IsingDraws &d) {
+    auto draw = [&](uint32_t r, IsingDraws<kSym> &d) {
         const uint32_t g0 = r * p.G + 4u * k;
 #pragma unroll
-        for (int w = 0; w < 4; ++w)
-            top_halves(philox_item(pp, g0 + (uint32_t)w, (uint32_t)kColour), d.p01[w], d.p23[w]);
+        for (int w = 0; w < 4; ++w) {
+            const U4 u = philox_item(pp, g0 + (uint32_t)w, (uint32_t)kColour);
+            if constexpr (kSym) top_halves(u, d.p01[w], d.p23[w]);
+            else d.u[w] = u;
+        }
     };
     {
         Row16<kAligned> a, b;
@@ -204,68 +238,74 @@ LAT_D void ising_walk(const IsingPlanes<kColour> &p, const uint32_t (&acc)[8], c
         row_words<kAligned>(qb, b, R[1]);
     }
     uint32_t redo = 0, first = y;   // undecided rows first + i
-    for (bool more = true; more;) {
+    // Row y at step s of four (a constant, so that R and draws stay in registers); whether there is another.
+    auto row = [&](auto which) {
+        constexpr int s = decltype(which)::value;
+        const uint32_t at = y * p.half + cc.j0;
+        const bool odd = ((kColour + y) & 1u) != 0u, more = y + 1u < y1;
+        IsingChunk c;
+        uint32_t C[4];
+        row_words<kAligned>(p.pS + at, nS, c.S);
+        row_words<kAligned>(other_row(y + 1u == p.L ? 0u : y + 1u), nD, R[(s + 2) & 3]);
+        shifted_row<kAligned>(cc, odd, nb_next, R[(s + 1) & 3], c.X);
 #pragma unroll
-        for (int s = 0; s < 4; ++s) {
-            const uint32_t at = y * p.half + cc.j0;
-            const bool odd = ((kColour + y) & 1u) != 0u;
-            IsingChunk c;
-            uint32_t C[4];
-            row_words<kAligned>(p.pS + at, nS, c.S);
-            row_words<kAligned>(other_row(y + 1u == p.L ? 0u : y + 1u), nD, R[(s + 2) & 3]);
-            shifted_row<kAligned>(cc, odd, nb_next, R[(s + 1) & 3], c.X);
+        for (int w = 0; w < 4; ++w) {
+            c.U[w] = R[s][w];
+            c.O[w] = R[(s + 1) & 3][w];
+            c.D[w] = R[(s + 2) & 3][w];
+            C[w] = nC[w];
+        }
+        auto step = [&]() {
+            ising_neighbours<kDis, false>(c, C, odd);
+            uint32_t F[4], Sn[4];
+            bool tie = false;
+            if constexpr (kSym) tie = flips16<true>(acc, c.n, c.St, draws[s & 1].p01, draws[s & 1].p23, F);
+            else ising_flips<kDis>(c, sthr, draws[s & 1].u, F);
 #pragma unroll
-            for (int w = 0; w < 4; ++w) {
-                c.U[w] = R[s][w];
-                c.O[w] = R[(s + 1) & 3][w];
-                c.D[w] = R[(s + 2) & 3][w];
-                C[w] = nC[w];
-            }
-            more = y + 1u < y1;
-            auto step = [&]() {
-                ising_neighbours<kDis>(c, C, odd);
-                uint32_t F[4], Sn[4];
-                const bool tie = flips16<kSym>(acc, c.n, c.St, draws[s & 1].p01, draws[s & 1].p23, F);
+            for (int w = 0; w < 4; ++w) Sn[w] = c.S[w] ^ F[w];
+            store16_any<kAligned>(p.dS + at, cc.nv, Sn);
+            ising_count<kColour, kDis, kAligned>(c, Sn, cc.vm, cnt);
+            if constexpr (kColour == 1) {
 #pragma unroll
-                for (int w = 0; w < 4; ++w) Sn[w] = c.S[w] ^ F[w];
-                store16_any<kAligned>(p.dS + at, cc.nv, Sn);
-                ising_count<kColour, kDis, kAligned>(c, Sn, cc.vm, cnt);
-                if constexpr (kColour == 1) {
+                for (int w = 0; w < 4; ++w) cnt.mag = dot4(R[(s + 1) & 3][w], 0x01010101u & cc.vm[w], cnt.mag);
+                if constexpr (kRef) {
+                    uint32_t R1[4], R0[4];
+                    load16_any<kAligned>(p.r1 + at, cc.nv, R1);
+                    load16_any<kAligned>(p.r0 + at, cc.nv, R0);
 #pragma unroll
                     for (int w = 0; w < 4; ++w)
-                        cnt.mag = dot4(R[(s + 1) & 3][w], 0x01010101u & cc.vm[w], cnt.mag);
-                    if constexpr (kRef) {
-                        uint32_t R1[4], R0[4];
-                        load16_any<kAligned>(p.r1 + at, cc.nv, R1);
-                        load16_any<kAligned>(p.r0 + at, cc.nv, R0);
-#pragma unroll
-                        for (int w = 0; w < 4; ++w)
-                            cnt.acf = dot4(Sn[w] & cc.vm[w], R1[w],
-                                           dot4(R[(s + 1) & 3][w] & cc.vm[w], R0[w], cnt.acf));
-                    }
+                        cnt.acf = dot4(Sn[w] & cc.vm[w], R1[w], dot4(R[(s + 1) & 3][w] & cc.vm[w], R0[w], cnt.acf));
                 }
-                if (tie) redo |= 1u << (y - first);
-            };
-            if (!more) {
-                step();
-                break;
             }
+            if (tie) redo |= 1u << (y - first);
+        };
+        if (more) {   // the next row's loads and draws in the same block
             fetch(y + 1u);
             draw(y + 1u, draws[(s + 1) & 1]);
             step();
             ++y;
+        } else {
+            step();
         }
-        if (!more || y - first >= 28u) {
-            while (redo != 0u) {
-                const uint32_t i = (uint32_t)__ffs((int)redo) - 1u;
-                redo &= redo - 1u;
-                const Counts d = ising_redo<kColour, kRef, kDis, kAligned>(p, sthr, sweep, key0, key1, k, first + i);
-                cnt.bond += d.bond;
-                cnt.mag += d.mag;
-                cnt.fld += d.fld;
-                cnt.acf += d.acf;
+        return more;
+    };
+    for (bool more = true; more;) {
+        more = row(std::integral_constant<int, 0>()) && row(std::integral_constant<int, 1>()) &&
+               row(std::integral_constant<int, 2>()) && row(std::integral_constant<int, 3>());
+        if constexpr (kSym) {
+            if (!more || y - first >= 28u) {
+                while (redo != 0u) {
+                    const uint32_t i = (uint32_t)__ffs((int)redo) - 1u;
+                    redo &= redo - 1u;
+                    const Counts d =
+                        ising_redo<kColour, kRef, kDis, kAligned>(p, sthr, sweep, key0, key1, k, first + i);
+                    cnt.bond += d.bond;
+                    cnt.mag += d.mag;
+                    cnt.fld += d.fld;
+                    cnt.acf += d.acf;
+                }
+                first = y;
             }
-            first = y;
         }
     }
     if constexpr (kColour == 1) cnt.up += (cnt.mag + 2 * (int)(cc.nv * rows)) / 2;
@@ -273,9 +313,8 @@ LAT_D void ising_walk(const IsingPlanes<kColour> &p, const uint32_t (&acc)[8], c
 
 // Row y's chunk of column k alone (lattices with little more than one chunk
 // a thread).
-template <int kColour, bool kRef, int kDis, bool kSym, bool kAligned>
-LAT_D void ising_one(const IsingPlanes<kColour> &p, const uint32_t (&acc)[8], const uint32_t *sthr,
-                     unsigned long long sweep, uint32_t key0, uint32_t key1, uint32_t k, uint32_t y, Counts &cnt)
+template <int kColour, bool kRef, int kDis, bool kAligned>
+LAT_D void ising_one(const IsingPlanes<kColour> &p, const uint32_t *sthr, unsigned long long sweep, uint32_t key0, uint32_t key1, uint32_t k, uint32_t y, Counts &cnt)
 {
     const ChunkCol<kAligned> cc = chunk_col<kAligned>(k, p.half);
     const size_t at = (size_t)y * p.half + cc.j0;
@@ -288,19 +327,24 @@ LAT_D void ising_one(const IsingPlanes<kColour> &p, const uint32_t (&acc)[8], co
     load16_any<kAligned>(p.pO + (size_t)(y + 1u == p.L ? 0u : y + 1u) * p.half + cc.j0, cc.nv, c.D);
     const uint32_t nb = (uint32_t)(uint8_t)p.pO[(size_t)y * p.half + (odd ? cc.jn : cc.jp)];
     if constexpr (kDis != kUniform) load_words<4>(p.pC + at, C);
-    IsingDraws d;
+    [[maybe_unused]] uint32_t R1[4], R0[4];
+    if constexpr (kColour == 1 && kRef) {
+        load16_any<kAligned>(p.r1 + at, cc.nv, R1);
+        load16_any<kAligned>(p.r0 + at, cc.nv, R0);
+    }
+    U4 u[4];
     {   // while the loads are on their way
         PhiloxPre pp;
         philox_prepare(pp, (uint32_t)sweep, (uint32_t)(sweep >> 32), key0, key1);
 #pragma unroll
         for (int w = 0; w < 4; ++w)
-            top_halves(philox_item(pp, y * p.G + 4u * k + (uint32_t)w, (uint32_t)kColour), d.p01[w], d.p23[w]);
+            u[w] = philox_item(pp, y * p.G + 4u * k + (uint32_t)w, (uint32_t)kColour);
     }
     shifted_row<kAligned>(cc, odd, nb, O, c.X);
 #pragma unroll
     for (int w = 0; w < 4; ++w) c.O[w] = O[w];
-    ising_neighbours<kDis>(c, C, odd);
-    const bool tie = flips16<kSym>(acc, c.n, c.St, d.p01, d.p23, F);
+    ising_neighbours<kDis, false>(c, C, odd);
+    ising_flips<kDis>(c, sthr, u, F);
 #pragma unroll
     for (int w = 0; w < 4; ++w) Sn[w] = c.S[w] ^ F[w];
     store16_any<kAligned>(p.dS + at, cc.nv, Sn);
@@ -309,20 +353,10 @@ LAT_D void ising_one(const IsingPlanes<kColour> &p, const uint32_t (&acc)[8], co
 #pragma unroll
         for (int w = 0; w < 4; ++w) cnt.mag = dot4(O[w], 0x01010101u & cc.vm[w], cnt.mag);
         if constexpr (kRef) {
-            uint32_t R1[4], R0[4];
-            load16_any<kAligned>(p.r1 + at, cc.nv, R1);
-            load16_any<kAligned>(p.r0 + at, cc.nv, R0);
 #pragma unroll
             for (int w = 0; w < 4; ++w)
                 cnt.acf = dot4(Sn[w] & cc.vm[w], R1[w], dot4(O[w] & cc.vm[w], R0[w], cnt.acf));
         }
-    }
-    if (tie) {
-        const Counts r = ising_redo<kColour, kRef, kDis, kAligned>(p, sthr, sweep, key0, key1, k, y);
-        cnt.bond += r.bond;
-        cnt.mag += r.mag;
-        cnt.fld += r.fld;
-        cnt.acf += r.acf;
     }
     if constexpr (kColour == 1) cnt.up += (cnt.mag + 2 * (int)cc.nv) / 2;
 }

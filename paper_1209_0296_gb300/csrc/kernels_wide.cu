@@ -240,11 +240,11 @@ constexpr int kWalkMinB = 2;   // (3, with fewer registers: 24 us a sweep at L =
 // each); else a thread per (chunk column, band of consecutive rows), in one
 // wave of at least cpr threads.
 template <int kColour, bool kRef, int kDis, bool kSym, bool kAligned, bool kOne>
-__global__ void __launch_bounds__(kThreads, kWalkMinB) k_ising_walk(Geom g, SweepAt at)
+__global__ void __launch_bounds__(kThreads, kOne && kAligned && kDis != kFields ? 4 : kWalkMinB) k_ising_walk(Geom g, SweepAt at)
 {
-    __shared__ uint32_t sthr[16];
+    __shared__ uint32_t sthr[kDis == kFields ? 32 : 16];
     __shared__ int red[kThreads / 32][5];
-    if (threadIdx.x < 16) sthr[threadIdx.x] = g.thr16[threadIdx.x];
+    ising_table<kDis>(g.thr16, sthr);
     __syncthreads();
     dep_wait();
     const unsigned long long sweep = sweep_of(g.ctrl, at);
@@ -257,11 +257,10 @@ __global__ void __launch_bounds__(kThreads, kWalkMinB) k_ising_walk(Geom g, Swee
     if (band < nb) {
         const IsingPlanes<kColour> p = ising_planes<kColour>(v, sweep);
         if constexpr (kOne) {
-            ising_one<kColour, kRef, kDis, kSym, kAligned>(p, g.acc, sthr, sweep, g.key0, g.key1, gt - band * cpr,
-                                                           band, cnt);
+            ising_one<kColour, kRef, kDis, kAligned>(p, sthr, sweep, g.key0, g.key1, gt - band * cpr, band, cnt);
         } else {
             uint32_t y, y1;
-            band_rows(band, nb, L, y, y1);
+            walk_rows(band, nb, L, y, y1);
             ising_walk<kColour, kRef, kDis, kSym, kAligned>(p, g.acc, sthr, sweep, g.key0, g.key1, gt - band * cpr, y,
                                                             y1, cnt);
         }
@@ -1311,33 +1310,33 @@ cudaError_t launch_sweep_wide(const Geom &g, bool fields, SweepAt at, cudaStream
         cudaError_t e = launch_pdl(ne[al][ref][0], grid, kThreads, st, k, at.off);
         return e == cudaSuccess ? launch_pdl(ne[al][ref][1], grid, kThreads, st, k, at.off) : e;
     }
-    // kinds: uniform at any even L with a general or a symmetric table; then
-    // L % 32 == 0: the same, bonds with either table, fields
     using K = void (*)(Geom, SweepAt);
-#define LAT_WALK(ref, dis, sym, al, one) {k_ising_walk<0, ref, dis, sym, al, one>, k_ising_walk<1, ref, dis, sym, al, one>}
-#define LAT_KIND(dis, sym, al)                                                              \
-    {{LAT_WALK(false, dis, sym, al, false), LAT_WALK(true, dis, sym, al, false)},           \
-     {LAT_WALK(false, dis, sym, al, true), LAT_WALK(true, dis, sym, al, true)}}
-    static const K is[7][2][2][2] = {LAT_KIND(kUniform, false, false), LAT_KIND(kUniform, true, false),
-                                     LAT_KIND(kUniform, false, true),  LAT_KIND(kUniform, true, true),
-                                     LAT_KIND(kBonds, false, true),    LAT_KIND(kBonds, true, true),
-                                     LAT_KIND(kFields, false, true)};
-#undef LAT_KIND
+#define LAT_WALK(dis, sym, al, one)                                                          \
+    {{k_ising_walk<0, false, dis, sym, al, one>, k_ising_walk<1, false, dis, sym, al, one>}, \
+     {k_ising_walk<0, true, dis, sym, al, one>, k_ising_walk<1, true, dis, sym, al, one>}}
+    // [uniform at any even L, then L % 32 == 0: uniform, bonds, fields][reference][colour]
+    static const K one[4][2][2] = {LAT_WALK(kUniform, false, false, true), LAT_WALK(kUniform, false, true, true),
+                                   LAT_WALK(kBonds, false, true, true), LAT_WALK(kFields, false, true, true)};
+    static const K walk[4][2][2] = {LAT_WALK(kUniform, false, false, false), LAT_WALK(kUniform, false, true, false),
+                                    LAT_WALK(kBonds, false, true, false), LAT_WALK(kFields, false, true, false)};
+    static const K top[3][2][2] = {LAT_WALK(kUniform, true, false, false), LAT_WALK(kUniform, true, true, false),
+                                   LAT_WALK(kBonds, true, true, false)};
 #undef LAT_WALK
-    static const unsigned wave = one_wave(reinterpret_cast<const void *>(is[3][0][0][1]));   // all: kWalkMinB per SM
-    const int sym = k.acc_sym ? 1 : 0;
-    const int m = g.cpl != nullptr ? (fields ? 6 : 4 + sym) : 2 * al + sym;
-    // one chunk a thread up to two waves of them: up to there the row walk's
-    // start-up costs more than its register reuse saves
-    const int one = blocks <= 2u * wave ? 1 : 0;
-    const unsigned grid = one ? (unsigned)blocks : wave;
-    cudaError_t e = launch_pdl(is[m][one][ref][0], grid, kThreads, st, k, at);
-    return e == cudaSuccess ? launch_pdl(is[m][one][ref][1], grid, kThreads, st, k, at) : e;
+    static const unsigned wave = one_wave(reinterpret_cast<const void *>(walk[1][0][1]));   // all: kWalkMinB per SM
+    const int m = g.cpl != nullptr ? (fields ? 3 : 2) : al;
+    // One chunk a thread up to two waves of them: up to there the row walk's
+    // start-up costs more than its register reuse saves.  The 16-bit
+    // acceptance of symmetric tables from 10 rows a thread on: its rows to be
+    // done again are a chain of memory trips at the end of every thread's walk
+    // (launches of a graph, 16-bit and look-ups: L = 3000, 3 rows, 20.0 and
+    // 17.6 us a sweep; 4096, 7 rows, 20.5 and 19.9; 6000, 15 rows, 55.0 and
+    // 56.2; 8192, 27 rows, 67.4 and 70.6).
+    const bool many = blocks > 2u * wave, sym = k.acc_sym != 0 && blocks >= 10u * wave;
+    const K *kern = !many ? one[m][ref] : (sym ? top[m][ref] : walk[m][ref]);
+    const unsigned grid = many ? wave : (unsigned)blocks;
+    cudaError_t e = launch_pdl(kern[0], grid, kThreads, st, k, at);
+    return e == cudaSuccess ? launch_pdl(kern[1], grid, kThreads, st, k, at) : e;
 }
-
-}  // namespace lat
-
-namespace lat {
 
 bool resident_supported(const Geom &g)
 {
@@ -1388,10 +1387,5 @@ cudaError_t launch_batch_resident(const Geom *geoms, const long long *n, int n_l
 }
 
 size_t resident_smem_bytes(const Geom &g) { return resident_bytes(g); }
-
-}  // namespace lat
-
-namespace lat {
-
 
 }  // namespace lat

@@ -109,6 +109,16 @@ LAT_D void band_rows(uint32_t b, uint32_t nb, uint32_t L, uint32_t &y0, uint32_t
     y1 = (uint32_t)((uint64_t)(b + 1u) * L / nb);
 }
 
+// The same for the threads of a streaming launch: the long bands come first.
+// (In turn with the short ones every warp takes the longer time: L = 2400, two
+// rows or three, 10.7 us a sweep for 9.2.)
+LAT_D void walk_rows(uint32_t b, uint32_t nb, uint32_t L, uint32_t &y0, uint32_t &y1)
+{
+    const uint32_t q = L / nb, r = L - q * nb;
+    y0 = b * q + min(b, r);
+    y1 = y0 + q + (b < r ? 1u : 0u);
+}
+
 // Bytes p[0 .. nv) (1 <= nv <= 16) as four words, byte b = p[b], the bytes
 // from nv on unspecified; an aligned word that holds none of them is not
 // read (the spin buffers are multiples of 4 bytes, so every word read is in
