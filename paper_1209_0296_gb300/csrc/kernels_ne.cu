@@ -68,7 +68,7 @@ LAT_D void ne_walk(const NeRows<kColour> &p, const PhiloxPre &pp, const NeRate r
     const int lane = threadIdx.x & 31;
     const unsigned below = (1u << lane) - 1u;
     const ChunkCol<kAligned> cc = chunk_col<kAligned>(k, p.half);
-    const NePlanes where{reinterpret_cast<uint8_t *>(p.dS), p.fl, p.r1, 0u, p.half, p.half};
+    const NePlanes where{reinterpret_cast<uint8_t *>(p.dS), p.fl, p.r1};
     int sites = 0;
     unsigned queued = 0;   // warp-uniform
     uint32_t R[4][4];      // rows of the other plane, row y - 1 + i in R[(s + i) & 3] at step s
@@ -95,11 +95,11 @@ LAT_D void ne_walk(const NeRows<kColour> &p, const PhiloxPre &pp, const NeRate r
         while (queued >= 32u) {
             queued -= 32u;
             const NeJob j = queue[queued + lane];
-            ne_job<kRef>(where, pp, rate, j, (uint32_t)kColour, cnt, j.g);
+            ne_job<kRef>(where, pp, rate, j, (uint32_t)kColour, cnt);
         }
         if (all && (unsigned)lane < queued) {
             const NeJob j = queue[lane];
-            ne_job<kRef>(where, pp, rate, j, (uint32_t)kColour, cnt, j.g);
+            ne_job<kRef>(where, pp, rate, j, (uint32_t)kColour, cnt);
         }
         __syncwarp();
     };
@@ -143,22 +143,9 @@ LAT_D void ne_walk(const NeRows<kColour> &p, const PhiloxPre &pp, const NeRate r
                 if (((sure[0] | sure[1] | sure[2] | sure[3]) & kB1) != 0u) {
                     const uint32_t chg = ne_changed(sure);
                     uint8_t *fp = p.fl + (size_t)y * p.G + 4u * k;
-                    if constexpr (kAligned) {
-                        uint32_t *f4 = reinterpret_cast<uint32_t *>(fp);
-                        const uint32_t was = *f4;
-                        *f4 = was | chg;
-                        cnt.unfl -= __popc(chg & ~was);
-                    } else {
-#pragma unroll
-                        for (int w = 0; w < 4; ++w) {
-                            const uint32_t b = (chg >> (8 * w)) & 0xFFu;
-                            if (b != 0u) {   // only groups that exist have valid sites
-                                const uint32_t was = fp[w];
-                                fp[w] = (uint8_t)(was | b);
-                                cnt.unfl -= __popc(b & ~was);
-                            }
-                        }
-                    }
+                    const uint32_t was = ne_flags<kAligned>(fp, cc.nv);
+                    cnt.unfl -= __popc(chg & ~was);
+                    ne_set_flags<kAligned>(fp, was, was | chg);
                 }
             }
             const uint32_t g0 = y * p.G + 4u * k;
@@ -181,73 +168,59 @@ LAT_D void ne_walk(const NeRows<kColour> &p, const PhiloxPre &pp, const NeRate r
 }
 
 // The chunk of row y and column k alone (lattices with no more chunks than
-// threads: nothing to keep in registers from row to row).
+// threads: nothing to keep in registers from row to row).  Such a pass is as
+// long as its chain of memory trips, so everything it reads is asked for at
+// once, and the thread draws for its own groups, all four, while that is on
+// its way.  (L = 1024, c = 0.3, launches of a graph: 5.0 us a sweep; with
+// persistence bits read once a move is known and the draws queued, 7.4.)
 template <int kColour, bool kRef, bool kAligned>
-LAT_D void ne_one(const NeRows<kColour> &p, const PhiloxPre &pp, const NeRate rate, uint32_t k, uint32_t y, bool act,
-                  NeJob *queue, Counts &cnt)
+LAT_D void ne_one(const NeRows<kColour> &p, const PhiloxPre &pp, const NeRate rate, uint32_t k, uint32_t y, Counts &cnt)
 {
-    const int lane = threadIdx.x & 31;
     const ChunkCol<kAligned> cc = chunk_col<kAligned>(k, p.half);
     const uint32_t at0 = y * p.half + cc.j0, g0 = y * p.G + 4u * k;
-    uint32_t cand[4], ws[4];
-    bool need[4] = {false, false, false, false};
-    int sites = 0;
-    if (act) {
-        auto other = [&](uint32_t r) { return p.pO + (size_t)r * p.half + cc.j0; };
-        const bool odd = ((kColour + y) & 1u) != 0u;
-        uint32_t U[4], O[4], D[4], S[4], X[4], E[4], W[4], Sn[4], sure[4];
-        load16_any<kAligned>(other(y == 0u ? p.L - 1u : y - 1u), cc.nv, U);
-        load16_any<kAligned>(other(y), cc.nv, O);
-        load16_any<kAligned>(other(y + 1u == p.L ? 0u : y + 1u), cc.nv, D);
-        load16_any<kAligned>(p.pS + (size_t)at0, cc.nv, S);
-        shifted_row<kAligned>(cc, odd, (uint32_t)(uint8_t)p.pO[(size_t)y * p.half + (odd ? cc.jn : cc.jp)], O, X);
-#pragma unroll
-        for (int w = 0; w < 4; ++w) {
-            E[w] = odd ? X[w] : O[w];
-            W[w] = odd ? O[w] : X[w];
-        }
-        ne_moves<kAligned>(U, D, E, W, S, cc.vm, rate, cand, sure, ws, Sn, need);
-        store16_any<kAligned>(p.dS + (size_t)at0, cc.nv, Sn);
-        const uint32_t chg = ne_changed(sure);
-        uint8_t *fp = p.fl + (size_t)y * p.G + 4u * k;
-#pragma unroll
-        for (int w = 0; w < 4; ++w) {
-            const uint32_t b = (chg >> (8 * w)) & 0xFFu;
-            if (b != 0u) {   // only groups that exist have valid sites
-                const uint32_t was = fp[w];
-                fp[w] = (uint8_t)(was | b);
-                cnt.unfl -= __popc(b & ~was);
-            }
-        }
-        if constexpr (kColour == 1) {
-            ne_count(Sn, U, D, O, X, cc.vm, cnt);
-            sites = 2 * (int)cc.nv;
-            if constexpr (kRef) {
-                uint32_t R1[4], R0[4];
-                load16_any<kAligned>(p.r1 + (size_t)at0, cc.nv, R1);
-                load16_any<kAligned>(p.r0 + (size_t)at0, cc.nv, R0);
-#pragma unroll
-                for (int w = 0; w < 4; ++w)
-                    cnt.acf = dot4(Sn[w] & cc.vm[w], R1[w], dot4(O[w] & cc.vm[w], R0[w], cnt.acf));
-            }
-        }
+    auto other = [&](uint32_t r) { return p.pO + (size_t)r * p.half + cc.j0; };
+    const bool odd = ((kColour + y) & 1u) != 0u;
+    uint32_t U[4], O[4], D[4], S[4], X[4], E[4], W[4], Sn[4], cand[4], moved[4], ws[4], rej[4];
+    bool need[4];
+    uint8_t *fp = p.fl + g0;
+    load16_any<kAligned>(other(y == 0u ? p.L - 1u : y - 1u), cc.nv, U);
+    load16_any<kAligned>(other(y), cc.nv, O);
+    load16_any<kAligned>(other(y + 1u == p.L ? 0u : y + 1u), cc.nv, D);
+    load16_any<kAligned>(p.pS + (size_t)at0, cc.nv, S);
+    const uint32_t nb = (uint32_t)(uint8_t)p.pO[(size_t)y * p.half + (odd ? cc.jn : cc.jp)];
+    [[maybe_unused]] uint32_t R1[4], R0[4];
+    if constexpr (kColour == 1 && kRef) {
+        load16_any<kAligned>(p.r1 + (size_t)at0, cc.nv, R1);
+        load16_any<kAligned>(p.r0 + (size_t)at0, cc.nv, R0);
     }
-    unsigned queued = 0;
+    const uint32_t was = ne_flags<kAligned>(fp, cc.nv);
+#pragma unroll
+    for (int w = 0; w < 4; ++w) rej[w] = ne_rejected(philox_item(pp, g0 + (uint32_t)w, (uint32_t)kColour), rate.K);
+    shifted_row<kAligned>(cc, odd, nb, O, X);
 #pragma unroll
     for (int w = 0; w < 4; ++w) {
-        const unsigned bal = __ballot_sync(0xffffffffu, need[w]);
-        if (need[w])
-            queue[queued + __popc(bal & ((1u << lane) - 1u))] =
-                NeJob{g0 + (uint32_t)w, at0 + 4u * (uint32_t)w, cand[w], ws[w]};
-        queued += __popc(bal);
+        E[w] = odd ? X[w] : O[w];
+        W[w] = odd ? O[w] : X[w];
     }
-    __syncwarp();
-    const NePlanes where{reinterpret_cast<uint8_t *>(p.dS), p.fl, p.r1, 0u, p.half, p.half};
-    for (unsigned i = (unsigned)lane; i < queued; i += 32u) {
-        const NeJob j = queue[i];
-        ne_job<kRef>(where, pp, rate, j, (uint32_t)kColour, cnt, j.g);
+    ne_moves<kAligned>(U, D, E, W, S, cc.vm, rate, cand, moved, ws, Sn, need);
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+        moved[w] |= cand[w] & ~rej[w];
+        Sn[w] = S[w] ^ (moved[w] & 0xFEFEFEFEu);
     }
-    if constexpr (kColour == 1) cnt.up += (cnt.mag + sites) / 2;
+    store16_any<kAligned>(p.dS + (size_t)at0, cc.nv, Sn);
+    const uint32_t chg = ne_changed(moved), now = was | chg;
+    cnt.unfl -= __popc(chg & ~was);
+    ne_set_flags<kAligned>(fp, was, now);
+    if constexpr (kColour == 1) {
+        ne_count(Sn, U, D, O, X, cc.vm, cnt);
+        cnt.up += (cnt.mag + 2 * (int)cc.nv) / 2;
+        if constexpr (kRef) {
+#pragma unroll
+            for (int w = 0; w < 4; ++w)
+                cnt.acf = dot4(Sn[w] & cc.vm[w], R1[w], dot4(O[w] & cc.vm[w], R0[w], cnt.acf));
+        }
+    }
 }
 
 // kOne: a thread per chunk (the launch has one for each); else a thread per
@@ -256,7 +229,7 @@ template <int kColour, bool kRef, bool kAligned, bool kOne>
 __global__ void __launch_bounds__(kThreads, kNeMinB) k_ne_walk(Geom g, SweepAt at)
 {
     __shared__ int red[kWarps][5];
-    __shared__ NeJob queue[kWarps][kNeQueue];
+    __shared__ NeJob queue[kOne ? 1 : kWarps][kOne ? 1 : kNeQueue];
     dep_wait();
     const unsigned long long sweep = sweep_of(g.ctrl, at);
     const SweepView v = sweep_view(g);
@@ -271,10 +244,10 @@ __global__ void __launch_bounds__(kThreads, kNeMinB) k_ne_walk(Geom g, SweepAt a
     const uint32_t k = act ? gt - band * cpr : 0u;
     const NeRows<kColour> p = ne_rows<kColour>(v, sweep);
     if constexpr (kOne) {
-        ne_one<kColour, kRef, kAligned>(p, pp, ne_rate(g.thr16), k, act ? band : 0u, act, queue[threadIdx.x >> 5], cnt);
+        if (act) ne_one<kColour, kRef, kAligned>(p, pp, ne_rate(g.thr16), k, band, cnt);
     } else {
         uint32_t y = 0, y1 = 0;
-        if (act) band_rows(band, nb, L, y, y1);
+        if (act) walk_rows(band, nb, L, y, y1);
         ne_walk<kColour, kRef, kAligned>(p, pp, ne_rate(g.thr16), k, y, y1, act, queue[threadIdx.x >> 5], cnt);
     }
     dep_launch();   // main work done: the next kernel may be scheduled

@@ -21,26 +21,26 @@ struct __align__(16) NeJob {
     uint32_t g, at, cand, ws;
 };
 
-// The draw threshold (accept iff u <= K), and the flag flip that marks the
-// state which draws (0: down spins, all ones: up spins).
+// The draw threshold (accept iff u <= K), the flag flip that marks the state
+// which draws (0: down spins, all ones: up spins), and whether any does (all
+// ones; 0 at c = 1/2, where both moves are certain).
 struct NeRate {
-    uint32_t K, inv;
+    uint32_t K, inv, draws;
 };
 
 LAT_D NeRate ne_rate(const uint32_t *thr16)
 {
     // index sd << 3 | nd; in c-mode every nd has the same entry
     const bool up_draws = thr16[8] == 0xFFFFFFFFu && thr16[0] != 0xFFFFFFFFu;
-    return NeRate{up_draws ? thr16[0] : thr16[8], up_draws ? 0xFFFFFFFFu : 0u};
+    const uint32_t K = up_draws ? thr16[0] : thr16[8];
+    return NeRate{K, up_draws ? 0xFFFFFFFFu : 0u, K == 0xFFFFFFFFu ? 0u : 0xFFFFFFFFu};
 }
 
-// Where a queued move is applied: the colour's spins (row pitch `pitch`),
-// its persistence bytes (one per group, at a quarter of the spins' offset)
-// and the reference plane 1 (row pitch `half`, first row y0).
+// Where a queued move is applied: the colour's spins, its persistence bytes
+// (one per group) and the reference plane 1.
 struct NePlanes {
     uint8_t *spins, *flags;
     const int8_t *ref;
-    uint32_t y0, half, pitch;
 };
 
 // 0xFF at the sites whose draw is above K.
@@ -59,7 +59,7 @@ LAT_D uint32_t ne_rejected(const U4 &u, uint32_t K)
 // One queued group: draw, accept, apply.
 template <bool kRef>
 LAT_D void ne_job(const NePlanes &p, const PhiloxPre &pp, const NeRate rate, const NeJob job, uint32_t colour,
-                  Counts &cnt, uint32_t flag_at = 0xFFFFFFFFu)
+                  Counts &cnt)
 {
     const U4 u = philox_item(pp, job.g, colour);
     const uint32_t rej = ne_rejected(u, rate.K);
@@ -71,7 +71,7 @@ LAT_D void ne_job(const NePlanes &p, const PhiloxPre &pp, const NeRate rate, con
     for (int b = 0; b < 4; ++b)
         if (f & (2u << (8 * b))) d[b] = now;
     const uint32_t bits = (uint32_t)dot4(f, 0x08040201u, 0) >> 1;
-    uint8_t *fl = p.flags + (flag_at == 0xFFFFFFFFu ? job.at >> 2 : flag_at);
+    uint8_t *fl = p.flags + job.g;
     const uint32_t was = *fl;
     *fl = (uint8_t)(was | bits);
     cnt.unfl -= __popc(bits & ~was);
@@ -81,11 +81,9 @@ LAT_D void ne_job(const NePlanes &p, const PhiloxPre &pp, const NeRate rate, con
         cnt.mag += sg * n;
         cnt.bond += sg * (4 * n - 2 * side);
         if constexpr (kRef) {
-            const uint32_t row = job.at / p.pitch;
-            const int8_t *r = p.ref + (size_t)(p.y0 + row) * p.half + (job.at - row * p.pitch);
 #pragma unroll
             for (int b = 0; b < 4; ++b)
-                if (f & (2u << (8 * b))) cnt.acf += sg * (int)r[b];
+                if (f & (2u << (8 * b))) cnt.acf += sg * (int)p.ref[job.at + b];
         }
     }
 }
@@ -102,8 +100,9 @@ LAT_D void ne_moves(const uint32_t (&U)[4], const uint32_t (&D)[4], const uint32
 #pragma unroll
     for (int w = 0; w < 4; ++w) {
         const uint32_t open = kFull ? ~(U[w] | E[w]) : ~(U[w] | E[w]) & vm[w];
-        cand[w] = open & (S[w] ^ rate.inv);
-        sure[w] = open & ~(S[w] ^ rate.inv);
+        const uint32_t undecided = (S[w] ^ rate.inv) & rate.draws;
+        cand[w] = open & undecided;
+        sure[w] = open & ~undecided;
         need[w] = (cand[w] & kB1) != 0u;
         Sn[w] = S[w] ^ (sure[w] & 0xFEFEFEFEu);
         ws[w] = (W[w] & kB1) | (D[w] & ~kB1);
@@ -117,6 +116,36 @@ LAT_D uint32_t ne_changed(const uint32_t (&sure)[4])
 #pragma unroll
     for (int w = 2; w >= 0; --w) c = dot4(sure[w] & kB1, 0x08040201u, c * 256);
     return (uint32_t)c >> 1;
+}
+
+// The persistence bits of a chunk of nv sites, byte w = group w (the bytes of
+// groups that do not exist are unspecified).  Unaligned: by whole words, so
+// that a row waits for memory once and not once a group (L = 3000, c = 0.4,
+// launches of a graph: 34.1 us a sweep with a byte read each, 21.4).  The
+// words' other bytes are other threads'; a word that holds none of the
+// chunk's is not read (the buffer is a multiple of 4 bytes, so every word read
+// is in bounds).
+template <bool kAligned>
+LAT_D uint32_t ne_flags(const uint8_t *fp, uint32_t nv)
+{
+    if constexpr (kAligned) return *reinterpret_cast<const uint32_t *>(fp);
+    const uintptr_t a = reinterpret_cast<uintptr_t>(fp);
+    const uint32_t sh = (uint32_t)(a & 3u);
+    const uint32_t *q = reinterpret_cast<const uint32_t *>(a - sh);
+    return __funnelshift_r(q[0], sh + (nv + 3u) / 4u > 4u ? q[1] : 0u, 8u * sh);
+}
+
+// Write the bytes that changed.
+template <bool kAligned>
+LAT_D void ne_set_flags(uint8_t *fp, uint32_t was, uint32_t now)
+{
+    if constexpr (kAligned) {
+        if (now != was) *reinterpret_cast<uint32_t *>(fp) = now;
+    } else {
+#pragma unroll
+        for (int w = 0; w < 4; ++w)   // (only groups that exist have moves)
+            if (((now ^ was) >> (8 * w) & 0xFFu) != 0u) fp[w] = (uint8_t)(now >> (8 * w));
+    }
 }
 
 // Colour 1: bonds of the new spins, both planes' magnetisation.
