@@ -237,7 +237,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_bits_walk(Geom g, int off)
         philox_prepare(pp, (uint32_t)sweep, (uint32_t)(sweep >> 32), g.key0, g.key1);
         const SymK sk = bits_sym(g.thr16);
         uint32_t y, y1;
-        band_rows(band, nb, L, y, y1);
+        walk_rows(band, nb, L, y, y1);
         const uint32_t rows = y1 - y;
         uint32_t U = pO[(size_t)(y == 0 ? L - 1 : y - 1) * bw + k], O = pO[(size_t)y * bw + k];
         uint32_t nD = pO[(size_t)(y + 1 == L ? 0 : y + 1) * bw + k], nS = pS[(size_t)y * bw + k];
@@ -301,8 +301,13 @@ cudaError_t launch_sweep_bitpacked(const Geom &g, int off, cudaStream_t st)
                                      one_wave(reinterpret_cast<const void *>(kern[1][1])),
                                      one_wave(reinterpret_cast<const void *>(kern[2][1])),
                                      one_wave(reinterpret_cast<const void *>(kern[3][1]))};
-    const int m = g.model == LAT_NE ? 3 : (k.acc_sym ? (g.ref_bits != nullptr ? 1 : 0) : 2);
     const uint64_t words = (uint64_t)g.L * g.bw;
+    // One word a thread: the table look-ups' shorter chain wins (launches of a
+    // graph, look-ups and two draws a compare: L = 1024 5.6 and 6.9 us a sweep,
+    // 2048 8.5 and 9.5, 2560 10.5 and 11.0; with more words a thread 3072 13.9
+    // and 13.6, 4096 20.4 and 19.6, 8192 69.0 and 58.3).
+    const bool pipe = words <= (uint64_t)kThreads * wave[2];
+    const int m = g.model == LAT_NE ? 3 : (k.acc_sym && !pipe ? (g.ref_bits != nullptr ? 1 : 0) : 2);
     const unsigned blocks = (unsigned)std::min<uint64_t>((words + kThreads - 1) / kThreads, wave[m]);
     cudaError_t e = launch_pdl(kern[m][0], blocks, kThreads, st, k, off);
     return e == cudaSuccess ? launch_pdl(kern[m][1], blocks, kThreads, st, k, off) : e;
