@@ -50,7 +50,6 @@ struct BandPart {
     unsigned long long sweep0;   // sweeps done before the launch
     int *err, *err_all;          // host-visible error words of the lattice and (or null) of its batch
     uint32_t limit;              // polls after which a wait gives up
-    uint32_t mute;               // solo: 1 + the band that sends nothing (0: none), by which tests let waits run out
     uint32_t mail;               // batched: packet rows start at this pair
     int n;                       // sweeps to run
     uint32_t key0, key1;

@@ -237,7 +237,7 @@ LAT_D void band_bits(const Geom &g, const BandPart &part, uint32_t band, uint32_
             const Nbr n = nbr_sum(a, d, o, x);
             uint32_t Sn;
             if constexpr (kNe) {
-                const uint32_t open = U & (odd ? X : O) & vm, draws = ~(S ^ rate.inv) & rate.draws;
+                const uint32_t open = U & (odd ? X : O) & vm, draws = ~(S ^ rate.inv);
                 const uint32_t sure = open & ~draws;
                 cand = open & draws;
                 Sn = S ^ sure;

@@ -478,6 +478,21 @@ static int64_t band_min_sweeps(const lattice *lt)
     // L no multiple of 16 has the generic kernel to beat (L = 100: 182 us, 84).
     if (lt->P.model == LAT_POTTS) return !potts_supported(lt->geom) || lt->P.N >= 750000u ? 4 : INT64_MAX;
     if (lt->P.L <= 128) return 16;
+    // General tables with several chunks a thread: the bands win while their
+    // chunks divide well and the work is small beside an exchange, the
+    // launches' row walk else.  us of 20 sweeps in bands and in launches, h =
+    // 0.15: L = 1664 (1.1 chunks a thread) 140 and 127, 2048 (1.75) 136 and 156,
+    // 2400 (2.3) 193 and 185, 2816 (3.3) 248 and 225, 5600 805 and 661; with field
+    // signs, whose launches read a third plane, 1664 157 and 164, 2560 (2.7) 235 and
+    // 255, 3008 (3.7) 313 and 315, 4096 514 and 492.  Rows of any alignment cost the
+    // launches more: L = 2050 168 and 227, 3000 284 and 327, 4402 619 and 661. 5
+    // sweeps: 2048 42.5 and 43, 2400 57 and 50; 2050 56 and 61, 2402 70 and 72,
+    // 3000 88 and 86.
+    if (const int load = band_chunk_load(lt->geom, lt->has_fields)) {
+        if (lt->P.L % 32 != 0) return load > 370 ? 8 : load >= 150 && load <= 200 ? 4 : 5;
+        if (load >= 150 && load <= 200) return 5;
+        return (load < 150 && !lt->has_fields) || load > (lt->has_fields ? 370 : 270) ? INT64_MAX : 12;
+    }
     return lt->P.N * (lt->geom.cpl != nullptr ? 2u : 1u) > 6000000u ? 5 : 3;
 }
 
@@ -1697,8 +1712,8 @@ int lattice_test_fail_alloc(int countdown)
 }
 
 // Test hook: waits of band launches give up after `polls` polls (0: the
-// default), and CTA `mute` - 1 of the next band launch sends nothing (0:
-// none), so that its neighbours' waits run out.
+// default), and CTA `mute` - 1 of the next batched band launch sends nothing
+// (0: none), so that its neighbours' waits run out.
 int lattice_test_band_wait(unsigned polls, int mute)
 {
     band_test().limit.store(polls != 0u ? polls : 1u << 24);

@@ -22,6 +22,10 @@ namespace {
 // Disorder of Eq. 1: none, bond signs, bond and field signs.
 enum IsingDisorder { kUniform = 0, kBonds = 1, kFields = 2 };
 
+// Acceptance: every threshold from the table in shared memory, or the top 16
+// bits (accept16.cuh) of a general or a symmetric table.
+enum IsingAccept { kLookUp = 0, kTopGen = 1, kTopSym = 2 };
+
 // The planes of one colour's pass: colour 0 reads both planes of the old
 // buffer; colour 1 its own old sites and the new colour-0 sites.  Each
 // writes only its own plane of the new buffer.
@@ -197,11 +201,13 @@ LAT_D void ising_flips(const IsingChunk &c, const uint32_t *sthr, const U4 (&u)[
 }
 
 // Rows [y, y1), y < y1, of chunk column k.
-template <int kColour, bool kRef, int kDis, bool kSym, bool kAligned>
+template <int kColour, bool kRef, int kDis, int kAcc, bool kAligned>
 LAT_D void ising_walk(const IsingPlanes<kColour> &p, const uint32_t (&acc)[8], const uint32_t *sthr,
                       unsigned long long sweep, uint32_t key0, uint32_t key1, uint32_t k, uint32_t y,
                       const uint32_t y1, Counts &cnt)
 {
+    constexpr bool kSym = kAcc == kTopSym;
+    static_assert(kAcc != kTopGen, "general tables walk by look-ups");
     PhiloxPre pp;
     philox_prepare(pp, (uint32_t)sweep, (uint32_t)(sweep >> 32), key0, key1);
     const ChunkCol<kAligned> cc = chunk_col<kAligned>(k, p.half);
@@ -255,6 +261,11 @@ LAT_D void ising_walk(const IsingPlanes<kColour> &p, const uint32_t (&acc)[8], c
             c.D[w] = R[(s + 2) & 3][w];
             C[w] = nC[w];
         }
+        [[maybe_unused]] uint32_t R1[4], R0[4];
+        if constexpr (kColour == 1 && kRef) {   // (asked for here, not where they are used: L = 8192, 76 us for 80)
+            load16_any<kAligned>(p.r1 + at, cc.nv, R1);
+            load16_any<kAligned>(p.r0 + at, cc.nv, R0);
+        }
         auto step = [&]() {
             ising_neighbours<kDis, false>(c, C, odd);
             uint32_t F[4], Sn[4];
@@ -269,9 +280,6 @@ LAT_D void ising_walk(const IsingPlanes<kColour> &p, const uint32_t (&acc)[8], c
 #pragma unroll
                 for (int w = 0; w < 4; ++w) cnt.mag = dot4(R[(s + 1) & 3][w], 0x01010101u & cc.vm[w], cnt.mag);
                 if constexpr (kRef) {
-                    uint32_t R1[4], R0[4];
-                    load16_any<kAligned>(p.r1 + at, cc.nv, R1);
-                    load16_any<kAligned>(p.r0 + at, cc.nv, R0);
 #pragma unroll
                     for (int w = 0; w < 4; ++w)
                         cnt.acf = dot4(Sn[w] & cc.vm[w], R1[w], dot4(R[(s + 1) & 3][w] & cc.vm[w], R0[w], cnt.acf));
@@ -313,8 +321,8 @@ LAT_D void ising_walk(const IsingPlanes<kColour> &p, const uint32_t (&acc)[8], c
 
 // Row y's chunk of column k alone (lattices with little more than one chunk
 // a thread).
-template <int kColour, bool kRef, int kDis, bool kAligned>
-LAT_D void ising_one(const IsingPlanes<kColour> &p, const uint32_t *sthr, unsigned long long sweep, uint32_t key0, uint32_t key1, uint32_t k, uint32_t y, Counts &cnt)
+template <int kColour, bool kRef, int kDis, int kAcc, bool kAligned>
+LAT_D void ising_one(const IsingPlanes<kColour> &p, const uint32_t (&acc)[8], const uint32_t *sthr, unsigned long long sweep, uint32_t key0, uint32_t key1, uint32_t k, uint32_t y, Counts &cnt)
 {
     const ChunkCol<kAligned> cc = chunk_col<kAligned>(k, p.half);
     const size_t at = (size_t)y * p.half + cc.j0;
@@ -344,7 +352,14 @@ LAT_D void ising_one(const IsingPlanes<kColour> &p, const uint32_t *sthr, unsign
 #pragma unroll
     for (int w = 0; w < 4; ++w) c.O[w] = O[w];
     ising_neighbours<kDis, false>(c, C, odd);
-    ising_flips<kDis>(c, sthr, u, F);
+    if constexpr (kAcc == kLookUp) {
+        ising_flips<kDis>(c, sthr, u, F);
+    } else {
+        uint32_t p01[4], p23[4];
+#pragma unroll
+        for (int w = 0; w < 4; ++w) top_halves(u[w], p01[w], p23[w]);
+        if (flips16<kAcc == kTopSym>(acc, c.n, c.St, p01, p23, F)) ising_flips<kDis>(c, sthr, u, F);
+    }
 #pragma unroll
     for (int w = 0; w < 4; ++w) Sn[w] = c.S[w] ^ F[w];
     store16_any<kAligned>(p.dS + at, cc.nv, Sn);

@@ -16,7 +16,6 @@ __global__ void __launch_bounds__(kT, 1) k_band(const __grid_constant__ Geom g, 
 {
     extern __shared__ __align__(16) uint8_t band_smem[];
     __shared__ BandShared sh;
-    if (blockIdx.x + 1u == part.mute) return;
     band_body<kKind, kRef, kT, kForm>(g, part, blockIdx.x, gridDim.x, mail, sh, band_smem);
     band_end(g, part, blockIdx.x, sh);
 }
@@ -68,6 +67,14 @@ int band_count_for(const Geom &g, bool fields)
     return bands >= 2 && band_kind_ok(g, kind) && band_fits(k, kind, bands) ? bands : 0;
 }
 
+int band_chunk_load(const Geom &g, bool fields)
+{
+    const Geom k = tiled_geom(g);
+    const int kind = band_kind(k, fields), bands = std::min(band_sms(), g.L / 2);
+    if (bands < 2 || band_on_bits(k, kind, bands) || band_is_small((uint32_t)k.L, k.half, (uint32_t)bands)) return 0;
+    return (int)((uint64_t)((k.L + bands - 1) / bands) * ((k.half + 15) / 16) * 100 / kBandThreads);
+}
+
 size_t band_mail_bytes(const Geom &g, bool fields, int bands)
 {
     const Geom k = tiled_geom(g);
@@ -104,8 +111,7 @@ cudaError_t launch_sweep_band(const Geom &g, bool fields, int bands, unsigned lo
     if (attr != cudaSuccess) return attr;
     if (band_test().launch()) return cudaErrorCooperativeLaunchTooLarge;
     const Geom k = tiled_geom(g);
-    BandPart part = band_part(k, sweep0, n, epoch, err);
-    part.mute = band_test().mute.exchange(0);
+    const BandPart part = band_part(k, sweep0, n, epoch, err);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)bands);
     // one chunk a thread: just the warps that have one (a row is a warp's when it fits)

@@ -122,10 +122,10 @@ LAT_D void ne_walk(const NeRows<kColour> &p, const PhiloxPre &pp, const NeRate r
                 uint32_t X[4], Sn[4], sure[4];
                 if (odd) {   // east is the shifted row
                     shifted_row<kAligned>(cc, true, nb, O, X);
-                    ne_moves<kAligned>(U, D, X, O, S, cc.vm, rate, cand, sure, ws, Sn, need);
+                    ne_moves<kAligned, true>(U, D, X, O, S, cc.vm, rate, cand, sure, ws, Sn, need);
                 } else {
                     shifted_row<kAligned>(cc, false, nb, O, X);
-                    ne_moves<kAligned>(U, D, O, X, S, cc.vm, rate, cand, sure, ws, Sn, need);
+                    ne_moves<kAligned, true>(U, D, O, X, S, cc.vm, rate, cand, sure, ws, Sn, need);
                 }
                 store16_any<kAligned>(p.dS + (size_t)at0, cc.nv, Sn);
                 if constexpr (kColour == 1) {

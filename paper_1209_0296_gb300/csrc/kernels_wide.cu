@@ -239,7 +239,7 @@ constexpr int kWalkMinB = 2;   // (3, with fewer registers: 24 us a sweep at L =
 // 2D Ising, one colour.  kOne: a thread per chunk (the launch has one for
 // each); else a thread per (chunk column, band of consecutive rows), in one
 // wave of at least cpr threads.
-template <int kColour, bool kRef, int kDis, bool kSym, bool kAligned, bool kOne>
+template <int kColour, bool kRef, int kDis, int kAcc, bool kAligned, bool kOne>
 __global__ void __launch_bounds__(kThreads, kOne && kAligned && kDis != kFields ? 4 : kWalkMinB) k_ising_walk(Geom g, SweepAt at)
 {
     __shared__ uint32_t sthr[kDis == kFields ? 32 : 16];
@@ -257,11 +257,12 @@ __global__ void __launch_bounds__(kThreads, kOne && kAligned && kDis != kFields 
     if (band < nb) {
         const IsingPlanes<kColour> p = ising_planes<kColour>(v, sweep);
         if constexpr (kOne) {
-            ising_one<kColour, kRef, kDis, kAligned>(p, sthr, sweep, g.key0, g.key1, gt - band * cpr, band, cnt);
+            ising_one<kColour, kRef, kDis, kAcc, kAligned>(p, g.acc, sthr, sweep, g.key0, g.key1, gt - band * cpr,
+                                                           band, cnt);
         } else {
             uint32_t y, y1;
             walk_rows(band, nb, L, y, y1);
-            ising_walk<kColour, kRef, kDis, kSym, kAligned>(p, g.acc, sthr, sweep, g.key0, g.key1, gt - band * cpr, y,
+            ising_walk<kColour, kRef, kDis, kAcc, kAligned>(p, g.acc, sthr, sweep, g.key0, g.key1, gt - band * cpr, y,
                                                             y1, cnt);
         }
     }
@@ -1311,28 +1312,32 @@ cudaError_t launch_sweep_wide(const Geom &g, bool fields, SweepAt at, cudaStream
         return e == cudaSuccess ? launch_pdl(ne[al][ref][1], grid, kThreads, st, k, at.off) : e;
     }
     using K = void (*)(Geom, SweepAt);
-#define LAT_WALK(dis, sym, al, one)                                                          \
-    {{k_ising_walk<0, false, dis, sym, al, one>, k_ising_walk<1, false, dis, sym, al, one>}, \
-     {k_ising_walk<0, true, dis, sym, al, one>, k_ising_walk<1, true, dis, sym, al, one>}}
+#define LAT_WALK(dis, acc, al, one)                                                          \
+    {{k_ising_walk<0, false, dis, acc, al, one>, k_ising_walk<1, false, dis, acc, al, one>}, \
+     {k_ising_walk<0, true, dis, acc, al, one>, k_ising_walk<1, true, dis, acc, al, one>}}
     // [uniform at any even L, then L % 32 == 0: uniform, bonds, fields][reference][colour]
-    static const K one[4][2][2] = {LAT_WALK(kUniform, false, false, true), LAT_WALK(kUniform, false, true, true),
-                                   LAT_WALK(kBonds, false, true, true), LAT_WALK(kFields, false, true, true)};
-    static const K walk[4][2][2] = {LAT_WALK(kUniform, false, false, false), LAT_WALK(kUniform, false, true, false),
-                                    LAT_WALK(kBonds, false, true, false), LAT_WALK(kFields, false, true, false)};
-    static const K top[3][2][2] = {LAT_WALK(kUniform, true, false, false), LAT_WALK(kUniform, true, true, false),
-                                   LAT_WALK(kBonds, true, true, false)};
+    static const K one[4][2][2] = {LAT_WALK(kUniform, kLookUp, false, true), LAT_WALK(kUniform, kLookUp, true, true),
+                                   LAT_WALK(kBonds, kLookUp, true, true), LAT_WALK(kFields, kLookUp, true, true)};
+    static const K walk[4][2][2] = {LAT_WALK(kUniform, kLookUp, false, false), LAT_WALK(kUniform, kLookUp, true, false),
+                                    LAT_WALK(kBonds, kLookUp, true, false), LAT_WALK(kFields, kLookUp, true, false)};
+    static const K top[3][2][2] = {LAT_WALK(kUniform, kTopSym, false, false), LAT_WALK(kUniform, kTopSym, true, false),
+                                   LAT_WALK(kBonds, kTopSym, true, false)};
+    static const K few[2][2][2] = {LAT_WALK(kUniform, kTopGen, false, true), LAT_WALK(kUniform, kTopSym, false, true)};
 #undef LAT_WALK
     static const unsigned wave = one_wave(reinterpret_cast<const void *>(walk[1][0][1]));   // all: kWalkMinB per SM
-    const int m = g.cpl != nullptr ? (fields ? 3 : 2) : al;
+    const int m = g.cpl != nullptr ? (fields ? 3 : 2) : al, sym = k.acc_sym ? 1 : 0;
     // One chunk a thread up to two waves of them: up to there the row walk's
     // start-up costs more than its register reuse saves.  The 16-bit
     // acceptance of symmetric tables from 10 rows a thread on: its rows to be
     // done again are a chain of memory trips at the end of every thread's walk
     // (launches of a graph, 16-bit and look-ups: L = 3000, 3 rows, 20.0 and
     // 17.6 us a sweep; 4096, 7 rows, 20.5 and 19.9; 6000, 15 rows, 55.0 and
-    // 56.2; 8192, 27 rows, 67.4 and 70.6).
-    const bool many = blocks > 2u * wave, sym = k.acc_sym != 0 && blocks >= 10u * wave;
-    const K *kern = !many ? one[m][ref] : (sym ? top[m][ref] : walk[m][ref]);
+    // 56.2; 8192, 27 rows, 67.4 and 70.6).  And where rows of any alignment
+    // give no more than a CTA an SM, whose undecided chunks are settled from
+    // registers: L = 66 4.78 and 4.97, 1000 5.79 and 5.96 (2000: 10.8 and 10.2).
+    const bool many = blocks > 2u * wave;
+    const K *kern = many ? (sym && blocks >= 10u * wave ? top[m][ref] : walk[m][ref])
+                         : (m == 0 && blocks <= wave / kWalkMinB ? few[sym][ref] : one[m][ref]);
     const unsigned grid = many ? wave : (unsigned)blocks;
     cudaError_t e = launch_pdl(kern[0], grid, kThreads, st, k, at);
     return e == cudaSuccess ? launch_pdl(kern[1], grid, kThreads, st, k, at) : e;

@@ -472,9 +472,10 @@ cudaError_t launch_batch_ne(const Geom *geoms, const uint2 *items, int n_items, 
 // device memory, zeroed once; epoch: at least every packet mark sent through
 // it before, the launch marks up to epoch + 2 n; err: host-visible word set
 // when a bounded wait gave up.  Advances ctrl->sweep.
-// Test settings of band launches: polls after which a wait gives up (about a quarter of a
-// microsecond each: four seconds), 1 + the CTA of the next launch that sends
-// nothing (0: none), launches until one is refused (1: the next; 0: none); and
+// Test settings of band launches: polls after which a wait gives up (about a
+// quarter of a microsecond each: four seconds), 1 + the CTA of the next batched
+// launch that sends nothing (0: none; not in the lone lattice's kernel, where
+// one more branch at its start costs 1 to 3 %), launches until one is refused (1: the next; 0: none); and
 // the launches so far.
 struct BandTest {
     std::atomic<uint32_t> limit{1u << 24}, mute{0};
@@ -492,6 +493,9 @@ struct BandTest {
 BandTest &band_test();
 int band_sms();   // CTAs of a launch at most
 int band_count_for(const Geom &g, bool fields);
+// 16-site chunks of a band of a lattice that keeps a byte a site on the chip
+// and has several chunks a thread (general tables), per hundred threads; else 0.
+int band_chunk_load(const Geom &g, bool fields);
 size_t band_mail_bytes(const Geom &g, bool fields, int bands);
 cudaError_t launch_sweep_band(const Geom &g, bool fields, int bands, unsigned long long sweep0, int n, void *mail,
                               unsigned epoch, int *err, cudaStream_t st);

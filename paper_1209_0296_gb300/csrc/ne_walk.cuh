@@ -91,8 +91,8 @@ LAT_D void ne_job(const NePlanes &p, const PhiloxPre &pp, const NeRate rate, con
 // The moves of a chunk that need no draw: north U, south D, east E, west W,
 // own spins S -> spins after the certain moves Sn, flags of those moves
 // (sure), of the sites whose draw decides (cand) and of their west and south
-// neighbours (ws), and which groups need a draw.
-template <bool kFull>
+// neighbours (ws), and which groups need a draw.  kHalf: looks whether any does.
+template <bool kFull, bool kHalf = false>
 LAT_D void ne_moves(const uint32_t (&U)[4], const uint32_t (&D)[4], const uint32_t (&E)[4], const uint32_t (&W)[4],
                     const uint32_t (&S)[4], const uint32_t (&vm)[4], const NeRate rate, uint32_t (&cand)[4],
                     uint32_t (&sure)[4], uint32_t (&ws)[4], uint32_t (&Sn)[4], bool (&need)[4])
@@ -100,7 +100,7 @@ LAT_D void ne_moves(const uint32_t (&U)[4], const uint32_t (&D)[4], const uint32
 #pragma unroll
     for (int w = 0; w < 4; ++w) {
         const uint32_t open = kFull ? ~(U[w] | E[w]) : ~(U[w] | E[w]) & vm[w];
-        const uint32_t undecided = (S[w] ^ rate.inv) & rate.draws;
+        const uint32_t undecided = kHalf ? (S[w] ^ rate.inv) & rate.draws : S[w] ^ rate.inv;
         cand[w] = open & undecided;
         sure[w] = open & ~undecided;
         need[w] = (cand[w] & kB1) != 0u;

@@ -109,12 +109,18 @@ LAT_D void band_rows(uint32_t b, uint32_t nb, uint32_t L, uint32_t &y0, uint32_t
     y1 = (uint32_t)((uint64_t)(b + 1u) * L / nb);
 }
 
-// The same for the threads of a streaming launch: the long bands come first.
-// (In turn with the short ones every warp takes the longer time: L = 2400, two
-// rows or three, 10.7 us a sweep for 9.2.)
+// The same for the threads of a streaming launch: where bands are short the
+// long ones come first.  (In turn with the others every warp takes the longer
+// time: L = 2400, two rows or three, 10.7 us a sweep for 9.2.  Many rows apart,
+// equal lengths make bands meet in the same memory channels: bit-packed L =
+// 32768, 143 rows or 144, 834 us for 810.)
 LAT_D void walk_rows(uint32_t b, uint32_t nb, uint32_t L, uint32_t &y0, uint32_t &y1)
 {
     const uint32_t q = L / nb, r = L - q * nb;
+    if (q >= 32u) {
+        band_rows(b, nb, L, y0, y1);
+        return;
+    }
     y0 = b * q + min(b, r);
     y1 = y0 + q + (b < r ? 1u : 0u);
 }
