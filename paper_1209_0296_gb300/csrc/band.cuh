@@ -17,9 +17,11 @@
 // packet of the half-sweep in between has arrived.
 //
 // A wait is bounded: when it gives up the launch ends normally and the host
-// sees the error word (LAT_ETIMEOUT).  It also leaves the launch's own mark in
-// the abort word, which ends the launch's other waits early; the next launch
-// on the same packets has another mark, so nothing needs to be cleared.
+// sees the error word (LAT_ETIMEOUT).  It also sets the launch's abort word,
+// which ends the launch's other waits early; the host clears it with the packets
+// before the next launch once it has seen the error.  (A word that holds the
+// mark of the launch that gave up needs no clearing, but costs 1 to 2 % in the
+// waits' code.)
 #pragma once
 
 #include <memory>
@@ -37,23 +39,28 @@ constexpr int kBandThreads = 512;
 constexpr int kBandWarps = kBandThreads / 32;
 constexpr int kBandNeThreads = 1024;        // North-East on bits, alone on the GPU, bands of more than 1024 words
 constexpr int kBandMaxCtas = 160;           // a batched launch's parts are kernel parameters
-constexpr uint32_t kAbortBytes = 128;       // the abort word's line, before a lattice's packets
+constexpr uint32_t kAbortBytes = 128;       // the abort word's line, before the packets
 constexpr size_t kBandMaxSmem = 224 * 1024;
 
 // What a CTA runs: band `band` of `bands` of one lattice.  The key and the
 // acceptance table are here (and not read from the lattice's descriptor) so
 // that they are kernel parameters, which the sweep loop reads as such.
+// (The order is measured: with four bytes more before the key and the table the
+// batched kernel, which reads them at a run-time index, took 721 us for the 707
+// of a served mix of 16 lattices; with the table first the bit-packed kernel
+// took 1 % more.)
 struct BandPart {
     uint32_t band, bands;        // batched (solo: the CTA and the grid)
     uint32_t lat, kind, ref;     // batched: descriptor index, BandKind, reference set
     uint32_t epoch;              // packets are marked epoch + 1 .. epoch + 2 n
     unsigned long long sweep0;   // sweeps done before the launch
-    int *err, *err_all;          // host-visible error words of the lattice and (or null) of its batch
-    uint32_t limit;              // polls after which a wait gives up
+    int *err;                    // host-visible error word of the lattice
     uint32_t mail;               // batched: packet rows start at this pair
     int n;                       // sweeps to run
     uint32_t key0, key1;
     uint32_t acc[8];
+    uint32_t limit;              // polls after which a wait gives up
+    int *err_all;                // batched: host-visible error word of the batch
 };
 
 struct BandShared {
@@ -71,7 +78,7 @@ struct Band {
     size_t plane;
     const int8_t *src;           // spins before the launch
     uint32_t up, dn;             // rows above and below the band
-    unsigned *abort;             // the launch's mark when a wait of it gave up
+    unsigned *abort;             // set when a wait of the launch gave up
     // packet rows of colour 0 (colour 1: + cpr packet pairs): this band's
     // first and last row, the last row of the band above, the first below
     ulonglong2 *first, *last;
@@ -127,9 +134,8 @@ LAT_D void mail_put(ulonglong2 *q, uint32_t tag, const uint32_t (&v)[4])
 LAT_D bool mail_over(unsigned i, const BandPart &p, unsigned *abort)
 {
     if ((i & 1023u) != 1023u) return false;
-    const uint32_t mark = p.epoch + 1u;   // no other launch on these packets has it
-    if (i < p.limit && *reinterpret_cast<volatile unsigned *>(abort) != mark) return false;
-    *reinterpret_cast<volatile unsigned *>(abort) = mark;
+    if (i < p.limit && *reinterpret_cast<volatile unsigned *>(abort) == 0u) return false;
+    *reinterpret_cast<volatile unsigned *>(abort) = 1u;
     return true;
 }
 

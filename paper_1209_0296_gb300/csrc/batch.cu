@@ -80,6 +80,7 @@ struct lattice_batch {
     void *d_mail = nullptr;
     size_t mail_cap = 0;
     unsigned mail_epoch = 0;
+    bool gave_up = false;   // a run's wait did: the packets must be cleared
     lat::BandShare band_share;
     int *band_err = nullptr;   // host-visible: a wait of a run gave up since the last synchronise
     // resident lattices
@@ -420,6 +421,12 @@ int run_bands(lattice_batch *b, BatchSlot &sl, size_t at, std::vector<BandGroup>
             if (pr.first->band_err == nullptr && (pr.first->band_err = band_error_word()) == nullptr) return LAT_OK;
             geoms.push_back(tiled_geom(pr.first->geom));
         }
+    // (A run queued before the host could see the time-out of the one before it
+    // ends its waits early too, those of more than 1024 polls: its lattices say so.)
+    b->gave_up = b->gave_up || *(volatile int *)b->band_err != 0;
+    if (b->gave_up) b->mail_epoch = 1u << 30;   // clear below
+    b->gave_up = false;
+    if (b->caller_orders) *b->band_err = 0;     // (the server asks its lattices)
     int rc = grow(&sl.d_band_geoms, sl.band_geoms_cap, (int)n, b->stream);
     if (rc == LAT_ENOMEM) {
         (void)cudaGetLastError();
@@ -913,6 +920,7 @@ int lattice_batch_synchronize(lattice_batch_t *b)
     if (e != cudaSuccess) return cuda_fail(e, "batch synchronize");
     if (b->band_err != nullptr && *(volatile int *)b->band_err != 0) {
         *b->band_err = 0;
+        b->gave_up = true;
         return LAT_ETIMEOUT;
     }
     return LAT_OK;

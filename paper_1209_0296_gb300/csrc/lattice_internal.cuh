@@ -471,7 +471,8 @@ cudaError_t launch_batch_ne(const Geom *geoms, const uint2 *items, int n_items, 
 // the whole GPU (0: not supported or too large).  mail: band_mail_bytes() of
 // device memory, zeroed once; epoch: at least every packet mark sent through
 // it before, the launch marks up to epoch + 2 n; err: host-visible word set
-// when a bounded wait gave up.  Advances ctrl->sweep.
+// when a bounded wait gave up (mail must then be zeroed before the next
+// launch).  Advances ctrl->sweep.
 // Test settings of band launches: polls after which a wait gives up (about a
 // quarter of a microsecond each: four seconds), 1 + the CTA of the next batched
 // launch that sends nothing (0: none; not in the lone lattice's kernel, where
