@@ -408,6 +408,7 @@ void plan_bands(Work &work, std::vector<BandGroup> &groups, size_t at_least)
 // flight), and then the step loop takes the rest.
 int run_bands(lattice_batch *b, BatchSlot &sl, size_t at, std::vector<BandGroup> &groups, bool clear)
 {
+    const BesideCapture beside;
     size_t n = 0, mail = 0;
     for (auto &g : groups) {
         n += g.work.size();

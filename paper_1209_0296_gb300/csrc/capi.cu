@@ -69,6 +69,7 @@ public:
             p_ = g_bounce_free.back();
             g_bounce_free.pop_back();
         } else if (g_bounce_made < kBounceMost) {
+            const BesideCapture beside;
             if (cudaHostAlloc(&p_, kBounceBytes, cudaHostAllocPortable) == cudaSuccess) {
                 ++g_bounce_made;
                 g_bounce_free.reserve(kBounceMost);
@@ -350,6 +351,7 @@ int *band_error_word() { return error_words().take(); }
 void band_error_word_back(int *w, cudaStream_t st, bool busy)
 {
     if (w == nullptr) return;
+    const BesideCapture beside;
     cudaEvent_t ev = nullptr;
     if (busy && (cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess ||
                  cudaEventRecord(ev, st) != cudaSuccess)) {
@@ -394,6 +396,8 @@ bool band_place(cudaStream_t st, int &dev, unsigned long long &id)
 
 bool idle_stream(cudaStream_t st)
 {
+    if (st == nullptr || st == cudaStreamLegacy || st == cudaStreamPerThread) return false;   // (blocking)
+    const BesideCapture beside;
     unsigned flags = 0;
     const bool idle = cudaStreamGetFlags(st, &flags) == cudaSuccess && (flags & cudaStreamNonBlocking) != 0u &&
                       cudaStreamQuery(st) == cudaSuccess;
@@ -403,12 +407,13 @@ bool idle_stream(cudaStream_t st)
 
 bool band_may(cudaStream_t st, BandShare *me)
 {
-    int dev = 0;
-    unsigned long long id = 0;
-    if (!band_place(st, dev, id)) return false;
     std::lock_guard<std::mutex> g(g_band_mu);
     if (me->yield == 0) return true;
     --me->yield;
+    const BesideCapture beside;
+    int dev = 0;
+    unsigned long long id = 0;
+    if (!band_place(st, dev, id)) return false;
     const BandLast &l = g_band_last[dev];
     if (in_flight(l, id)) {
         me->yield = kBandYield;
@@ -531,6 +536,7 @@ static int band_bands(lattice *lt, int64_t n)
 static int band_sweeps(lattice *lt, int bands, int64_t n, bool clear, int64_t *done)
 {
     *done = 0;
+    const BesideCapture beside;
     if (lt->band_err == nullptr && (lt->band_err = band_error_word()) == nullptr) return LAT_OK;
     const size_t bytes = band_mail_bytes(lt->geom, lt->has_fields, bands);
     if (bytes > lt->band_mail_cap) {

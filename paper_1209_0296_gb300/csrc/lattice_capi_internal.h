@@ -28,6 +28,18 @@ int create_impl(struct ::lattice **out, int dims, int L, int two_S, int model, d
                 double T_or_c, uint64_t seed, int init, int layout, void *cuda_stream);
 int sweep_impl(struct ::lattice *lt, int64_t n);
 int choose_kernel(const struct ::lattice *lt);
+// While one lives, this thread's allocations and queries break no capture that
+// the caller has going on another stream (in the global mode they would).
+class BesideCapture {
+public:
+    BesideCapture() { cudaThreadExchangeStreamCaptureMode(&mode_); }
+    ~BesideCapture() { cudaThreadExchangeStreamCaptureMode(&mode_); }
+    BesideCapture(const BesideCapture &) = delete;
+    BesideCapture &operator=(const BesideCapture &) = delete;
+
+private:
+    cudaStreamCaptureMode mode_ = cudaStreamCaptureModeRelaxed;
+};
 // A host-visible error word for band launches, zeroed (null: no memory), the
 // owner's until it is given back; busy: launches on st may still write it.
 int *band_error_word();
