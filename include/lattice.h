@@ -156,7 +156,11 @@ int lattice_create(lattice_t **out, int dims, int L, int two_S, int model,
 
 /* Queue n >= 0 checkerboard sweeps (§III.A steps 5-8; §III.B rule) on the
  * handle's stream; returns without waiting.  After each sweep t the four
- * exact int64 counters of lattice_series are recorded on the device. */
+ * exact int64 counters of lattice_series are recorded on the device.  A call
+ * while the stream is captured is captured: replays of it go on from the
+ * device's count of sweeps, as later calls then do, and the handle's own count
+ * (lattice_info, the bounds of lattice_series, which of its two buffers is read
+ * back) counts the captured call once. */
 int lattice_sweep(lattice_t *lat, int64_t n);
 
 /* Per-site observables of the current configuration (waits for the

@@ -365,7 +365,7 @@ void plan_bands(Work &work, std::vector<BandGroup> &groups, size_t at_least)
     Work fit, rest;
     for (auto &pr : work) {
         const lattice *lt = pr.first;
-        const bool ok = pr.second >= kMinSweeps && !lt->graph_pinned && choose_kernel(lt) == LAT_KERNEL_WIDE &&
+        const bool ok = pr.second >= kMinSweeps && !lt->captured && !lt->graph_pinned && choose_kernel(lt) == LAT_KERNEL_WIDE &&
                         band_min_ctas(lt->geom) > 0;
         (ok ? fit : rest).push_back(pr);
     }
@@ -731,6 +731,10 @@ int lattice_batch_run(lattice_batch_t *b)
             const int rc = band_status(pr.first);
             if (rc != LAT_OK) return rc;
         }
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    const bool outside = cudaStreamIsCapturing(b->stream, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone;
+    if (!outside && cs != cudaStreamCaptureStatusNone)
+        for (auto &pr : work) pr.first->captured = true;
     // Counter space for every sweep of the run (queued on each lattice's own
     // stream), then the batch stream waits for the work queued so far on
     // each distinct lattice stream (lattices often share one): an event
@@ -779,9 +783,7 @@ int lattice_batch_run(lattice_batch_t *b)
     // Lattices that fit the chip's shared memory: all their sweeps in a few launches.
     std::vector<BandGroup> groups;
     // (the launches carry the host's sweep numbers: not while the caller captures the stream)
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(b->stream, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone &&
-        band_may(b->stream, &b->band_share))
+    if (outside && band_may(b->stream, &b->band_share))
         plan_bands(work, groups, b->caller_orders ? 2 : 1);
     // the resident and band lattices' uploads sit at the front of the staging
     size_t res_bytes = res.empty() ? 0 : ((res.size() * (sizeof(Geom) + sizeof(long long)) + 64 + 15) & ~(size_t)15);

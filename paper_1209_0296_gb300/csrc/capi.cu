@@ -501,32 +501,35 @@ static int64_t band_min_sweeps(const lattice *lt)
     return lt->P.N * (lt->geom.cpl != nullptr ? 2u : 1u) > 6000000u ? 5 : 3;
 }
 
-// Whether the host's sweep number may go into a launch on st: not while the
-// caller captures the stream.
-static bool not_capturing(cudaStream_t st)
+// Whether the host's sweep number may go into a launch: not while the caller
+// captures the stream, and not once a call was captured, since the caller's
+// replays move the device's count alone.
+static bool host_counts(lattice *lt)
 {
+    if (lt->captured) return false;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) {
+    if (cudaStreamIsCapturing(lt->stream, &cs) != cudaSuccess) {
         (void)cudaGetLastError();
         return false;
     }
-    return cs == cudaStreamCaptureStatusNone;
+    lt->captured = cs != cudaStreamCaptureStatusNone;
+    return !lt->captured;
 }
 
 // CTAs of the band-resident kernel for a call of n sweeps, or 0: lattices on
 // the wide kernel that fit the chip's shared memory, unless the caller chose
-// a graph size (which asks for launches) or is capturing the stream (the
-// launch carries the host's sweep number, so it cannot be replayed).
+// a graph size (which asks for launches) or the host's count may be behind (the
+// launch carries the host's sweep number).
 static int band_bands(lattice *lt, int64_t n)
 {
-    if (n < band_min_sweeps(lt) || lt->graph_pinned || lt->dynamics != LAT_DYNAMICS_CHECKERBOARD) return 0;
+    if (lt->captured || n < band_min_sweeps(lt) || lt->graph_pinned || lt->dynamics != LAT_DYNAMICS_CHECKERBOARD) return 0;
     // (3-state Potts at sizes without a wide kernel too, unless the generic one was asked for)
     if (lt->P.layout == LAT_INT8 && choose_kernel(lt) != LAT_KERNEL_WIDE &&
         !(lt->P.model == LAT_POTTS && lt->kernel != LAT_KERNEL_GENERIC))
         return 0;
     const int bands = band_count_for(lt->geom, lt->has_fields);
     if (bands == 0) return 0;
-    return not_capturing(lt->stream) && band_may(lt->stream, &lt->band_share) ? bands : 0;
+    return band_may(lt->stream, &lt->band_share) ? bands : 0;
 }
 
 // Queue n sweeps on the band-resident kernel (sets *done to the sweeps
@@ -916,6 +919,7 @@ int sweep_impl(lattice *lt, int64_t n)
     if (n < 0) return LAT_EINVAL;
     if (n == 0) return LAT_OK;
     int rc = band_status(lt);
+    const bool counts = host_counts(lt);
     const bool clear = n >= band_min_sweeps(lt) && idle_stream(lt->stream);
     if (rc == LAT_OK) rc = ensure_series(lt, (unsigned long long)(lt->sweeps + n));
     if (rc != LAT_OK) return rc;
@@ -928,7 +932,7 @@ int sweep_impl(lattice *lt, int64_t n)
         n -= lt->sweeps - before;   // sweeps already done (and counted) by the tuner
         if (left == 0) return LAT_OK;
     }
-    if (const int bands = band_bands(lt, left)) {
+    if (const int bands = counts ? band_bands(lt, left) : 0) {
         int64_t done = 0;
         rc = band_sweeps(lt, bands, left, clear, &done);
         lt->sweeps += done;
@@ -950,7 +954,7 @@ int sweep_impl(lattice *lt, int64_t n)
     }
     if (left > 0) {
         lt->sweeps += n - left;   // graph replays queued above
-        rc = enqueue_sweeps(lt, left, lt->stream, not_capturing(lt->stream));
+        rc = enqueue_sweeps(lt, left, lt->stream, counts);
         lt->sweeps -= n - left;
         if (rc != LAT_OK) return rc;
     }

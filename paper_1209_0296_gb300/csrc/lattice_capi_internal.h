@@ -137,6 +137,7 @@ struct lattice {
     unsigned long long *scratch4 = nullptr;
     std::vector<lat::TabEntry> host_tab;
     int64_t sweeps = 0;        // sweeps done (global index of the next sweep)
+    bool captured = false;     // a caller captured sweeps of it: replays move the device's count alone
     int64_t series_first = 0;  // first sweep index recorded in the series buffer
     int64_t unfl_base = 0;     // unflipped sites before that sweep (North-East)
     int kernel = 0, tile_w = 0, tile_h = 0, graph_sweeps = 0;
