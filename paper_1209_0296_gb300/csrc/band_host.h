@@ -3,6 +3,7 @@
 #pragma once
 
 #include <cstddef>
+#include <deque>
 #include <mutex>
 #include <utility>
 #include <vector>
@@ -24,16 +25,7 @@ public:
     {
         std::lock_guard<std::mutex> g(mu_);
         try {
-            for (size_t i = 0; i < pending_.size();) {
-                if (done_(pending_[i].second)) {
-                    int *w = pending_[i].first;
-                    pending_[i] = pending_.back();
-                    pending_.pop_back();
-                    free_.push_back(w);
-                } else {
-                    ++i;
-                }
-            }
+            if (free_.empty()) collect(pending_.size());
             if (free_.empty()) {
                 free_.reserve(words_);
                 int *p = page_(words_);
@@ -49,24 +41,36 @@ public:
         return w;
     }
 
-    // Give w back, free once event is complete (null: at once).
+    // Give w back, free once event is complete (null: at once).  The oldest such
+    // words are looked at here, so that taking one asks nothing.
     void give(int *w, void *event)
     {
         std::lock_guard<std::mutex> g(mu_);
         try {
             if (event == nullptr) free_.push_back(w);
             else pending_.emplace_back(w, event);
+            collect(2);
         } catch (...) {
         }
     }
 
 private:
+    // Free the words of the `most` oldest events that are complete.
+    void collect(size_t most)
+    {
+        while (most-- > 0 && !pending_.empty() && done_(pending_.front().second)) {
+            int *w = pending_.front().first;
+            pending_.pop_front();
+            free_.push_back(w);
+        }
+    }
+
     const Page page_;
     const Done done_;
     const size_t words_;
     std::mutex mu_;
     std::vector<int *> free_;
-    std::vector<std::pair<int *, void *>> pending_;
+    std::deque<std::pair<int *, void *>> pending_;
 };
 
 // A value found once per device (function attributes and SM counts belong to

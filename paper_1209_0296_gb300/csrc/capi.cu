@@ -487,16 +487,17 @@ static int64_t band_min_sweeps(const lattice *lt)
     // chunks divide well and the work is small beside an exchange, the
     // launches' row walk else.  us of 20 sweeps in bands and in launches, h =
     // 0.15: L = 1664 (1.1 chunks a thread) 140 and 127, 2048 (1.75) 136 and 156,
-    // 2400 (2.3) 193 and 185, 2816 (3.3) 248 and 225, 5600 805 and 661; with field
-    // signs, whose launches read a third plane, 1664 157 and 164, 2560 (2.7) 235 and
-    // 255, 3008 (3.7) 313 and 315, 4096 514 and 492.  Rows of any alignment cost the
-    // launches more: L = 2050 168 and 227, 3000 284 and 327, 4402 619 and 661. 5
-    // sweeps: 2048 42.5 and 43, 2400 57 and 50; 2050 56 and 61, 2402 70 and 72,
-    // 3000 88 and 86.
+    // 2400 (2.3) 193 and 185, 2816 (3.3) 248 and 225, 5600 805 and 661.  Rows of any
+    // alignment cost the launches more: L = 2050 168 and 227, 3000 284 and 327, 4402
+    // 619 and 661.  With disorder the launches read a third plane, and no tuner
+    // has made their graph before the first long call, which costs 0.15 ms: field
+    // signs 1664 157 and 164, 2560 235 and 255, 4096 514 and 492 (a first call 535
+    // and 643; without a graph 530).  5 sweeps: 2048 42.5 and 43, 2400 57 and 50;
+    // 2050 56 and 61, 2402 70 and 72, 3000 88 and 86; field signs 4096 142 and 127.
     if (const int load = band_chunk_load(lt->geom, lt->has_fields)) {
         if (lt->P.L % 32 != 0) return load > 370 ? 8 : load >= 150 && load <= 200 ? 4 : 5;
         if (load >= 150 && load <= 200) return 5;
-        return (load < 150 && !lt->has_fields) || load > (lt->has_fields ? 370 : 270) ? INT64_MAX : 12;
+        return lt->geom.cpl == nullptr && (load < 150 || load > 270) ? INT64_MAX : 12;
     }
     return lt->P.N * (lt->geom.cpl != nullptr ? 2u : 1u) > 6000000u ? 5 : 3;
 }
@@ -609,8 +610,9 @@ int enqueue_sweeps(lattice *lt, int64_t k, cudaStream_t st, bool direct = false)
     }
     int kern = choose_kernel(lt);
     // Under AUTO a short call on a small lattice takes the kernel that is
-    // cheaper for it, tuned or not: two launches for one sweep (L = 64: 4.0
-    // us, resident 5.8), one resident launch for more (0.8 us a sweep on top).
+    // cheaper for it, tuned or not: two launches for one sweep (L = 64, calls in
+    // a row: 4.3 us, resident 6.2), one resident launch for more (two sweeps:
+    // 7.6 in launches, 6.2; from there 0.8 us a sweep on top).
     if (direct && lt->kernel == LAT_KERNEL_AUTO && lt->P.L <= 128 && resident_supported(lt->geom) &&
         lt->geom.cpl == nullptr && (kern == LAT_KERNEL_WIDE || kern == LAT_KERNEL_RESIDENT) && sweep_at_known(lt->geom))
         kern = k == 1 ? LAT_KERNEL_WIDE : LAT_KERNEL_RESIDENT;

@@ -1,13 +1,15 @@
 // ising_walk.cuh -- one colour of one thread's column of 16-site chunks for
-// 2D spin-1/2 Ising lattices (uniform, or with the disorder of Eq. 1),
-// shared by the solo and the batched kernels.
+// 2D spin-1/2 Ising lattices (uniform, or with the disorder of Eq. 1): the
+// two-launch kernels of a lone lattice (kernels_wide.cu), and the neighbours and
+// counters of a chunk, which the band-resident forms use too.
 //
 // The thread walks consecutive rows.  The three rows of the other plane
 // that a chunk touches stay in registers and turn over by renaming, so a row
 // costs one new load of each plane; the next row's loads and Philox draws
-// share each instruction block with this row's acceptance.  Acceptance is by
-// the top 16 bits (accept16.cuh); rows with an undecided site are marked and
-// done again exactly, from memory, after the walk (one chunk in 2700).
+// share each instruction block with this row's acceptance.  Acceptance looks
+// every threshold up, or, on long walks of symmetric tables, goes by the top 16
+// bits (accept16.cuh); there rows with an undecided site are marked and done
+// again exactly, from memory, after the walk (one chunk in 2700).
 #pragma once
 
 #include <type_traits>
@@ -320,7 +322,7 @@ LAT_D void ising_walk(const IsingPlanes<kColour> &p, const uint32_t (&acc)[8], c
 }
 
 // Row y's chunk of column k alone (lattices with little more than one chunk
-// a thread).
+// a thread).  Everything it reads is asked for before its draws.
 template <int kColour, bool kRef, int kDis, int kAcc, bool kAligned>
 LAT_D void ising_one(const IsingPlanes<kColour> &p, const uint32_t (&acc)[8], const uint32_t *sthr, unsigned long long sweep, uint32_t key0, uint32_t key1, uint32_t k, uint32_t y, Counts &cnt)
 {

@@ -28,13 +28,15 @@ template <int kKind, bool kRef, int kVar>
 constexpr BandKernel band_kernel()
 {
     constexpr bool kNe = kKind == kBandNe || kKind == kBandNeFull || kKind == kBandPackedNe;
+    // on bits a partial last chunk makes no difference
+    constexpr int kBits = kKind == kBandSym ? kBandSymFull : kKind == kBandNe ? kBandNeFull : kKind;
     if constexpr (kVar == 0) {
         if constexpr (kKind >= kBandPacked) return nullptr;
         else return k_band<kKind, kRef, kBandThreads, 0>;
     } else if constexpr (kVar == 1) {
-        return k_band<kKind, kRef, kBandThreads, 1>;
+        return k_band<kBits, kRef, kBandThreads, 1>;
     } else {
-        if constexpr (kNe) return k_band<kKind, kRef, kBandNeThreads, 1>;
+        if constexpr (kNe) return k_band<kBits, kRef, kBandNeThreads, 1>;
         else return nullptr;
     }
 }

@@ -1,7 +1,7 @@
-// ne_walk.cuh -- the pieces of a c-mode North-East half-sweep shared by the
-// streaming kernels (kernels_ne.cu) and the band-resident ones
-// (kernels_band.cu): the constraint and the certain moves of a 16-site
-// chunk, the queued draws, counters.
+// ne_walk.cuh -- the pieces of a c-mode North-East half-sweep: the constraint
+// and the certain moves of a 16-site chunk and its counters, which the streaming
+// kernels (kernels_ne.cu) and the band-resident ones (band.cuh) share, and the
+// streaming kernels' queued draws.
 #pragma once
 
 #include "accept16.cuh"
