@@ -367,6 +367,7 @@ namespace {
 struct BandLast {
     cudaEvent_t ev = nullptr;        // recorded after it
     unsigned long long stream = 0;   // cudaStreamGetId: a handle may be used again, an id is not
+    bool launching = false;          // a thread is queueing one now: ev, stream, clear and depth are its alone
     bool clear = false;
     int depth = 0;                   // band launches of other streams it waits for
     uint64_t sites = 0;
@@ -415,7 +416,7 @@ bool band_may(cudaStream_t st, BandShare *me)
     unsigned long long id = 0;
     if (!band_place(st, dev, id)) return false;
     const BandLast &l = g_band_last[dev];
-    if (in_flight(l, id)) {
+    if (l.launching || in_flight(l, id)) {
         me->yield = kBandYield;
         if (l.owner != nullptr) l.owner->yield = kBandYield;
     }
@@ -432,41 +433,44 @@ void band_forget(BandShare *me)
 BandTurn::BandTurn(cudaStream_t st, BandShare *me, uint64_t sites, bool clear)
     : st_(st), me_(me), clear_(clear), sites_(sites)
 {
-    g_band_mu.lock();
-    if (!band_place(st, dev_, id_)) {
-        dev_ = -1;
-        return;
-    }
-    BandLast &l = g_band_last[dev_];
-    go = true;
-    if (in_flight(l, id_)) {
-        const uint64_t least = std::min(sites, l.sites);
-        if (l.clear && (least >= kBandLarge || (least >= kBandTwo && l.depth == 0))) {
-            status = cudaStreamWaitEvent(st, l.ev, 0);
+    if (!band_place(st, dev_, id_)) return;
+    bool wait = false;
+    {
+        std::lock_guard<std::mutex> g(g_band_mu);
+        BandLast &l = g_band_last[dev_];
+        go = true;
+        if (l.launching || in_flight(l, id_)) {
+            const uint64_t least = std::min(sites, l.sites);
+            wait = !l.launching && l.clear && (least >= kBandLarge || (least >= kBandTwo && l.depth == 0));
             depth_ = l.depth + 1;
-        } else {
-            go = false;
-            if (least < kBandLarge) {
-                me->yield = kBandYield;
-                if (l.owner != nullptr) l.owner->yield = kBandYield;
+            if (!wait) {
+                go = false;
+                if (least < kBandLarge) {
+                    me->yield = kBandYield;
+                    if (l.owner != nullptr) l.owner->yield = kBandYield;
+                }
+                return;
             }
         }
+        l.launching = true;   // the record is this turn's until its end
+        l.owner = me;
+        l.sites = sites;
     }
-    if (go && status == cudaSuccess && l.ev == nullptr) status = cudaEventCreateWithFlags(&l.ev, cudaEventDisableTiming);
+    BandLast &l = g_band_last[dev_];
+    if (wait) status = cudaStreamWaitEvent(st, l.ev, 0);
+    else if (l.ev == nullptr) status = cudaEventCreateWithFlags(&l.ev, cudaEventDisableTiming);
 }
 
 BandTurn::~BandTurn()
 {
-    if (go && status == cudaSuccess) {
-        BandLast &l = g_band_last[dev_];
-        cudaEventRecord(l.ev, st_);
-        l.stream = id_;
-        l.clear = clear_;
-        l.depth = depth_;
-        l.sites = sites_;
-        l.owner = me_;
-    }
-    g_band_mu.unlock();
+    if (!go) return;
+    BandLast &l = g_band_last[dev_];
+    if (l.ev != nullptr) cudaEventRecord(l.ev, st_);
+    std::lock_guard<std::mutex> g(g_band_mu);
+    l.launching = false;
+    l.stream = id_;
+    l.clear = clear_;
+    l.depth = depth_;
 }
 
 // The band-resident kernel takes calls of at least this many sweeps: its

@@ -58,7 +58,7 @@ int band_status(const struct ::lattice *lt);
 // bands alone for their next kBandYield calls: small lattices on streams of
 // their own overlap their launches.  Launches side by side and bands in turn,
 // ms: 16 x L = 256, 100 sweeps 1.0 and 3.7; 2 x L = 512 0.42 and 0.47; 2, 4, 8 x
-// L = 1000 0.76 and 0.52, 0.97 and 1.02, 1.45 and 2.02; 4 x L = 2048, 20 sweeps
+// L = 1000 0.76 and 0.52, 0.98 and 1.02, 1.70 and 2.02; 4 x L = 2048, 20 sweeps
 // 0.49 and 0.43.
 struct BandShare {
     int yield = 0;   // calls that still do without bands
@@ -74,7 +74,9 @@ bool idle_stream(cudaStream_t st);
 // Before *me is freed.
 void band_forget(BandShare *me);
 
-// Held while one band launch is queued on st.
+// Lives while one band launch is queued on st.  No lock is held meanwhile (a
+// launch waits on the host when the stream's queue is full): other threads'
+// band launches are refused until it is.
 class BandTurn {
 public:
     // clear: the launch waits for no other work than this call's and bands like it.
@@ -86,7 +88,7 @@ public:
 private:
     cudaStream_t st_;
     BandShare *me_;
-    int dev_ = -1;
+    int dev_ = 0;
     unsigned long long id_ = 0;
     bool clear_;
     int depth_ = 0;

@@ -105,3 +105,41 @@ def test_batches_on_two_streams():
             _check(g, o, 20)
     for b in bs:
         b.close()
+
+
+# threads with a lattice and a stream each: whoever meets whom, the sweeps are the same
+def test_threads():
+    import threading
+
+    sizes = [300, 512, 1000, 1632, 1632, 300]
+    make = lambda i, s: lt.Lattice(2, sizes[i], 1, lt.ISING, 1.0, 0.0, 2.2, seed=80 + i, init=lt.INIT_RANDOM, stream=s)
+    lats = [make(i, torch.cuda.Stream()) for i in range(len(sizes))]
+    for g in lats:
+        g.set_kernel(lt.KERNEL_WIDE)
+    failed = []
+
+    def work(g):
+        try:
+            for k in range(60):
+                g.sweep(5 + k % 7)
+                if k % 5 == 0:
+                    g.synchronize()
+            g.synchronize()
+        except Exception as e:
+            failed.append(e)
+
+    threads = [threading.Thread(target=work, args=(g,)) for g in lats]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed
+    n = sum(5 + k % 7 for k in range(60))
+    for i, g in enumerate(lats):
+        f = make(i, None)
+        f.set_kernel(lt.KERNEL_WIDE, 0, 0, 8)    # launches
+        f.sweep(n)
+        assert np.array_equal(f.get_spins(), g.get_spins())
+        assert np.array_equal(f.series(0, n)["bond"], g.series(0, n)["bond"])
+        f.close()
+        g.close()
